@@ -6,12 +6,12 @@ namespace cass {
 
 // Workspace carve-up (all offsets 256-byte aligned).
 struct EncWs {
-    uint32_t* keepbm;        // [n_pad][k_pad/32]
-    uint32_t* cnt_fw;        // [n_pad][n_seg]  field words of the row in that segment
-    uint32_t* ubits;         // [n_pad][n_seg]  code bits of the row in that segment
-    unsigned long long* hist;   // [256]
-    uint8_t* exp_to_rank;    // [256]
+    uint32_t* keepbm;        // [n][k_pad/32]
+    uint2* sb_size;          // [n_rb * n_seg]  of each superblock's rows: most kept values, most code words
+    unsigned long long* hist;   // [256] exponents of the kept values; zeroed by the caller, as is abort_flag behind it
     uint32_t* abort_flag;    // [1]
+    uint8_t* exp_to_rank;    // [256]
+    size_t zero_bytes;       // hist and abort_flag
     size_t bytes;
 };
 
@@ -19,12 +19,12 @@ static EncWs carve(void* base, int n_pad, int k_pad, int n_seg) {
     EncWs w;
     size_t off = 0;
     auto take = [&](size_t b) { size_t o = off; off = align_up(off + b, 256); return (char*)base + o; };
-    w.keepbm = (uint32_t*)take((size_t)n_pad * (k_pad / 32) * 4);
-    w.cnt_fw = (uint32_t*)take((size_t)n_pad * n_seg * 4);
-    w.ubits = (uint32_t*)take((size_t)n_pad * n_seg * 4);
     w.hist = (unsigned long long*)take(256 * 8);
-    w.exp_to_rank = (uint8_t*)take(256);
     w.abort_flag = (uint32_t*)take(256);
+    w.zero_bytes = off;
+    w.exp_to_rank = (uint8_t*)take(256);
+    w.keepbm = (uint32_t*)take((size_t)n_pad * (k_pad / 32) * 4);
+    w.sb_size = (uint2*)take((size_t)(n_pad / kRowsPerBlock) * n_seg * 8);
     w.bytes = off;
     return w;
 }
@@ -56,58 +56,214 @@ static int make_geom(const cass_format* fmt, int rows, int cols, EncGeom* g) {
     return CASS_OK;
 }
 
-// ---- E1: per-row selection of the kept set -------------------------------------------------------------
-// One block per row.  Score bits (non-negative fp32, so the integer order is the float order) are staged in
-// shared memory; the composite key (score << 20 | column) is unique, so "prune the n_prune smallest keys"
-// is the rule "lowest score first, lower column first among equals".  The threshold key is found by a
-// bitwise binary search on the count of smaller keys.
-__global__ void __launch_bounds__(256) k_select(const uint16_t* __restrict__ W, const float* __restrict__ act, EncGeom g,
-                                                uint32_t* __restrict__ keepbm, unsigned long long* __restrict__ hist) {
-    extern __shared__ uint32_t s_score[];            // [k]
-    __shared__ unsigned int s_hist[256];
-    __shared__ int s_part[8];
-    const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint16_t* wr = W + (size_t)row * g.k;
-    s_hist[tid] = 0;
-    for (int c = tid; c < g.k; c += 256) {
-        float mag = bf16_bits_to_float(wr[c] & 0x7FFFu);
-        float a = act ? act[c] : 1.0f;
-        s_score[c] = __float_as_uint(__fmul_rn(mag, a));
+// Eight columns a lane: byte `lane` of 8 bitmap words that lanes j0 .. j0 + 7 hold, and the row's 8 values from p on (two a
+// word), of which those without a bit may be anything.
+__device__ __forceinline__ uint32_t row_byte(uint32_t bm_lane, int j0, int lane) {
+    return (__shfl_sync(0xffffffffu, bm_lane, j0 + (lane >> 2)) >> (24 - 8 * (lane & 3))) & 0xFFu;
+}
+__device__ __forceinline__ void row_load8(const uint16_t* __restrict__ p, uint32_t byte, bool vec, uint32_t (&v)[4]) {
+    v[0] = v[1] = v[2] = v[3] = 0;
+    if (vec) {                                                             // rows of whole 16-byte groups: one load
+        if (byte) {
+            const uint4 q = __ldg(reinterpret_cast<const uint4*>(p));
+            v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        }
+        return;
     }
-    __syncthreads();
-    unsigned long long thr = 0;                      // smallest kept key
-    if (g.n_prune > 0) {
-        for (int bit = 51; bit >= 0; --bit) {
-            unsigned long long cand = thr | (1ull << bit);
-            int c_lt = 0;
-            for (int c = tid; c < g.k; c += 256) {
-                unsigned long long key = ((unsigned long long)s_score[c] << 20) | (unsigned)c;
-                c_lt += key < cand;
-            }
-            c_lt = __reduce_add_sync(0xffffffffu, c_lt);
-            if (lane == 0) s_part[warp] = c_lt;
-            __syncthreads();
-            int tot = 0;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) tot += s_part[i];
-            if (tot <= g.n_prune) thr = cand;
-            __syncthreads();
-        }
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t lo = byte & (0x80u >> (2 * i)) ? __ldg(p + 2 * i) : 0u, hi = byte & (0x40u >> (2 * i)) ? __ldg(p + 2 * i + 1) : 0u;
+        v[i] = lo | (hi << 16);
     }
-    const int words = g.k_pad / 32;
-    for (int j = warp; j < words; j += 8) {
-        int c = j * 32 + lane;
-        bool keep = false;
-        if (c < g.k) {
-            unsigned long long key = ((unsigned long long)s_score[c] << 20) | (unsigned)c;
-            keep = key >= thr;
-            if (keep) atomicAdd(&s_hist[(wr[c] >> 7) & 0xFF], 1u);
+}
+
+// ---- E1: per-row selection of the kept set -------------------------------------------------------------
+// Keys (score bits, column) are unique and scores are non-negative floats, whose integer order is the float order, so
+// "prune the n_prune smallest keys" is the rule "lowest score first, lower column first among equals".  The smallest
+// kept key is found in two steps: the top 16 bits of its score by a bitwise search that counts smaller ones two at a time
+// (packed bf16 compare and add: the scores' upper halves order as bf16 numbers), then the handful of keys that share
+// those bits are ranked against each other.
+// A row is read once, 8 columns a lane, and its scores' upper halves stay in registers, NV values a lane; the few values
+// of which more is needed are read again.  Up to 4096 columns one warp holds a row and no barrier is needed; WPR warps
+// hold a longer one.
+// Bound: the integer pipe, which starts a warp instruction every other cycle (packed compare and add: 1.4 cycles a value
+// and round); loads have to be issued well ahead of their use, hence the clamped, unconditional ones.
+constexpr int kSelList = 512;
+constexpr int sel_threads(int wpr) { return wpr < 4 ? 128 : 32 * wpr; }
+
+__device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t v) {
+    __nv_bfloat162 r;
+    *reinterpret_cast<uint32_t*>(&r) = v;
+    return r;
+}
+
+template <int NV, int WPR>
+__global__ void __launch_bounds__(sel_threads(WPR), 512 / sel_threads(WPR)) k_select(const uint16_t* __restrict__ W,
+                                                                                     const float* __restrict__ act, EncGeom g,
+                                                                                     uint32_t* __restrict__ keepbm,
+                                                                                     unsigned long long* __restrict__ hist) {
+    constexpr int NT = sel_threads(WPR), ROWS = NT / (32 * WPR), NG = NV / 8, HW = NV >= 32 ? NV / 32 : 1;
+    __shared__ unsigned int s_exp[256];
+    __shared__ unsigned long long s_list[ROWS][kSelList], s_thr[ROWS];
+    __shared__ uint32_t s_cnt[2][ROWS][WPR], s_m[ROWS];
+    const int tid = threadIdx.x, lane = tid & 31, warp = (tid >> 5) % WPR, slot = tid / (32 * WPR);
+    // the warps of a row meet at a barrier of their own: another row of the CTA may be elsewhere, or done
+    auto row_sync = [&]() {
+        if (WPR == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(32 * WPR) : "memory");
+    };
+    int turn = 0;
+    auto row_sum = [&](uint32_t v) {                                     // sum over the row's lanes; two buffers in turn, one barrier
+        v = __reduce_add_sync(0xffffffffu, v);
+        if (WPR == 1) return v;
+        turn ^= 1;
+        if (lane == 0) s_cnt[turn][slot][warp] = v;
+        row_sync();
+        return __reduce_add_sync(0xffffffffu, lane < WPR ? s_cnt[turn][slot][lane] : 0u);
+    };
+    for (int i = tid; i < 256; i += NT) s_exp[i] = 0;
+    pdl_wait();
+    __syncthreads();
+    const int step = (int)gridDim.x * ROWS, row_bytes = g.k_pad / 8;
+    const bool vec = g.k % 8 == 0 && (((uintptr_t)W | (uintptr_t)act) & 15) == 0;
+    const int k_last = vec ? g.k - 8 : 0;
+    for (int row = (int)blockIdx.x * ROWS + slot; row < g.n; row += step) {     // the same row for all of its warps
+        const uint16_t* wr = W + (size_t)row * g.k;
+        auto score_of = [&](int c) { return __float_as_uint(__fmul_rn(bf16_bits_to_float(wr[c] & 0x7FFFu), act ? __ldg(act + c) : 1.0f)); };
+        auto col_of = [&](int i) { return ((warp + (i / 8) * WPR) * 32 + lane) * 8 + (i & 7); };       // column of the lane's value i
+        uint32_t x[NV / 2];                                              // upper halves of scores 2 i (low) and 2 i + 1
+        int later = 0;
+#pragma unroll
+        for (int q = 0; q < NG; ++q) {
+            // four groups' loads at a time: all of them at once would not fit the registers
+            if (q > 0 && q % 4 == 0) asm volatile("" : "+r"(later) : "r"(x[q * 4 - 1]), "r"(x[q * 4 - 5]), "r"(x[q * 4 - 9]), "r"(x[q * 4 - 13]));
+            const int c = col_of(q * 8) + later;
+            uint32_t w[4];
+            float a[8];
+            if (vec) {
+                const int cc = min(c, k_last);
+                const uint4 wv = __ldg(reinterpret_cast<const uint4*>(wr + cc));
+                w[0] = wv.x; w[1] = wv.y; w[2] = wv.z; w[3] = wv.w;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[i] = 1.0f;
+                if (act) {
+                    const float4 lo = __ldg(reinterpret_cast<const float4*>(act + cc)), hi = __ldg(reinterpret_cast<const float4*>(act + cc + 4));
+                    a[0] = lo.x; a[1] = lo.y; a[2] = lo.z; a[3] = lo.w; a[4] = hi.x; a[5] = hi.y; a[6] = hi.z; a[7] = hi.w;
+                }
+            } else {
+                uint32_t h[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int ci = min(c + i, g.k - 1);
+                    h[i] = __ldg(wr + ci);
+                    a[i] = act ? __ldg(act + ci) : 1.0f;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) w[i] = h[2 * i] | (h[2 * i + 1] << 16);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t lo = __float_as_uint(__fmul_rn(__uint_as_float((w[i] << 16) & 0x7FFF0000u), a[2 * i]));
+                const uint32_t hi = __float_as_uint(__fmul_rn(__uint_as_float(w[i] & 0x7FFF0000u), a[2 * i + 1]));
+                uint32_t v = __byte_perm(lo, hi, 0x7632);
+                if (c + 2 * i >= g.k) v |= 0x7FFFu;                      // beyond the row: a NaN, which is neither below nor above anything
+                if (c + 2 * i + 1 >= g.k) v |= 0x7FFF0000u;
+                x[q * 4 + i] = v;
+            }
         }
-        uint32_t b = __brev(__ballot_sync(0xffffffffu, keep));     // column c at bit 31 - c%32
-        if (lane == 0) keepbm[(size_t)row * words + j] = b;
+        uint32_t top = 0, below = 0;                                     // upper half of the smallest kept score; scores below it
+        uint32_t hit[HW] = {};                                           // which of the lane's values share it
+        unsigned long long thr = 0;                                      // smallest kept key
+        if (g.n_prune > 0) {
+            if (lane == 0 && warp == 0) s_m[slot] = 0;
+#pragma unroll 1
+            for (int bit = 14; bit >= 0; --bit) {
+                const uint32_t cand = top | (1u << bit);
+                // below the normal numbers the packed compare may flush: those scores are one bin; beyond infinity there is none
+                if (cand < 0x0080u || cand > 0x7F80u) continue;
+                const __nv_bfloat162 c2 = as_bf162(cand | (cand << 16));
+                __nv_bfloat162 n[2] = {as_bf162(0), as_bf162(0)};
+#pragma unroll
+                for (int i = 0; i < NV / 2; ++i) n[i & 1] = __hadd2(n[i & 1], __hlt2(as_bf162(x[i]), c2));     // at most 32 in a counter: exact
+                const __nv_bfloat162 sum = __hadd2(n[0], n[1]);
+                const uint32_t cnt = row_sum((uint32_t)(int)(__low2float(sum) + __high2float(sum)));
+                if (cnt <= (uint32_t)g.n_prune) { top = cand; below = cnt; }
+            }
+            const uint32_t top2 = top | (top << 16), sel = top ? 0xFFFFFFFFu : 0xFF80FF80u;
+#pragma unroll
+            for (int i = 0; i < NV / 2; ++i) {
+                const uint32_t d = (x[i] ^ top2) & sel;
+                if ((d & 0xFFFFu) == 0) hit[i / 16] |= 1u << (2 * i & 31);
+                if (d < 0x10000u) hit[i / 16] |= 2u << (2 * i & 31);
+            }
+            row_sync();                                                  // s_m is zero
+#pragma unroll
+            for (int h = 0; h < HW; ++h)
+                for (uint32_t b = hit[h]; b; b &= b - 1) {
+                    const int c = col_of(h * 32 + __ffs(b) - 1);
+                    const uint32_t at = atomicAdd(&s_m[slot], 1u);
+                    if (at < (uint32_t)kSelList) s_list[slot][at] = ((unsigned long long)score_of(c) << 20) | (unsigned)c;
+                }
+            const uint32_t want = (uint32_t)g.n_prune - below;           // rank of the smallest kept key among them
+            row_sync();                                                  // the list is complete
+            const int m = (int)s_m[slot];
+            if (m <= kSelList) {
+                for (int i = warp * 32 + lane; i < m; i += 32 * WPR) {
+                    const unsigned long long mine = s_list[slot][i];
+                    uint32_t less = 0;
+                    for (int j = 0; j < m; ++j) less += s_list[slot][j] < mine;
+                    if (less == want) s_thr[slot] = mine;
+                }
+                row_sync();
+                thr = s_thr[slot];
+            } else {
+                // many equal scores (a constant row): bit by bit over the keys that share the upper half
+                for (int bit = 51; bit >= 0; --bit) {
+                    const unsigned long long cand = thr | (1ull << bit);
+                    uint32_t less = 0;
+#pragma unroll
+                    for (int h = 0; h < HW; ++h)
+                        for (uint32_t b = hit[h]; b; b &= b - 1) {
+                            const int c = col_of(h * 32 + __ffs(b) - 1);
+                            less += (((unsigned long long)score_of(c) << 20) | (unsigned)c) < cand;
+                        }
+                    if (row_sum(less) <= want) thr = cand;
+                }
+            }
+            row_sync();                                                  // the list and s_thr are free again
+        }
+        // kept: the values above the shared upper half, and those of the list from the threshold on
+        const __nv_bfloat162 t2 = as_bf162(top ? top | (top << 16) : 0x007F007Fu);
+        uint8_t* keep_row = reinterpret_cast<uint8_t*>(keepbm) + (size_t)row * row_bytes;
+#pragma unroll
+        for (int q = 0; q < NG; ++q) {
+            const int c = col_of(q * 8);
+            uint32_t kb = 0;                                             // column c + i at bit 7 - i
+            if (g.n_prune > 0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) kb |= __hgt2_mask(as_bf162(x[q * 4 + i]), t2) & (0x00400080u >> (2 * i));
+                kb = (kb | (kb >> 16)) & 0xFFu;
+                for (uint32_t b = (hit[q / 4] >> (8 * (q & 3))) & 0xFFu; b; b &= b - 1) {
+                    const int i = __ffs(b) - 1;
+                    if ((((unsigned long long)score_of(c + i) << 20) | (unsigned)(c + i)) >= thr) kb |= 0x80u >> i;
+                }
+            } else {
+                kb = c + 8 <= g.k ? 0xFFu : c < g.k ? (0xFF00u >> (g.k - c)) & 0xFFu : 0u;
+            }
+            // byte of column c in its word: the first column at the most significant end
+            if (c / 8 < row_bytes) keep_row[(c / 8) ^ 3] = (uint8_t)kb;
+            if (!g.mx) {
+                uint32_t v[4];
+                row_load8(wr + c, kb, vec, v);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (kb & (0x80u >> i)) atomicAdd(&s_exp[((i & 1) ? v[i / 2] >> 23 : v[i / 2] >> 7) & 0xFF], 1u);
+            }
+        }
     }
     __syncthreads();
-    if (s_hist[tid]) atomicAdd(&hist[tid], (unsigned long long)s_hist[tid]);
+    for (int e = tid; e < 256; e += NT)
+        if (s_exp[e]) atomicAdd(&hist[e], (unsigned long long)s_exp[e]);
 }
 
 // ---- E3: codebook: rank exponents by (count desc, exponent asc) -----------------------------------------
@@ -115,223 +271,344 @@ __global__ void k_codebook(const unsigned long long* __restrict__ hist, uint8_t*
                            uint8_t* __restrict__ exp_to_rank) {
     __shared__ unsigned long long s[256];
     int e = threadIdx.x;
+    pdl_wait();
     s[e] = hist[e];
     __syncthreads();
     unsigned long long mine = s[e];
     int rank = 0;
+#pragma unroll 16
     for (int o = 0; o < 256; ++o) rank += (s[o] > mine) || (s[o] == mine && o < e);
     rank_to_exp[rank] = (uint8_t)e;
     exp_to_rank[e] = (uint8_t)rank;
 }
 
-// ---- E4: per (row, segment) sizes: kept values and code bits ------------------------------------------------
-__global__ void k_sizes(const uint16_t* __restrict__ W, EncGeom g, const uint32_t* __restrict__ keepbm,
-                        const uint8_t* __restrict__ exp_to_rank, uint32_t* __restrict__ cnt_kept,
-                        uint32_t* __restrict__ ubits) {
-    int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (gw >= g.n_pad * g.n_seg) return;
-    int row = gw / g.n_seg, seg = gw % g.n_seg;
-    uint32_t kept_n = 0, ub = 0;
+// ---- E4: superblock sizes: the most kept values and code words among its 32 rows (one CTA a superblock, a warp a row) ----
+__global__ void __launch_bounds__(1024) k_sizes(const uint16_t* __restrict__ W, EncGeom g, const uint32_t* __restrict__ keepbm,
+                                                const uint8_t* __restrict__ exp_to_rank, uint2* __restrict__ sb_size) {
+    __shared__ uint32_t s_len[512], s_kept[kRowsPerBlock], s_words[kRowsPerBlock];
+    const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+    const int rb = blockIdx.x / g.n_seg, seg = blockIdx.x % g.n_seg, row = rb * kRowsPerBlock + r;
+    pdl_wait();
+    if (!g.mx && threadIdx.x < 512) s_len[threadIdx.x] = exp_to_rank[threadIdx.x & 255] + 1u;     // by sign and exponent
+    __syncthreads();
+    uint32_t kept = 0, bits = 0;
     if (row < g.n) {
-        const int words = g.k_pad / 32;
-        int scols = seg_cols_of(g.k_pad, g.seg_cols, seg);
-        int w0 = seg * (g.seg_cols / 32), nw = scols / 32;
-        for (int j = 0; j < nw; ++j) {
-            uint32_t bm = keepbm[(size_t)row * words + w0 + j];
-            bool kept = (bm >> (31 - lane)) & 1u;
-            uint32_t len = 0;
-            if (kept) len = exp_to_rank[(W[(size_t)row * g.k + (w0 + j) * 32 + lane] >> 7) & 0xFF] + 1u;
-            ub += __reduce_add_sync(0xffffffffu, len);
-            kept_n += __popc(bm);
+        const int w0 = seg * (g.seg_cols / 32), nw = seg_cols_of(g.k_pad, g.seg_cols, seg) / 32;       // at most 64 words
+        const uint32_t* bmr = keepbm + (size_t)row * (g.k_pad / 32) + w0;
+        const uint32_t bm0 = lane < nw ? bmr[lane] : 0u, bm1 = lane + 32 < nw ? bmr[lane + 32] : 0u;
+        kept = __reduce_add_sync(0xffffffffu, __popc(bm0) + __popc(bm1));
+        if (!g.mx) {
+            const uint16_t* wr = W + (size_t)row * g.k + w0 * 32;
+            const bool vec = g.k % 8 == 0 && ((uintptr_t)W & 15) == 0;
+            for (int j0 = 0; j0 < nw; j0 += 8) {                         // 256 columns, 8 a lane
+                const uint32_t byte = row_byte(j0 < 32 ? bm0 : bm1, j0 & 31, lane);
+                uint32_t v[4];
+                row_load8(wr + (j0 * 32 + lane * 8), byte, vec, v);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (byte & (0x80u >> i)) bits += s_len[(i & 1) ? v[i / 2] >> 23 : (v[i / 2] >> 7) & 0x1FFu];
+            }
+            bits = __reduce_add_sync(0xffffffffu, bits);
+        } else {
+            bits = 8u * ((kept + kMxBlock - 1) / kMxBlock);              // one exponent byte per block of 32 kept values
         }
     }
-    if (g.mx) ub = 8u * ((kept_n + kMxBlock - 1) / kMxBlock);        // one exponent byte per block of 32 kept values
-    if (lane == 0) { cnt_kept[gw] = kept_n; ubits[gw] = ub; }
+    if (lane == 0) { s_kept[r] = kept; s_words[r] = (bits + 31u) / 32u; }
+    __syncthreads();
+    if (r == 0) {
+        const uint32_t mk = __reduce_max_sync(0xffffffffu, s_kept[lane]), mw = __reduce_max_sync(0xffffffffu, s_words[lane]);
+        if (lane == 0) sb_size[blockIdx.x] = make_uint2(mk, mw);
+    }
 }
 
 // ---- E5: directory (exclusive scan of superblock sizes) and header -------------------------------------
-__global__ void __launch_bounds__(1024) k_directory(EncGeom g, const uint32_t* __restrict__ cnt_fw,
-                                                    const uint32_t* __restrict__ ubits, uint32_t* __restrict__ blob,
+__global__ void __launch_bounds__(1024) k_directory(EncGeom g, const uint2* __restrict__ sb_size, uint32_t* __restrict__ blob,
                                                     unsigned long long blob_cap, uint32_t* abort_flag, int32_t* d_status) {
-    __shared__ unsigned long long s_scan[1024];
-    __shared__ unsigned long long s_carry;
+    __shared__ unsigned long long s_sum[32];
     __shared__ unsigned int s_maxsb;
-    const int tid = threadIdx.x, n_sb = g.n_rb * g.n_seg;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_sb = g.n_rb * g.n_seg;
     const unsigned long long body_off = align_up((size_t)kBlobDirOffset + 16ull * n_sb, 128);
-    if (tid == 0) { s_carry = body_off; s_maxsb = 0; }
+    if (tid == 0) s_maxsb = 0;
+    pdl_wait();
     __syncthreads();
     uint32_t* dir = blob + kBlobDirOffset / 4;
+    unsigned long long carry = body_off;
+    unsigned int max_bytes = 0;
     for (int base = 0; base < n_sb; base += 1024) {
-        int sb = base + tid;
+        const int sb = base + tid;
         unsigned long long bytes = 0;
         uint32_t wf = 0, wu = 0, max_kept = 0;
         int n_ch = 0;
         if (sb < n_sb) {
-            int rb = sb / g.n_seg, seg = sb % g.n_seg;
             const uint32_t per = 32u / (8u - (uint32_t)g.t);
-            for (int r = 0; r < kRowsPerBlock; ++r) {
-                int row = rb * kRowsPerBlock + r;
-                max_kept = max(max_kept, cnt_fw[row * g.n_seg + seg]);
-                wu = max(wu, (ubits[row * g.n_seg + seg] + 31u) / 32u);
-            }
+            const uint2 mx = sb_size[sb];
+            max_kept = mx.x;
+            wu = mx.y;
             wf = (max_kept + per - 1) / per;
-            int scols = seg_cols_of(g.k_pad, g.seg_cols, seg);
+            const int scols = seg_cols_of(g.k_pad, g.seg_cols, sb % g.n_seg);
             n_ch = ceil_div(scols, g.chunk_cols);
             bytes = (unsigned long long)SbGeom::make(n_ch, scols, (int)wf, (int)wu).total * 4ull;
-            atomicMax(&s_maxsb, (unsigned int)bytes);
+            max_bytes = max(max_bytes, (unsigned int)bytes);
         }
-        s_scan[tid] = bytes;
+        unsigned long long incl = bytes;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) s_sum[warp] = incl;
         __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {          // inclusive Hillis-Steele scan
-            unsigned long long v = tid >= o ? s_scan[tid - o] : 0;
-            __syncthreads();
-            s_scan[tid] += v;
-            __syncthreads();
+        unsigned long long below = lane < warp ? s_sum[lane] : 0ull, all = s_sum[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            below += __shfl_xor_sync(0xffffffffu, below, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
         }
-        unsigned long long excl = s_scan[tid] - bytes + s_carry;
         if (sb < n_sb) {
-            dir[sb * 4 + 0] = (uint32_t)(excl / 16);
-            dir[sb * 4 + 1] = wf;
-            dir[sb * 4 + 2] = wu;
             const int e_chunk = g.mx ? mx_chunk_elems_for((int)max_kept, n_ch) : chunk_elems_for((int)max_kept, n_ch);
-            dir[sb * 4 + 3] = (uint32_t)n_ch | ((uint32_t)e_chunk << 8);
+            reinterpret_cast<uint4*>(dir)[sb] = make_uint4((uint32_t)((carry + below + incl - bytes) / 16), wf, wu,
+                                                           (uint32_t)n_ch | ((uint32_t)e_chunk << 8));
         }
-        __syncthreads();
-        if (tid == 1023) s_carry += s_scan[1023];
+        carry += all;
         __syncthreads();
     }
+    atomicMax(&s_maxsb, max_bytes);
+    __syncthreads();
+    if (tid < kBlobHeaderBytes / 4) blob[tid] = 0;
+    // the padding between directory and first body
+    for (unsigned long long o = kBlobDirOffset + 16ull * n_sb + 4ull * tid; o < body_off; o += 4096) blob[o / 4] = 0;
+    __syncthreads();
     if (tid == 0) {
-        unsigned long long total = s_carry;
         uint32_t* h = blob;
-        for (int i = 0; i < kBlobHeaderBytes / 4; ++i) h[i] = 0;
         h[H_MAGIC] = kBlobMagic; h[H_VERSION] = kBlobVersion; h[H_ROWS] = g.n; h[H_COLS] = g.k; h[H_P] = g.p; h[H_T] = g.t;
         h[H_SEG] = g.seg_cols; h[H_CHUNK] = g.chunk_cols; h[H_NSEG] = g.n_seg; h[H_NRB] = g.n_rb;
         h[H_KEPT] = g.k - g.n_prune; h[H_DIROFF] = kBlobDirOffset; h[H_BODYOFF] = (uint32_t)body_off;
-        h[H_TOTLO] = (uint32_t)total; h[H_TOTHI] = (uint32_t)(total >> 32); h[H_MAXSB] = s_maxsb;
+        h[H_TOTLO] = (uint32_t)carry; h[H_TOTHI] = (uint32_t)(carry >> 32); h[H_MAXSB] = s_maxsb;
         h[H_MODE] = g.mx ? kBlobModeMx : kBlobModeUnary;
-        // zero the padding between directory and first body
-        for (unsigned long long o = kBlobDirOffset + 16ull * n_sb; o < body_off; o += 4) blob[o / 4] = 0;
-        if (total > blob_cap) {
+        if (carry > blob_cap) {
             *abort_flag = 1;
             if (d_status) *d_status = CASS_ERR_CAPACITY;
         }
     }
 }
 
-// ---- E6: pack one superblock (32 warps = 32 rows) -------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_pack(const uint16_t* __restrict__ W, EncGeom g,
-                                               const uint32_t* __restrict__ keepbm,
-                                               const uint8_t* __restrict__ exp_to_rank, uint32_t* __restrict__ blob,
-                                               const uint32_t* __restrict__ abort_flag) {
+// ---- E6: pack one superblock (a CTA of 16 warps, two of the 32 rows a warp) -------------------------------------------
+// A warp takes 256 columns of its row at a time, 8 a lane, and compacts the kept values into a ring in shared memory;
+// whenever 256 are there it packs them, 8 consecutive ones a lane: a lane forms whole field words (t = 4: one; t = 0:
+// two), and its code bits in one word of its own that is then shifted to where a warp scan of the lengths puts it, so
+// that a lane needs two atomics for 8 codewords.
+// The body is built in shared memory, its 32-word lines one word apart (a row's words would share a bank otherwise), and
+// leaves as contiguous stores; one that does not fit (code words of 5 bits a value and more at p = 0) is built in place.
+// Cassandra-2 (MX): four lanes hold a block of 32 values, whose largest exponent is their shared one.
+// T: truncated bits, or -1: any (from the geometry).
+// Bound: instruction issue.  Two atomics a kept value on global memory, as before, took 0.6 ms of a 4096 x 14336 matrix.
+constexpr int kPackRing = 512;
+constexpr int kPackThreads = 512;                                          // two CTAs an SM: one's stores overlap the other's packing
+constexpr int kPackRingBytes = kPackThreads / 32 * kPackRing * 2;
+constexpr int kPackBodyBytes = 92 * 1024;
+constexpr int kPackSmem = kPackRingBytes + kPackBodyBytes;
+
+template <bool MX, int T>
+__global__ void __launch_bounds__(kPackThreads, 2) k_pack(const uint16_t* __restrict__ W, EncGeom g, const uint32_t* __restrict__ keepbm,
+                                                          const uint8_t* __restrict__ exp_to_rank, uint32_t* __restrict__ blob,
+                                                          const uint32_t* __restrict__ abort_flag) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ uint32_t s_len[MX ? 1 : 512];                               // code length by sign and exponent
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_wait();
     if (*abort_flag) return;
     const int sb = blockIdx.x, rb = sb / g.n_seg, seg = sb % g.n_seg;
-    const int tid = threadIdx.x, lane = tid & 31, r = tid >> 5;
-    const uint32_t* dir = blob + kBlobDirOffset / 4 + sb * 4;
+    const uint4 dir = reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4)[sb];
     const int scols = seg_cols_of(g.k_pad, g.seg_cols, seg);
-    const int n_ch = dir_n_ch(dir[3]);
-    const uint32_t E = (uint32_t)dir_chunk_elems(dir[3]);
-    const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir[1], (int)dir[2]);
-    uint32_t* body = blob + (size_t)dir[0] * 4;
-    for (int i = tid; i < sg.total / 4; i += 1024) reinterpret_cast<uint4*>(body)[i] = make_uint4(0, 0, 0, 0);
+    const int n_ch = dir_n_ch(dir.w);
+    const uint32_t E = (uint32_t)dir_chunk_elems(dir.w);
+    const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir.y, (int)dir.z);
+    uint32_t* gbody = blob + (size_t)dir.x * 4;
+    uint16_t* ring = reinterpret_cast<uint16_t*>(smem) + warp * kPackRing;
+    const bool staged = sg.total / 32 * 33 * 4 <= kPackBodyBytes;
+    const int ls = staged ? 33 : 32;                                       // words between two lines of the body
+    uint32_t* body = staged ? reinterpret_cast<uint32_t*>(smem + kPackRingBytes) : gbody;
+    if (!MX) s_len[tid] = exp_to_rank[tid & 255] + 1u;
+    static_assert(kPackThreads == 512, "one table entry a thread");
+    for (int i = tid; i < sg.total / 32 * ls; i += kPackThreads) body[i] = 0;
     __syncthreads();
 
-    const int row = rb * kRowsPerBlock + r;
-    const int t = g.t, F = 8 - t, per = 32 / F;
-    const int words = g.k_pad / 32;
+    const int t = T >= 0 ? T : g.t, F = 8 - t;
+    const uint32_t per = 32u / (uint32_t)F;
     const int w0 = seg * (g.seg_cols / 32);
-    uint32_t ub = 0, k_base = 0;
-    for (int j = 0; j < sg.bm_words; ++j) {
-        uint32_t bm = row < g.n ? keepbm[(size_t)row * words + w0 + j] : 0u;
-        if (lane == 0) body[sg.bm + j * 32 + r] = bm;
-        bool kept = (bm >> (31 - lane)) & 1u;
-        uint32_t len = 0, field = 0;
-        if (kept) {
-            uint32_t b = W[(size_t)row * g.k + (w0 + j) * 32 + lane];
-            len = exp_to_rank[(b >> 7) & 0xFF] + 1u;
-            field = ((b >> 15) << (7 - t)) | ((b & 0x7Fu) >> t);
-        }
-        uint32_t incl = len;
+    const bool vec = g.k % 8 == 0 && ((uintptr_t)W & 15) == 0;
+#pragma unroll 1
+    for (int r = warp; r < kRowsPerBlock; r += kPackThreads / 32) {
+        const int row = rb * kRowsPerBlock + r;
+        const uint16_t* wr = W + (size_t)row * g.k + w0 * 32;
+        const uint32_t* bmr = keepbm + (size_t)row * (g.k_pad / 32) + w0;
+        uint32_t* tab_r = body + sg.tab / 32 * ls + r;
+        uint32_t* bm_r = body + sg.bm / 32 * ls + r;
+        uint32_t* fl_r = body + sg.fl / 32 * ls + r;
+        uint32_t* un_r = body + sg.un / 32 * ls + r;
+        uint32_t ub = 0, k_cnt = 0, k_done = 0, next_ch = 0, done_ch = 0;  // code bits packed; values compacted; packed; chunks whose column, whose entry is written
+
+        const int n_blk = row < g.n ? ceil_div(sg.bm_words, 8) : 0;
+        uint32_t bm8 = 0, v[4], byte = 0;
+        auto fetch = [&](int blk) {                                        // bitmap words and values of the blk-th 256 columns
+            bm8 = lane < 8 && blk * 8 + lane < sg.bm_words ? __ldg(bmr + blk * 8 + lane) : 0u;
+            byte = row_byte(bm8, 0, lane);
+            row_load8(wr + blk * 256 + lane * 8, byte, vec, v);
+        };
+        if (n_blk > 0) fetch(0);
+#pragma unroll 1
+        for (int blk = 0; blk < n_blk || k_cnt > k_done; ++blk) {
+            if (blk < n_blk) {
+                if (lane < 8 && blk * 8 + lane < sg.bm_words) bm_r[(blk * 8 + lane) * ls] = bm8;
+                const uint32_t cnt = __popc(byte);
+                uint32_t incl = cnt;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += x;
+                }
+                uint32_t k = k_cnt + incl - cnt;                           // index of the lane's first kept value
+                k_cnt += __shfl_sync(0xffffffffu, incl, 31);
+                while (next_ch < (uint32_t)n_ch && next_ch * E < k_cnt) {  // a chunk starts in these columns: where
+                    const uint32_t nth = next_ch * E - k;                  // of the lane's kept values
+                    if (nth < cnt) {
+                        uint32_t b = byte;
+                        for (uint32_t i = 0; i < nth; ++i) b &= ~(0x80000000u >> __clz(b));
+                        tab_r[next_ch * ls] = (uint32_t)(blk * 256 + lane * 8 + __clz(b) - 24) << 20;
+                    }
+                    ++next_ch;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (byte & (0x80u >> i)) {
+                        ring[k & (kPackRing - 1)] = (uint16_t)((i & 1) ? v[i / 2] >> 16 : v[i / 2]);
+                        ++k;
+                    }
+                if (blk + 1 < n_blk) fetch(blk + 1);                       // the next columns travel while these are packed
+                __syncwarp();
+                if (k_cnt - k_done < 256u && blk + 1 < n_blk) continue;
+            }
+            // ---- pack the values k_done .. k_done + n - 1, 8 a lane ----
+            const uint32_t n = min(256u, k_cnt - k_done);
+            const uint32_t kk = k_done + (uint32_t)lane * 8u;
+            const uint4 raw = *reinterpret_cast<const uint4*>(ring + (kk & (kPackRing - 1)));
+            const uint32_t rw[4] = {raw.x, raw.y, raw.z, raw.w};
+            const int nv = min(8, max(0, (int)n - lane * 8));
+            uint32_t e[8], entry = 0;                                      // values; the lane's first code bit or 8 x its block
+#pragma unroll
+            for (int i = 0; i < 8; ++i) e[i] = (i & 1) ? rw[i / 2] >> 16 : rw[i / 2] & 0xFFFFu;
+            if (MX) {
+                uint32_t e_blk = 0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) if (i < nv) e_blk = max(e_blk, (e[i] >> 7) & 0xFFu);
+                e_blk = max(e_blk, __shfl_xor_sync(0xffffffffu, e_blk, 1));
+                e_blk = max(e_blk, __shfl_xor_sync(0xffffffffu, e_blk, 2));
+                const uint32_t b = kk / kMxBlock;
+                if ((lane & 3) == 0 && nv > 0) atomicOr(&un_r[(b / 4) * ls], e_blk << (24 - 8 * (b % 4)));
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {                              // field: sign, magnitude in the block's unit
+                    const uint32_t ex = (e[i] >> 7) & 0xFFu, shift = 1u + e_blk - ex;
+                    const uint32_t m7 = (shift < 8u && ex > 0u && e_blk >= 7u) ? (0x80u | (e[i] & 0x7Fu)) >> shift : 0u;
+                    e[i] = ((e[i] >> 15) << (7 - t)) | (m7 >> t);
+                }
+                entry = 8u * b;
+            } else {
+                uint32_t off = 0, bits = 0;                                // the lane's codewords from bit 31 of a word of its own
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (i < nv) {
+                        off += s_len[e[i] >> 7];
+                        bits |= off <= 32u ? 0x80000000u >> (off - 1u) : 0u;
+                    }
+                uint32_t incl = off;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += x;
+                }
+                uint32_t pos = ub + incl - off;
+                entry = pos;
+                if (off <= 32u) {
+                    const uint32_t hi = bits >> (pos & 31u), lo = __funnelshift_r(0u, bits, pos & 31u);
+                    if (hi) atomicOr(&un_r[(pos >> 5) * ls], hi);
+                    if (lo) atomicOr(&un_r[((pos >> 5) + 1) * ls], lo);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (i < nv) {
+                            pos += s_len[e[i] >> 7];
+                            atomicOr(&un_r[((pos - 1) >> 5) * ls], 0x80000000u >> ((pos - 1) & 31));
+                        }
+                }
+                ub += __shfl_sync(0xffffffffu, incl, 31);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) e[i] = ((e[i] >> 15) << (7 - t)) | ((e[i] & 0x7Fu) >> t);
+            }
+            while (done_ch < (uint32_t)n_ch && done_ch * E < k_done + n) { // chunks that start here (a multiple of 8: some lane's first value)
+                if (kk == done_ch * E) tab_r[done_ch * ls] |= entry;
+                ++done_ch;
+            }
+            if (nv > 0) {
+                if (per == 8 || per == 4) {                                // the lane's own words
+#pragma unroll
+                    for (int h = 0; h < 8; h += 4) {
+                        uint32_t acc = 0;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int j = per == 8 ? h + i : i;
+                            if (h + i < nv) acc |= MX ? e[h + i] << (32 - F * (j + 1)) : field_bits_in_word(e[h + i], j, t);
+                        }
+                        if (h < nv) fl_r[((kk + h) / per) * ls] |= acc;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (i < nv) {
+                            const uint32_t k = kk + i;
+                            atomicOr(&fl_r[(k / per) * ls], MX ? e[i] << (32 - F * (k % per + 1)) : field_bits_in_word(e[i], k % per, t));
+                        }
+                }
+            }
+            k_done += n;
+            __syncwarp();
         }
-        if (kept) {
-            uint32_t pre = lane ? __popc(bm >> (32 - lane)) : 0u;
-            uint32_t k = k_base + pre;
-            atomicOr(&body[sg.fl + (k / per) * 32 + r], field_bits_in_word(field, k % per, t));
-            uint32_t pos = ub + incl - 1;                                   // the codeword's terminating one
-            atomicOr(&body[sg.un + (pos >> 5) * 32 + r], 0x80000000u >> (pos & 31));
-            if (k % E == 0 && k / E < (uint32_t)n_ch)                       // first value of a chunk: its column and first code bit
-                body[sg.tab + (k / E) * 32 + r] = ((uint32_t)(j * 32 + lane) << 20) | (pos + 1 - len);
+        // chunks the row has no value for, and the totals
+        const uint32_t end = MX ? 8u * ((k_cnt + kMxBlock - 1) / kMxBlock) : ub;
+        for (int c = lane; c <= n_ch; c += 32) {
+            if (c == n_ch) tab_r[c * ls] = (k_cnt << 20) | end;
+            else if ((uint32_t)c * E >= k_cnt) tab_r[c * ls] = ((uint32_t)scols << 20) | end;
         }
-        ub += __shfl_sync(0xffffffffu, incl, 31);
-        k_base += __popc(bm);
     }
-    // chunks the row has no value for, and the totals
-    for (int c = lane; c <= n_ch; c += 32) {
-        if (c == n_ch) body[sg.tab + c * 32 + r] = (k_base << 20) | ub;
-        else if ((uint32_t)c * E >= k_base) body[sg.tab + c * 32 + r] = ((uint32_t)scols << 20) | ub;
-    }
+    if (!staged) return;
+    __syncthreads();
+    for (int i = tid; i < sg.total; i += kPackThreads) gbody[i] = body[i / 32 * 33 + i % 32];
 }
 
-// ---- E6 for Cassandra-2: the same superblock with shared exponents (Sec. 4.2, MX) --------------------------
-// Pass 1 finds the largest exponent of every block of 32 kept values of every row (shared memory), pass 2 writes the
-// bitmap, the magnitudes relative to their block's exponent, the exponent bytes and the chunk table.
-__global__ void __launch_bounds__(1024) k_pack_mx(const uint16_t* __restrict__ W, EncGeom g,
-                                                  const uint32_t* __restrict__ keepbm, uint32_t* __restrict__ blob,
-                                                  const uint32_t* __restrict__ abort_flag) {
-    __shared__ uint32_t s_exp[kRowsPerBlock][2048 / kMxBlock];
-    if (*abort_flag) return;
-    const int sb = blockIdx.x, rb = sb / g.n_seg, seg = sb % g.n_seg;
-    const int tid = threadIdx.x, lane = tid & 31, r = tid >> 5;
-    const uint32_t* dir = blob + kBlobDirOffset / 4 + sb * 4;
-    const int scols = seg_cols_of(g.k_pad, g.seg_cols, seg);
-    const int n_ch = dir_n_ch(dir[3]);
-    const uint32_t E = (uint32_t)dir_chunk_elems(dir[3]);
-    const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir[1], (int)dir[2]);
-    uint32_t* body = blob + (size_t)dir[0] * 4;
-    for (int i = tid; i < sg.total / 4; i += 1024) reinterpret_cast<uint4*>(body)[i] = make_uint4(0, 0, 0, 0);
-    for (int i = lane; i < 2048 / kMxBlock; i += 32) s_exp[r][i] = 0;
-    __syncthreads();
+// CTAs of k_select: as many as run at once (each takes rows in turn, so that the counts of kept exponents reach global
+// memory once per CTA).
+template <int NV, int WPR>
+static int launch_select_as(const uint16_t* W, const float* act, const EncGeom& g, const EncWs& ws, cudaStream_t stream) {
+    constexpr int NT = sel_threads(WPR), ROWS = NT / (32 * WPR);
+    int dev = 0, sms = 148, per_sm = 1;
+    CASS_CUDA_CHECK(cudaGetDevice(&dev));
+    CASS_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    CASS_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_select<NV, WPR>, NT, 0));
+    const int most = sms * (per_sm < 1 ? 1 : per_sm), need = ceil_div(g.n, ROWS);
+    CASS_PDL_LAUNCH((k_select<NV, WPR>), dim3(need < most ? need : most), dim3(NT), 0, stream, W, act, g, ws.keepbm, ws.hist);
+    return CASS_OK;
+}
 
-    const int row = rb * kRowsPerBlock + r;
-    const int t = g.t, F = 8 - t, per = 32 / F;
-    const int words = g.k_pad / 32;
-    const int w0 = seg * (g.seg_cols / 32);
-    uint32_t k_base = 0;
-    for (int j = 0; j < sg.bm_words; ++j) {                      // pass 1: block maxima
-        uint32_t bm = row < g.n ? keepbm[(size_t)row * words + w0 + j] : 0u;
-        if ((bm >> (31 - lane)) & 1u) {
-            uint32_t k = k_base + (lane ? __popc(bm >> (32 - lane)) : 0u);
-            atomicMax(&s_exp[r][k / kMxBlock], ((uint32_t)W[(size_t)row * g.k + (w0 + j) * 32 + lane] >> 7) & 0xFFu);
-        }
-        k_base += __popc(bm);
-    }
-    __syncwarp();
-    const uint32_t n_blk = (k_base + kMxBlock - 1) / kMxBlock;
-    for (uint32_t b = lane; b < n_blk; b += 32) atomicOr(&body[sg.un + (b / 4) * 32 + r], s_exp[r][b] << (24 - 8 * (b % 4)));
-    k_base = 0;
-    for (int j = 0; j < sg.bm_words; ++j) {                      // pass 2: bitmap, fields, table
-        uint32_t bm = row < g.n ? keepbm[(size_t)row * words + w0 + j] : 0u;
-        if (lane == 0) body[sg.bm + j * 32 + r] = bm;
-        if ((bm >> (31 - lane)) & 1u) {
-            const uint32_t b = W[(size_t)row * g.k + (w0 + j) * 32 + lane];
-            const uint32_t k = k_base + (lane ? __popc(bm >> (32 - lane)) : 0u);
-            const uint32_t e = (b >> 7) & 0xFFu, e_blk = s_exp[r][k / kMxBlock];
-            const uint32_t shift = 1u + e_blk - e;
-            const uint32_t m7 = (shift < 8u && e > 0u && e_blk >= 7u) ? (0x80u | (b & 0x7Fu)) >> shift : 0u;
-            const uint32_t field = ((b >> 15) << (7 - t)) | (m7 >> t);
-            atomicOr(&body[sg.fl + (k / per) * 32 + r], field << (32 - F * (k % per + 1)));
-            if (k % E == 0 && k / E < (uint32_t)n_ch)
-                body[sg.tab + (k / E) * 32 + r] = ((uint32_t)(j * 32 + lane) << 20) | (8u * (k / kMxBlock));
-        }
-        k_base += __popc(bm);
-    }
-    for (int c = lane; c <= n_ch; c += 32) {
-        if (c == n_ch) body[sg.tab + c * 32 + r] = (k_base << 20) | (8u * n_blk);
-        else if ((uint32_t)c * E >= k_base) body[sg.tab + c * 32 + r] = ((uint32_t)scols << 20) | (8u * n_blk);
-    }
+// One warp a row while its lanes' registers hold it (128 values a lane), then as many warps as it takes.
+static int launch_select(const uint16_t* W, const float* act, const EncGeom& g, const EncWs& ws, cudaStream_t stream) {
+    const int k = g.k;
+    if (k <= 512) return launch_select_as<16, 1>(W, act, g, ws, stream);
+    if (k <= 1024) return launch_select_as<32, 1>(W, act, g, ws, stream);
+    if (k <= 2048) return launch_select_as<64, 1>(W, act, g, ws, stream);
+    if (k <= 4096) return launch_select_as<128, 1>(W, act, g, ws, stream);
+    if (k <= 8192) return launch_select_as<128, 2>(W, act, g, ws, stream);
+    if (k <= 16384) return launch_select_as<128, 4>(W, act, g, ws, stream);
+    if (k <= 32768) return launch_select_as<128, 8>(W, act, g, ws, stream);
+    return launch_select_as<128, 16>(W, act, g, ws, stream);
 }
 
 // ---- test hook: zero-padded reconstruction of the whole blob ---------------------------------------------
@@ -427,25 +704,23 @@ extern "C" int cass_encode_weights(const cass_format* fmt, const void* W_bf16, c
     const uint16_t* W = (const uint16_t*)W_bf16;
     uint32_t* b32 = (uint32_t*)blob;
 
-    CASS_CUDA_CHECK(cudaMemsetAsync(workspace, 0, ws.bytes, stream));
-    size_t smem = (size_t)g.k * 4;
-    CASS_CUDA_CHECK(cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_select<<<g.n, 256, smem, stream>>>(W, act_norm, g, ws.keepbm, ws.hist);
-    CASS_LAUNCH_CHECK();
+    CASS_CUDA_CHECK(cudaMemsetAsync(workspace, 0, ws.zero_bytes, stream));
+    rc = launch_select(W, act_norm, g, ws, stream);
+    if (rc) return rc;
     if (g.mx) {
         CASS_CUDA_CHECK(cudaMemsetAsync((uint8_t*)blob + kBlobHeaderBytes, 0, kBlobCodebookBytes, stream));    // no codebook
     } else {
-        k_codebook<<<1, 256, 0, stream>>>(ws.hist, (uint8_t*)blob + kBlobHeaderBytes, ws.exp_to_rank);
-        CASS_LAUNCH_CHECK();
+        CASS_PDL_LAUNCH(k_codebook, dim3(1), dim3(256), 0, stream, (const unsigned long long*)ws.hist, (uint8_t*)blob + kBlobHeaderBytes,
+                        ws.exp_to_rank);
     }
-    int warps = g.n_pad * g.n_seg;
-    k_sizes<<<ceil_div(warps, 8), 256, 0, stream>>>(W, g, ws.keepbm, ws.exp_to_rank, ws.cnt_fw, ws.ubits);
-    CASS_LAUNCH_CHECK();
-    k_directory<<<1, 1024, 0, stream>>>(g, ws.cnt_fw, ws.ubits, b32, (unsigned long long)blob_cap, ws.abort_flag, d_status);
-    CASS_LAUNCH_CHECK();
-    if (g.mx) k_pack_mx<<<(unsigned)n_sb, 1024, 0, stream>>>(W, g, ws.keepbm, b32, ws.abort_flag);
-    else k_pack<<<(unsigned)n_sb, 1024, 0, stream>>>(W, g, ws.keepbm, ws.exp_to_rank, b32, ws.abort_flag);
-    CASS_LAUNCH_CHECK();
+    CASS_PDL_LAUNCH(k_sizes, dim3((unsigned)n_sb), dim3(1024), 0, stream, W, g, (const uint32_t*)ws.keepbm, (const uint8_t*)ws.exp_to_rank,
+                    ws.sb_size);
+    CASS_PDL_LAUNCH(k_directory, dim3(1), dim3(1024), 0, stream, g, (const uint2*)ws.sb_size, b32, (unsigned long long)blob_cap,
+                    ws.abort_flag, d_status);
+    auto pack = g.mx ? (g.t == 4 ? k_pack<true, 4> : k_pack<true, -1>) : (g.t == 4 ? k_pack<false, 4> : k_pack<false, -1>);
+    CASS_CUDA_CHECK(cudaFuncSetAttribute(pack, cudaFuncAttributeMaxDynamicSharedMemorySize, kPackSmem));
+    CASS_PDL_LAUNCH(pack, dim3((unsigned)n_sb), dim3(kPackThreads), (size_t)kPackSmem, stream, W, g, (const uint32_t*)ws.keepbm,
+                    (const uint8_t*)ws.exp_to_rank, b32, (const uint32_t*)ws.abort_flag);
     return CASS_OK;
 }
 
