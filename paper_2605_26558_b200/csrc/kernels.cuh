@@ -190,8 +190,13 @@ bool rope_kv_fusable(const KvGeom& g);
 int launch_rope_kv_append(const KvGeom& g, const KvComp& ck, const KvComp& cv, uint16_t* k_cache, uint16_t* v_cache,
                           Partials pp, const float* cos_t, const float* sin_t, uint16_t* qkv, int n_q, int use_inflight,
                           int rps, int flags, DevState* st, int n_seq, cudaStream_t s);
-int launch_kv_codebook(const KvGeom& g, const KvComp& ck, const KvComp& cv, const uint16_t* k_cache,
-                       const uint16_t* v_cache, int n_tokens, cudaStream_t s);
+// Many tokens at a time (kv_span.cu); start_pos as a number.
+int launch_kv_span(const KvGeom& g, const KvComp& ck, const KvComp& cv, uint16_t* k_cache, uint16_t* v_cache, const uint16_t* src_k,
+                   const uint16_t* src_v, int row_stride, int start_pos, int n_new, int flags, DevState* st, int seq0, int n_seq, cudaStream_t s);
+// Codebooks of every layer and sequence from the first n_tokens positions of the bf16 caches, and those positions' records
+// (caches given for layer 0 and sequence 0; layers lie layer_stride bytes apart).
+int launch_kv_codebook(const KvGeom& g, const KvComp& ck, const KvComp& cv, uint16_t* k_cache, uint16_t* v_cache, int n_layers,
+                       size_t layer_stride, int n_seq, int n_tokens, DevState* st, cudaStream_t s);
 
 // ---- attention ----------------------------------------------------------------------------------------
 struct AttnScratch {

@@ -1,5 +1,5 @@
 // Online KV encoder (Sec. 4.2: per-token magnitude pruning of K and V, mantissa truncation, unary exponent
-// code; Sec. 5.1 encoder): one warp formats one (token, KV head, K|V) record; records are appended to the
+// code; Sec. 5.1 encoder) for the rows of a decode step (kv_span.cu: for prompts): one warp formats one (token, KV head, K|V) record; records are appended to the
 // compressed cache and, on request, the raw bf16 rows go to the target's cache.
 #include "kernels.cuh"
 
@@ -43,44 +43,6 @@ __device__ __forceinline__ void kv_select(const uint32_t (&bits)[kKvMaxPerLane],
     }
 #pragma unroll
     for (int j = 0; j < kKvMaxPerLane; ++j) keep[j] = j < nj && key[j] >= thr;
-}
-
-__global__ void __launch_bounds__(256) k_kv_hist(KvGeom g, KvComp ck, KvComp cv, const uint16_t* __restrict__ k_cache,
-                                                 const uint16_t* __restrict__ v_cache, int n_tokens) {
-    __shared__ unsigned int s_hist[256];
-    const int head = blockIdx.x, kind = blockIdx.y;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint16_t* cache = kind ? v_cache : k_cache;
-    s_hist[threadIdx.x] = 0;
-    __syncthreads();
-    const int nj = g.d / 32;
-    for (int t = blockIdx.z * kKvWarps + warp; t < n_tokens; t += gridDim.z * kKvWarps) {
-        uint32_t bits[kKvMaxPerLane];
-        bool keep[kKvMaxPerLane];
-        const uint16_t* src = cache + ((size_t)t * g.n_kv + head) * g.d;
-#pragma unroll
-        for (int j = 0; j < kKvMaxPerLane; ++j) bits[j] = j < nj ? src[lane + 32 * j] : 0;
-        kv_select(bits, nj, g.n_prune, lane, keep);
-#pragma unroll
-        for (int j = 0; j < kKvMaxPerLane; ++j)
-            if (keep[j]) atomicAdd(&s_hist[(bits[j] >> 7) & 0xFF], 1u);
-    }
-    __syncthreads();
-    unsigned long long* hist = kind ? cv.hist : ck.hist;
-    if (s_hist[threadIdx.x]) atomicAdd(&hist[threadIdx.x], (unsigned long long)s_hist[threadIdx.x]);
-}
-
-__global__ void k_kv_rank(KvComp ck, KvComp cv) {
-    __shared__ unsigned long long s[256];
-    KvComp c = blockIdx.x ? cv : ck;
-    int e = threadIdx.x;
-    s[e] = c.hist[e];
-    __syncthreads();
-    unsigned long long mine = s[e];
-    int rank = 0;
-    for (int o = 0; o < 256; ++o) rank += (s[o] > mine) || (s[o] == mine && o < e);
-    c.rank_to_exp[rank] = (uint8_t)e;
-    c.exp_to_rank[e] = (uint8_t)rank;
 }
 
 // grid (n_kv, 2): block of 8 warps walks the n_new tokens in batches of 8; offsets into the unary arena are
@@ -333,6 +295,9 @@ int launch_kv_append(const KvGeom& g, const KvComp& ck, const KvComp& cv, uint16
                      const uint16_t* src_k, const uint16_t* src_v, int row_stride, int start_pos, int use_inflight,
                      int n_new, int flags, DevState* st, int seq0, int n_seq, cudaStream_t s) {
     if (n_new <= 0 || n_seq <= 0) return CASS_OK;
+    // two rounds of 8 tokens inside one CTA per head cost less than the span encoder's three launches; more do not
+    if (n_new > 2 * kKvWarps && start_pos >= 0)
+        return launch_kv_span(g, ck, cv, k_cache, v_cache, src_k, src_v, row_stride, start_pos, n_new, flags, st, seq0, n_seq, s);
     dim3 grid(g.n_kv, 2, n_seq);
     CASS_PDL_LAUNCH(k_kv_append<false>, grid, dim3(256), 0, s, g, ck, cv, k_cache, v_cache, src_k, src_v, row_stride, start_pos,
                     use_inflight, n_new, flags, st, seq0, RopeSrc{});
@@ -350,20 +315,6 @@ int launch_rope_kv_append(const KvGeom& g, const KvComp& ck, const KvComp& cv, u
     dim3 grid(g.n_kv + q_blocks, 2, n_seq);
     CASS_PDL_LAUNCH(k_kv_append<true>, grid, dim3(256), 0, s, g, ck, cv, k_cache, v_cache, (const uint16_t*)nullptr,
                     (const uint16_t*)nullptr, 0, -1, use_inflight, rps, flags, st, 0, RopeSrc{pp, cos_t, sin_t, qkv, n_q});
-    return CASS_OK;
-}
-
-int launch_kv_codebook(const KvGeom& g, const KvComp& ck, const KvComp& cv, const uint16_t* k_cache,
-                       const uint16_t* v_cache, int n_tokens, cudaStream_t s) {
-    CASS_CUDA_CHECK(cudaMemsetAsync(ck.hist, 0, 256 * 8, s));
-    CASS_CUDA_CHECK(cudaMemsetAsync(cv.hist, 0, 256 * 8, s));
-    if (n_tokens > 0) {
-        dim3 grid(g.n_kv, 2, min(64, ceil_div(n_tokens, kKvWarps)));
-        k_kv_hist<<<grid, 256, 0, s>>>(g, ck, cv, k_cache, v_cache, n_tokens);
-        CASS_LAUNCH_CHECK();
-    }
-    k_kv_rank<<<2, 256, 0, s>>>(ck, cv);
-    CASS_LAUNCH_CHECK();
     return CASS_OK;
 }
 

@@ -375,17 +375,12 @@ extern "C" int cass_kv_build_codebook(void* session, int n_tokens, void* stream_
     if (!session) return CASS_ERR_INVALID_ARG;
     Session* s = (Session*)session;
     if (n_tokens < 0 || n_tokens > s->d.max_seq) return CASS_ERR_INVALID_ARG;
-    cudaStream_t stream = (cudaStream_t)stream_;
-    const size_t ss = s->kg.seq_stride;
-    for (auto& L : s->layers)
-        for (int b = 0; b < s->B; ++b) {       // every sequence has its own codebooks, built from its own prompt
-            const uint16_t *kc = of_seq(L.kc, b, ss), *vc = of_seq(L.vc, b, ss);
-            int rc = launch_kv_codebook(s->kg, of_seq(L.ck, b, ss), of_seq(L.cv, b, ss), kc, vc, n_tokens, stream);
-            if (rc) return rc;
-            rc = launch_kv_append(s->kg, L.ck, L.cv, L.kc, L.vc, kc, vc, s->kg.n_kv * s->kg.d, 0, 0, n_tokens,
-                                  CASS_KV_COMPRESSED, s->st, b, 1, stream);
-            if (rc) return rc;
-        }
+    // every sequence has its own codebooks, built from its own prompt; the layers' storage is laid out alike
+    LayerDev& L0 = s->layers[0];
+    const size_t layer_stride = s->layers.size() > 1 ? (size_t)((uint8_t*)s->layers[1].kc - (uint8_t*)L0.kc) : 0;
+    const int rc = launch_kv_codebook(s->kg, L0.ck, L0.cv, L0.kc, L0.vc, (int)s->layers.size(), layer_stride, s->B, n_tokens, s->st,
+                                      (cudaStream_t)stream_);
+    if (rc) return rc;
     s->codebooks_ready = true;
     return CASS_OK;
 }

@@ -1,0 +1,116 @@
+"""Edges of the two encoders' kernels: row lengths around the register and warp splits of the weight selection, rows with
+many equal scores, and spans of tokens against the same tokens appended a few at a time."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from oracle import layout, mx
+
+pytestmark = pytest.mark.gpu
+
+
+def _bits(t):
+    return t.detach().cpu().contiguous().view(torch.int16).numpy().astype(np.uint16)
+
+
+@pytest.fixture(scope="module")
+def cass():
+    import paper_2605_26558_b200 as m
+    from paper_2605_26558_b200 import engine
+    m.engine = engine
+    return m
+
+
+def _blob(cass, w, act, fmt):
+    bound, ws_bytes = cass.cass_encoded_weight_bytes(fmt, *w.shape)
+    blob = torch.zeros(bound // 4, dtype=torch.int32, device="cuda")
+    ws = torch.full((ws_bytes,), 0xA5, dtype=torch.uint8, device="cuda")       # the scratch holds whatever was there
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    cass.cass_encode_weights(fmt, w.cuda(), torch.from_numpy(act).cuda(), blob, ws, status)
+    info = cass.cass_weight_blob_info(blob)
+    assert int(status.item()) == 0
+    return blob[: info.total_bytes // 4].cpu().numpy().view(np.uint32)
+
+
+@pytest.mark.parametrize("cols", [1, 31, 511, 513, 1024, 1027, 2047, 2056, 4095, 4096, 4104, 8193, 16384, 16391, 32769])
+@pytest.mark.parametrize("mode", [1, 2])
+def test_rows_around_the_splits(cass, cols, mode):
+    rows = 3 if cols > 4096 else 37
+    w = synth.student_t_weight(rows, cols, 1, f"edge/w{cols}")
+    if cols > 64:
+        w[1] = 0.25                                  # every score of the row equal under equal norms
+        w[2, : cols // 2] = 0.0                      # half of the row zero: the threshold lies at a tie
+        w[0, 5:40] = w[0, 5]
+    act = (np.abs(np.random.default_rng(cols).standard_normal(cols)) + 0.05).astype(np.float32)
+    act[::2] = 1.0
+    fmt = cass.default_format(mode=mode)
+    got = _blob(cass, w, act, fmt)
+    enc = layout.encode_weight_blob if mode == 1 else mx.encode_weight_blob
+    assert np.array_equal(got, enc(_bits(w), act, 400, 4)[0])
+
+
+def test_constant_rows_and_no_pruning(cass):
+    w = torch.full((40, 3000), 0.5, dtype=torch.bfloat16)
+    w[7] = 0.0
+    act = np.ones(3000, dtype=np.float32)
+    for p, t in ((400, 4), (0, 0), (999, 3)):
+        got = _blob(cass, w, act, cass.default_format(w_p=p, w_t=t))
+        assert np.array_equal(got, layout.encode_weight_blob(_bits(w), act, p, t)[0]), (p, t)
+
+
+def _records(cass, eng, layer, seq):
+    base, mem, out = eng.mem.data_ptr(), eng.mem.view(torch.int32), []
+    for kind in (0, 1):
+        v = cass.cass_kv_query(eng.session, layer, kind, 0, seq=seq)
+        h, n = eng.shape.n_kv_heads, eng.desc.max_seq
+        for ptr, words in ((v.fixed, h * ((n + 31) // 32) * v.fixed_words_per_token * 32), (v.arena, h * v.arena_words),
+                           (v.offsets, h * (n + 1)), (v.codebook, 64)):
+            o = (ptr - base) // 4
+            out.append(mem[o: o + words].clone())
+    return out
+
+
+@pytest.mark.parametrize("d,kv_p,kv_t,kv_mode", [(32, 400, 4, 1), (64, 400, 4, 1), (128, 400, 4, 1), (128, 0, 0, 1), (256, 300, 4, 1),
+                                                 (96, 400, 0, 2), (128, 400, 4, 2), (256, 0, 0, 2)])
+@pytest.mark.parametrize("n_new", [17, 40, 301])
+def test_span_of_tokens_equals_tokens_in_turn(cass, d, kv_p, kv_t, kv_mode, n_new):
+    """Two layers, two sequences: the codebook's prompt and a later span give the records, offsets and codebooks that
+    appending up to 16 tokens a call gives, rows with ties, zeros and exponents that the codebook knows badly included."""
+    shape = synth.ModelShape(n_layers=2, hidden=256, n_q_heads=4, n_kv_heads=2, head_dim=d, ffn=256, vocab=256)
+    wt = synth.model_weights(shape, 0, device="cuda")
+    gw = {"layers": [cass.engine.fuse_layer_weights(lw) for lw in wt["layers"]], "embed": wt["embed"], "lm_head": wt["lm_head"],
+          "norm_final": wt["norm_final"]}
+    fmt = cass.default_format(kv_p=kv_p, kv_t=kv_t, kv_mode=kv_mode)
+    n0 = 21
+    engs = [cass.engine.Engine(shape, gw, fmt=fmt, max_seq=384, gamma_max=4, batch=2) for _ in range(2)]
+    for layer in range(2):
+        for seq in range(2):
+            k, v = (x.cuda() for x in synth.kv_fill(n0 + n_new, 2, d, 10 * layer + seq, "edge/kv"))
+            k[3], v[n0 + 1] = 0.0, 1.5
+            k[n0 + 2] *= torch.exp2(torch.arange(d, device="cuda") % 37).to(torch.bfloat16)
+            k[n0 + 4, :, ::3] = 0.75
+            for e in engs:
+                cass.cass_kv_append(e.session, layer, k[:n0].contiguous(), v[:n0].contiguous(), 0, n0, cass.KV_BF16, seq=seq)
+    for e in engs:
+        e.n_prompt = n0
+        e.build_kv_codebook()
+        for layer in range(2):
+            for seq in range(2):
+                k, v = (x.cuda() for x in synth.kv_fill(n0 + n_new, 2, d, 10 * layer + seq, "edge/kv"))
+                v[n0 + 1] = 1.5
+                k[n0 + 2] *= torch.exp2(torch.arange(d, device="cuda") % 37).to(torch.bfloat16)
+                k[n0 + 4, :, ::3] = 0.75
+                step = n_new if e is engs[0] else 16
+                for i in range(0, n_new, step):
+                    m = min(step, n_new - i)
+                    cass.cass_kv_append(e.session, layer, k[n0 + i: n0 + i + m].contiguous(), v[n0 + i: n0 + i + m].contiguous(),
+                                        n0 + i, m, cass.KV_BF16 | cass.KV_COMPRESSED, seq=seq)
+    torch.cuda.synchronize()
+    for layer in range(2):
+        for seq in range(2):
+            for i, (a, b) in enumerate(zip(_records(cass, engs[0], layer, seq), _records(cass, engs[1], layer, seq))):
+                assert torch.equal(a, b), (layer, seq, i)
+    for e in engs:
+        assert e.status()[0] == 0
+        e.close()
