@@ -284,6 +284,13 @@ int cass_draft_step(void* session, const int32_t* tok_in, int32_t* tok_out, int 
 int cass_verify(void* session, const int32_t* toks, int g, int32_t* target_argmax, float* logits_opt,
                 void* stream);
 
+/* Target pass over the prompts (Sec. 2.2: prefill of the target model): toks[b][i], i < n, sits at position i of sequence b
+ * (all sequences equally long, n <= max_seq - 16).  Writes K/V of those positions into the bf16 cache, and into the compressed
+ * one if the codebooks are built; the greedy token after each prompt goes to target_argmax[b]; every length becomes n and no
+ * draft is in flight.  While calibration is on, the statistics of every row are accumulated.  The passes are wider than those
+ * of cass_verify and the results the same.  toks: device [max_batch][n]; target_argmax: device [max_batch]. */
+int cass_prefill(void* session, const int32_t* toks, int n, int32_t* target_argmax, void* stream);
+
 /* Stand-alone draft attention of one layer (Sec. 4.1 draft inference over the KV speculation data of Sec. 4.2):
  * q: bf16 [max_batch][n_q_heads][head_dim] (post-RoPE); sequence b's query sees the first len_b + 1 positions of its
  * compressed cache of that layer (len = committed length, see cass_set_len; no draft in flight);

@@ -52,6 +52,7 @@ constexpr int kGroupCodes = 4;             // codewords per unary-walk group
 constexpr int kMaxVerifyRows = 16;         // rows of one sequence in one verification call; also the margin kept at the end of a cache
 constexpr int kMaxBatch = 8;               // sequences per session
 constexpr int kMaxRows = 64;               // rows of all sequences in one call
+constexpr int kPrefillRows = 128;          // rows of all sequences in one pass of a prefill
 
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 __host__ __device__ inline size_t align_up(size_t a, size_t b) { return (a + b - 1) / b * b; }
@@ -91,6 +92,11 @@ __device__ __forceinline__ uint16_t float_to_bf16_bits(float f) {
 }
 
 __device__ __forceinline__ float round_bf16(float f) { return __bfloat162float(__float2bfloat16_rn(f)); }
+
+// Rotation of a pair (RoPE), the roundings spelled out: every kernel that rotates gives the same bits.
+__device__ __forceinline__ float2 rope_pair(float a, float b, float c, float s) {
+    return make_float2(__fmaf_rn(a, c, -__fmul_rn(b, s)), __fmaf_rn(a, s, __fmul_rn(b, c)));
+}
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll

@@ -5,13 +5,13 @@
 namespace cass {
 
 // Merge the chunk partials of every (row, query head): out = sum_c e^{m_c - M} o_c / sum_c e^{m_c - M} l_c.
-// Row r (the (r % rps)-th of sequence r / rps) sees positions < len + (draft: inflight + 1 | verify: r % rps + 1);
+// Row i of a sequence sees positions < len + (draft: inflight + 1 | verify: i + 1);
 // chunks hold `chunk_tokens` positions.
 // The reductions run in a fixed order that depends on the number of visible chunks only.
 constexpr int kMergeThreads = 256;
 constexpr int kMergeWarps = kMergeThreads / 32;
 
-__global__ void __launch_bounds__(kMergeThreads) k_attn_merge(AttnScratch sc, int n_chunks_alloc, int chunk_tokens, int rps, int n_q, int d,
+__global__ void __launch_bounds__(kMergeThreads) k_attn_merge(AttnScratch sc, int chunk_tokens, AttnRows ar, int n_q, int d,
                                                               const DevState* __restrict__ st, int draft_mode, int draft_units,
                                                               uint16_t* __restrict__ out) {
     extern __shared__ __align__(16) float w_s[];    // [n_chunks_alloc] weights e^{m_c - M}, then [kMergeWarps][d] partial outputs
@@ -20,8 +20,9 @@ __global__ void __launch_bounds__(kMergeThreads) k_attn_merge(AttnScratch sc, in
     pdl_wait();
     const int hq = blockIdx.x, r = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int seq = r / rps;
-    const int vis = st->len[seq] + (draft_mode ? st->inflight[seq] + 1 : r % rps + 1);
+    const int sub = ar.hi - ar.lo, seq = r / sub, n_chunks_alloc = ar.chunks;
+    const int row = ar.lo + r % sub;                                        // of the sequence's rps rows
+    const int vis = st->len[seq] + (draft_mode ? st->inflight[seq] + 1 : row + 1);
     if (draft_units < 0) chunk_tokens = tc_run_tokens(vis, -draft_units);     // the draft attention's runs follow the visible length
     const int n_ch = ceil_div(vis, chunk_tokens);
     const size_t pair = (size_t)r * n_q + hq;
@@ -94,22 +95,85 @@ __global__ void __launch_bounds__(kMergeThreads) k_attn_merge(AttnScratch sc, in
         float acc = part_s[dim];
 #pragma unroll
         for (int w = 1; w < kMergeWarps; ++w) acc += part_s[w * d + dim];
-        out[((size_t)r * n_q + hq) * d + dim] = float_to_bf16_bits(acc / L);
+        out[(((size_t)seq * ar.rps + row) * n_q + hq) * d + dim] = float_to_bf16_bits(acc / L);
     }
 }
 
-int launch_attn_merge(const AttnScratch& sc, int n_chunks_alloc, int chunk_tokens, int rows, int rps, int n_q, int d,
+// The same for at most MC chunks: one warp a (row, query head), lane = chunk for the statistics, then four dims a lane with all
+// chunks requested at once.  Every sum is formed in the order of k_attn_merge (eight interleaved chains, added in turn), so
+// the bits are the same.  A CTA of 8 warps and three barriers a pair, most of it idle, took 13.5 us for the 4096 pairs of a
+// prefill pass.
+template <int MC>
+__global__ void __launch_bounds__(kMergeThreads) k_attn_merge_few(AttnScratch sc, int chunk_tokens, AttnRows ar, int n_pairs, int n_q, int d,
+                                                                  const DevState* __restrict__ st, int draft_mode, int draft_units,
+                                                                  uint16_t* __restrict__ out) {
+    pdl_early<3>();
+    pdl_wait();
+    const int pair = blockIdx.x * kMergeWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (pair >= n_pairs) return;
+    const int r = pair / n_q, hq = pair % n_q, sub = ar.hi - ar.lo, seq = r / sub, row = ar.lo + r % sub;
+    const int vis = st->len[seq] + (draft_mode ? st->inflight[seq] + 1 : row + 1);
+    if (draft_units < 0) chunk_tokens = tc_run_tokens(vis, -draft_units);
+    const int n_ch = ceil_div(vis, chunk_tokens);
+    const size_t base = (size_t)pair * ar.chunks;
+    const float* op = sc.o + base * d;
+    const float m = lane < n_ch ? __ldcg(sc.m + base + lane) : -INFINITY, l = lane < n_ch ? __ldcg(sc.l + base + lane) : 0.f;
+    float M = 0.f, L = 0.f, w = 0.f;
+    for (int d0 = 0; d0 < d; d0 += 128) {
+        const int dim = min(d0 + lane * 4, d - 4);                        // lanes beyond the head repeat its last dims
+        float4 o[MC];
+#pragma unroll
+        for (int c = 0; c < MC; ++c) o[c] = __ldcg(reinterpret_cast<const float4*>(op + (size_t)min(c, n_ch - 1) * d + dim));
+        if (d0 == 0) {
+            M = warp_max(m);
+            w = lane < n_ch ? expf(m - M) : 0.f;
+            L = warp_sum(w * l);
+        }
+        float4 total = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int c0 = 0; c0 < kMergeWarps; ++c0) {
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int c = c0; c < MC; c += kMergeWarps) {
+                const float wc = __shfl_sync(0xffffffffu, w, c);
+                if (c < n_ch) {
+                    acc.x = fmaf(wc, o[c].x, acc.x); acc.y = fmaf(wc, o[c].y, acc.y);
+                    acc.z = fmaf(wc, o[c].z, acc.z); acc.w = fmaf(wc, o[c].w, acc.w);
+                }
+            }
+            total.x = c0 ? total.x + acc.x : acc.x; total.y = c0 ? total.y + acc.y : acc.y;
+            total.z = c0 ? total.z + acc.z : acc.z; total.w = c0 ? total.w + acc.w : acc.w;
+        }
+        const uint32_t b[4] = {float_to_bf16_bits(total.x / L), float_to_bf16_bits(total.y / L), float_to_bf16_bits(total.z / L),
+                               float_to_bf16_bits(total.w / L)};
+        *reinterpret_cast<uint2*>(out + (((size_t)seq * ar.rps + row) * n_q + hq) * d + dim) = make_uint2(b[0] | (b[1] << 16), b[2] | (b[3] << 16));
+    }
+}
+
+int launch_attn_merge(const AttnScratch& sc, int chunk_tokens, int n_seq, const AttnRows& ar, int n_q, int d,
                       const DevState* st, int draft_mode, int draft_units, uint16_t* out, cudaStream_t s) {
     if (d % 4) return CASS_ERR_UNSUPPORTED;
-    dim3 grid(n_q, rows);
-    const size_t smem = ((size_t)((n_chunks_alloc + 3) & ~3) + (size_t)kMergeWarps * d) * 4;
+    dim3 grid(n_q, n_seq * (ar.hi - ar.lo));
+    const int pairs = n_q * n_seq * (ar.hi - ar.lo);
+    // a warp a pair where few chunks are possible (by the cache's size, not by what is visible now), or where pairs abound
+#define CASS_MERGE_FEW(MC)                                                                                                              \
+    do {                                                                                                                                \
+        CASS_PDL_LAUNCH(k_attn_merge_few<MC>, dim3(ceil_div(pairs, kMergeWarps)), dim3(kMergeThreads), 0, s, sc, chunk_tokens, ar, pairs, n_q, \
+                        d, st, draft_mode, draft_units, out);                                                                           \
+        return CASS_OK;                                                                                                                 \
+    } while (0)
+    if (ar.chunks <= 8) CASS_MERGE_FEW(8);
+    if (ar.chunks <= 16 && pairs >= 1024) CASS_MERGE_FEW(16);
+    if (ar.chunks <= 32 && pairs >= 1024) CASS_MERGE_FEW(32);
+#undef CASS_MERGE_FEW
+    const size_t smem = ((size_t)((ar.chunks + 3) & ~3) + (size_t)kMergeWarps * d) * 4;
     if (smem > 200 * 1024) return CASS_ERR_CAPACITY;
     static size_t attr = 48 * 1024;
     if (smem > attr) {
         CASS_CUDA_CHECK(cudaFuncSetAttribute(k_attn_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr = smem;
     }
-    CASS_PDL_LAUNCH(k_attn_merge, grid, dim3(kMergeThreads), smem, s, sc, n_chunks_alloc, chunk_tokens, rps, n_q, d, st, draft_mode,
+    CASS_PDL_LAUNCH(k_attn_merge, grid, dim3(kMergeThreads), smem, s, sc, chunk_tokens, ar, n_q, d, st, draft_mode,
                     draft_units, out);
     return CASS_OK;
 }

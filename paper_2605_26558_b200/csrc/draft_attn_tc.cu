@@ -562,9 +562,6 @@ __global__ void __launch_bounds__(kTcThreads) k_draft_attn_tc(KvGeom g, KvComp c
     }
 }
 
-int launch_attn_merge(const AttnScratch& sc, int n_chunks_alloc, int chunk_tokens, int rows, int rps, int n_q, int d,
-                      const DevState* st, int draft_mode, int draft_units, uint16_t* out, cudaStream_t s);
-
 size_t draft_attn_tc_smem_bytes(const KvGeom& g) {
     const size_t ks = (size_t)g.d + kTcPad;
     return (2 * kTcTok + kTcHeads) * ks * 2 + (size_t)tc_fix_words(g) * 4 + (size_t)4 * tc_una_rows(g) * 32 * 4 + (size_t)tc_lut_words(g) * 4 + 3 * kTcHeads * 4 + 64;
@@ -600,7 +597,7 @@ int launch_draft_attn_tc(const KvGeom& g, const KvComp& ck, const KvComp& cv, co
     // the runs of every (sequence, query head) are merged by a kernel of their own: one CTA per head with the runs spread
     // over its warps (a merge by the last CTA of a KV head, as the slice-parallel kernel does it, is one CTA adding up to
     // 74 runs for the whole group in sequence: measured 32.6 instead of 16.7 us at 4096 positions)
-    return launch_attn_merge(sc, n_chunks, kTcTok, n_seq, 1, n_q, g.d, st, 1, -g.n_kv * n_seq, out, s);
+    return launch_attn_merge(sc, kTcTok, n_seq, attn_all_rows(1, n_chunks), n_q, g.d, st, 1, -g.n_kv * n_seq, out, s);
 }
 
 }  // namespace cass

@@ -109,6 +109,25 @@ __device__ __forceinline__ float4 parts_sum4(const Partials& pp, size_t off) {
     }
     return acc;
 }
+// Two such quadruples whose loads travel together.
+__device__ __forceinline__ void parts_sum4_pair(const Partials& pp, size_t off_a, size_t off_b, float4& a, float4& b) {
+    a = b = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < pp.n_seg; s0 += 4) {
+        float4 va[4], vb[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float* p = pp.p + (size_t)min(s0 + i, pp.n_seg - 1) * pp.seg_stride;          // unconditional: all of them travel at once
+            va[i] = __ldcg(reinterpret_cast<const float4*>(p + off_a));
+            vb[i] = __ldcg(reinterpret_cast<const float4*>(p + off_b));
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (s0 + i < pp.n_seg) {
+                a.x += va[i].x; a.y += va[i].y; a.z += va[i].z; a.w += va[i].w;
+                b.x += vb[i].x; b.y += vb[i].y; b.z += vb[i].z; b.w += vb[i].w;
+            }
+    }
+}
 // The same for N offsets at once: all loads of a batch of parts travel together.
 template <int N>
 __device__ __forceinline__ void parts_sum_n(const Partials& pp, const size_t (&off)[N], const bool (&on)[N], float (&acc)[N]) {
@@ -144,8 +163,8 @@ inline Partials draft_gemv_partials(const float* partial, const cass_blob_info& 
 
 // ---- small ops (ops.cu) -------------------------------------------------------------------------------
 int launch_rope_table(float* cos_t, float* sin_t, int max_seq, int d, float theta, cudaStream_t s);
-// row r takes token toks[r * tok_stride]
-int launch_embed(const int32_t* toks, int tok_stride, const uint16_t* embed, uint16_t* h, int rows, int hidden, cudaStream_t s);
+// row r (the (r % rps)-th of sequence r / rps) takes token toks[(r / rps) * seq_stride + r % rps]
+int launch_embed(const int32_t* toks, int rps, int seq_stride, const uint16_t* embed, uint16_t* h, int rows, int hidden, cudaStream_t s);
 int launch_rmsnorm(const uint16_t* h, const uint16_t* gain, uint16_t* out, int rows, int hidden, float eps,
                    cudaStream_t s);
 // h = bf16(h + y); out = rmsnorm(h) * gain.  y comes either as bf16 [rows][hidden] or (rows == 1) as fp32 split-K
@@ -164,6 +183,8 @@ int launch_swiglu(const uint16_t* gu_bf16, Partials pp, uint16_t* act, int rows,
 // Row r's token goes to out[r * out_stride].
 int launch_argmax(const float* logits, Partials pp, int rows, int vocab, int32_t* out, int out_stride,
                   float* logits_copy, float* tmp_v, int32_t* tmp_i, DevState* st, int bump_inflight, cudaStream_t s);
+int launch_set_len(DevState* st, int len, cudaStream_t s);
+int launch_last_rows(const uint16_t* src, int n_seq, int rps, int take, int cols, uint16_t* dst, cudaStream_t s);
 int launch_accept(DevState* st, int n_seq, const int32_t* draft, int draft_stride, const int32_t* target, int g, int32_t* n_acc,
                   int32_t* out_tokens, int32_t* next_tok, int next_stride, cudaStream_t s);
 // Sampling-based acceptance (sampling.cu): p [n_seq][g+1][vocab], q [n_seq][g][vocab] probabilities, r [n_seq][g] and
@@ -208,23 +229,35 @@ struct AttnScratch {
 // sequence's compressed cache (caches given for sequence 0).
 int launch_draft_attn(const KvGeom& g, const KvComp& ck, const KvComp& cv, const uint16_t* qkv, int qkv_stride, int n_q,
                       int n_seq, const DevState* st, const AttnScratch& sc, uint16_t* out, cudaStream_t s);
-// Verify: rps rows per sequence at positions len + i over that sequence's bf16 cache, causal.
-int launch_verify_attn(const KvGeom& g, const uint16_t* k_cache, const uint16_t* v_cache, const uint16_t* qkv,
-                       int n_seq, int rps, int n_q, const DevState* st, const AttnScratch& sc, uint16_t* out, cudaStream_t s);
+// Rows of a verification or prefill call that one attention launch covers: rows lo .. hi - 1 of each sequence's rps rows (row
+// i sits at position len + i), `group` of them a CTA.  Scratch holds hi - lo rows a sequence, `chunks` partial results a
+// pair (at least what position len + hi - 1 needs).
+struct AttnRows {
+    int rps, lo, hi, group, chunks;
+};
+inline AttnRows attn_all_rows(int rps, int chunks) { return AttnRows{rps, 0, rps, rps, chunks}; }
 
-// Tensor-core version (verify_attn_tc.cu) for head_dim 128 and rps * (n_q / n_kv) <= 64.  np_cols = 32 or 64: the
-// MMA's pair columns (>= rps * group); a pair's result does not depend on it, but a session keeps one value for
-// all its decode calls.
+// Verify: causal attention of those rows over each sequence's bf16 cache.
+int launch_verify_attn(const KvGeom& g, const uint16_t* k_cache, const uint16_t* v_cache, const uint16_t* qkv,
+                       int n_seq, const AttnRows& ar, int n_q, const DevState* st, const AttnScratch& sc, uint16_t* out, cudaStream_t s);
+
+// Tensor-core version (verify_attn_tc.cu) for head_dim 128 and group * (n_q / n_kv) <= 64.  np_cols = 32 or 64: the
+// MMA's pair columns (>= group * (n_q / n_kv)); a pair's result does not depend on it, but a session keeps one value for
+// all its decode calls.  Rows below `fine` of a sequence (a multiple of the group) keep their probabilities in two bf16
+// terms, as accurate as the fp32-pipe kernel.
 bool verify_attn_tc_usable(const KvGeom& g, int rps, int n_q);
 int launch_verify_attn_tc(const KvGeom& g, const uint16_t* k_cache, const uint16_t* v_cache, const uint16_t* qkv, int n_seq,
-                          int rps, int n_q, int np_cols, const DevState* st, const AttnScratch& sc, uint16_t* out,
+                          const AttnRows& ar, int fine, int n_q, int np_cols, const DevState* st, const AttnScratch& sc, uint16_t* out,
                           int32_t* d_status, cudaStream_t s);
+// Combines the partial results of rows lo .. hi - 1 (draft attention: ar.rps = 1, draft_units < 0, see draft_attn.cu).
+int launch_attn_merge(const AttnScratch& sc, int chunk_tokens, int n_seq, const AttnRows& ar, int n_q, int d, const DevState* st,
+                      int draft_mode, int draft_units, uint16_t* out, cudaStream_t s);
 
 // ---- verification GEMM (verify_gemm.cu): Y[r][n] = sum_k W[n][k] X[r][k], bf16 in, fp32 accumulate (tcgen05) ----
-// X is a buffer of `bn` rows of k values (bn = 16, 32 or 64 token columns of the MMA; the first `rows` are used);
+// X is a buffer of `bn` rows of k values (bn = 16, 32, 64 or 128 token columns of the MMA; the first `rows` are used);
 // partial: fp32 scratch of verify_gemm_partial_floats.
 // With both outputs null only the partial sums are produced: [splits][bn][n], see verify_gemm_partials().
-inline int verify_gemm_bn(int rows) { return rows <= 16 ? 16 : rows <= 32 ? 32 : 64; }
+inline int verify_gemm_bn(int rows) { return rows <= 16 ? 16 : rows <= 32 ? 32 : rows <= 64 ? 64 : 128; }
 size_t verify_gemm_partial_floats(int n, int k, int bn);
 Partials verify_gemm_partials(const float* partial, int n, int k, int bn);
 // w_static: W is not the output of a kernel that may still be running when this one is scheduled (the bf16 matrices of

@@ -97,8 +97,9 @@ __global__ void __launch_bounds__(256) k_kv_append(KvGeom g, KvComp ck, KvComp c
             float ab[2];
             parts_sum_n<2>(pp, offs, on2, ab);
             const float a = round_bf16(ab[0]), b = round_bf16(ab[1]);
-            rs.qkv[r * qkv_dim + ia] = float_to_bf16_bits(a * c - b * sn);
-            rs.qkv[r * qkv_dim + ib] = float_to_bf16_bits(b * c + a * sn);
+            const float2 rot = rope_pair(a, b, c, sn);
+            rs.qkv[r * qkv_dim + ia] = float_to_bf16_bits(rot.x);
+            rs.qkv[r * qkv_dim + ib] = float_to_bf16_bits(rot.y);
         }
         return;
     }
@@ -148,9 +149,9 @@ __global__ void __launch_bounds__(256) k_kv_append(KvGeom g, KvComp ck, KvComp c
                     for (int j = 0; j < kKvMaxPerLane / 2; ++j) {
                         if (j < hj) {
                             const float c = rc[j], sn = rsn[j];
-                            const float a = val[j], b = val[j + hj];
-                            val[j] = bf16_bits_to_float(float_to_bf16_bits(a * c - b * sn));
-                            val[j + hj] = bf16_bits_to_float(float_to_bf16_bits(b * c + a * sn));
+                            const float2 rot = rope_pair(val[j], val[j + hj], c, sn);
+                            val[j] = bf16_bits_to_float(float_to_bf16_bits(rot.x));
+                            val[j + hj] = bf16_bits_to_float(float_to_bf16_bits(rot.y));
                         }
                     }
                 }

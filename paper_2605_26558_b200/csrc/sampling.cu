@@ -31,7 +31,7 @@ __device__ __forceinline__ float block_reduce(float v, bool is_max, float* s_red
 constexpr int kSoftmaxThreads = 512;
 
 template <int NV>
-__global__ void __launch_bounds__(kSoftmaxThreads) k_softmax_rows(const float* __restrict__ logits, int vocab, int per, float inv_t,
+__global__ void __launch_bounds__(kSoftmaxThreads, 2) k_softmax_rows(const float* __restrict__ logits, int vocab, int per, float inv_t,
                                                                   float* __restrict__ probs) {
     __shared__ float s_red[kSoftmaxThreads / 32], s_cta[2];
     cg::cluster_group cluster = cg::this_cluster();

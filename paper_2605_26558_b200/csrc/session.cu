@@ -38,9 +38,11 @@ struct Session {
     int B, R;                // sequences; row capacity of one call (16, 32 or 64 = token columns of the verification MMA)
     // activations (R rows)
     uint16_t *h, *xn, *qkv, *attn, *y, *gu, *act;
+    uint16_t *ph, *pxn, *pqkv, *pattn, *pact;      // the same of a prefill pass (kPrefillRows rows)
     float *logits, *partial, *vg_partial;
     size_t partial_floats;
     AttnScratch asc;
+    size_t attn_parts;       // partial results (row, head, chunk) that asc holds
     int32_t* argmax_tmp;
     float* argmax_val;
     bool have_blobs, codebooks_ready, calib_host;
@@ -129,6 +131,12 @@ static size_t layout(Session* s, uint8_t* base) {
     s->y = (uint16_t*)at(p.take((size_t)R * d.hidden * 2));
     s->gu = (uint16_t*)at(p.take((size_t)R * 2 * d.ffn * 2));
     s->act = (uint16_t*)at(p.take((size_t)R * d.ffn * 2));
+    const size_t W = kPrefillRows;
+    s->ph = (uint16_t*)at(p.take(W * d.hidden * 2));
+    s->pxn = (uint16_t*)at(p.take(W * d.hidden * 2));
+    s->pqkv = (uint16_t*)at(p.take(W * s->qkv_dim * 2));
+    s->pattn = (uint16_t*)at(p.take(W * d.n_q_heads * d.head_dim * 2));
+    s->pact = (uint16_t*)at(p.take(W * d.ffn * 2));
     s->logits = (float*)at(p.take((size_t)R * d.vocab * 4));
     // split-K partials of the draft GEMVs: segments (<= ceil(K/256)) x padded rows
     size_t nmax = (size_t)d.vocab;
@@ -146,18 +154,23 @@ static size_t layout(Session* s, uint8_t* base) {
     s->partial_floats = pf;                                   // per vector of a draft GEMV
     s->partial = (float*)at(p.take(pf * 4 * s->B));
     {   // split-K scratch of the verification GEMMs
-        size_t c[5] = {verify_gemm_partial_floats(s->qkv_dim, d.hidden, R), verify_gemm_partial_floats(d.hidden, d.n_q_heads * d.head_dim, R),
-                       verify_gemm_partial_floats(2 * d.ffn, d.hidden, R), verify_gemm_partial_floats(d.hidden, d.ffn, R),
+        size_t c[5] = {verify_gemm_partial_floats(s->qkv_dim, d.hidden, kPrefillRows), verify_gemm_partial_floats(d.hidden, d.n_q_heads * d.head_dim, kPrefillRows),
+                       verify_gemm_partial_floats(2 * d.ffn, d.hidden, kPrefillRows), verify_gemm_partial_floats(d.hidden, d.ffn, kPrefillRows),
                        verify_gemm_partial_floats(d.vocab, d.hidden, R)};
         size_t m = 0;
         for (size_t v : c) if (v > m) m = v;
         s->vg_partial = (float*)at(p.take(m * 4));
     }
+    // attention scratch: what the rows of one verification call can need and, up to 64 MB, those of a prefill pass
     const int n_chunks = ceil_div(d.max_seq, kAttnChunk);
-    size_t pairs = (size_t)R * d.n_q_heads;
-    s->asc.o = (float*)at(p.take(pairs * n_chunks * d.head_dim * 4));
-    s->asc.m = (float*)at(p.take(pairs * n_chunks * 4));
-    s->asc.l = (float*)at(p.take(pairs * n_chunks * 4));
+    size_t parts = (size_t)R * d.n_q_heads * n_chunks;
+    size_t wide = (size_t)kPrefillRows * d.n_q_heads * ceil_div(n_chunks, 2);
+    if (wide > ((size_t)16 << 20) / d.head_dim) wide = ((size_t)16 << 20) / d.head_dim;
+    if (wide > parts) parts = wide;
+    s->attn_parts = parts;
+    s->asc.o = (float*)at(p.take(parts * d.head_dim * 4));
+    s->asc.m = (float*)at(p.take(parts * 4));
+    s->asc.l = (float*)at(p.take(parts * 4));
     s->argmax_tmp = (int32_t*)at(p.take((size_t)R * 128 * 4));
     s->argmax_val = (float*)at(p.take((size_t)R * 128 * 4));
     s->layers.resize(d.n_layers);
@@ -274,6 +287,7 @@ extern "C" int cass_session_reset(void* session, void* stream_) {
                 CASS_CUDA_CHECK(cudaMemsetAsync(c.off, 0, (size_t)s->kg.n_kv * (s->kg.max_seq + 1) * 4, stream));
             }
     s->codebooks_ready = false;
+    s->calib_host = false;
     s->drafts_pending = 0;
     return CASS_OK;
 }
@@ -310,6 +324,7 @@ extern "C" int cass_session_rows(const cass_model_desc* desc) {
 extern "C" int cass_calib_enable(void* session, int on, void* stream_) {
     if (!session) return CASS_ERR_INVALID_ARG;
     Session* s = (Session*)session;
+    if (s->calib_host == (on != 0)) return CASS_OK;               // as it is: nothing to wait for
     int32_t v = on ? 1 : 0;
     CASS_CUDA_CHECK(cudaMemcpyAsync(&s->st->calib_on, &v, 4, cudaMemcpyHostToDevice, (cudaStream_t)stream_));
     CASS_CUDA_CHECK(cudaStreamSynchronize((cudaStream_t)stream_));
@@ -426,6 +441,11 @@ extern "C" int cass_debug_activation(void* session, int which, const void** d_pt
 
 #define RC(expr) do { int _rc = (expr); if (_rc) return _rc; } while (0)
 
+static bool simt_verify_attn() {
+    static const bool on = [] { const char* e = std::getenv("CASS_SIMT_VERIFY_ATTN"); return e && e[0] == '1'; }();
+    return on;
+}
+
 extern "C" int cass_verify(void* session, const int32_t* toks, int g, int32_t* target_argmax, float* logits_opt,
                            void* stream_) {
     if (!session || !toks || !target_argmax) return CASS_ERR_INVALID_ARG;
@@ -439,7 +459,7 @@ extern "C" int cass_verify(void* session, const int32_t* toks, int g, int32_t* t
     const bool fused = rope_kv_fusable(s->kg);       // RoPE and the KV append in one kernel
     // tensor-core attention where the shape allows (head_dim 128, rows x group <= 64); CASS_SIMT_VERIFY_ATTN=1 keeps
     // the fp32-pipe kernel.  For a given model shape every decode call of a session takes the same path.
-    static const bool simt_env = [] { const char* e = std::getenv("CASS_SIMT_VERIFY_ATTN"); return e && e[0] == '1'; }();
+    const bool simt_env = simt_verify_attn();
     const int grp = d.n_q_heads / d.n_kv_heads;
     // decode calls (rps <= gamma_max + 1) are classed by gamma_max, so that plain and speculative decoding agree
     const bool attn_tc = !simt_env && verify_attn_tc_usable(s->kg, rps <= d.gamma_max + 1 ? d.gamma_max + 1 : rps, d.n_q_heads);
@@ -455,7 +475,7 @@ extern "C" int cass_verify(void* session, const int32_t* toks, int g, int32_t* t
         if (rc) w_rc = rc;
         return s->vscratch;
     };
-    RC(launch_embed(toks, 1, (const uint16_t*)s->embed, s->h, rows, d.hidden, st));
+    RC(launch_embed(toks, rps, rps, (const uint16_t*)s->embed, s->h, rows, d.hidden, st));
     RC(launch_rmsnorm(s->h, (const uint16_t*)s->layers[0].w.norm_attn, s->xn, rows, d.hidden, d.rms_eps, st));
     const int kv_flags = CASS_KV_BF16 | (s->codebooks_ready ? CASS_KV_COMPRESSED : 0);
     const bool calib = s->calib_host;           // the accumulation kernels are only launched while calibration is on
@@ -474,8 +494,12 @@ extern "C" int cass_verify(void* session, const int32_t* toks, int g, int32_t* t
             RC(launch_kv_append(s->kg, L.ck, L.cv, L.kc, L.vc, s->qkv + qd, s->qkv + qd + d.n_kv_heads * d.head_dim, s->qkv_dim,
                                 -1, 0, rps, kv_flags, s->st, 0, B, st));
         }
-        if (attn_tc) RC(launch_verify_attn_tc(s->kg, L.kc, L.vc, s->qkv, B, rps, d.n_q_heads, np_cols, s->st, s->asc, s->attn, status, st));
-        else RC(launch_verify_attn(s->kg, L.kc, L.vc, s->qkv, B, rps, d.n_q_heads, s->st, s->asc, s->attn, st));
+        if (attn_tc)
+            RC(launch_verify_attn_tc(s->kg, L.kc, L.vc, s->qkv, B, attn_all_rows(rps, ceil_div(d.max_seq, 2 * kAttnChunk)), 0, d.n_q_heads,
+                                     np_cols, s->st, s->asc, s->attn, status, st));
+        else
+            RC(launch_verify_attn(s->kg, L.kc, L.vc, s->qkv, B, attn_all_rows(rps, ceil_div(d.max_seq, kAttnChunk)), d.n_q_heads, s->st,
+                                  s->asc, s->attn, st));
         if (calib) RC(launch_calib_accum(s->attn, rows, qd, L.calib[1], s->st, st));
         RC(launch_verify_gemm(weight(L.w.wo, L.blob[1], L.bi[1], L.vdata[1]), s->attn, rows, bn, d.hidden, qd, s->vg_partial, nullptr, nullptr, status, st, s->from_parts ? 0 : 1));
         RC(launch_residual_rmsnorm(s->h, nullptr, vparts(d.hidden, qd), (const uint16_t*)L.w.norm_ffn, s->xn,
@@ -496,6 +520,97 @@ extern "C" int cass_verify(void* session, const int32_t* toks, int g, int32_t* t
     return w_rc;
 }
 
+// Attention of a prefill pass: w rows of every sequence at positions pos .. pos + w - 1.  fine: rows whose probabilities are
+// kept in two terms (see launch_verify_attn_tc).
+static int prefill_attention(Session* s, const LayerDev& L, int pos, int w, int fine, cudaStream_t st) {
+    const cass_model_desc& d = s->d;
+    const bool tc = !simt_verify_attn() && verify_attn_tc_usable(s->kg, 1, d.n_q_heads);
+    const int tok = tc ? 2 * kAttnChunk : kAttnChunk, grp = d.n_q_heads / d.n_kv_heads;
+    // rows a CTA: what 64 pair columns hold, 16 at most (more would leave the long passes of few heads without CTAs)
+    int group = 16;
+    while (tc && group * grp > 64) group /= 2;
+    for (int lo = 0; lo < w;) {
+        // as many rows as the scratch holds at this context
+        int take = w - lo;
+        auto fits = [&](int rows) { return (size_t)rows * s->B * d.n_q_heads * ceil_div(pos + lo + rows, tok) <= s->attn_parts; };
+        while (take > 1 && !fits(take)) take = take > group ? (take - 1) / group * group : take / 2;
+        const AttnRows ar{w, lo, lo + take, group < take ? group : take, ceil_div(pos + lo + take, tok)};
+        if (tc) RC(launch_verify_attn_tc(s->kg, L.kc, L.vc, s->pqkv, s->B, ar, fine, d.n_q_heads, 64, s->st, s->asc, s->pattn, &s->st->status, st));
+        else RC(launch_verify_attn(s->kg, L.kc, L.vc, s->pqkv, s->B, ar, d.n_q_heads, s->st, s->asc, s->pattn, st));
+        lo += take;
+    }
+    return CASS_OK;
+}
+
+// The prompt in passes of kPrefillRows rows over all sequences: every pass reads the weights once for its rows (16 rows a
+// pass, as verification takes them, read them 8 times as often: 51.8 ms instead of 5.5 ms for 1000 tokens of four
+// 8B-shaped layers), and lm_head runs once.  A row's result is what cass_verify gives for it: the same K ranges, added in
+// the same order.
+extern "C" int cass_prefill(void* session, const int32_t* toks, int n, int32_t* target_argmax, void* stream_) {
+    if (!session || !toks || !target_argmax) return CASS_ERR_INVALID_ARG;
+    Session* s = (Session*)session;
+    const cass_model_desc& d = s->d;
+    const int B = s->B, qd = d.n_q_heads * d.head_dim, kvd = d.n_kv_heads * d.head_dim, grp = d.n_q_heads / d.n_kv_heads;
+    if (n < 1 || n + kMaxVerifyRows > d.max_seq) return CASS_ERR_INVALID_ARG;
+    cudaStream_t st = (cudaStream_t)stream_;
+    int32_t* status = &s->st->status;
+    const int w_max = kPrefillRows / B, chunk = kMaxVerifyRows < s->R / B ? kMaxVerifyRows : s->R / B;
+    // rows that calls of `chunk` rows would give to the fp32-pipe attention keep its accuracy
+    auto tc_rows = [&](int rps) { return verify_attn_tc_usable(s->kg, rps <= d.gamma_max + 1 ? d.gamma_max + 1 : rps, d.n_q_heads); };
+    const int rest = n % chunk;
+    const int fine = tc_rows(chunk) || n < chunk ? 0 : (rest && tc_rows(rest) ? n - rest : n);
+    const int kv_flags = CASS_KV_BF16 | (s->codebooks_ready ? CASS_KV_COMPRESSED : 0);
+    const bool calib = s->calib_host;
+    int w_rc = CASS_OK;
+    auto weight = [&](const void* bf16, const void* blob, const cass_blob_info& bi, const void* vd) -> const uint16_t* {
+        if (!s->from_parts) return (const uint16_t*)bf16;
+        const int rc = cass_decode_full(blob, &bi, vd, s->vscratch, stream_);
+        if (rc) w_rc = rc;
+        return s->vscratch;
+    };
+    const int w_static = s->from_parts ? 0 : 1;
+    int w = 0;
+    for (int pos = 0; pos < n; pos += w) {
+        w = n - pos < w_max ? n - pos : w_max;
+        const int rows = B * w, bn = verify_gemm_bn(rows);
+        auto parts = [&](int nn, int k) { return verify_gemm_partials(s->vg_partial, nn, k, bn); };
+        RC(launch_set_len(s->st, pos, st));
+        RC(launch_embed(toks + pos, w, n, (const uint16_t*)s->embed, s->ph, rows, d.hidden, st));
+        RC(launch_rmsnorm(s->ph, (const uint16_t*)s->layers[0].w.norm_attn, s->pxn, rows, d.hidden, d.rms_eps, st));
+        for (int l = 0; l < d.n_layers; ++l) {
+            LayerDev& L = s->layers[l];
+            if (calib) RC(launch_calib_accum(s->pxn, rows, d.hidden, L.calib[0], s->st, st));
+            RC(launch_verify_gemm(weight(L.w.wqkv, L.blob[0], L.bi[0], L.vdata[0]), s->pxn, rows, bn, s->qkv_dim, d.hidden, s->vg_partial, nullptr, nullptr, status, st, w_static));
+            RC(launch_qkv_rope(s->pqkv, parts(s->qkv_dim, d.hidden), s->cos_t, s->sin_t, s->st, 0, rows, w, d.n_q_heads, d.n_kv_heads, d.head_dim, st));
+            RC(launch_kv_span(s->kg, L.ck, L.cv, L.kc, L.vc, s->pqkv + qd, s->pqkv + qd + kvd, s->qkv_dim, pos, w, kv_flags, s->st, 0, B, st));
+            RC(prefill_attention(s, L, pos, w, fine - pos, st));
+            if (calib) RC(launch_calib_accum(s->pattn, rows, qd, L.calib[1], s->st, st));
+            RC(launch_verify_gemm(weight(L.w.wo, L.blob[1], L.bi[1], L.vdata[1]), s->pattn, rows, bn, d.hidden, qd, s->vg_partial, nullptr, nullptr, status, st, w_static));
+            RC(launch_residual_rmsnorm(s->ph, nullptr, parts(d.hidden, qd), (const uint16_t*)L.w.norm_ffn, s->pxn, rows, d.hidden, d.rms_eps, st));
+            if (calib) RC(launch_calib_accum(s->pxn, rows, d.hidden, L.calib[2], s->st, st));
+            RC(launch_verify_gemm(weight(L.w.wgu, L.blob[2], L.bi[2], L.vdata[2]), s->pxn, rows, bn, 2 * d.ffn, d.hidden, s->vg_partial, nullptr, nullptr, status, st, w_static));
+            RC(launch_swiglu(nullptr, parts(2 * d.ffn, d.hidden), s->pact, rows, d.ffn, st));
+            if (calib) RC(launch_calib_accum(s->pact, rows, d.ffn, L.calib[3], s->st, st));
+            RC(launch_verify_gemm(weight(L.w.wd, L.blob[3], L.bi[3], L.vdata[3]), s->pact, rows, bn, d.hidden, d.ffn, s->vg_partial, nullptr, nullptr, status, st, w_static));
+            const uint16_t* next_gain = (const uint16_t*)(l + 1 < d.n_layers ? s->layers[l + 1].w.norm_attn : s->norm_final);
+            RC(launch_residual_rmsnorm(s->ph, nullptr, parts(d.hidden, d.ffn), next_gain, s->pxn, rows, d.hidden, d.rms_eps, st));
+        }
+        if (calib) RC(launch_calib_accum(s->pxn, rows, d.hidden, s->calib_lm, s->st, st));
+    }
+    // each sequence's last rows where a verification call leaves its own (cass_debug_activation), and the last one through lm_head
+    const int last = (n - 1) % chunk + 1;
+    RC(launch_last_rows(s->ph, B, w, last, d.hidden, s->h, st));
+    RC(launch_last_rows(s->pqkv, B, w, last, s->qkv_dim, s->qkv, st));
+    RC(launch_last_rows(s->pattn, B, w, last, qd, s->attn, st));
+    RC(launch_last_rows(s->pxn, B, w, 1, d.hidden, s->xn, st));
+    RC(launch_verify_gemm(weight(s->lm_head, s->lm_blob, s->lm_bi, s->lm_vdata), s->xn, B, s->R, d.vocab, d.hidden, s->vg_partial, nullptr, nullptr, status, st, w_static));
+    RC(launch_argmax(nullptr, verify_gemm_partials(s->vg_partial, d.vocab, d.hidden, s->R), B, d.vocab, target_argmax, 1, nullptr,
+                     s->argmax_val, s->argmax_tmp, s->st, 0, st));
+    RC(launch_set_len(s->st, n, st));
+    s->drafts_pending = 0;
+    return w_rc;
+}
+
 extern "C" int cass_draft_step(void* session, const int32_t* tok_in, int32_t* tok_out, int tok_stride, float* logits_opt,
                                void* stream_) {
     if (!session || !tok_in || !tok_out || tok_stride < 1) return CASS_ERR_INVALID_ARG;
@@ -512,7 +627,7 @@ extern "C" int cass_draft_step(void* session, const int32_t* tok_in, int32_t* to
     const int B = s->B;
     auto draftp = [&](const cass_blob_info& b) { return draft_gemv_partials(s->partial, b); };
     const bool fused = rope_kv_fusable(s->kg);
-    RC(launch_embed(tok_in, tok_stride, (const uint16_t*)s->embed, s->h, B, d.hidden, st));
+    RC(launch_embed(tok_in, 1, tok_stride, (const uint16_t*)s->embed, s->h, B, d.hidden, st));
     RC(launch_rmsnorm(s->h, (const uint16_t*)s->layers[0].w.norm_attn, s->xn, B, d.hidden, d.rms_eps, st));
     for (int l = 0; l < d.n_layers; ++l) {
         LayerDev& L = s->layers[l];

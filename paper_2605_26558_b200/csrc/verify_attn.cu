@@ -13,16 +13,18 @@ constexpr int kVaMaxGroup = 8;
 constexpr int kVaMaxPairs = kVaRowBatch * kVaMaxGroup;      // (row, query head) pairs handled at a time
 constexpr int kVaHalfPairs = kVaMaxPairs / 2;
 
-// grid (chunk, KV head, sequence); `rows` = rows of each sequence in this call.
+// grid (chunk, KV head, sequence x row group)
 __global__ void __launch_bounds__(kVaThreads) k_verify_attn(KvGeom g, const uint16_t* __restrict__ k_cache0,
                                                             const uint16_t* __restrict__ v_cache0, const uint16_t* __restrict__ qkv0,
-                                                            int rows, int n_q, const DevState* __restrict__ st, AttnScratch sc,
-                                                            int n_chunks_alloc) {
+                                                            AttnRows ar, int n_groups, int n_q, const DevState* __restrict__ st,
+                                                            AttnScratch sc) {
     extern __shared__ __align__(16) uint8_t smem[];
     pdl_early<4>();
     pdl_wait();
-    const int chunk = blockIdx.x, head = blockIdx.y, seq = blockIdx.z;
-    const int len = st->len[seq];
+    const int chunk = blockIdx.x, head = blockIdx.y, seq = blockIdx.z / n_groups;
+    const int first = ar.lo + (int)(blockIdx.z % n_groups) * ar.group;            // the group's rows: row r of it sits at position len + r
+    const int rows = min(ar.group, ar.hi - first);
+    const int len = st->len[seq] + first;
     const uint16_t* __restrict__ k_cache = of_seq(k_cache0, seq, g.seq_stride);
     const uint16_t* __restrict__ v_cache = of_seq(v_cache0, seq, g.seq_stride);
     const int t0 = chunk * kAttnChunk;
@@ -30,7 +32,7 @@ __global__ void __launch_bounds__(kVaThreads) k_verify_attn(KvGeom g, const uint
     const int d = g.d, G = n_q / g.n_kv, ks = d + 8;                  // padded K row stride (elements)
     const int qkv_dim = (n_q + 2 * g.n_kv) * d;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint16_t* __restrict__ qkv = qkv0 + (size_t)seq * rows * qkv_dim;     // this sequence's rows
+    const uint16_t* __restrict__ qkv = qkv0 + ((size_t)seq * ar.rps + first) * qkv_dim;     // the group's rows
     uint16_t* k_s = reinterpret_cast<uint16_t*>(smem);                         // [64][d+8]
     uint16_t* v_s = k_s + kAttnChunk * ks;                                      // [64][d]
     float* q_s = reinterpret_cast<float*>(v_s + kAttnChunk * d);                // [pairs][d]
@@ -108,7 +110,7 @@ __global__ void __launch_bounds__(kVaThreads) k_verify_attn(KvGeom g, const uint
             s_s[p * kAttnChunk + 32 + lane] = b;
             const float l = warp_sum(a + b);
             __syncwarp();
-            const size_t pair = ((size_t)seq * rows + r) * n_q + head * G + gi;
+            const size_t pair = ((size_t)seq * (ar.hi - ar.lo) + first - ar.lo + r) * n_q + head * G + gi;
             for (int dim = lane * 4; dim < d; dim += 128) {             // four dims per lane, tokens in order
                 float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll 4
@@ -120,25 +122,22 @@ __global__ void __launch_bounds__(kVaThreads) k_verify_attn(KvGeom g, const uint
                     a2 = fmaf(pr, __uint_as_float(vv.y << 16), a2);
                     a3 = fmaf(pr, __uint_as_float(vv.y & 0xFFFF0000u), a3);
                 }
-                *reinterpret_cast<float4*>(sc.o + (pair * n_chunks_alloc + chunk) * d + dim) = make_float4(a0, a1, a2, a3);
+                *reinterpret_cast<float4*>(sc.o + (pair * ar.chunks + chunk) * d + dim) = make_float4(a0, a1, a2, a3);
             }
             if (lane == 0) {
-                sc.m[pair * n_chunks_alloc + chunk] = m;
-                sc.l[pair * n_chunks_alloc + chunk] = l;
+                sc.m[pair * ar.chunks + chunk] = m;
+                sc.l[pair * ar.chunks + chunk] = l;
             }
         }
     }
 }
 
-int launch_attn_merge(const AttnScratch& sc, int n_chunks_alloc, int chunk_tokens, int rows, int rps, int n_q, int d,
-                      const DevState* st, int draft_mode, int draft_units, uint16_t* out, cudaStream_t s);
-
 int launch_verify_attn(const KvGeom& g, const uint16_t* k_cache, const uint16_t* v_cache, const uint16_t* qkv, int n_seq,
-                       int rps, int n_q, const DevState* st, const AttnScratch& sc, uint16_t* out, cudaStream_t s) {
+                       const AttnRows& ar, int n_q, const DevState* st, const AttnScratch& sc, uint16_t* out, cudaStream_t s) {
     const int G = n_q / g.n_kv;
     if (G > kVaMaxGroup || g.d % 8) return CASS_ERR_UNSUPPORTED;
     static_assert(kAttnChunk == 64 && kVaThreads == 2 * kAttnChunk, "thread = (token, half of the pairs)");
-    const int n_chunks = ceil_div(g.max_seq, kAttnChunk);
+    const int n_groups = ceil_div(ar.hi - ar.lo, ar.group);
     size_t smem = (size_t)kAttnChunk * (g.d + 8) * 2 + (size_t)kAttnChunk * g.d * 2 + (size_t)kVaMaxPairs * g.d * 4 +
                   (size_t)kVaMaxPairs * kAttnChunk * 4;
     static size_t attr = 0;
@@ -146,9 +145,9 @@ int launch_verify_attn(const KvGeom& g, const uint16_t* k_cache, const uint16_t*
         CASS_CUDA_CHECK(cudaFuncSetAttribute(k_verify_attn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr = smem;
     }
-    dim3 grid(n_chunks, g.n_kv, n_seq);
-    CASS_PDL_LAUNCH(k_verify_attn, grid, dim3(kVaThreads), smem, s, g, k_cache, v_cache, qkv, rps, n_q, st, sc, n_chunks);
-    return launch_attn_merge(sc, n_chunks, kAttnChunk, n_seq * rps, rps, n_q, g.d, st, 0, 0, out, s);
+    dim3 grid(ar.chunks, g.n_kv, n_seq * n_groups);
+    CASS_PDL_LAUNCH(k_verify_attn, grid, dim3(kVaThreads), smem, s, g, k_cache, v_cache, qkv, ar, n_groups, n_q, st, sc);
+    return launch_attn_merge(sc, kAttnChunk, n_seq, ar, n_q, g.d, st, 0, 0, out, s);
 }
 
 }  // namespace cass

@@ -8,7 +8,9 @@
 // swizzled layout.  The V tile is used as it lies in memory (rows = tokens), i.e. as an M-contiguous A operand.
 // Chunk results (o, running maximum m, sum l) go to the split-K scratch and k_attn_merge combines the chunks, as for
 // the SIMT kernel.  A (row, head) pair is one accumulator column, so its result does not depend on the other rows.
-// Needs head_dim = 128 and rows x group <= 64; other shapes use k_verify_attn.
+// Needs head_dim = 128 and rows x group <= 64; other shapes use k_verify_attn.  More rows than that (prefill) are cut into
+// groups, one CTA each; where the fp32-pipe kernel would have taken them 16 at a time, P is kept as two bf16 terms and the
+// second product runs twice, so that the accuracy is that kernel's.
 #include "tc.cuh"
 #include "kernels.cuh"
 
@@ -22,7 +24,7 @@ constexpr int kVtTileBytes = kVtTok * 64 * 2;          // one TMA box: 128 token
 constexpr int vt_q_bytes(int np) { return np * 64 * 2; }               // one K-block of the Q or P operand: NP rows x 64 elements
 // K tiles (32 KB) | V tiles (32 KB) | Q (2 blocks) | [P (2 blocks) when np = 64] | barriers.  The scores (np x 128
 // floats) reuse the K tiles' memory, and with np = 32 so does P: both are written only after the first product has
-// finished reading K.
+// finished reading K.  The low term of P takes Q's place.
 constexpr int vt_smem(int np) { return 4 * kVtTileBytes + (np == 32 ? 2 : 4) * vt_q_bytes(np) + 256 + 1024; }
 static_assert(32 * kVtTok * 4 + 2 * vt_q_bytes(32) <= 2 * kVtTileBytes && 64 * kVtTok * 4 <= 2 * kVtTileBytes, "scores (and P) fit the K tiles");
 constexpr int vt_tmem_cols(int np) { return 2 * np; }                  // scores^T in columns 0..NP-1, out^T in columns NP..2NP-1
@@ -50,14 +52,17 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
 template <int NP>
 __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_constant__ CUtensorMap map_k,
                                                                 const __grid_constant__ CUtensorMap map_v,
-                                                                const uint16_t* __restrict__ qkv, int rows, int n_q, int n_kv,
-                                                                const DevState* __restrict__ st, AttnScratch sc, int n_chunks_alloc,
+                                                                const uint16_t* __restrict__ qkv, AttnRows ar, int n_groups, int fine,
+                                                                int n_q, int n_kv, const DevState* __restrict__ st, AttnScratch sc,
                                                                 int32_t* __restrict__ d_status) {
     extern __shared__ uint8_t smem_dyn[];
     pdl_early<4>();
     pdl_wait();
-    const int chunk = blockIdx.x, head = blockIdx.y, seq = blockIdx.z;
-    const int len = st->len[seq];
+    const int chunk = blockIdx.x, head = blockIdx.y, seq = blockIdx.z / n_groups;
+    const int first = ar.lo + (int)(blockIdx.z % n_groups) * ar.group;        // the group's rows: row r of it sits at position len + r
+    const int rows = min(ar.group, ar.hi - first);
+    const bool two_terms = first < fine;
+    const int len = st->len[seq] + first;
     const int t0 = chunk * kVtTok;
     if (t0 >= len + rows) return;                              // no row of this call sees the chunk
     constexpr int kVtPairs = NP, kVtQBytes = vt_q_bytes(NP), kVtTmemCols = vt_tmem_cols(NP);
@@ -73,6 +78,10 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
     uint64_t* bar_p = bar_k + 3;       // P written to shared memory (128 arrivals)
     uint64_t* bar_o = bar_k + 4;       // output complete in tensor memory
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_k + 5);
+    // per pair: the last position it sees (-1: no such pair), and its place in the scratch; divisions by the group size and
+    // 64-bit products for every pair and thread took most of the instructions
+    __shared__ __align__(16) int s_lim[NP];
+    __shared__ __align__(16) uint32_t s_at[NP];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int G = n_q / n_kv, P = rows * G;
@@ -92,10 +101,15 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kVtTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    if (warp == 1)
+        for (int p = lane; p < NP; p += 32) {
+            s_lim[p] = p < P ? len + p / G : -1;
+            s_at[p] = (uint32_t)((((size_t)seq * (ar.hi - ar.lo) + first - ar.lo + p / G) * n_q + head * G + p % G) * ar.chunks + chunk);
+        }
     if (warp >= 2) {
         // Q of this sequence's rows and this group's heads -> sQ (pair p = row * G + head-in-group), zero beyond P
         const int et = tid - 64;
-        const uint16_t* q0 = qkv + (size_t)seq * rows * qkv_dim + (size_t)head * G * kVtD;
+        const uint16_t* q0 = qkv + ((size_t)seq * ar.rps + first) * qkv_dim + (size_t)head * G * kVtD;
         for (int i = et; i < kVtPairs * (kVtD / 8); i += 128) {
             const int p = i / (kVtD / 8), c8 = i % (kVtD / 8);           // 8 dims = 16 bytes per item
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -138,6 +152,8 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
                 // B: block kk / 4 of P (64 tokens each), 32 bytes per 16 tokens inside the swizzled row
                 const uint64_t bd = tc_smem_desc(sP + (kk >> 2) * kVtQBytes) + (uint64_t)((kk & 3) * 2);
                 tc_mma(tmem + (uint32_t)NP, ad, bd, idesc2, (uint32_t)(kk != 0));
+                if (two_terms)
+                    tc_mma(tmem + (uint32_t)NP, ad, tc_smem_desc(sQ + (kk >> 2) * kVtQBytes) + (uint64_t)((kk & 3) * 2), idesc2, 1u);
             }
         } else if (ok) {
             atomicExch(d_status, CASS_ERR_TIMEOUT);
@@ -159,12 +175,13 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
                 const int p = c0 + i;
-                const bool vis = have && p < P && (t0 + et) <= len + p / G;
+                const bool vis = have && (t0 + et) <= s_lim[p];
                 sS[p * kVtTok + et] = vis ? __uint_as_float(v[i]) * scale : -INFINITY;
             }
         }
         named_sync_128();
         // chunk softmax of every pair (warp q: pairs q, q + 4, ...), numerators rounded to bf16 into the P operand
+#pragma unroll 2
         for (int p = q; p < kVtPairs; p += 4) {
             float a[4];
 #pragma unroll
@@ -175,15 +192,20 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
             for (int k = 0; k < 4; ++k) {
                 const float e = (m == -INFINITY) ? 0.f : expf(a[k] - m);
                 const uint16_t eb = float_to_bf16_bits(e);
-                l += bf16_bits_to_float(eb);                  // the sum of what the MMA multiplies
                 const int t = lane + 32 * k;
+                float used = bf16_bits_to_float(eb);
+                if (two_terms) {                              // Q has been consumed: the remainder goes there
+                    const uint16_t lo = float_to_bf16_bits(e - used);
+                    used += bf16_bits_to_float(lo);
+                    *reinterpret_cast<uint16_t*>(sQ + (t >> 6) * kVtQBytes + swz_off(p, t & 63)) = lo;
+                }
+                l += used;                                    // the sum of what the MMA multiplies
                 *reinterpret_cast<uint16_t*>(sP + (t >> 6) * kVtQBytes + swz_off(p, t & 63)) = eb;
             }
             l = warp_sum(l);
-            if (lane == 0 && p < P && t0 <= len + p / G) {
-                const size_t pair = ((size_t)seq * rows + p / G) * n_q + head * G + p % G;
-                sc.m[pair * n_chunks_alloc + chunk] = m;
-                sc.l[pair * n_chunks_alloc + chunk] = l;
+            if (lane == 0 && t0 <= s_lim[p]) {
+                sc.m[s_at[p]] = m;
+                sc.l[s_at[p]] = l;
             }
         }
         fence_proxy_async();
@@ -197,10 +219,7 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
                     const int p = c0 + i;
-                    if (p < P && t0 <= len + p / G) {
-                        const size_t pair = ((size_t)seq * rows + p / G) * n_q + head * G + p % G;
-                        sc.o[(pair * n_chunks_alloc + chunk) * kVtD + et] = __uint_as_float(v[i]);
-                    }
+                    if (t0 <= s_lim[p]) sc.o[(size_t)s_at[p] * kVtD + et] = __uint_as_float(v[i]);
                 }
             }
         } else {
@@ -215,18 +234,15 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
     }
 }
 
-int launch_attn_merge(const AttnScratch& sc, int n_chunks_alloc, int chunk_tokens, int rows, int rps, int n_q, int d,
-                      const DevState* st, int draft_mode, int draft_units, uint16_t* out, cudaStream_t s);
-
 bool verify_attn_tc_usable(const KvGeom& g, int rps, int n_q) {
     return g.d == kVtD && rps * (n_q / g.n_kv) <= kVtMaxPairs && (g.seq_stride % 16) == 0;
 }
 
 // caches: sequence 0's bf16 K and V of one layer ([max_seq][n_kv][128]); the other sequences lie seq_stride bytes apart.
 int launch_verify_attn_tc(const KvGeom& g, const uint16_t* k_cache, const uint16_t* v_cache, const uint16_t* qkv, int n_seq,
-                          int rps, int n_q, int np_cols, const DevState* st, const AttnScratch& sc, uint16_t* out,
+                          const AttnRows& ar, int fine, int n_q, int np_cols, const DevState* st, const AttnScratch& sc, uint16_t* out,
                           int32_t* d_status, cudaStream_t s) {
-    if (!verify_attn_tc_usable(g, rps, n_q) || (np_cols != 32 && np_cols != 64) || rps * (n_q / g.n_kv) > np_cols)
+    if (!verify_attn_tc_usable(g, ar.group, n_q) || (np_cols != 32 && np_cols != 64) || ar.group * (n_q / g.n_kv) > np_cols)
         return CASS_ERR_UNSUPPORTED;
     EncodeTiledFn fn = encode_fn();
     if (!fn) return CASS_ERR_CUDA;
@@ -241,26 +257,26 @@ int launch_verify_attn_tc(const KvGeom& g, const uint16_t* k_cache, const uint16
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return CASS_ERR_INVALID_ARG;
     }
-    const int n_chunks = ceil_div(g.max_seq, kVtTok);
-    dim3 grid(n_chunks, g.n_kv, n_seq);
+    const int n_groups = ceil_div(ar.hi - ar.lo, ar.group);
+    dim3 grid(ar.chunks, g.n_kv, n_seq * n_groups);
     if (np_cols == 32) {
         static bool attr = false;
         if (!attr) {
             CASS_CUDA_CHECK(cudaFuncSetAttribute(k_verify_attn_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, vt_smem(32)));
             attr = true;
         }
-        CASS_PDL_LAUNCH(k_verify_attn_tc<32>, grid, dim3(kVtThreads), (size_t)vt_smem(32), s, mk, mv, qkv, rps, n_q, g.n_kv, st, sc,
-                        n_chunks, d_status);
+        CASS_PDL_LAUNCH(k_verify_attn_tc<32>, grid, dim3(kVtThreads), (size_t)vt_smem(32), s, mk, mv, qkv, ar, n_groups, fine, n_q,
+                        g.n_kv, st, sc, d_status);
     } else {
         static bool attr = false;
         if (!attr) {
             CASS_CUDA_CHECK(cudaFuncSetAttribute(k_verify_attn_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, vt_smem(64)));
             attr = true;
         }
-        CASS_PDL_LAUNCH(k_verify_attn_tc<64>, grid, dim3(kVtThreads), (size_t)vt_smem(64), s, mk, mv, qkv, rps, n_q, g.n_kv, st, sc,
-                        n_chunks, d_status);
+        CASS_PDL_LAUNCH(k_verify_attn_tc<64>, grid, dim3(kVtThreads), (size_t)vt_smem(64), s, mk, mv, qkv, ar, n_groups, fine, n_q,
+                        g.n_kv, st, sc, d_status);
     }
-    return launch_attn_merge(sc, n_chunks, kVtTok, n_seq * rps, rps, n_q, g.d, st, 0, 0, out, s);
+    return launch_attn_merge(sc, kVtTok, n_seq, ar, n_q, g.d, st, 0, 0, out, s);
 }
 
 }  // namespace cass

@@ -2,7 +2,7 @@
 // memory-bound on the bf16 weights): Y[r][n] = sum_k W[n][k] X[r][k], bf16 operands, fp32 accumulation.
 //
 // tcgen05 version, "swap-AB": the weights are the M operand (128 output features per CTA), the token rows the N
-// operand (padded to BN = 16, 32 or 64 columns), the accumulator lives in tensor memory.  One CTA = one 128-feature tile x
+// operand (padded to BN = 16, 32, 64 or, in a prefill, 128 columns), the accumulator lives in tensor memory.  One CTA = one 128-feature tile x
 // one K range (split-K so that small matrices still fill the GPU); warp 0 streams 128x64 weight tiles and the
 // BNx64 activation tile through a ring of TMA loads (128-byte swizzle), warp 1 issues the MMAs, warps 2-5 read the
 // accumulator back and store fp32 partial sums; a second kernel adds the K ranges in fixed order.
@@ -15,12 +15,12 @@
 namespace cass {
 
 constexpr int kTcBM = 128, kTcBK = 64;
-constexpr int tc_stages(int bn) { return bn <= 16 ? 6 : bn <= 32 ? 5 : 4; }      // two CTAs per SM at every bn
+constexpr int tc_stages(int bn) { return bn <= 16 ? 6 : bn <= 32 ? 5 : bn <= 64 ? 4 : 3; }      // two CTAs per SM at every bn
 constexpr int kTcABytes = kTcBM * kTcBK * 2;
 constexpr int kTcThreads = 192;
 constexpr int tc_b_bytes(int bn) { return bn * kTcBK * 2; }
 constexpr int tc_smem(int bn) { return tc_stages(bn) * (kTcABytes + tc_b_bytes(bn)) + 256 + 1024; }     // + barriers + alignment slack
-constexpr int tc_tmem_cols(int bn) { return bn <= 32 ? 32 : 64; }                                   // a power of two >= 32
+constexpr int tc_tmem_cols(int bn) { return bn <= 32 ? 32 : bn; }                                   // a power of two >= 32
 
 // bf16 matrix [rows][cols] row-major -> map with a (box_rows x 64)-element box, 128-byte swizzle, zero fill outside.
 static int make_map(CUtensorMap* m, const void* ptr, int rows, int cols, int box_rows) {
@@ -215,7 +215,7 @@ static int launch_tc(const CUtensorMap& mw, const CUtensorMap& mx, float* partia
 
 int launch_verify_gemm(const uint16_t* W, const uint16_t* X, int rows, int bn, int n, int k, float* partial, uint16_t* y_bf16,
                        float* y_f32, int32_t* d_status, cudaStream_t s, int w_static) {
-    if (rows < 1 || rows > bn || (bn != 16 && bn != 32 && bn != 64) || (k % 8) || n < 1 || !partial || !d_status)
+    if (rows < 1 || rows > bn || (bn != 16 && bn != 32 && bn != 64 && bn != 128) || (k % 8) || n < 1 || !partial || !d_status)
         return CASS_ERR_INVALID_ARG;
     if (((uintptr_t)W & 15) || ((uintptr_t)X & 15)) return CASS_ERR_INVALID_ARG;
     CUtensorMap mw, mx;
@@ -227,6 +227,7 @@ int launch_verify_gemm(const uint16_t* W, const uint16_t* X, int rows, int bn, i
     split_plan(n, k, &kbt, &kbs, &ns);
     if (bn == 16) rc = launch_tc<16>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
     else if (bn == 32) rc = launch_tc<32>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
+    else if (bn == 128) rc = launch_tc<128>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
     else rc = launch_tc<64>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
     if (rc) return rc;
     if (!y_bf16 && !y_f32) return CASS_OK;          // the caller's next kernel adds the parts itself

@@ -81,23 +81,15 @@ class Engine:
         self.n_prompt = 0
 
     def prefill(self, prompt: torch.Tensor, calibrate: bool = False):
-        """Target pass over the prompt(s) ([n] or [batch][n] token ids, equal lengths) in chunks of up to 16 rows per
-        sequence (bf16 cache only); returns the first generated token (per sequence).  With calibrate, the Wanda
-        activation statistics are accumulated on the way."""
+        """Target pass over the prompt(s) ([n] or [batch][n] token ids, equal lengths; bf16 cache only); returns the first
+        generated token (per sequence).  With calibrate, the Wanda activation statistics are accumulated on the way."""
         prompt = prompt.to(self.device, torch.int32).reshape(self.batch, -1).contiguous()
         n = int(prompt.shape[1])
-        chunk = min(16, self.max_rows // self.batch)
         B.cass_calib_enable(self.session, calibrate)
-        pos, rows = 0, 0
-        while pos < n:
-            rows = min(chunk, n - pos)
-            B.cass_set_len(self.session, pos)
-            B.cass_verify(self.session, prompt[:, pos: pos + rows].contiguous(), rows - 1, self.targ)
-            pos += rows
+        B.cass_prefill(self.session, prompt, n, self.targ)
         B.cass_calib_enable(self.session, False)
-        B.cass_set_len(self.session, n)
         self.n_prompt = n
-        first = self.targ[: self.batch * rows].view(self.batch, rows)[:, rows - 1].clone()
+        first = self.targ[: self.batch].clone()
         self._stride = 1
         self.toks[: self.batch] = first
         return int(first[0].item()) if self.batch == 1 else first.tolist()
