@@ -1,6 +1,6 @@
 // Verification data (Sec. 4.1 target inference, Sec. 5.1 encoder): what the Cassandra-1 speculation data leaves out
 // -- the low t mantissa bits of the kept values and the pruned values as they are -- and the exact reconstruction
-// of the bf16 matrix from the two parts (k_decode_full).  A session told to verify from the two parts
+// of the bf16 matrix from the two parts (k_join).  A session told to verify from the two parts
 // (cass_session_verify_from_parts) rebuilds every matrix with it right before the verification GEMM reads it.
 //
 // Layout: header of 8 words {magic 'CASV', 1, rows, cols, kept per row, t, words per row, 0}; per row
@@ -17,157 +17,320 @@ constexpr int kVdataHeaderWords = 8;
 __host__ __device__ inline int vdata_lo_words(int kept, int t) { return (kept * t + 31) / 32; }
 __host__ __device__ inline int vdata_row_words(int cols, int kept, int t) { return vdata_lo_words(kept, t) + (cols - kept + 1) / 2; }
 
-// Bitmap word j (32 columns) of `row` inside the blob: superblock (row / 32, segment), bitmap section, interleaved.
-__device__ __forceinline__ uint32_t blob_bitmap_word(const uint32_t* __restrict__ blob, int row, int j, int seg_cols, int n_seg,
-                                                     int k_pad) {
-    const int seg = (j * 32) / seg_cols, jj = j - seg * (seg_cols / 32);
-    const uint32_t* dir = blob + kBlobDirOffset / 4 + ((row / kRowsPerBlock) * n_seg + seg) * 4;
-    const SbGeom g = SbGeom::make(dir_n_ch(dir[3]), seg_cols_of(k_pad, seg_cols, seg), (int)dir[1], (int)dir[2]);
-    return blob[(size_t)dir[0] * 4 + g.bm + jj * 32 + (row % kRowsPerBlock)];
-}
+// Verification data of a row by one warp, 256 columns at a time, 8 a lane.  Pruned values go straight to their places; the
+// low bits of kept values are collected in a ring and leave 8 values (t bytes) a lane.  Bound: latency and issue (about 80
+// instructions a lane and 8 columns); one column a lane with two global atomics a kept value took 307 us for a
+// 2825 x 11733 matrix.
+constexpr int kSplitWarps = 8;
+constexpr int kSplitRing = 512;
 
-// One warp per row.  ENCODE: W -> verification data.  otherwise: W_out (holding the draft reconstruction) |= low bits,
-// pruned positions <- raw values.
-template <bool ENCODE>
-__global__ void __launch_bounds__(256) k_vdata(const uint32_t* __restrict__ blob, const uint16_t* __restrict__ W,
-                                               uint32_t* __restrict__ vdata, uint16_t* __restrict__ W_out) {
-    const int n = blob[H_ROWS], k = blob[H_COLS], t = blob[H_T], seg_cols = blob[H_SEG], n_seg = blob[H_NSEG];
-    const int kept = blob[H_KEPT], k_pad = ceil_div(k, 32) * 32;
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(32 * kSplitWarps) k_split(const uint32_t* __restrict__ blob, const uint16_t* __restrict__ W,
+                                                            uint32_t* __restrict__ vdata, int n, int k, int kept, int t, int seg_cols,
+                                                            int n_seg) {
+    __shared__ __align__(8) uint8_t s_low[kSplitWarps][kSplitRing];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row = blockIdx.x * kSplitWarps + warp, k_pad = ceil_div(k, 32) * 32;
+    pdl_wait();
     if (row >= n) return;
     const int lo_words = vdata_lo_words(kept, t), row_words = vdata_row_words(k, kept, t);
     uint32_t* lo = vdata + kVdataHeaderWords + (size_t)row * row_words;
     uint16_t* raw = reinterpret_cast<uint16_t*>(lo + lo_words);
-    if (ENCODE) {
-        for (int w = lane; w < row_words; w += 32) lo[w] = 0u;
-        __syncwarp();
-    }
-    uint32_t k_base = 0, p_base = 0;
-    for (int j = 0; j < k_pad / 32; ++j) {
-        const uint32_t bm = blob_bitmap_word(blob, row, j, seg_cols, n_seg, k_pad);
-        const int c = j * 32 + lane;
-        const bool in = c < k, is_kept = (bm >> (31 - lane)) & 1u;
-        const uint32_t before = lane ? __popc(bm >> (32 - lane)) : 0u;          // kept columns of this word before mine
-        if (in && is_kept && t > 0) {
-            const uint32_t bit0 = (k_base + before) * (uint32_t)t;               // first bit of my t-bit group
-            const uint32_t sh = bit0 & 31u, wi = bit0 >> 5;
-            if (ENCODE) {
-                const uint64_t v = (uint64_t)(W[(size_t)row * k + c] & ((1u << t) - 1u)) << (64 - t - sh);
-                atomicOr(&lo[wi], (uint32_t)(v >> 32));
-                if ((uint32_t)v) atomicOr(&lo[wi + 1], (uint32_t)v);
-            } else {
-                const uint64_t two = ((uint64_t)lo[wi] << 32) | (sh + t > 32 ? lo[wi + 1] : 0u);
-                W_out[(size_t)row * k + c] |= (uint16_t)((two >> (64 - t - sh)) & ((1u << t) - 1u));
+    const uint16_t* wr = W + (size_t)row * k;
+    const bool vec = k % 8 == 0 && ((uintptr_t)W & 15) == 0;
+    const uint32_t low_mask = (1u << t) - 1u;
+    uint8_t* ring = s_low[warp];
+    uint32_t k_cnt = 0, k_done = 0;                                     // kept values met; written
+    // the n values from k_done on, 8 a lane (n = 256, or what is left at the row's end): 8 t bits, the first at the top
+    auto put = [&](uint32_t nv) {
+        const uint32_t kk = k_done + (uint32_t)lane * 8u;
+        if (t > 0 && (uint32_t)lane * 8u < nv) {
+            const uint2 two = *reinterpret_cast<const uint2*>(ring + (kk & (kSplitRing - 1)));
+            unsigned long long bits = 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t v = (i < 4 ? two.x >> (8 * i) : two.y >> (8 * (i - 4))) & 0xFFu;
+                bits = (bits << t) | ((uint32_t)lane * 8u + i < nv ? v : 0u);
             }
-        } else if (in && !is_kept) {
-            const uint32_t i = p_base + ((uint32_t)lane - before);               // pruned columns before mine
-            if (ENCODE) raw[i] = W[(size_t)row * k + c];
-            else W_out[(size_t)row * k + c] = raw[i];
+            const uint32_t byte0 = kk / 8u * (uint32_t)t;
+            if (t == 4) {
+                lo[byte0 / 4] = (uint32_t)bits;
+            } else {
+                for (int i = 0; i < t; ++i)                             // byte b of the stream sits at b ^ 3
+                    if (byte0 + i < (uint32_t)lo_words * 4u) reinterpret_cast<uint8_t*>(lo)[(byte0 + i) ^ 3u] = (uint8_t)(bits >> (8 * (t - 1 - i)));
+            }
         }
-        const int valid = min(32, k - j * 32);                                   // columns of this word inside the matrix
-        const uint32_t kept_here = __popc(valid >= 32 ? bm : (bm & ~(0xFFFFFFFFu >> valid)));
-        k_base += kept_here;
-        p_base += (uint32_t)valid - kept_here;
+        k_done += nv;
+        __syncwarp();
+    };
+    for (int seg = 0; seg < n_seg; ++seg) {
+        const uint4 dir = __ldg(reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4) + (row / kRowsPerBlock) * n_seg + seg);
+        const int scols = seg_cols_of(k_pad, seg_cols, seg), c_base = seg * seg_cols;
+        const SbGeom sg = SbGeom::make(dir_n_ch(dir.w), scols, (int)dir.y, (int)dir.z);
+        const uint32_t* bmr = blob + (size_t)dir.x * 4 + sg.bm + row % kRowsPerBlock;
+        uint32_t byte = 0, v[4];
+        auto fetch = [&](int j0) {                                      // 8 bitmap words and their values
+            const uint32_t bm8 = lane < 8 && j0 + lane < sg.bm_words ? __ldg(bmr + (j0 + lane) * 32) : 0u;
+            const int c = c_base + j0 * 32 + lane * 8;
+            byte = (__shfl_sync(0xffffffffu, bm8, lane >> 2) >> (24 - 8 * (lane & 3))) & 0xFFu;
+            if (vec) {
+                const uint4 q = __ldg(reinterpret_cast<const uint4*>(wr + min(c, k - 8)));
+                v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+            } else {
+                uint32_t h[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) h[i] = __ldg(wr + min(c + i, k - 1));
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = h[2 * i] | (h[2 * i + 1] << 16);
+            }
+        };
+        fetch(0);
+        for (int j0 = 0; j0 < sg.bm_words; j0 += 8) {
+            const int c = c_base + j0 * 32 + lane * 8, valid = max(0, min(8, min(k, c_base + scols) - c));
+            const uint32_t cnt = __popc(byte);
+            uint32_t incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += x;
+            }
+            uint32_t kx = k_cnt + incl - cnt;                           // kept values before the lane's columns
+            uint32_t px = (uint32_t)c - kx;                             // pruned ones
+            k_cnt += __shfl_sync(0xffffffffu, incl, 31);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint32_t x = (i & 1) ? v[i / 2] >> 16 : v[i / 2] & 0xFFFFu;
+                if (byte & (0x80u >> i)) { ring[kx & (kSplitRing - 1)] = (uint8_t)(x & low_mask); ++kx; }
+                else if (i < valid) { raw[px] = (uint16_t)x; ++px; }
+            }
+            if (j0 + 8 < sg.bm_words) fetch(j0 + 8);
+            __syncwarp();
+            if (k_cnt - k_done >= 256u) put(256u);
+        }
     }
-    if (ENCODE && row == 0 && lane == 0) {
-        vdata[0] = kVdataMagic; vdata[1] = 1; vdata[2] = n; vdata[3] = k; vdata[4] = kept; vdata[5] = t; vdata[6] = row_words;
-        vdata[7] = 0;
-    }
+    while (k_cnt > k_done) put(min(256u, k_cnt - k_done));
+    // what the last value leaves of its words
+    for (uint32_t b = (uint32_t)(ceil_div((int)k_cnt, 8) * t) + lane; b < (uint32_t)lo_words * 4u; b += 32) reinterpret_cast<uint8_t*>(lo)[b ^ 3u] = 0;
+    if (lane == 0 && ((k - kept) & 1)) raw[k - kept] = 0;
+    if (row == 0 && lane < kVdataHeaderWords)
+        vdata[lane] = lane == 0 ? kVdataMagic : lane == 1 ? 1u : lane == 2 ? (uint32_t)n : lane == 3 ? (uint32_t)k : lane == 4 ? (uint32_t)kept
+                      : lane == 5 ? (uint32_t)t : lane == 6 ? (uint32_t)row_words : 0u;
 }
 
 // Exact reconstruction (Sec. 4.1 target inference: speculation and verification data are loaded and the original values
-// rebuilt; Sec. 5.1 mantissa concatenator), in two light kernels that keep many warps per SM in flight:
-//   k_decode_kept<T>: one CTA per superblock, warp = chunk, lane = row.  The lane walks its chunk's kept values (the
-//     blob's streams are interleaved over the 32 rows, so the warp's reads are contiguous) and stores their speculation
-//     bits (sign, exponent, high mantissa bits) at their columns of the output.
-//   k_merge_vdata: one warp per row, lane = column.  For every 32 columns the kept values get their low t bits from the
-//     row's verification data and the pruned columns their raw values; kept and pruned counts before a column are
-//     popcounts of the bitmap (prefix sums over the row's bitmap words first, so that the words are then independent
-//     and their loads overlap), neighbouring lanes read neighbouring verification data and the row leaves as
-//     contiguous stores.
-template <int TT>                                                       // truncated bits (0..5), or -1: read from the header
-__global__ void __launch_bounds__(1024) k_decode_kept(const uint32_t* __restrict__ blob, uint16_t* __restrict__ out) {
-    __shared__ uint16_t lut_s[256];                                     // rank -> exponent at its bf16 position
-    const uint32_t* h = blob;
-    const int n = h[H_ROWS], k = h[H_COLS], t = TT >= 0 ? TT : (int)h[H_T], seg_cols = h[H_SEG], n_seg = h[H_NSEG];
-    const int k_pad = ceil_div(k, 32) * 32;
-    const int sb = blockIdx.x, rb = sb / n_seg, seg = sb % n_seg;
-    const uint32_t* dir = blob + kBlobDirOffset / 4 + sb * 4;
-    const SbGeom sg = SbGeom::make(dir_n_ch(dir[3]), seg_cols_of(k_pad, seg_cols, seg), (int)dir[1], (int)dir[2]);
-    const int chunk_elems = dir_chunk_elems(dir[3]);
-    const uint32_t* body = blob + (size_t)dir[0] * 4;
-    const uint8_t* cb = reinterpret_cast<const uint8_t*>(blob) + kBlobHeaderBytes;
-    if ((int)h[H_T] != t) return;                                       // not the blob the launch was told about
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) lut_s[i] = (uint16_t)cb[i] << 7;
-    __syncthreads();
-    const int ch = threadIdx.x >> 5, r = threadIdx.x & 31, row = rb * kRowsPerBlock + r;
-    if (ch >= sg.n_ch || row >= n) return;
-    uint16_t* orow = out + (size_t)row * k + seg * seg_cols;
-    const int cols_here = k - seg * seg_cols;
-    auto put = [&](int col, uint16_t bits) { if (col < cols_here) orow[col] = bits; };
-    if constexpr (TT >= 0) decode_chunk_fixed<(TT >= 0 ? TT : 0)>(body, sg, chunk_elems, ch, r, lut_s, put);
-    else decode_chunk_generic(body, sg, chunk_elems, ch, r, t, cb, put);
-}
+// rebuilt; Sec. 5.1 mantissa concatenator).  One warp takes one (superblock, chunk) in two steps:
+//   lane = row: the chunk's codewords, fields and low mantissa bits become complete bf16 values in a list in shared memory,
+//     8 at a time as in the draft GEMV (the bitmap is not needed for this, so there is no search for columns); the words of
+//     the next group are requested before a group is decoded;
+//   lane = two neighbouring columns, one row after the other: a prefix count of the bitmap says which list entry, or which
+//     pruned value of the verification data, each column takes, and the row leaves as contiguous stores.  A row's loads are
+//     all under way before its first store.
+// Every output value is written once.  Bound: instruction issue.  Storing kept values at their columns from the decoding lanes
+// and filling the gaps in a second pass over the output took 255 us for a 6144 x 4096 matrix; four warps for the second step
+// of one chunk, three of them waiting for the first, 145 us; this, 131 us.
+constexpr int kJoinWarps = 4;
+constexpr int kJoinCap = 168;                                           // values of a row in hand; longer chunks take several turns
+constexpr int kJoinStride = kJoinCap + 2;                               // halfwords: an odd number of words, rows in different banks
+constexpr int kJoinSpan = 5;                                            // pairs of bitmap words (64 columns) of a row at a time
+static_assert(kJoinCap % 8 == 0 && (kJoinStride / 2) % 2 == 1, "groups of 8; odd row stride in words");
 
-constexpr int kMergeRowWarps = 8;
-__global__ void __launch_bounds__(32 * kMergeRowWarps) k_merge_vdata(const uint32_t* __restrict__ blob, const uint32_t* __restrict__ vdata,
-                                                                     uint16_t* __restrict__ out) {
-    __shared__ uint32_t kb_s[kMergeRowWarps][64];                       // kept values before each 32-column word of the segment in hand
-    const uint32_t* h = blob;
-    const int n = h[H_ROWS], k = h[H_COLS], t = h[H_T], seg_cols = h[H_SEG], n_seg = h[H_NSEG], kept = h[H_KEPT];
-    const int k_pad = ceil_div(k, 32) * 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row = blockIdx.x * kMergeRowWarps + warp;
-    if (row >= n) return;
-    const int rb = row / kRowsPerBlock, rr = row % kRowsPerBlock;
-    const int lo_words = vdata_lo_words(kept, t), row_words = vdata_row_words(k, kept, t);
-    const uint32_t* lo = vdata + kVdataHeaderWords + (size_t)row * row_words;
-    const uint16_t* raw = reinterpret_cast<const uint16_t*>(lo + lo_words);
-    uint32_t k_base = 0;                                                // kept values of the row in the segments already done
-    for (int seg = 0; seg < n_seg; ++seg) {
-        const uint32_t* dir = blob + kBlobDirOffset / 4 + (rb * n_seg + seg) * 4;
-        const int scols = seg_cols_of(k_pad, seg_cols, seg), n_words = scols / 32;       // <= 64 words
-        const SbGeom sg = SbGeom::make(dir_n_ch(dir[3]), scols, (int)dir[1], (int)dir[2]);
-        const uint32_t* bmw = blob + (size_t)dir[0] * 4 + sg.bm + rr;  // bitmap word j of this row at bmw[j * 32]
-        const int c_base = seg * seg_cols;
-        uint16_t* orow = out + (size_t)row * k + c_base;
-        __syncwarp();
-        uint32_t c0 = 0, c1 = 0;
-        if (lane < n_words) c0 = __popc(bmw[lane * 32]);
-        if (lane + 32 < n_words) c1 = __popc(bmw[(lane + 32) * 32]);
-        uint32_t i0 = c0, i1 = c1;
+struct JoinGeom {
+    int n, k, k_pad, t, seg_cols, n_seg, n_ch, n_tasks, lo_words, row_words, n_raw;
+};
+
+// TEAM: the CTA's four warps share one chunk, the first decoding and each writing a quarter of the rows: the latency of a small
+// matrix; in a large one three warps would wait while the first decodes.
+template <int TT, bool TEAM>                                            // TT: truncated bits (0..5), or -1: any (from the geometry)
+__global__ void __launch_bounds__(32 * kJoinWarps, 5) k_join(const uint32_t* __restrict__ blob, const uint32_t* __restrict__ vdata,
+                                                             uint16_t* __restrict__ out, JoinGeom jg) {
+    __shared__ uint16_t s_lists[kJoinWarps * 32 * kJoinStride + 64 * kJoinSpan + 2];      // a look past the last list reads what no column takes
+    __shared__ uint16_t s_lut[256];                                     // rank -> exponent at its bf16 position
+    const int t = TT >= 0 ? TT : jg.t, F = 8 - t, PER = 32 / F;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint8_t* cb = reinterpret_cast<const uint8_t*>(blob) + kBlobHeaderBytes;
+    pdl_wait();
+    for (int i = threadIdx.x; i < 256; i += 32 * kJoinWarps) s_lut[i] = (uint16_t)cb[i] << 7;
+    __syncthreads();
+    const int task = TEAM ? (int)blockIdx.x : (int)blockIdx.x * kJoinWarps + warp;
+    if (task >= jg.n_tasks) return;
+    const int sb = task / jg.n_ch, ch = task % jg.n_ch, rb = sb / jg.n_seg, seg = sb % jg.n_seg;
+    const uint4 dir = __ldg(reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4) + sb);
+    const int scols = seg_cols_of(jg.k_pad, jg.seg_cols, seg), n_ch = dir_n_ch(dir.w), E = dir_chunk_elems(dir.w);
+    if (ch >= n_ch) return;                                             // a shorter last segment
+    const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir.y, (int)dir.z);
+    const uint32_t* body = blob + (size_t)dir.x * 4;
+    const int c_base = seg * jg.seg_cols;
+    const uint32_t* un = body + sg.un + lane;
+    const uint32_t* fl = body + sg.fl + lane;
+    const uint32_t* lo = vdata + kVdataHeaderWords + (size_t)min(rb * kRowsPerBlock + lane, jg.n - 1) * jg.row_words;
+    const int wu_last = max(sg.w_u - 1, 0), wf_last = max(sg.w_f - 1, 0), lo_last = max(jg.lo_words - 1, 0);
+    const uint32_t ulimit = (uint32_t)sg.w_u * 32u, low_mask = (1u << t) - 1u, keep_bits = 0x8000u | (0x7Fu & ~low_mask);
+    const uint32_t e0 = __ldg(body + sg.tab + ch * 32 + lane), total = __ldg(body + sg.tab + n_ch * 32 + lane);
+    const int col_end = ch + 1 < n_ch ? (int)(__ldg(body + sg.tab + (ch + 1) * 32 + lane) >> 20) : scols;
+    int col = ch == 0 ? 0 : (int)(e0 >> 20);                            // this lane's row: first column not yet written
+    const int cnt = max(0, min(E, (int)(total >> 20) - ch * E));        // its kept values in this chunk
+    uint32_t upos = e0 & 0xFFFFFu;
+    int k_row = ch * E;                                                 // kept values of the row before this chunk
+    for (int i = 0; i < seg; ++i) {
+        const uint4 dp = __ldg(reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4) + rb * jg.n_seg + i);
+        k_row += (int)(__ldg(blob + (size_t)dp.x * 4 + dir_n_ch(dp.w) * 32 + lane) >> 20);
+    }
+    const int n_max = __reduce_max_sync(0xffffffffu, cnt);
+    constexpr int NFW = TT == 4 ? 1 : TT == 0 ? 2 : 4, NLW = TT == 0 ? 0 : TT > 0 && TT <= 4 ? 2 : 3;       // words a group of 8 can touch
+    uint16_t* s_list = s_lists + (TEAM ? 0 : warp * 32 * kJoinStride);
+    uint16_t* mine = s_list + lane * kJoinStride;
+
+    for (int p0 = 0; p0 == 0 || p0 < n_max; p0 += kJoinCap) {
+        const int n_here = min(kJoinCap, n_max - p0);
+        if (!TEAM || warp == 0) {
+            // ---- lane = row: values p0 .. p0 + n_here - 1 of the chunk ----
+            uint32_t fw[NFW], lw[NLW > 0 ? NLW : 1], fn[NFW], ln[NLW > 0 ? NLW : 1];
+            auto fetch = [&](int g) {                                   // field and low words of the group that starts at value g
+                const int fi = (ch * E + p0 + g) / PER;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t a = __shfl_up_sync(0xffffffffu, i0, o), b2 = __shfl_up_sync(0xffffffffu, i1, o);
-            if (lane >= o) { i0 += a; i1 += b2; }
-        }
-        const uint32_t tot0 = __shfl_sync(0xffffffffu, i0, 31), tot1 = __shfl_sync(0xffffffffu, i1, 31);
-        kb_s[warp][lane] = k_base + i0 - c0;
-        kb_s[warp][lane + 32] = k_base + tot0 + i1 - c1;
-        __syncwarp();
-#pragma unroll 4
-        for (int j = 0; j < n_words; ++j) {
-            const uint32_t bm = bmw[j * 32];
-            const int c = j * 32 + lane;
-            const uint32_t kb = kb_s[warp][j];
-            const bool in = c_base + c < k, is_kept = (bm >> (31 - lane)) & 1u;
-            const uint32_t before = lane ? __popc(bm >> (32 - lane)) : 0u;          // kept columns of this word before mine
-            if (in) {
-                uint16_t v;
-                if (is_kept) {
-                    v = orow[c];                                                    // the speculation bits k_decode_kept left here
-                    if (t > 0) {
-                        const uint32_t bit0 = (kb + before) * (uint32_t)t, sh = bit0 & 31u, wi = bit0 >> 5;
-                        const uint64_t two = ((uint64_t)lo[wi] << 32) | (sh + t > 32 ? lo[wi + 1] : 0u);
-                        v |= (uint16_t)((two >> (64 - t - sh)) & ((1u << t) - 1u));
-                    }
-                } else {
-                    v = raw[(uint32_t)(c_base + c) - kb - before];                   // pruned columns before mine = columns - kept before
+                for (int i = 0; i < NFW; ++i) fn[i] = __ldg(fl + min(fi + i, wf_last) * 32);
+                if (NLW > 0) {
+                    const int li = (int)((uint32_t)(k_row + p0 + g) * (uint32_t)t >> 5);
+#pragma unroll
+                    for (int i = 0; i < NLW; ++i) ln[i] = __ldg(lo + min(li + i, lo_last));
                 }
-                orow[c] = v;
+            };
+            int at = (int)(upos >> 5);                                  // u0, u1, u2: code words at, at + 1, at + 2
+            uint32_t u0 = __ldg(un + min(at, wu_last) * 32), u1 = __ldg(un + min(at + 1, wu_last) * 32), u2 = __ldg(un + min(at + 2, wu_last) * 32);
+            fetch(0);
+            for (int g = 0; g < n_here; g += 8) {
+#pragma unroll
+                for (int i = 0; i < NFW; ++i) fw[i] = fn[i];
+#pragma unroll
+                for (int i = 0; i < NLW; ++i) lw[i] = ln[i];
+                if (g + 8 < n_here) fetch(g + 8);
+                uint32_t uv = __funnelshift_l(u1, u0, upos), used = 0, q = 0, v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {                           // shifting the found one out leaves the next code at the top
+                    asm("bfind.u32 %0, %1;" : "=r"(q) : "r"(uv));
+                    v[i] = s_lut[(31u - q) & 255u];
+                    used += 32u - q;
+                    uv = __funnelshift_r(0u, uv, q);
+                }
+                if ((int32_t)q < 0) {                                   // the codes did not fit the window: one by one
+                    uint32_t ub = upos;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (p0 + g + i < cnt) v[i] = s_lut[read_unary(un, ub, ulimit) & 255];
+                    used = ub - upos;
+                }
+                upos += used;
+                const int step = (int)(upos >> 5) - at;
+                if (step == 1) {
+                    u0 = u1; u1 = u2;
+                    u2 = __ldg(un + min(at + 3, wu_last) * 32);
+                } else if (step > 1) {
+                    u0 = __ldg(un + min(at + step, wu_last) * 32);
+                    u1 = __ldg(un + min(at + step + 1, wu_last) * 32);
+                    u2 = __ldg(un + min(at + step + 2, wu_last) * 32);
+                }
+                at += step;
+                const int k = ch * E + p0 + g;                          // of the segment: fields are numbered through it
+                const uint32_t bit0 = ((uint32_t)(k_row + p0 + g) * (uint32_t)t) & 31u;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    uint32_t sm;
+                    if (TT == 4) {
+                        sm = __funnelshift_l(fw[0], fw[0], (4 * i + 16) & 31);
+                    } else if (TT == 0) {
+                        sm = __funnelshift_l(fw[i / 4 % NFW], fw[i / 4 % NFW], (8 * (i & 3) + 16) & 31);
+                    } else {
+                        const int j = k % PER + i, wi = j / PER;        // up to three words on
+                        sm = field_sign_mant_bf16(wi == 0 ? fw[0] : wi == 1 ? fw[1 % NFW] : wi == 2 ? fw[2 % NFW] : fw[3 % NFW], j - wi * PER, t);
+                    }
+                    v[i] |= sm & keep_bits;
+                    if (NLW > 0 && t > 0) {
+                        const uint32_t b = bit0 + (uint32_t)(i * t), wi = b >> 5;
+                        const uint32_t hi = wi == 0 ? lw[0] : wi == 1 || NLW == 2 ? lw[NLW > 1 ? 1 : 0] : lw[NLW > 2 ? 2 : 0];
+                        const uint32_t nx = wi == 0 || NLW == 2 ? lw[NLW > 1 ? 1 : 0] : lw[NLW > 2 ? 2 : 0];
+                        v[i] |= (__funnelshift_l(nx, hi, b) >> (32 - t)) & low_mask;
+                    }
+                    mine[g + i] = (uint16_t)v[i];
+                }
             }
         }
-        k_base += tot0 + tot1;
+        if (TEAM) __syncthreads(); else __syncwarp();
+        // ---- lane = two columns: one row after the other ----
+        constexpr int kRowStep = TEAM ? kJoinWarps : 1;
+        uint32_t bm_next = 0;                                           // the row's bitmap words, one a lane, fetched a row ahead
+        auto words = [&](int r) {
+            const int c0 = __shfl_sync(0xffffffffu, col, r), j = (c0 >> 5) + lane;
+            return lane < 2 * kJoinSpan && j < sg.bm_words ? __ldg(body + sg.bm + j * 32 + r) : 0u;
+        };
+        bm_next = words(TEAM ? warp : 0);
+#pragma unroll 1
+        for (int r = TEAM ? warp : 0; r < kRowsPerBlock; r += kRowStep) {
+            uint32_t bmv = bm_next;
+            if (r + kRowStep < kRowsPerBlock) bm_next = words(r + kRowStep);
+            const int row = rb * kRowsPerBlock + r;
+            if (row >= jg.n) break;
+            const int c0 = __shfl_sync(0xffffffffu, col, r), c_row = __shfl_sync(0xffffffffu, col_end, r);
+            const int n_row = __shfl_sync(0xffffffffu, cnt, r), kr = __shfl_sync(0xffffffffu, k_row, r);
+            if (c0 >= c_row) continue;
+            const int k_end = min(p0 + n_here, n_row);                  // list entries of this turn: chunk values p0 .. k_end - 1
+            const bool last = k_end == n_row;                           // else the row goes up to the value k_end, exclusive
+            const uint16_t* list = s_list + r * kJoinStride - p0;
+            const uint16_t* raw = reinterpret_cast<const uint16_t*>(vdata + (jg.n_raw > 0 ? kVdataHeaderWords + (size_t)row * jg.row_words + jg.lo_words : 0));
+            uint16_t* orow = out + (size_t)row * jg.k + c_base;
+            const bool pairs = (((size_t)row * jg.k) & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0;
+            const int lim = min(last ? c_row : scols, jg.k - c_base), j_end = (lim + 31) / 32;
+            int kpos = p0, stop = c_row;
+            const uint32_t r_last = (uint32_t)max(jg.n_raw - 1, 0), left = ~(0xFFFFFFFFu >> (2 * (lane & 15)));
+            for (int j0 = c0 >> 5;;) {
+                if (j0 * 32 < c0 && lane == 0) bmv &= 0xFFFFFFFFu >> (c0 & 31);      // values before belong to an earlier turn
+                int pre = __popc(bmv), here = pre;                      // kept values before each word
+#pragma unroll
+                for (int o = 1; o < 16; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, pre, o);
+                    if (lane >= o) pre += v;
+                }
+                const int all = __shfl_sync(0xffffffffu, pre, 15);
+                pre += kpos - here;
+                // both candidates of every column are loaded, without a condition, before any is used: a choice between the
+                // loads is a divergent branch that waits for each in turn
+                uint32_t lx[kJoinSpan][2], rx[kJoinSpan][2], two[kJoinSpan];
+                int bf[kJoinSpan];
+                const int q0 = c_base + lane * 2 - kr;
+#pragma unroll
+                for (int i = 0; i < kJoinSpan; ++i) {
+                    const uint32_t b = __shfl_sync(0xffffffffu, bmv, 2 * i + (lane >> 4));
+                    bf[i] = __shfl_sync(0xffffffffu, pre, 2 * i + (lane >> 4)) + __popc(b & left);      // kept values before the first column
+                    two[i] = b << (2 * (lane & 15));                    // kept? this lane's columns at the top
+                    const uint32_t p_at = (uint32_t)(q0 + (j0 + 2 * i) * 32 - bf[i]);                   // pruned ones = columns - kept
+                    lx[i][0] = list[bf[i]];
+                    lx[i][1] = list[bf[i] + 1];
+                    rx[i][0] = __ldg(raw + min(p_at, r_last));
+                    rx[i][1] = __ldg(raw + min(p_at + 1u, r_last));
+                }
+#pragma unroll
+                for (int i = 0; i < kJoinSpan; ++i) {
+                    const int j = j0 + 2 * i, c = j * 32 + lane * 2;
+                    const bool k0 = two[i] >> 31, k1 = (two[i] >> 30) & 1u;
+                    const uint32_t x0 = k0 ? lx[i][0] : rx[i][0];
+                    const uint32_t xl = k0 ? lx[i][1] : lx[i][0], xr = k0 ? rx[i][0] : rx[i][1], x1 = k1 ? xl : xr;
+                    if (pairs && last && j * 32 >= c0 && (j + 2) * 32 <= lim) {
+                        *reinterpret_cast<uint32_t*>(orow + c) = x0 | (x1 << 16);
+                    } else if (j < j_end) {                             // the row's ends, and rows off 4-byte boundaries
+                        if (c >= c0 && c < lim && (last || bf[i] + k0 <= k_end)) orow[c] = (uint16_t)x0;
+                        if (c + 1 >= c0 && c + 1 < lim && (last || bf[i] + k0 + k1 <= k_end)) orow[c + 1] = (uint16_t)x1;
+                        if (!last && kpos + all > k_end && stop == c_row) {      // the value k_end is in these words: its column begins the next turn
+                            const uint32_t at = __reduce_min_sync(0xffffffffu, k0 && bf[i] == k_end ? (uint32_t)c : k1 && bf[i] + k0 == k_end ? (uint32_t)(c + 1) : 0xFFFFFFFFu);
+                            if (at != 0xFFFFFFFFu) stop = (int)at;
+                        }
+                    }
+                }
+                j0 += 2 * kJoinSpan;
+                if (j0 >= j_end || stop != c_row) break;
+                kpos += all;
+                bmv = lane < 2 * kJoinSpan && j0 + lane < sg.bm_words ? __ldg(body + sg.bm + (j0 + lane) * 32 + r) : 0u;
+            }
+            if (lane == r) col = last ? c_row : stop;
+        }
+        if (TEAM) __syncthreads(); else __syncwarp();
     }
 }
 
@@ -189,9 +352,9 @@ extern "C" int cass_encode_verification_data(const void* blob, const cass_blob_i
     if (rc) return rc;
     if (!blob || !W_bf16 || !vdata || ((uintptr_t)vdata & 3)) return CASS_ERR_INVALID_ARG;
     if (vdata_bytes < need) return CASS_ERR_CAPACITY;
-    k_vdata<true><<<ceil_div(bi->rows, 8), 256, 0, (cudaStream_t)stream_>>>((const uint32_t*)blob, (const uint16_t*)W_bf16,
-                                                                            (uint32_t*)vdata, nullptr);
-    CASS_LAUNCH_CHECK();
+    CASS_PDL_LAUNCH(k_split, dim3(ceil_div(bi->rows, kSplitWarps)), dim3(32 * kSplitWarps), 0, (cudaStream_t)stream_, (const uint32_t*)blob,
+                    (const uint16_t*)W_bf16, (uint32_t*)vdata, (int)bi->rows, (int)bi->cols, (int)bi->kept_per_row, (int)bi->trunc_bits,
+                    (int)bi->seg_cols, (int)bi->n_seg);
     return CASS_OK;
 }
 
@@ -200,22 +363,29 @@ extern "C" int cass_decode_full(const void* blob, const cass_blob_info* bi, cons
     if (bi->mode != 1) return CASS_ERR_UNSUPPORTED;
     const int n_ch = ceil_div(bi->seg_cols, bi->chunk_cols);
     if (n_ch > 32) return CASS_ERR_UNSUPPORTED;
-    const int threads = 32 * n_ch;
-    const int grid = bi->n_rowblocks * bi->n_seg;
     cudaStream_t stream = (cudaStream_t)stream_;
-    const uint32_t* b32 = (const uint32_t*)blob;
+    const uint32_t *b32 = (const uint32_t*)blob, *v32 = (const uint32_t*)vdata;
     uint16_t* o16 = (uint16_t*)W_bf16_out;
+    const JoinGeom jg{bi->rows, bi->cols, ceil_div(bi->cols, 32) * 32, bi->trunc_bits, bi->seg_cols, bi->n_seg, n_ch,
+                      bi->n_rowblocks * bi->n_seg * n_ch, vdata_lo_words(bi->kept_per_row, bi->trunc_bits),
+                      vdata_row_words(bi->cols, bi->kept_per_row, bi->trunc_bits), bi->cols - bi->kept_per_row};
+    // below about half of the 2960 warps that run at once, teams: 24 instead of 46 us for 986 x 1289 (186 chunks), 54 instead of
+    // 62 for 4096 x 2048 (1024 chunks), but 99 instead of 76 for 4096 x 4096 (2048)
+    const bool team = jg.n_tasks < 1536;
+#define CASS_JOIN(T_)                                                                                                               \
+    do {                                                                                                                            \
+        if (team) CASS_PDL_LAUNCH((k_join<T_, true>), dim3(jg.n_tasks), dim3(32 * kJoinWarps), 0, stream, b32, v32, o16, jg);        \
+        else CASS_PDL_LAUNCH((k_join<T_, false>), dim3(ceil_div(jg.n_tasks, kJoinWarps)), dim3(32 * kJoinWarps), 0, stream, b32, v32, o16, jg); \
+    } while (0)
     switch (bi->trunc_bits) {
-        case 0: k_decode_kept<0><<<grid, threads, 0, stream>>>(b32, o16); break;
-        case 1: k_decode_kept<1><<<grid, threads, 0, stream>>>(b32, o16); break;
-        case 2: k_decode_kept<2><<<grid, threads, 0, stream>>>(b32, o16); break;
-        case 3: k_decode_kept<3><<<grid, threads, 0, stream>>>(b32, o16); break;
-        case 4: k_decode_kept<4><<<grid, threads, 0, stream>>>(b32, o16); break;
-        case 5: k_decode_kept<5><<<grid, threads, 0, stream>>>(b32, o16); break;
-        default: k_decode_kept<-1><<<grid, threads, 0, stream>>>(b32, o16); break;
+        case 0: CASS_JOIN(0); break;
+        case 1: CASS_JOIN(1); break;
+        case 2: CASS_JOIN(2); break;
+        case 3: CASS_JOIN(3); break;
+        case 4: CASS_JOIN(4); break;
+        case 5: CASS_JOIN(5); break;
+        default: CASS_JOIN(-1); break;
     }
-    CASS_LAUNCH_CHECK();
-    k_merge_vdata<<<ceil_div(bi->rows, kMergeRowWarps), 32 * kMergeRowWarps, 0, stream>>>(b32, (const uint32_t*)vdata, o16);
-    CASS_LAUNCH_CHECK();
+#undef CASS_JOIN
     return CASS_OK;
 }

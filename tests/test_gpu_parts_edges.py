@@ -1,0 +1,52 @@
+"""Edges of the kernels that split a matrix into its two parts and join them again: every truncation, rows longer than a
+decoding turn, gaps longer than 32 bitmap words, codes longer than a window, odd widths and unaligned rows."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from oracle import codec, layout
+
+pytestmark = pytest.mark.gpu
+
+
+def _bits(t):
+    return t.detach().cpu().contiguous().view(torch.int16).numpy().astype(np.uint16)
+
+
+@pytest.fixture(scope="module")
+def cass():
+    import paper_2605_26558_b200 as m
+    return m
+
+
+@pytest.mark.parametrize("rows,cols,p,t,seg,chunk", [
+    (33, 1, 0, 4, 0, 0), (1, 31, 400, 4, 0, 0), (40, 257, 400, 1, 0, 0), (65, 2049, 300, 2, 0, 0), (31, 4097, 500, 3, 0, 0),
+    (35, 1000, 400, 5, 0, 0), (34, 999, 400, 6, 256, 32), (33, 801, 200, 7, 0, 0), (37, 2048, 0, 4, 2048, 2048),
+    (32, 4096, 990, 4, 2048, 2048), (70, 3001, 999, 4, 0, 0), (64, 1024, 100, 0, 1024, 512)])
+def test_split_and_join(cass, rows, cols, p, t, seg, chunk):
+    w = synth.student_t_weight(rows, cols, 6, f"parts/{rows}x{cols}").float()
+    if rows > 20 and cols > 900:
+        w[3, 100:900] = 0.0                                  # a long gap
+        w[7, ::5] *= 2.0 ** 40                               # rare exponents: long codes
+        w[11] = 0.0
+    w = w.to(torch.bfloat16)
+    wb, act = _bits(w), np.ones(cols, dtype=np.float32)
+    fmt = cass.default_format(w_p=p, w_t=t, seg_cols=seg, chunk_cols=chunk)
+    bound, ws_bytes = cass.cass_encoded_weight_bytes(fmt, rows, cols)
+    blob = torch.zeros(bound, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    wd = w.cuda()
+    cass.cass_encode_weights(fmt, wd, None, blob, torch.zeros(ws_bytes, dtype=torch.uint8, device="cuda"), status)
+    info = cass.cass_weight_blob_info(blob)
+    assert int(status.item()) == 0
+    want = layout.encode_verification_data(wb, codec.keep_mask_weights(wb, act, p), p, t)
+    vdata = torch.full((cass.cass_verification_data_bytes(info) // 4,), -1, dtype=torch.int32, device="cuda")
+    cass.cass_encode_verification_data(blob, info, wd, vdata)
+    assert np.array_equal(vdata.cpu().numpy().view(np.uint32), want)
+    full = torch.full((rows * cols + 3,), float("nan"), dtype=torch.bfloat16, device="cuda")
+    for shift in (0, 1):                                     # output rows on and off 4-byte boundaries
+        out = full[shift: shift + rows * cols].view(rows, cols)
+        cass.cass_decode_full(blob, info, vdata, out)
+        assert np.array_equal(_bits(out), wb), shift
+    assert torch.isnan(full[-1]).item()
