@@ -8,17 +8,21 @@
 // overlap each other's copies and decodes.  Warp c decodes chunk c with lane = row: every lane
 // walks its own bitmap, field and unary streams, which are interleaved word by word over the 32 rows so that
 // all shared-memory reads of the streams are conflict free.
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "wblob.cuh"
 #include "kernels.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace cass {
 
 constexpr int kGemvStages = 1;         // stages of the copy ring per CTA; several CTAs share an SM, so their copies and decodes overlap
 constexpr int kXSlack = 288;           // readable floats after the x slice: a window walk may run up to 8 x 32 + 8 columns past its start
 
-static size_t gemv_stage_bytes(const cass_blob_info& bi) { return align_up((size_t)bi.max_superblock_bytes + 256, 128); }
+static size_t gemv_stage_bytes(const cass_blob_info& bi) { return align_up((size_t)bi.max_superblock_bytes + 384, 512); }
 
 // Bytes per column of the x slice in shared memory: one vector is kept as fp32, several as packed bf16 [col][nb].
 __host__ __device__ constexpr int x_col_bytes(int nb) { return nb == 1 ? 4 : 2 * nb; }
@@ -65,12 +69,12 @@ struct WalkState {
 template <int NB>
 struct XRaw { uint32_t w[NB == 1 ? 1 : NB / 2]; };
 
-template <int NB>
+template <int NB, int OFF = 0>
 __device__ __forceinline__ XRaw<NB> x_load(uint32_t addr) {
     XRaw<NB> r;
-    if constexpr (NB <= 2) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(r.w[0]) : "r"(addr));
-    else if constexpr (NB == 4) asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(r.w[0]), "=r"(r.w[1]) : "r"(addr));
-    else asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]) : "r"(addr));
+    if constexpr (NB <= 2) asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(r.w[0]) : "r"(addr), "n"(OFF));
+    else if constexpr (NB == 4) asm volatile("ld.shared.v2.u32 {%0,%1}, [%2+%3];" : "=r"(r.w[0]), "=r"(r.w[1]) : "r"(addr), "n"(OFF));
+    else asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4+%5];" : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]) : "r"(addr), "n"(OFF));
     return r;
 }
 
@@ -130,12 +134,20 @@ __device__ __forceinline__ uint32_t lds_u32_off(uint32_t addr) {
     return v;
 }
 
-// Dot product of one chunk (32 rows, lane = row) with x.  T = truncated mantissa bits (0 or 4).  Every lane walks
-// its row in groups of 8 kept values through 32-bit windows: one bitmap window per group, one unary window per 4
-// codewords.  A group whose 8 kept columns span more than 32 columns, or whose 4 codewords take more than 32 bits,
-// shows up as a window that ran dry (no bit left to find); that lane then redoes the group with the careful
-// walk while the others wait.  The walk addresses shared memory through 32-bit shared-space addresses.
-template <int T, int NB>
+// Dot product of one chunk (32 rows, lane = row) with x.  T = truncated mantissa bits (0 to 5).  Every lane walks its row in
+// groups of 8 kept values: 32 bitmap bits and 64 code bits from its cursors on.  The highest set bit of the bitmap window is
+// the next kept column, the highest one of the code window the next terminator; one funnel shift by its position drops it
+// and everything above, so the next search starts at the top again and a search gives a distance: the running address of x
+// moves by the columns skipped, and the position itself indexes the rank -> exponent table.
+// A group whose 8 kept columns span more than 32 columns (wide: four of them), or four of whose codewords take more than 32
+// bits, shows up as a window that ran dry (nothing left to find); that lane then redoes the group with the careful walk while
+// the others wait.
+// Bound: about 16 warp instructions a kept value and lane, of which 7 on the integer pipe (one every other cycle), two bit
+// searches (one every 8 cycles) and 3 shared-memory loads (the gather of x meets a bank two to three times): issue slots 76 %,
+// shared memory 61 %, integer pipe 58 %, searches 55 % busy.  Clearing the used bit with a shift and a mask, positions kept
+// absolute and a code window for every 4 values took 19: 58.6 -> 53.0 us on 28672 x 4096 with the results added in the kernel.
+// Finding some terminators by a conversion to float instead of a search: 54.5 to 56 us.
+template <int T, int NB, bool WIDE>
 __device__ __forceinline__ void chunk_dot_fast(const uint32_t* __restrict__ sb, const SbGeom& g, int ch, int lane,
                                                int chunk_elems, const float* __restrict__ xs,
                                                const uint32_t* __restrict__ lut, float (&acc)[NB]) {
@@ -145,6 +157,7 @@ __device__ __forceinline__ void chunk_dot_fast(const uint32_t* __restrict__ sb, 
     constexpr uint32_t MASK = 0x80000000u | (((1u << (7 - T)) - 1u) << (16 + T));   // sign + kept mantissa of a binary32
     static_assert(ROT ? (PER == 4 || PER == 8) : (PER >= 4 && PER <= 10), "fast path: 4 to 10 fields per word");
     constexpr uint32_t XS = (uint32_t)x_col_bytes(NB);            // bytes per column of the x slice
+    constexpr uint32_t XL = XS == 4 ? 2 : XS == 8 ? 3 : 4;
     const uint32_t e0 = sb[g.tab + ch * 32 + lane];            // where this row's value ch * chunk_elems sits
     const uint32_t fw = (uint32_t)(ch * chunk_elems) / PER;    // the word of the chunk's first field (fields are numbered through the segment)
     uint32_t upos = e0 & 0xFFFFFu;
@@ -159,76 +172,87 @@ __device__ __forceinline__ void chunk_dot_fast(const uint32_t* __restrict__ sb, 
     const int m = max(0, min(chunk_elems, kept - ch * chunk_elems));
     const int n_full = __reduce_min_sync(0xffffffffu, m) / kGroupCols;
     const int n_groups = ceil_div(__reduce_max_sync(0xffffffffu, m), kGroupCols);
-    uint32_t bpos = e0 >> 20;
-    const uint32_t bpos_lim = (uint32_t)(g.bm_words * 32), upos_lim = (uint32_t)(g.w_u * 32);
+    uint32_t xc = xs_a + (e0 >> 20) * XS;                       // address of the cursor's column in the x slice
+    const uint32_t xc_lim = xs_a + (uint32_t)(g.bm_words * 32) * XS, upos_lim = (uint32_t)(g.w_u * 32);
+    const uint32_t bm_x = bm_a - xs_a;
 
-    // Bit positions are counted from the least significant end (bfind): a window keeps its place and the bit
-    // just used is cleared, so a kept column is x[bpos + 31 - p] and a codeword's rank is the distance between two
-    // consecutive terminators.  A window that ran dry gives p = -1; once dry it stays dry, so the sign of the last
-    // position of each window tells whether the whole group fitted.
     auto group = [&](int grp, auto tail_c) {
         constexpr bool tail = decltype(tail_c)::value;         // two specialisations: full groups carry no per-value tests
         WalkState<NB> st0;
 #pragma unroll
         for (int b = 0; b < NB; ++b) st0.acc[b] = acc[b];
-        st0.bpos = bpos; st0.upos = upos;
-        const uint32_t ba = bm_a + (bpos >> 5) * 128u;
-        uint32_t bv = __funnelshift_l(lds_u32_off<128>(ba), lds_u32(ba), bpos);    // 32 columns from bpos on
-        const uint32_t xg = xs_a + bpos * XS + 31u * XS;                           // address of x[bpos + 31]
+        st0.upos = upos;
+        // the x slice starts at a multiple of 512 bytes, so that the address itself gives the bit (modulo 32) and the word
+        const uint32_t xc0 = xc, bpos = xc >> XL;
+        const uint32_t ba = XL == 2 ? (xc & ~127u) + bm_x : (((xc - xs_a) >> (XL - 2)) & ~127u) + bm_a;
+        const uint32_t bw1 = lds_u32_off<128>(ba), bv0 = __funnelshift_l(bw1, lds_u32(ba), bpos);      // 32 columns from the cursor on
+        uint32_t bv = bv0;
+        const uint32_t ua = un_a + (upos & ~31u) * 4u;
+        const uint32_t u1 = lds_u32_off<128>(ua);
+        const uint32_t uv0 = __funnelshift_l(u1, lds_u32(ua), upos);                       // 64 code bits from the cursor on
+        const uint32_t uv1 = __funnelshift_l(lds_u32_off<256>(ua), u1, upos);
+        uint32_t uv = uv0;
         uint32_t fwd[NFW];
         fwd[0] = lds_u32(fl_a);
         if (NFW > 1) fwd[1] = lds_u32_off<128>(fl_a);
         if (NFW > 2) fwd[2] = lds_u32_off<256>(fl_a);
         const int rem = m - grp * kGroupCols;
         uint32_t dry = 0;                           // sign bit set: a window ran dry under a value that counts
-        uint32_t p = 0;
-#pragma unroll
-        for (int half = 0; half < kGroupCols / kGroupCodes; ++half) {
-            const uint32_t ua = un_a + (upos >> 5) * 128u;
-            uint32_t uv = __funnelshift_l(lds_u32_off<128>(ua), lds_u32(ua), upos);   // 32 code bits from upos on
-            uint32_t la = lut_a + 124u;             // lut + 4 * (position of the previous terminator - 1); none yet: 32
-            uint32_t q = 0;
-#pragma unroll
-            for (int j = 0; j < kGroupCodes; ++j) {
-                const int e = half * kGroupCodes + j;
-                p = bfind_u32(bv);                                   // next kept column
-                const XRaw<NB> xv = x_load<NB>(mad_lo(p, 0u - XS, xg));
-                bv &= ~shl_sat(1u, p);
-                q = bfind_u32(uv);                                   // next terminator
-                const uint32_t eb = lds_u32(mad_lo(q, 0xFFFFFFFCu, la));          // lut[previous - q - 1]
-                la = mad_lo(q, 4u, lut_a - 4u);
-                uv &= ~shl_sat(1u, q);
-                uint32_t wb;
-                if constexpr (ROT) {
-                    const uint32_t fword = fwd[e / PER];
-                    const uint32_t a = __funnelshift_l(fword, fword, (F * (e % PER)) & 31);
-                    wb = (a & MASK) | eb;
-                } else {
-                    const uint32_t jj = j0 + (uint32_t)e;                 // field jj of the group's (up to three) words
-                    const uint32_t wsel = jj >= 2u * PER ? 2u : (jj >= (uint32_t)PER ? 1u : 0u);
-                    const uint32_t fword = wsel == 2u ? fwd[NFW - 1] : (wsel == 1u ? fwd[1] : fwd[0]);
-                    wb = packed_field_f32<T>(fword, jj - wsel * PER) | eb;
-                }
-                if (!tail) {
-                    x_fma<NB>(xv, wb, acc);
-                } else if (e < rem) {
-                    x_fma<NB>(xv, wb, acc);
-                    dry |= p | q;
-                }
+        uint32_t p = 0, xg = xc;                    // the cursor's column, less XS * 32 for every value found
+        auto take = [&](auto e_c) {
+            constexpr int e = decltype(e_c)::value, j = e % kGroupCodes;
+            p = bfind_u32(bv);                                       // next kept column: 31 - p columns on
+            xg = mad_lo(p, 0u - XS, xg);
+            const XRaw<NB> xv = x_load<NB, (32 * (e + 1) - 1) * (int)XS>(xg);
+            bv = __funnelshift_r(0u, bv, p);
+            const uint32_t q = bfind_u32(uv);                        // next terminator: the code's rank is 31 - q
+            const uint32_t eb = lds_u32(mad_lo(q, 0xFFFFFFFCu, lut_a + 124u));
+            uv = __funnelshift_r(0u, uv, q);
+            upos -= q;
+            uint32_t wb;
+            if constexpr (ROT) {
+                const uint32_t fword = fwd[e / PER];
+                const uint32_t a = __funnelshift_l(fword, fword, (F * (e % PER)) & 31);
+                wb = (a & MASK) | eb;
+            } else {
+                const uint32_t jj = j0 + (uint32_t)e;                 // field jj of the group's (up to three) words
+                const uint32_t wsel = jj >= 2u * PER ? 2u : (jj >= (uint32_t)PER ? 1u : 0u);
+                const uint32_t fword = wsel == 2u ? fwd[NFW - 1] : (wsel == 1u ? fwd[1] : fwd[0]);
+                wb = packed_field_f32<T>(fword, jj - wsel * PER) | eb;
             }
-            upos += 32u - q;                                         // bits up to and including the last terminator
-            if (tail) upos = min(upos, upos_lim);                    // rows that ran out of values stay inside the buffers
-            else dry |= q;
+            if constexpr (!tail) {
+                x_fma<NB>(xv, wb, acc);
+                if (j == kGroupCodes - 1) dry |= WIDE ? p | q : q;
+            } else if (e < rem) {
+                x_fma<NB>(xv, wb, acc);
+                dry |= p | q;
+            }
+        };
+        take(std::integral_constant<int, 0>{}); take(std::integral_constant<int, 1>{});
+        take(std::integral_constant<int, 2>{}); take(std::integral_constant<int, 3>{});
+        const uint32_t used = upos + 4u * 32u - st0.upos;            // bits up to and including the fourth terminator: at most 32
+        uv = __funnelshift_lc(uv1, uv0, used);
+        if constexpr (WIDE) {                                                  // and the columns up to the fourth value's: the next 32 from there
+            const uint32_t cols = (uint32_t)((int32_t)(xg - xc0) >> XL) + 4u * 32u;
+            bv = __funnelshift_lc(__funnelshift_l(lds_u32_off<256>(ba), bw1, bpos), bv0, cols);
         }
-        bpos += 32u - p;
-        if (tail) bpos = min(bpos, bpos_lim);
-        else dry |= p;
+        take(std::integral_constant<int, 4>{}); take(std::integral_constant<int, 5>{});
+        take(std::integral_constant<int, 6>{}); take(std::integral_constant<int, 7>{});
+        upos += 8u * 32u;                                            // 32 - q bits a code
+        xc = xg + 8u * 32u * XS;
+        if (tail) {                                                  // rows that ran out of values stay inside the buffers
+            upos = min(upos, upos_lim);
+            xc = min(xc, xc_lim);
+        } else {
+            dry |= p;
+        }
         if ((int32_t)dry < 0) {
+            st0.bpos = (xc0 - xs_a) >> XL;
             const WalkState<NB> r = group_slow<T, NB>(bmS, unS, flS, (uint32_t)(ch * chunk_elems + grp * kGroupCols), min(rem, kGroupCols),
-                                                      st0, bpos_lim, upos_lim, xs, lut);
+                                                      st0, (xc_lim - xs_a) >> XL, upos_lim, xs, lut);
 #pragma unroll
             for (int b = 0; b < NB; ++b) acc[b] = r.acc[b];
-            bpos = r.bpos; upos = r.upos;
+            xc = xs_a + (r.bpos << XL); upos = r.upos;
         }
         if constexpr (ROT) {
             fl_a += NFW * 128u;
@@ -267,11 +291,12 @@ __device__ __noinline__ WalkState<NB> group_slow_mx(const uint32_t* bmS, uint32_
     return st;
 }
 
-template <int NB>
+template <int NB, bool WIDE>
 __device__ __forceinline__ void chunk_dot_mx4(const uint32_t* __restrict__ sb, const SbGeom& g, int ch, int lane,
                                               int chunk_elems, const float* __restrict__ xs,
                                               const float* __restrict__ nlut, float (&acc)[NB]) {
     constexpr uint32_t XS = (uint32_t)x_col_bytes(NB);
+    constexpr uint32_t XL = XS == 4 ? 2 : XS == 8 ? 3 : 4;
     const uint32_t e0 = sb[g.tab + ch * 32 + lane];
     const uint32_t* bmS = sb + g.bm + lane;
     const uint32_t bm_a = smem_u32(bmS), xs_a = smem_u32(xs), nl_a = smem_u32(nlut);      // nlut is 64-byte aligned
@@ -281,9 +306,9 @@ __device__ __forceinline__ void chunk_dot_mx4(const uint32_t* __restrict__ sb, c
     const int m = max(0, min(chunk_elems, kept - ch * chunk_elems));
     const int n_full = __reduce_min_sync(0xffffffffu, m) / kGroupCols;
     const int n_groups = ceil_div(__reduce_max_sync(0xffffffffu, m), kGroupCols);
-    uint32_t bpos = e0 >> 20;
+    uint32_t xc = xs_a + (e0 >> 20) * XS;                       // address of the cursor's column in the x slice
     const uint32_t blk0 = (e0 & 0xFFFFFu) >> 3;                 // index of the chunk's first exponent byte
-    const uint32_t bpos_lim = (uint32_t)(g.bm_words * 32);
+    const uint32_t xc_lim = xs_a + (uint32_t)(g.bm_words * 32) * XS, bm_x = bm_a - xs_a;
     float blk[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b) blk[b] = 0.f;
@@ -293,35 +318,48 @@ __device__ __forceinline__ void chunk_dot_mx4(const uint32_t* __restrict__ sb, c
         WalkState<NB> st0;
 #pragma unroll
         for (int b = 0; b < NB; ++b) st0.acc[b] = blk[b];
-        st0.bpos = bpos; st0.upos = 0;
-        const uint32_t ba = bm_a + (bpos >> 5) * 128u;
-        uint32_t bv = __funnelshift_l(lds_u32_off<128>(ba), lds_u32(ba), bpos);
-        const uint32_t xg = xs_a + bpos * XS + 31u * XS;
+        st0.upos = 0;
+        // the x slice starts at a multiple of 512 bytes, so that the address itself gives the bit (modulo 32) and the word
+        const uint32_t xc0 = xc, bpos = xc >> XL;
+        const uint32_t ba = XL == 2 ? (xc & ~127u) + bm_x : (((xc - xs_a) >> (XL - 2)) & ~127u) + bm_a;
+        const uint32_t bw1 = lds_u32_off<128>(ba), bv0 = __funnelshift_l(bw1, lds_u32(ba), bpos);
+        uint32_t bv = bv0;
         const uint32_t fword = lds_u32(fl_a);
         const int rem = m - grp * kGroupCols;
-        uint32_t dry = 0, p = 0;
-#pragma unroll
-        for (int e = 0; e < kGroupCols; ++e) {
-            p = bfind_u32(bv);
-            const XRaw<NB> xv = x_load<NB>(mad_lo(p, 0u - XS, xg));
-            bv &= ~shl_sat(1u, p);
+        uint32_t dry = 0, p = 0, xg = xc;
+        auto take = [&](auto e_c) {
+            constexpr int e = decltype(e_c)::value;
+            p = bfind_u32(bv);                                       // next kept column: 31 - p columns on
+            xg = mad_lo(p, 0u - XS, xg);
+            const XRaw<NB> xv = x_load<NB, (32 * (e + 1) - 1) * (int)XS>(xg);
+            bv = __funnelshift_r(0u, bv, p);
             const uint32_t off = e < 7 ? (fword >> (26 - 4 * e)) : (fword << 2);
             const uint32_t wb = lds_u32((off & 0x3Cu) | nl_a);                         // +-(magnitude << 4) as a float
-            if (!tail) {
+            if constexpr (!tail) {
                 x_fma<NB>(xv, wb, blk);
             } else if (e < rem) {
                 x_fma<NB>(xv, wb, blk);
                 dry |= p;
             }
+        };
+        take(std::integral_constant<int, 0>{}); take(std::integral_constant<int, 1>{});
+        take(std::integral_constant<int, 2>{}); take(std::integral_constant<int, 3>{});
+        if constexpr (WIDE) {                                                  // the next 32 columns from the fourth value's on
+            if (!tail) dry |= p;
+            const uint32_t cols = (uint32_t)((int32_t)(xg - xc0) >> XL) + 4u * 32u;
+            bv = __funnelshift_lc(__funnelshift_l(lds_u32_off<256>(ba), bw1, bpos), bv0, cols);
         }
-        bpos += 32u - p;
-        if (tail) bpos = min(bpos, bpos_lim);
+        take(std::integral_constant<int, 4>{}); take(std::integral_constant<int, 5>{});
+        take(std::integral_constant<int, 6>{}); take(std::integral_constant<int, 7>{});
+        xc = xg + 8u * 32u * XS;
+        if (tail) xc = min(xc, xc_lim);
         else dry |= p;
         if ((int32_t)dry < 0) {
-            const WalkState<NB> r = group_slow_mx<NB>(bmS, fword, min(rem, kGroupCols), st0, bpos_lim, xs, nlut);
+            st0.bpos = (xc0 - xs_a) >> XL;
+            const WalkState<NB> r = group_slow_mx<NB>(bmS, fword, min(rem, kGroupCols), st0, (xc_lim - xs_a) >> XL, xs, nlut);
 #pragma unroll
             for (int b = 0; b < NB; ++b) blk[b] = r.acc[b];
-            bpos = r.bpos;
+            xc = xs_a + (r.bpos << XL);
         }
         fl_a += 128u;
         if ((grp & 3) == 3 || grp == n_groups - 1) {              // a block of 32 values is complete: apply its scale
@@ -342,195 +380,251 @@ __device__ __forceinline__ void chunk_dot_mx4(const uint32_t* __restrict__ sb, c
 // grid = (n_seg, G): CTA (seg, j) handles the superblocks (rb, seg) for rb = j, j + G, ...
 // NB vectors x[b] (bf16 [NB][k]) are multiplied in the same pass: every decoded weight is used NB times, and each
 // vector's sums are formed in the same order as with NB = 1.
-template <int T, int NB>
+// out = 1: the matrix is one segment wide, a sum is the result.  out = 2: the n_seg CTAs of a row block are a cluster with one
+// tile each, and the first adds the others' sums in segment order.  (A kernel of its own for these additions costs a launch,
+// 2 us of the 10 us that a small matrix takes.)  out = 0: only `partial` is written.
+template <int T, int NB, bool WIDE>
 __global__ void __launch_bounds__(1024) k_draft_gemv(const uint32_t* __restrict__ blob, const uint16_t* __restrict__ x,
                                                      float* __restrict__ partial, int32_t* __restrict__ d_status,
                                                      int stage_bytes, int max_sb, int n, int k, int t, int seg_cols,
-                                                     int chunk_cols, int n_seg, int n_rb, unsigned long long blob_bytes) {
-    extern __shared__ __align__(128) uint8_t smem_raw[];
-    // The geometry comes from the host's copy of the header (the launch sized shared memory from it); the header
-    // itself is fetched now and compared once it has arrived, so that its latency is off the critical path.
-    const uint32_t* h = blob;
-    const uint32_t h_n = h[H_ROWS], h_k = h[H_COLS], h_t = h[H_T], h_seg = h[H_SEG], h_chunk = h[H_CHUNK], h_nseg = h[H_NSEG],
-                   h_nrb = h[H_NRB], h_magic = h[H_MAGIC];
-    const int k_pad = ceil_div(k, 32) * 32;
-    const int seg = blockIdx.x, rb0 = blockIdx.y, rb_step = gridDim.y;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = blockDim.x >> 5;
-
-    float* xs = reinterpret_cast<float*>(smem_raw + (size_t)kGemvStages * stage_bytes);
-    uint32_t* lut = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(xs) + (size_t)(seg_cols + kXSlack) * x_col_bytes(NB));
-    float* red = reinterpret_cast<float*>(lut + 256);                       // NB = 1: [2][n_warps][32], else [NB][n_warps][32]
-    uint64_t* bar = reinterpret_cast<uint64_t*>(red + (NB < 2 ? 2 : NB) * n_warps * 32);    // [kGemvStages]
-    __shared__ int s_skip[kGemvStages];
-
-    const int scols = seg_cols_of(k_pad, seg_cols, seg);
-    const int n_ch = ceil_div(scols, chunk_cols);
-    // The launch sized shared memory from the host's copy of the header; a blob that does not match it is
-    // refused instead of overrunning the buffers.
-    if (seg >= n_seg || (int)blockDim.x < 32 * n_ch || n_ch > 32 || (T == 104 && (smem_u32(lut) & 63u))) {
-        if (tid == 0 && d_status) atomicExch(d_status, CASS_ERR_INVALID_ARG);
-        return;
-    }
-    const int n_tiles = rb0 < n_rb ? (n_rb - rb0 + rb_step - 1) / rb_step : 0;
-
-    if (tid == 0) {
-        for (int s = 0; s < kGemvStages; ++s) mbar_init(&bar[s], 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-
-    // thread 0: start the copy of tile i into stage i % kGemvStages.  Nothing is read beyond blob + blob_bytes (the
-    // size the caller's description gives): a directory entry that points outside is skipped and flagged.
-    auto issue = [&](int i) {
-        const int s = i % kGemvStages;
-        const int sb_i = (rb0 + i * rb_step) * n_seg + seg;
-        const uint32_t* dir = blob + kBlobDirOffset / 4 + sb_i * 4;
-        const bool dir_ok = (unsigned long long)kBlobDirOffset + ((unsigned long long)sb_i + 1ull) * 16ull <= blob_bytes;
-        const uint32_t d0 = dir_ok ? dir[0] : 0u, d1 = dir_ok ? dir[1] : 0u, d2 = dir_ok ? dir[2] : 0u, d3 = dir_ok ? dir[3] : 0u;
-        const SbGeom g = SbGeom::make(dir_n_ch(d3), scols, (int)d1, (int)d2);
-        const uint32_t bytes = (uint32_t)g.total * 4u;
-        if (!dir_ok || bytes > (uint32_t)max_sb || dir_n_ch(d3) != n_ch || d1 > 0xFFFFu || d2 > 0xFFFFu ||
-            (unsigned long long)d0 * 16ull + bytes > blob_bytes) {                // does not fit: skip the tile, flag it
-            s_skip[s] = 1;
-            if (d_status) atomicExch(d_status, CASS_ERR_INVALID_ARG);
-            mbar_expect_tx(&bar[s], 0);
-            return;
-        }
-        s_skip[s] = 0;
-        const uint8_t* src = reinterpret_cast<const uint8_t*>(blob) + (size_t)d0 * 16;
-        uint8_t* dst = smem_raw + (size_t)s * stage_bytes;
-        mbar_expect_tx(&bar[s], bytes);
-        for (uint32_t off = 0; off < bytes; off += 32768u) bulk_g2s(dst + off, src + off, min(32768u, bytes - off), &bar[s]);
+                                                     int chunk_cols, int n_seg, int n_rb, unsigned long long blob_bytes,
+                                                     int out, uint16_t* __restrict__ y_bf16, float* __restrict__ y_f32) {
+    extern __shared__ __align__(512) uint8_t smem_raw[];
+    __shared__ float s_sum[NB][32];                     // out = 2: this segment's sums
+    const int lane = threadIdx.x & 31;
+    auto store = [&](int b, int row, float sum) {
+        if (y_f32) y_f32[(size_t)b * n + row] = sum;
+        if (y_bf16) y_bf16[(size_t)b * n + row] = float_to_bf16_bits(sum);
     };
-    if (tid == 0) {
-        for (int i = 0; i < kGemvStages && i < n_tiles; ++i) issue(i);
-    }
-    // the rank -> exponent table, pre-shifted into place
-    const uint8_t* cb = reinterpret_cast<const uint8_t*>(blob) + kBlobHeaderBytes;
-    if (T == 104) {
-        // signed magnitudes of the 16 field values, as floats: (+-) (m << 4)
-        if (tid < 16) reinterpret_cast<float*>(lut)[tid] = (tid & 8 ? -16.f : 16.f) * (float)(tid & 7);
-    } else {
-        for (int i = tid; i < 256; i += blockDim.x) lut[i] = (uint32_t)cb[i] << 23;
-    }
-    // Everything above touches only the blob, which no kernel writes.  When the launch allows this grid to start
-    // before its predecessor in the stream has finished, wait here: x and the scratch `partial` are the predecessor's.
-    pdl_wait();
-    // x of this segment (fp32), zero beyond the matrix
-    const int c0 = seg * seg_cols;
-    if constexpr (NB > 1) {
-        // packed bf16 [col][NB]: all vectors' values of one column side by side
-        uint16_t* xs16 = reinterpret_cast<uint16_t*>(xs);
-        if ((k & 7) == 0 && ((uintptr_t)x & 15) == 0) {
-            const int n_oct = (seg_cols + kXSlack) / 8;
-            for (int it = tid; it < n_oct * NB; it += blockDim.x) {
-                const int i = (it / NB) * 8, b = it % NB;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (i < scols && c0 + i < k) v = *reinterpret_cast<const uint4*>(x + (size_t)b * k + c0 + i);
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    auto result = [&](int b, int row, float sum) {      // a segment's sum of one row
+        if (out == 1) store(b, row, sum);
+        else if (out == 2) s_sum[b][lane] = sum;
+    };
+    auto tiles = [&]() -> bool {
+        // The geometry comes from the host's copy of the header (the launch sized shared memory from it); the header
+        // itself is fetched now and compared once it has arrived, so that its latency is off the critical path.
+        const uint32_t* h = blob;
+        uint32_t hw[9] = {};                                   // thread 32: what the header says, and what it should
+        const uint32_t want[9] = {(uint32_t)n, (uint32_t)k, (uint32_t)t, (uint32_t)seg_cols, (uint32_t)chunk_cols, (uint32_t)n_seg, (uint32_t)n_rb,
+                                  kBlobMagic, (T == 104 || T == -2) ? kBlobModeMx : kBlobModeUnary};
+        const bool checks = threadIdx.x == (blockDim.x > 32 ? 32u : 0u);
+        if (checks) {
+            const int at[9] = {H_ROWS, H_COLS, H_T, H_SEG, H_CHUNK, H_NSEG, H_NRB, H_MAGIC, H_MODE};
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    xs16[(size_t)(i + 2 * q) * NB + b] = (uint16_t)(w[q] & 0xFFFFu);
-                    xs16[(size_t)(i + 2 * q + 1) * NB + b] = (uint16_t)(w[q] >> 16);
+            for (int i = 0; i < 9; ++i) hw[i] = __ldg(h + at[i]);
+        }
+        const int k_pad = ceil_div(k, 32) * 32;
+        const int seg = blockIdx.x, rb0 = blockIdx.y, rb_step = gridDim.y;
+        const int tid = threadIdx.x, warp = tid >> 5, n_warps = blockDim.x >> 5;
+
+        float* xs = reinterpret_cast<float*>(smem_raw + (size_t)kGemvStages * stage_bytes);
+        uint32_t* lut = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(xs) + (size_t)(seg_cols + kXSlack) * x_col_bytes(NB));
+        float* red = reinterpret_cast<float*>(lut + 256);                       // NB = 1: [2][n_warps][32], else [NB][n_warps][32]
+        uint64_t* bar = reinterpret_cast<uint64_t*>(red + (NB < 2 ? 2 : NB) * n_warps * 32);    // [kGemvStages]
+        __shared__ int s_skip[kGemvStages], s_bad;
+        __shared__ uint32_t s_dir[kGemvStages][3];          // sizes of the tile in each stage
+
+        const int scols = seg_cols_of(k_pad, seg_cols, seg);
+        const int n_ch = scols == seg_cols ? (int)blockDim.x / 32 : ceil_div(scols, chunk_cols);
+        // The launch sized shared memory from the host's copy of the header; a blob that does not match it is
+        // refused instead of overrunning the buffers.
+        if (seg >= n_seg || (int)blockDim.x < 32 * n_ch || n_ch > 32 || (T == 104 && (smem_u32(lut) & 63u)) ||
+            (smem_u32(xs) & (32u * x_col_bytes(NB) - 1u))) {
+            if (tid == 0 && d_status) atomicExch(d_status, CASS_ERR_INVALID_ARG);
+            return false;
+        }
+        const int n_tiles = rb0 >= n_rb ? 0 : rb_step >= n_rb ? 1 : (n_rb - rb0 + rb_step - 1) / rb_step;
+
+        if (tid == 0) {
+            for (int s = 0; s < kGemvStages; ++s) mbar_init(&bar[s], 1);
+            fence_mbar_init();
+        }
+        __syncthreads();
+
+        // thread 0: start the copy of tile i into stage i % kGemvStages.  Nothing is read beyond blob + blob_bytes (the
+        // size the caller's description gives): a directory entry that points outside is skipped and flagged.
+        auto issue = [&](int i) {
+            const int s = i % kGemvStages;
+            const int sb_i = (rb0 + i * rb_step) * n_seg + seg;
+            const uint32_t* dir = blob + kBlobDirOffset / 4 + sb_i * 4;
+            const bool dir_ok = (unsigned long long)kBlobDirOffset + ((unsigned long long)sb_i + 1ull) * 16ull <= blob_bytes;
+            const uint32_t d0 = dir_ok ? dir[0] : 0u, d1 = dir_ok ? dir[1] : 0u, d2 = dir_ok ? dir[2] : 0u, d3 = dir_ok ? dir[3] : 0u;
+            const SbGeom g = SbGeom::make(dir_n_ch(d3), scols, (int)d1, (int)d2);
+            const uint32_t bytes = (uint32_t)g.total * 4u;
+            if (!dir_ok || bytes > (uint32_t)max_sb || dir_n_ch(d3) != n_ch || d1 > 0xFFFFu || d2 > 0xFFFFu ||
+                (unsigned long long)d0 * 16ull + bytes > blob_bytes) {                // does not fit: skip the tile, flag it
+                s_skip[s] = 1;
+                if (d_status) atomicExch(d_status, CASS_ERR_INVALID_ARG);
+                mbar_expect_tx(&bar[s], 0);
+                return;
+            }
+            s_skip[s] = 0;
+            s_dir[s][0] = d1; s_dir[s][1] = d2; s_dir[s][2] = d3;
+            const uint8_t* src = reinterpret_cast<const uint8_t*>(blob) + (size_t)d0 * 16;
+            uint8_t* dst = smem_raw + (size_t)s * stage_bytes;
+            mbar_expect_tx(&bar[s], bytes);
+            for (uint32_t off = 0; off < bytes; off += 32768u) bulk_g2s(dst + off, src + off, min(32768u, bytes - off), &bar[s]);
+        };
+        if (tid == 0) {
+            for (int i = 0; i < kGemvStages && i < n_tiles; ++i) issue(i);
+        }
+        // the rank -> exponent table, pre-shifted into place
+        const uint8_t* cb = reinterpret_cast<const uint8_t*>(blob) + kBlobHeaderBytes;
+        if (T == 104) {
+            // signed magnitudes of the 16 field values, as floats: (+-) (m << 4)
+            if (tid < 16) reinterpret_cast<float*>(lut)[tid] = (tid & 8 ? -16.f : 16.f) * (float)(tid & 7);
+        } else {
+            for (int i = tid; i < 256; i += blockDim.x) lut[i] = (uint32_t)cb[i] << 23;
+        }
+        if (checks) {
+            bool bad = false;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) bad = bad || hw[i] != want[i];
+            s_bad = bad;
+        }
+        // Everything above touches only the blob, which no kernel writes.  When the launch allows this grid to start
+        // before its predecessor in the stream has finished, wait here: x and the scratch `partial` are the predecessor's.
+        pdl_wait();
+        // x of this segment (fp32), zero beyond the matrix
+        const int c0 = seg * seg_cols;
+        if constexpr (NB > 1) {
+            // packed bf16 [col][NB]: all vectors' values of one column side by side
+            uint16_t* xs16 = reinterpret_cast<uint16_t*>(xs);
+            if ((k & 7) == 0 && ((uintptr_t)x & 15) == 0) {
+                const int n_oct = (seg_cols + kXSlack) / 8;
+                for (int it = tid; it < n_oct * NB; it += blockDim.x) {
+                    const int i = (it / NB) * 8, b = it % NB;
+                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                    if (i < scols && c0 + i < k) v = *reinterpret_cast<const uint4*>(x + (size_t)b * k + c0 + i);
+                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        xs16[(size_t)(i + 2 * q) * NB + b] = (uint16_t)(w[q] & 0xFFFFu);
+                        xs16[(size_t)(i + 2 * q + 1) * NB + b] = (uint16_t)(w[q] >> 16);
+                    }
+                }
+            } else {
+                for (int it = tid; it < (seg_cols + kXSlack) * NB; it += blockDim.x) {
+                    const int i = it / NB, b = it % NB, c = c0 + i;
+                    xs16[it] = (i < scols && c < k) ? x[(size_t)b * k + c] : (uint16_t)0;
                 }
             }
+        } else if ((k & 7) == 0 && ((uintptr_t)x & 15) == 0) {
+            // eight values per 16-byte load: one round trip to L2 for the whole slice
+            for (int i = tid * 8; i < seg_cols + kXSlack; i += blockDim.x * 8) {
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (i < scols && c0 + i < k) v = *reinterpret_cast<const uint4*>(x + c0 + i);
+                float4 lo = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
+                                        __uint_as_float(v.y & 0xFFFF0000u));
+                float4 hi = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u), __uint_as_float(v.w << 16),
+                                        __uint_as_float(v.w & 0xFFFF0000u));
+                *reinterpret_cast<float4*>(xs + i) = lo;
+                *reinterpret_cast<float4*>(xs + i + 4) = hi;
+            }
         } else {
-            for (int it = tid; it < (seg_cols + kXSlack) * NB; it += blockDim.x) {
-                const int i = it / NB, b = it % NB, c = c0 + i;
-                xs16[it] = (i < scols && c < k) ? x[(size_t)b * k + c] : (uint16_t)0;
+            for (int i = tid; i < seg_cols + kXSlack; i += blockDim.x) {
+                int c = c0 + i;
+                xs[i] = (i < scols && c < k) ? bf16_bits_to_float(x[c]) : 0.f;
             }
         }
-    } else if ((k & 7) == 0 && ((uintptr_t)x & 15) == 0) {
-        // eight values per 16-byte load: one round trip to L2 for the whole slice
-        for (int i = tid * 8; i < seg_cols + kXSlack; i += blockDim.x * 8) {
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (i < scols && c0 + i < k) v = *reinterpret_cast<const uint4*>(x + c0 + i);
-            float4 lo = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
-                                    __uint_as_float(v.y & 0xFFFF0000u));
-            float4 hi = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u), __uint_as_float(v.w << 16),
-                                    __uint_as_float(v.w & 0xFFFF0000u));
-            *reinterpret_cast<float4*>(xs + i) = lo;
-            *reinterpret_cast<float4*>(xs + i + 4) = hi;
+        __syncthreads();
+        if (s_bad) {
+            // not the blob the caller described: flag it, let the copies already started land, produce nothing
+            if (tid == 0 && d_status) atomicExch(d_status, CASS_ERR_INVALID_ARG);
+            for (int j = 0; j < n_tiles && j < kGemvStages; ++j) mbar_wait_bounded(&bar[j % kGemvStages], 0u);
+            return false;
         }
-    } else {
-        for (int i = tid; i < seg_cols + kXSlack; i += blockDim.x) {
-            int c = c0 + i;
-            xs[i] = (i < scols && c < k) ? bf16_bits_to_float(x[c]) : 0.f;
-        }
-    }
-    __syncthreads();
-    if (h[H_MODE] != ((T == 104 || T == -2) ? kBlobModeMx : kBlobModeUnary) || h_magic != kBlobMagic || (int)h_n != n || (int)h_k != k || (int)h_t != t || (int)h_seg != seg_cols ||
-        (int)h_chunk != chunk_cols || (int)h_nseg != n_seg || (int)h_nrb != n_rb) {
-        // not the blob the caller described: flag it, let the copies already started land, produce nothing
-        if (tid == 0 && d_status) atomicExch(d_status, CASS_ERR_INVALID_ARG);
-        for (int j = 0; j < n_tiles && j < kGemvStages; ++j) mbar_wait_bounded(&bar[j % kGemvStages], 0u);
-        return;
-    }
 
-    for (int i = 0; i < n_tiles; ++i) {
-        const int s = i % kGemvStages;
-        const int rb = rb0 + i * rb_step;
-        if (!mbar_wait_bounded(&bar[s], (uint32_t)(i / kGemvStages) & 1u)) {
-            // give up: flag the error, let the copies still in flight into this CTA's buffers land (bounded), leave
-            if (d_status) atomicExch(d_status, CASS_ERR_TIMEOUT);
-            for (int j = i; j < n_tiles && j < i + kGemvStages; ++j)
-                mbar_wait_bounded(&bar[j % kGemvStages], (uint32_t)(j / kGemvStages) & 1u);
-            return;
-        }
-        const uint32_t* sb = reinterpret_cast<const uint32_t*>(smem_raw + (size_t)s * stage_bytes);
-        float acc[NB];
+        for (int i = 0; i < n_tiles; ++i) {
+            const int s = i % kGemvStages;
+            const int rb = rb0 + i * rb_step;
+            if (!mbar_wait_bounded(&bar[s], (uint32_t)(i / kGemvStages) & 1u)) {
+                // give up: flag the error, let the copies still in flight into this CTA's buffers land (bounded), leave
+                if (d_status) atomicExch(d_status, CASS_ERR_TIMEOUT);
+                for (int j = i; j < n_tiles && j < i + kGemvStages; ++j)
+                    mbar_wait_bounded(&bar[j % kGemvStages], (uint32_t)(j / kGemvStages) & 1u);
+                return false;
+            }
+            const uint32_t* sb = reinterpret_cast<const uint32_t*>(smem_raw + (size_t)s * stage_bytes);
+            float acc[NB];
 #pragma unroll
-        for (int b = 0; b < NB; ++b) acc[b] = 0.f;
-        if (warp < n_ch && !s_skip[s]) {
-            const uint32_t* dir = blob + kBlobDirOffset / 4 + (rb * n_seg + seg) * 4;
-            const SbGeom g = SbGeom::make(n_ch, scols, (int)dir[1], (int)dir[2]);
-            if (T == 104) {
-                chunk_dot_mx4<NB>(sb, g, warp, lane, dir_chunk_elems(dir[3]), xs, reinterpret_cast<const float*>(lut), acc);
-            } else if (T == -2) {
-                const uint32_t xs_a = smem_u32(xs);
-                decode_chunk_generic_mx(sb, g, dir_chunk_elems(dir[3]), warp, lane, t, [&](int col, uint16_t bits) {
-                    x_fma<NB>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
-                });
-            } else if (T >= 0) {
-                chunk_dot_fast<(T >= 0 && T <= 5 ? T : 0), NB>(sb, g, warp, lane, dir_chunk_elems(dir[3]), xs, lut, acc);
+            for (int b = 0; b < NB; ++b) acc[b] = 0.f;
+            if (warp < n_ch && !s_skip[s]) {
+                const uint32_t* dir = s_dir[s] - 1;                   // written before the copy was started; its arrival orders the read
+                const SbGeom g = SbGeom::make(n_ch, scols, (int)dir[1], (int)dir[2]);
+                if (T == 104) {
+                    chunk_dot_mx4<NB, WIDE>(sb, g, warp, lane, dir_chunk_elems(dir[3]), xs, reinterpret_cast<const float*>(lut), acc);
+                } else if (T == -2) {
+                    const uint32_t xs_a = smem_u32(xs);
+                    decode_chunk_generic_mx(sb, g, dir_chunk_elems(dir[3]), warp, lane, t, [&](int col, uint16_t bits) {
+                        x_fma<NB>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
+                    });
+                } else if (T >= 0) {
+                    chunk_dot_fast<(T >= 0 && T <= 5 ? T : 0), NB, WIDE>(sb, g, warp, lane, dir_chunk_elems(dir[3]), xs, lut, acc);
+                } else {
+                    const uint32_t xs_a = smem_u32(xs);
+                    decode_chunk_generic(sb, g, dir_chunk_elems(dir[3]), warp, lane, t, cb, [&](int col, uint16_t bits) {
+                        x_fma<NB>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
+                    });
+                }
+            }
+            const size_t n_pad = (size_t)n_rb * kRowsPerBlock;
+            const int row = rb * kRowsPerBlock + lane;
+            if constexpr (NB == 1) {
+                float* red_i = red + (i & 1) * n_warps * 32;
+                red_i[warp * 32 + lane] = acc[0];
+                __syncthreads();                              // all reads of stage s are done; partial sums are visible
+                if (tid == 0 && i + kGemvStages < n_tiles) {
+                    fence_proxy_async();
+                    issue(i + kGemvStages);
+                }
+                if (warp == 0) {
+                    float sum = 0.f;
+                    for (int w = 0; w < n_ch; ++w) sum += red_i[w * 32 + lane];
+                    if (row < n) {
+                        partial[(size_t)seg * n_pad + row] = sum;
+                        result(0, row, sum);
+                    }
+                }
             } else {
-                const uint32_t xs_a = smem_u32(xs);
-                decode_chunk_generic(sb, g, dir_chunk_elems(dir[3]), warp, lane, t, cb, [&](int col, uint16_t bits) {
-                    x_fma<NB>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
-                });
+#pragma unroll
+                for (int b = 0; b < NB; ++b) red[(b * n_warps + warp) * 32 + lane] = acc[b];
+                __syncthreads();
+                if (tid == 0 && i + kGemvStages < n_tiles) {
+                    fence_proxy_async();
+                    issue(i + kGemvStages);
+                }
+                for (int b = warp; b < NB; b += n_warps) {    // vector b's chunk sums, added in chunk order as with NB = 1
+                    float sum = 0.f;
+                    for (int w = 0; w < n_ch; ++w) sum += red[(b * n_warps + w) * 32 + lane];
+                    if (row < n) {
+                        partial[((size_t)b * n_seg + seg) * n_pad + row] = sum;
+                        result(b, row, sum);
+                    }
+                }
+                __syncthreads();                              // the sums are read before the next tile overwrites them
             }
         }
-        const size_t n_pad = (size_t)n_rb * kRowsPerBlock;
-        const int row = rb * kRowsPerBlock + lane;
-        if constexpr (NB == 1) {
-            float* red_i = red + (i & 1) * n_warps * 32;
-            red_i[warp * 32 + lane] = acc[0];
-            __syncthreads();                              // all reads of stage s are done; partial sums are visible
-            if (tid == 0 && i + kGemvStages < n_tiles) {
-                fence_proxy_async();
-                issue(i + kGemvStages);
-            }
-            if (warp == 0) {
-                float sum = 0.f;
-                for (int w = 0; w < n_ch; ++w) sum += red_i[w * 32 + lane];
-                if (row < n) partial[(size_t)seg * n_pad + row] = sum;
-            }
-        } else {
+        return true;
+    };
+    const bool done = tiles();
+    if (out != 2) return;
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();                                     // every CTA comes here, also one that gave up
+    if (done && cluster.block_rank() == 0 && threadIdx.x < 32) {
+        const int row = (int)blockIdx.y * kRowsPerBlock + lane;
+        for (int b = 0; b < NB; ++b) {
+            float part[8];
 #pragma unroll
-            for (int b = 0; b < NB; ++b) red[(b * n_warps + warp) * 32 + lane] = acc[b];
-            __syncthreads();
-            if (tid == 0 && i + kGemvStages < n_tiles) {
-                fence_proxy_async();
-                issue(i + kGemvStages);
-            }
-            for (int b = warp; b < NB; b += n_warps) {    // vector b's chunk sums, added in chunk order as with NB = 1
-                float sum = 0.f;
-                for (int w = 0; w < n_ch; ++w) sum += red[(b * n_warps + w) * 32 + lane];
-                if (row < n) partial[((size_t)b * n_seg + seg) * n_pad + row] = sum;
-            }
-            __syncthreads();                              // the sums are read before the next tile overwrites them
+            for (int s = 0; s < 8; ++s) part[s] = *cluster.map_shared_rank(&s_sum[b][lane], min(s, n_seg - 1));
+            float sum = 0.f;
+#pragma unroll
+            for (int s = 0; s < 8; ++s)
+                if (s < n_seg) sum += part[s];
+            if (row < n) store(b, row, sum);
         }
     }
+    cluster.sync();                                     // nobody leaves while its sums may be read
 }
 
 // grid.y = vector b: partial [b][n_seg][n_pad] -> y [b][n]
@@ -557,8 +651,9 @@ static int gemv_sm_count() {
     return n;
 }
 
-int launch_draft_gemv(const void* blob, const cass_blob_info& bi, const void* x_bf16, int nb, float* partial,
-                      int32_t* d_status, cudaStream_t stream) {
+// y_bf16 / y_f32 (either may be null): [nb][rows] results.  Both null: only `partial`, which the caller's next kernel adds.
+static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x_bf16, int nb, float* partial, uint16_t* y_bf16,
+                       float* y_f32, int32_t* d_status, cudaStream_t stream) {
     const int n_ch = ceil_div(bi.seg_cols, bi.chunk_cols);
     if (n_ch > 32) return CASS_ERR_UNSUPPORTED;
     if (nb != 1 && nb != 2 && nb != 4 && nb != 8) return CASS_ERR_UNSUPPORTED;
@@ -579,36 +674,51 @@ int launch_draft_gemv(const void* blob, const cass_blob_info& bi, const void* x_
         if (g > bi.n_rowblocks) g = bi.n_rowblocks;
     }
     if (g < 1) g = 1;
+    // results inside the kernel where the segments of a row block are one CTA, or a cluster of CTAs with one tile each
+    const bool want = y_bf16 || y_f32;
+    const int out = !want ? 0 : bi.n_seg == 1 ? 1 : (bi.n_seg <= 8 && g == bi.n_rowblocks) ? 2 : 0;
+    // with q = 1 - p kept, 8 kept columns span 8 / q columns, give or take sqrt(8 p) / q: more than 32 about once in 10^4 groups
+    // of a lane at p = 50 %, once in 40 at 60 %, and one lane's long gap costs its warp a careful walk (359 x 1467 at p = 60 %:
+    // 26 us without the second window, 12.8 with it)
+    const bool wide = bi.prune_permille > 520;
     dim3 grid(bi.n_seg, g), block(threads);
     const uint32_t* b = (const uint32_t*)blob;
     const uint16_t* x = (const uint16_t*)x_bf16;
     const int stage = (int)gemv_stage_bytes(bi);
-#define CASS_GEMV_LAUNCH(TT, NN)                                                                               \
+#define CASS_GEMV_LAUNCH(TT, NN, WW)                                                                             \
     do {                                                                                                       \
         static int attr_smem = 0;      /* largest size already granted to this instantiation */              \
         if ((int)smem > attr_smem) {                                                                           \
-            CASS_CUDA_CHECK(cudaFuncSetAttribute(k_draft_gemv<TT, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,\
+            CASS_CUDA_CHECK(cudaFuncSetAttribute((k_draft_gemv<TT, NN, WW>), cudaFuncAttributeMaxDynamicSharedMemorySize,\
                                                  (int)smem));                                                  \
             attr_smem = (int)smem;                                                                             \
         }                                                                                                      \
         cudaLaunchConfig_t cfg = {};                                                                           \
         cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;            \
-        cudaLaunchAttribute at[1];                                                                             \
+        cudaLaunchAttribute at[2];                                                                             \
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   /* prologue may overlap the predecessor */ \
         at[0].val.programmaticStreamSerializationAllowed = pdl_enabled();                                                  \
-        cfg.attrs = at; cfg.numAttrs = 1;                                                                      \
-        CASS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, k_draft_gemv<TT, NN>, b, x, partial, d_status, stage,         \
+        at[1].id = cudaLaunchAttributeClusterDimension;                                                        \
+        at[1].val.clusterDim.x = bi.n_seg; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;             \
+        cfg.attrs = at; cfg.numAttrs = out == 2 ? 2 : 1;                                                       \
+        CASS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, k_draft_gemv<TT, NN, WW>, b, x, partial, d_status, stage,         \
                                            (int)bi.max_superblock_bytes, (int)bi.rows, (int)bi.cols,           \
                                            (int)bi.trunc_bits, (int)bi.seg_cols, (int)bi.chunk_cols,           \
                                            (int)bi.n_seg, (int)bi.n_rowblocks,                                 \
-                                           (unsigned long long)bi.total_bytes));                               \
+                                           (unsigned long long)bi.total_bytes, out, y_bf16, y_f32));     \
     } while (0)
 #define CASS_GEMV_LAUNCH_NB(TT)                                                                                \
     do {                                                                                                       \
-        if (nb == 1) CASS_GEMV_LAUNCH(TT, 1);                                                                  \
-        else if (nb == 2) CASS_GEMV_LAUNCH(TT, 2);                                                             \
-        else if (nb == 4) CASS_GEMV_LAUNCH(TT, 4);                                                             \
-        else CASS_GEMV_LAUNCH(TT, 8);                                                                          \
+        constexpr bool kHasWide = TT >= 0;          /* the generic decoders search any distance */               \
+        if (wide && kHasWide) {                                                                                \
+            if (nb == 1) CASS_GEMV_LAUNCH(TT, 1, kHasWide);                                                    \
+            else if (nb == 2) CASS_GEMV_LAUNCH(TT, 2, kHasWide);                                               \
+            else if (nb == 4) CASS_GEMV_LAUNCH(TT, 4, kHasWide);                                               \
+            else CASS_GEMV_LAUNCH(TT, 8, kHasWide);                                                            \
+        } else if (nb == 1) CASS_GEMV_LAUNCH(TT, 1, false);                                                    \
+        else if (nb == 2) CASS_GEMV_LAUNCH(TT, 2, false);                                                      \
+        else if (nb == 4) CASS_GEMV_LAUNCH(TT, 4, false);                                                      \
+        else CASS_GEMV_LAUNCH(TT, 8, false);                                                                   \
     } while (0)
     if (bi.mode == 2 && bi.trunc_bits == 4) CASS_GEMV_LAUNCH_NB(104);
     else if (bi.mode == 2) CASS_GEMV_LAUNCH_NB(-2);
@@ -622,7 +732,17 @@ int launch_draft_gemv(const void* blob, const cass_blob_info& bi, const void* x_
 #undef CASS_GEMV_LAUNCH_NB
 #undef CASS_GEMV_LAUNCH
     CASS_LAUNCH_CHECK();
+    if (want && out == 0) {
+        const int n_pad = bi.n_rowblocks * kRowsPerBlock;
+        CASS_PDL_LAUNCH(k_gemv_finish, dim3(ceil_div(bi.rows, 256), nb), dim3(256), 0, stream, (const float*)partial, (int)bi.rows, n_pad,
+                        (int)bi.n_seg, y_bf16, y_f32);
+    }
     return CASS_OK;
+}
+
+int launch_draft_gemv(const void* blob, const cass_blob_info& bi, const void* x_bf16, int nb, float* partial,
+                      int32_t* d_status, cudaStream_t stream) {
+    return launch_gemv(blob, bi, x_bf16, nb, partial, nullptr, nullptr, d_status, stream);
 }
 
 }  // namespace cass
@@ -630,32 +750,16 @@ int launch_draft_gemv(const void* blob, const cass_blob_info& bi, const void* x_
 using namespace cass;
 
 extern "C" int cass_draft_gemv(const void* blob, const cass_blob_info* h_info, const void* x_bf16, float* partial,
-                               void* y_bf16, float* y_f32, int32_t* d_status, void* stream_) {
+                               void* y_bf16, float* y_f32, int32_t* d_status, void* stream) {
     if (!blob || !h_info || !x_bf16 || !partial) return CASS_ERR_INVALID_ARG;
-    cudaStream_t stream = (cudaStream_t)stream_;
-    int rc = launch_draft_gemv(blob, *h_info, x_bf16, 1, partial, d_status, stream);
-    if (rc) return rc;
-    if (!y_bf16 && !y_f32) return CASS_OK;
-    int n_pad = h_info->n_rowblocks * kRowsPerBlock;
-    k_gemv_finish<<<ceil_div(h_info->rows, 256), 256, 0, stream>>>(partial, h_info->rows, n_pad, h_info->n_seg,
-                                                                    (uint16_t*)y_bf16, y_f32);
-    CASS_LAUNCH_CHECK();
-    return CASS_OK;
+    return launch_gemv(blob, *h_info, x_bf16, 1, partial, (uint16_t*)y_bf16, y_f32, d_status, (cudaStream_t)stream);
 }
 
 extern "C" int cass_draft_gemv_batch(const void* blob, const cass_blob_info* h_info, const void* x_bf16, int n_vec,
-                                     float* partial, void* y_bf16, float* y_f32, int32_t* d_status, void* stream_) {
+                                     float* partial, void* y_bf16, float* y_f32, int32_t* d_status, void* stream) {
     if (!blob || !h_info || !x_bf16 || !partial) return CASS_ERR_INVALID_ARG;
     if (n_vec != 1 && n_vec != 2 && n_vec != 4 && n_vec != 8) return CASS_ERR_INVALID_ARG;
-    cudaStream_t stream = (cudaStream_t)stream_;
-    int rc = launch_draft_gemv(blob, *h_info, x_bf16, n_vec, partial, d_status, stream);
-    if (rc) return rc;
-    if (!y_bf16 && !y_f32) return CASS_OK;
-    int n_pad = h_info->n_rowblocks * kRowsPerBlock;
-    k_gemv_finish<<<dim3(ceil_div(h_info->rows, 256), n_vec), 256, 0, stream>>>(partial, h_info->rows, n_pad, h_info->n_seg,
-                                                                                 (uint16_t*)y_bf16, y_f32);
-    CASS_LAUNCH_CHECK();
-    return CASS_OK;
+    return launch_gemv(blob, *h_info, x_bf16, n_vec, partial, (uint16_t*)y_bf16, y_f32, d_status, (cudaStream_t)stream);
 }
 
 // ---- variant with built-in scratch ------------------------------------------------------------------------
@@ -682,12 +786,5 @@ extern "C" int cass_draft_gemv_static(const void* blob, const cass_blob_info* h_
         s_scratch[dev] = ptr;
     }
     float* partial = s_scratch[dev];
-    cudaStream_t stream = (cudaStream_t)stream_;
-    int rc = launch_draft_gemv(blob, *h_info, x_bf16, 1, partial, d_status, stream);
-    if (rc) return rc;
-    const int n_pad = h_info->n_rowblocks * kRowsPerBlock;
-    k_gemv_finish<<<ceil_div(h_info->rows, 256), 256, 0, stream>>>(partial, h_info->rows, n_pad, h_info->n_seg,
-                                                                    (uint16_t*)y_bf16, y_f32);
-    CASS_LAUNCH_CHECK();
-    return CASS_OK;
+    return launch_gemv(blob, *h_info, x_bf16, 1, partial, (uint16_t*)y_bf16, y_f32, d_status, (cudaStream_t)stream_);
 }
