@@ -1,4 +1,4 @@
-"""In-tree build of the CUDA library (sm_100a only) with nvcc; no torch extension machinery."""
+"""In-tree build of the CUDA library (sm_100a only) with nvcc and of its CPython entry points with g++; no torch extension machinery."""
 from __future__ import annotations
 
 import concurrent.futures
@@ -9,6 +9,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcass.so")
+FASTCALL = os.path.join(HERE, "_fastcall.so")          # CPython entry points of the library (csrc/fastcall.cpp)
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
          "--expt-relaxed-constexpr"]
@@ -23,6 +24,25 @@ def _stale(target: str, deps: list[str]) -> bool:
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _build_fastcall(header: str, force: bool) -> None:
+    src = os.path.join(CSRC, "fastcall.cpp")
+    if not force and not _stale(FASTCALL, [src, header]):
+        return
+    import sysconfig
+
+    import torch
+
+    troot = os.path.dirname(torch.__file__)
+    inc = [os.path.join(troot, "include"), os.path.join(troot, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")]
+    cmd = (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] +
+           [f"-I{i}" for i in inc] + [src, "-o", FASTCALL, "-L" + HERE, "-l:libcass.so", "-L" + os.path.join(troot, "lib"), "-ltorch_python", "-ltorch_cpu",
+                                     "-ltorch", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"])
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for {src}:\n{r.stdout}\n{r.stderr}")
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -55,6 +75,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
+    _build_fastcall(os.path.join(os.path.dirname(HERE), "include", "cass.h"), force)
     return LIB
 
 
