@@ -77,9 +77,15 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
     const uint32_t tmem = *tmem_slot;
     // Barriers and tensor memory are set up.  The weights are nobody's output: the first ring of weight tiles is
     // requested ahead of the wait for the preceding kernels, whose results are the activations and the scratch.
-    // (w_static = 0: the weights too come from a preceding kernel, e.g. rebuilt from their two parts: nothing is early)
+    // (kWeightsRebuilt: the weights too come from a preceding kernel, e.g. rebuilt from their two parts: nothing is early)
     const int n_pre = nkb < kTcStages ? nkb : kTcStages;
-    if (warp == 0 && lane == 0 && w_static) {
+    // (kWeightsInput: a caller's matrix, which a preceding kernel may be writing: its first tiles are asked for as far as L2,
+    // where a later write still finds them; memory is then busy while the previous call's parts are added: 12.1 instead of
+    // 13.1 us a call on 6144 x 4096)
+    if (warp == 0 && lane == 0 && w_static == kWeightsInput) {
+        for (int kb = 0; kb < n_pre; ++kb) tma_prefetch_2d(&map_w, (kb0 + kb) * kTcBK, m0);
+    }
+    if (warp == 0 && lane == 0 && w_static == kWeightsStatic) {
         for (int kb = 0; kb < n_pre; ++kb) {                 // stages are empty at the start: nothing to wait for
             mbar_expect_tx(&full[kb], kTcABytes + kTcBBytes);
             tma_load_2d(sA + kb * kTcABytes, &map_w, (kb0 + kb) * kTcBK, m0, &full[kb]);
@@ -91,7 +97,7 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
     if (warp == 0 && lane == 0) {
         // ---- producer: TMA loads into the ring ----
         for (int kb = 0; kb < n_pre; ++kb) {
-            if (!w_static) {
+            if (w_static != kWeightsStatic) {
                 mbar_expect_tx(&full[kb], kTcABytes + kTcBBytes);
                 tma_load_2d(sA + kb * kTcABytes, &map_w, (kb0 + kb) * kTcBK, m0, &full[kb]);
             }
@@ -156,12 +162,11 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
 
 __global__ void k_verify_gemm_finish(const float* __restrict__ partial, int rows, int bn, int n, int n_split,
                                      uint16_t* __restrict__ y_bf16, float* __restrict__ y_f32) {
-    pdl_early<5>();
+    pdl_launch_dependents();             // a few small CTAs: the next call's may come in beside them and start on their weights
     pdl_wait();
     const int j = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
     if (j >= n || r >= rows) return;
-    float acc = 0.f;
-    for (int s = 0; s < n_split; ++s) acc += partial[((size_t)s * bn + r) * n + j];
+    const float acc = parts_sum(Partials{partial, n_split, (size_t)bn * n, (size_t)n}, (size_t)r * n + j);
     if (y_f32) y_f32[(size_t)r * n + j] = acc;
     if (y_bf16) y_bf16[(size_t)r * n + j] = float_to_bf16_bits(acc);
 }
@@ -251,5 +256,5 @@ extern "C" int cass_verify_gemm(const void* W_bf16, const void* X_bf16, int rows
     if (n < 1 || k < 1 || scratch_bytes < cass_verify_gemm_scratch_bytes(n, k)) return CASS_ERR_CAPACITY;
     if (rows < 1 || rows > kMaxRows) return CASS_ERR_INVALID_ARG;
     return launch_verify_gemm((const uint16_t*)W_bf16, (const uint16_t*)X_bf16, rows, verify_gemm_bn(rows), n, k, (float*)scratch,
-                              (uint16_t*)y_bf16, y_f32, d_status, (cudaStream_t)stream);
+                              (uint16_t*)y_bf16, y_f32, d_status, (cudaStream_t)stream, kWeightsInput);
 }
