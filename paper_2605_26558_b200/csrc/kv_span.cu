@@ -10,7 +10,7 @@
 //   k_kv_codes     exponent words into the arena
 // One warp a record throughout; a record's words sit 128 bytes apart (32-token blocks), so the 8 warps of a CTA take
 // consecutive tokens and share sectors.  Bound: instruction issue of the selection (about 350 a record).
-#include "kernels.cuh"
+#include "kv_record.cuh"
 
 namespace cass {
 
@@ -24,76 +24,6 @@ struct KvSpan {
 };
 __device__ __forceinline__ size_t span_shift(const KvGeom& g, const KvSpan& sp, int z) {
     return (size_t)(z / sp.n_seq) * sp.layer_stride + (size_t)(sp.seq0 + z % sp.n_seq) * g.seq_stride;
-}
-
-// lane holds elements lane + 32 j.  bm[j] (the same in every lane): bit `lane` set for the kept ones, the d - n_prune
-// largest |x| (ties: the lower channel is pruned first).  Keys (|x| bits, channel) are unique; a threshold with exactly
-// n_prune keys below it is searched two bits at a time (three counts packed into one reduction) and the search ends with
-// the first one found.  It starts six binades below the largest value, where the threshold of an ordinary row lies, and
-// from zero if too many keys lie below that.
-template <int NJ>
-__device__ __forceinline__ void span_select(const uint32_t (&bits)[NJ], int nj, int n_prune, int lane, uint32_t (&bm)[NJ]) {
-    uint32_t key[NJ], big = 0;
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-        key[j] = j < nj ? (((bits[j] & 0x7FFFu) << 8) | (uint32_t)(lane + 32 * j)) : 0xFFFFFFFFu;
-        big = j < nj ? max(big, key[j]) : big;
-    }
-    uint32_t thr = 0;
-    if (n_prune > 0) {
-        big = __reduce_max_sync(0xffffffffu, big);
-        int bit = 20;                                                   // the next two bits to decide: bit + 1 and bit
-        uint32_t base = 0;
-        bool done = false;
-        if (big >= (6u << 15)) {
-            uint32_t c = 0;
-            const uint32_t low = big - (6u << 15);
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) c += key[j] < low;
-            c = __reduce_add_sync(0xffffffffu, c);
-            if ((int)c <= n_prune) { base = low; bit = 16; done = (int)c == n_prune; }      // within 6 x 2^15 < 2^18 of it
-        }
-        if (base == 0) {                                                // 23 key bits: the top one alone
-            uint32_t c = 0;
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) c += key[j] < (1u << 22);
-            if ((int)__reduce_add_sync(0xffffffffu, c) <= n_prune) base = 1u << 22;
-        }
-        thr = base;
-#pragma unroll 1
-        for (; bit >= 0 && !done; bit -= 2) {
-            const uint32_t c1 = thr + (1u << bit), c2 = thr + (2u << bit), c3 = thr + (3u << bit);
-            uint32_t c = 0;                                             // three counts of at most 256 each in one word
-#pragma unroll
-            for (int j = 0; j < NJ; ++j)
-                c += (uint32_t)(key[j] < c1) + ((uint32_t)(key[j] < c2) << 10) + ((uint32_t)(key[j] < c3) << 20);
-            c = __reduce_add_sync(0xffffffffu, c);
-            const int n1 = (int)(c & 1023u), n2 = (int)((c >> 10) & 1023u), n3 = (int)(c >> 20);      // n1 <= n2 <= n3
-            if (n3 <= n_prune) { thr = c3; done = n3 == n_prune; }
-            else if (n2 <= n_prune) { thr = c2; done = n2 == n_prune; }
-            else if (n1 <= n_prune) { thr = c1; done = n1 == n_prune; }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) bm[j] = __ballot_sync(0xffffffffu, j < nj && key[j] >= thr);
-}
-
-// Code lengths of a record's slices -> entry words and arena words (R: raw exponents where the codes take more room).
-template <int NJ>
-__device__ __forceinline__ uint32_t span_entries(const KvGeom& g, const uint32_t (&len)[NJ], int nj, uint32_t (&entry)[3]) {
-    uint32_t ub = 0;
-    entry[0] = entry[1] = entry[2] = 0;
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-        if (j >= nj) break;
-        if (j > 0) entry[(j - 1) / 3] |= (ub & 0x3FFu) << (20 - 10 * ((j - 1) % 3));
-        ub += __reduce_add_sync(0xffffffffu, len[j]);
-    }
-    if (ub > (uint32_t)kv_code_budget(g.kept)) {
-        entry[0] = kKvRawFlag; entry[1] = entry[2] = 0;
-        return (uint32_t)ceil_div(g.kept, 4);
-    }
-    return (ub + 31) / 32;
 }
 
 // grid ((tokens / 8, cut off), n_kv * 2, layers * sequences)
@@ -133,7 +63,7 @@ __global__ void __launch_bounds__(32 * kSpanWarps) k_kv_form(KvGeom g, KvComp ck
         }
         if (!(flags & CASS_KV_COMPRESSED)) continue;
         uint32_t bm[NJ];
-        span_select<NJ>(bits, nj, g.n_prune, lane, bm);
+        kv_select<NJ>(bits, nj, g.n_prune, lane, bm);
         const bool mx = g.mode == 2;
         const int bm0 = g.e_words;                                      // the bitmap's place in the record
         uint32_t len[NJ], kbase = 0, xw[2] = {0, 0};
@@ -143,13 +73,9 @@ __global__ void __launch_bounds__(32 * kSpanWarps) k_kv_form(KvGeom g, KvComp ck
             if (j >= nj) break;
             const bool keep = (bm[j] >> lane) & 1u;
             const uint32_t e = (bits[j] >> 7) & 0xFFu, k = kbase + __popc(bm[j] & lanemask_lt());
-            uint32_t field = ((bits[j] >> 15) << (7 - T)) | ((bits[j] & 0x7Fu) >> T);
-            if (mx) {                                                   // sign, magnitude in the slice's unit
-                const uint32_t E = __reduce_max_sync(0xffffffffu, keep ? e : 0u), sh = 1u + E - e;
-                const uint32_t m7 = (sh < 8u && e > 0u && E >= 7u) ? ((0x80u | (bits[j] & 0x7Fu)) >> sh) : 0u;
-                field = ((bits[j] >> 15) << (7 - T)) | (m7 >> T);
-                xw[j / 4] |= E << (24 - 8 * (j % 4));
-            }
+            uint32_t E;
+            const uint32_t field = kv_field<T>(bits[j], keep, mx, E);
+            xw[j / 4] |= E << (24 - 8 * (j % 4));
             if (keep) {
                 s_fld[warp][k] = (uint8_t)field;
                 if (HIST) atomicAdd(&s_len[e], 1u);
@@ -161,7 +87,7 @@ __global__ void __launch_bounds__(32 * kSpanWarps) k_kv_form(KvGeom g, KvComp ck
         if (!HIST) {
             uint32_t entry[3], nw = 0;
             if (!mx) {
-                nw = span_entries<NJ>(g, len, nj, entry);
+                nw = kv_entries<NJ>(g, len, nj, entry);
                 if (lane < g.e_words) rec[lane] = lane == 0 ? entry[0] : lane == 1 ? entry[1] : entry[2];
             }
             if (lane == 0) c.off[(size_t)head * (g.max_seq + 1) + pos + 1] = nw;       // k_kv_scan makes it an offset
@@ -170,20 +96,7 @@ __global__ void __launch_bounds__(32 * kSpanWarps) k_kv_form(KvGeom g, KvComp ck
         }
         if (mx && lane < g.x_words) rec[bm0 + nj + g.f_words + lane] = lane ? xw[1] : xw[0];
         __syncwarp();
-        for (int w = lane; w < g.f_words; w += 32) {
-            uint32_t acc = 0;
-#pragma unroll
-            for (int q = 0; q < PER; q += 4) {
-                const uint32_t four = *reinterpret_cast<const uint32_t*>(&s_fld[warp][w * PER + q]);
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const uint32_t f = (four >> (8 * b)) & 0xFFu;
-                    const uint32_t v = mx ? f << (32 - F * (q + b + 1)) : field_bits_in_word(f, q + b, T);
-                    acc |= w * PER + q + b < g.kept ? v : 0u;
-                }
-            }
-            rec[bm0 + nj + w] = acc;
-        }
+        kv_field_words<T>(g, s_fld[warp], rec + bm0 + nj, lane);
         __syncwarp();
         uint32_t* blk = c.fixed + ((size_t)head * g.n_blocks + pos / 32) * g.wpt * 32 + pos % 32;
         for (int w = (HIST ? g.e_words : 0) + lane; w < g.wpt; w += 32) blk[w * 32] = rec[w];
@@ -239,7 +152,7 @@ __global__ void __launch_bounds__(32 * kSpanWarps) k_kv_lengths(KvGeom g, KvComp
         }
 #pragma unroll
         for (int j = 0; j < NJ; ++j) len[j] = (bm[j] << lane) >> 31 ? s_len[(bits[j] >> 7) & 0xFFu] : 0u;
-        nw = span_entries<NJ>(g, len, nj, entry);
+        nw = kv_entries<NJ>(g, len, nj, entry);
         if (lane < g.e_words) blk[lane * 32] = lane == 0 ? entry[0] : lane == 1 ? entry[1] : entry[2];
         if (lane == 0) c.off[(size_t)head * (g.max_seq + 1) + pos + 1] = nw;
     }
