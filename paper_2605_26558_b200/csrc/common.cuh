@@ -177,13 +177,14 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 
 // Which kernel classes release their successor (griddepcontrol.launch_dependents) before they finish (bit per class:
 // 0 small operators, 1 KV encoder, 2 draft attention, 3 attention merge, 4 verification attention, 5 verification
-// GEMM).  A kernel outside the mask releases its successor when it exits; every kernel still starts with
-// griddepcontrol.wait, and the draft GEMV does its set-up (barriers, table, first weight copy) before that wait.
-// Measured on the full model (ms per speculative step / plain tokens per s): none 25.5 / 249, small operators + GEMM
-// 25.7 / 252, all but the KV encoder about the same, with the KV encoder 26.6 / 224, all 27.1 / 226: an early release
-// mostly lets the successor's CTAs take SM resources while they wait, so the default releases nothing early.
+// GEMM, 6 draft GEMV).  A kernel outside the mask releases its successor when it exits.  The release always comes after the
+// kernel's own griddepcontrol.wait, so that whoever starts finds everything before its predecessor complete, and after its
+// tensor-memory allocation.  The successor's set-up (barriers, tables, its first weight copies) then runs while the last CTAs
+// finish: decode step of the 8B shape 6.73 -> 6.54 ms, smallest draft GEMV 6.3 -> 5.3 us a call, projection 12.2 -> 10.6.
+// (Released before the wait, waiting CTAs took the predecessor's place: 25.5 -> 27.1 ms on the full model.)
+// Draft attention and the merge keep their successors out: 14.3 -> 13.5 us a stand-alone attention, the step the same.
 #ifndef CASS_PDL_EARLY_MASK
-#define CASS_PDL_EARLY_MASK 0x00
+#define CASS_PDL_EARLY_MASK 0x73
 #endif
 template <int CLS>
 __device__ __forceinline__ void pdl_early() {

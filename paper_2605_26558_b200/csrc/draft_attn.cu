@@ -16,8 +16,8 @@ __global__ void __launch_bounds__(kMergeThreads) k_attn_merge(AttnScratch sc, in
                                                               uint16_t* __restrict__ out) {
     extern __shared__ __align__(16) float w_s[];    // [n_chunks_alloc] weights e^{m_c - M}, then [kMergeWarps][d] partial outputs
     __shared__ float s_red[kMergeWarps];
-    pdl_early<3>();
     pdl_wait();
+    pdl_early<3>();
     const int hq = blockIdx.x, r = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int sub = ar.hi - ar.lo, seq = r / sub, n_chunks_alloc = ar.chunks;
@@ -107,8 +107,8 @@ template <int MC>
 __global__ void __launch_bounds__(kMergeThreads) k_attn_merge_few(AttnScratch sc, int chunk_tokens, AttnRows ar, int n_pairs, int n_q, int d,
                                                                   const DevState* __restrict__ st, int draft_mode, int draft_units,
                                                                   uint16_t* __restrict__ out) {
-    pdl_early<3>();
     pdl_wait();
+    pdl_early<3>();
     const int pair = blockIdx.x * kMergeWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (pair >= n_pairs) return;
     const int r = pair / n_q, hq = pair % n_q, sub = ar.hi - ar.lo, seq = r / sub, row = ar.lo + r % sub;

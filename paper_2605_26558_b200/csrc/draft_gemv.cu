@@ -485,6 +485,7 @@ __global__ void __launch_bounds__(1024) k_draft_gemv(const uint32_t* __restrict_
         // Everything above touches only the blob, which no kernel writes.  When the launch allows this grid to start
         // before its predecessor in the stream has finished, wait here: x and the scratch `partial` are the predecessor's.
         pdl_wait();
+        pdl_early<6>();
         // x of this segment (fp32), zero beyond the matrix
         const int c0 = seg * seg_cols;
         if constexpr (NB > 1) {

@@ -76,8 +76,8 @@ __global__ void __launch_bounds__(32 * kKvWarps) k_kv_append(KvGeom g, KvComp ck
     // The codebook tables were written when the codebook was frozen, long before this launch's predecessor: they may be
     // read ahead of the wait, which hides their latency.
     if (coded && (!FUSED || head < g.n_kv)) s_len[threadIdx.x] = of_seq((kind ? cv : ck).exp_to_rank, seq, g.seq_stride)[threadIdx.x] + 1u;
-    pdl_early<1>();
     pdl_wait();
+    pdl_early<1>();
     int start_pos = start_pos_arg;
     if (FUSED || start_pos < 0) start_pos = st->len[seq] + (use_inflight ? st->inflight[seq] : 0);
     if (FUSED && head >= g.n_kv) {

@@ -17,8 +17,8 @@ __global__ void k_rope_table(float* __restrict__ cos_t, float* __restrict__ sin_
 
 __global__ void k_embed(const int32_t* __restrict__ toks, int rps, int seq_stride, const uint16_t* __restrict__ embed,
                         uint16_t* __restrict__ h, int hidden) {
-    pdl_early<0>();
     pdl_wait();
+    pdl_early<0>();
     int r = blockIdx.x;
     const uint16_t* src = embed + (size_t)toks[(size_t)(r / rps) * seq_stride + r % rps] * hidden;
     uint16_t* dst = h + (size_t)r * hidden;
@@ -68,8 +68,8 @@ __global__ void __launch_bounds__(1024) k_residual_rmsnorm(uint16_t* __restrict_
         const int i = threadIdx.x * 4 + it * (int)blockDim.x * 4;
         gvs[it] = (out && i < hidden) ? __ldg(reinterpret_cast<const uint2*>(gain + i)) : make_uint2(0u, 0u);
     }
-    pdl_early<0>();
     pdl_wait();
+    pdl_early<0>();
     const int r = blockIdx.x;
     uint16_t* hr = h + (size_t)r * hidden;
     float vals[ITERS][4];
@@ -130,8 +130,8 @@ __global__ void __launch_bounds__(1024) k_residual_rmsnorm(uint16_t* __restrict_
 __global__ void __launch_bounds__(128) k_qkv_rope(uint16_t* __restrict__ qkv, Partials pp,
                                                   const float* __restrict__ cos_t, const float* __restrict__ sin_t,
                                                   const DevState* __restrict__ st, int use_inflight, int rps, int n_q, int n_kv, int d) {
-    pdl_early<0>();
     pdl_wait();
+    pdl_early<0>();
     const int r = blockIdx.y, half = d / 2;
     const int qkv_dim = (n_q + 2 * n_kv) * d;
     const int b = r / rps;
@@ -181,8 +181,8 @@ __global__ void __launch_bounds__(128) k_qkv_rope(uint16_t* __restrict__ qkv, Pa
 // Four features a thread: 16-byte loads of the parts, one address for four.  (One a thread was bound by instruction issue in a
 // prefill pass: 18.3 us for 128 rows of 14336, 29 MB of parts.)
 __global__ void __launch_bounds__(128) k_swiglu(const uint16_t* __restrict__ gu, Partials pp, uint16_t* __restrict__ act, int ffn) {
-    pdl_early<0>();
     pdl_wait();
+    pdl_early<0>();
     const int r = blockIdx.y;
     for (int i = (blockIdx.x * blockDim.x + threadIdx.x) * 4; i < ffn; i += gridDim.x * blockDim.x * 4) {
         float g[4], u[4];
@@ -219,8 +219,8 @@ __global__ void __launch_bounds__(256) k_argmax_part(const float* __restrict__ l
                                                      int32_t* __restrict__ tmp_i, float* __restrict__ logits_copy) {
     __shared__ float s_v[8];
     __shared__ int s_i[8];
-    pdl_early<0>();
     pdl_wait();
+    pdl_early<0>();
     const int r = blockIdx.y, nsl = gridDim.x;
     const int per = ceil_div(vocab, nsl);
     const int lo = blockIdx.x * per, hi = min(vocab, lo + per);
@@ -256,8 +256,8 @@ __global__ void __launch_bounds__(kArgmaxSlices) k_argmax_final(const float* __r
                                                                 int bump_inflight) {
     __shared__ float s_v[kArgmaxSlices / 32];
     __shared__ int s_i[kArgmaxSlices / 32];
-    pdl_early<0>();
     pdl_wait();
+    pdl_early<0>();
     const int r = blockIdx.x;
     float best = -INFINITY;
     int best_i = 0x7fffffff;
@@ -286,8 +286,8 @@ __global__ void __launch_bounds__(kArgmaxSlices) k_argmax_final(const float* __r
 // next_tok[b * next_stride].
 __global__ void k_accept(DevState* st, const int32_t* __restrict__ draft, int draft_stride, const int32_t* __restrict__ target, int g,
                          int32_t* n_acc, int32_t* out_tokens, int32_t* next_tok, int next_stride) {
-    pdl_early<0>();
     pdl_wait();
+    pdl_early<0>();
     if (threadIdx.x != 0) return;
     const int b = blockIdx.x;
     draft += (size_t)b * draft_stride;
@@ -311,8 +311,8 @@ __global__ void k_accept(DevState* st, const int32_t* __restrict__ draft, int dr
 
 __global__ void k_calib_accum(const uint16_t* __restrict__ x, int rows, int cols, float* __restrict__ sumsq,
                               const DevState* __restrict__ st) {
-    pdl_early<0>();
     pdl_wait();
+    pdl_early<0>();
     if (!st->calib_on) return;
     int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= cols) return;

@@ -19,8 +19,8 @@ __global__ void __launch_bounds__(kVaThreads) k_verify_attn(KvGeom g, const uint
                                                             AttnRows ar, int n_groups, int n_q, const DevState* __restrict__ st,
                                                             AttnScratch sc) {
     extern __shared__ __align__(16) uint8_t smem[];
-    pdl_early<4>();
     pdl_wait();
+    pdl_early<4>();
     const int chunk = blockIdx.x, head = blockIdx.y, seq = blockIdx.z / n_groups;
     const int first = ar.lo + (int)(blockIdx.z % n_groups) * ar.group;            // the group's rows: row r of it sits at position len + r
     const int rows = min(ar.group, ar.hi - first);

@@ -56,7 +56,6 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
                                                                 int n_q, int n_kv, const DevState* __restrict__ st, AttnScratch sc,
                                                                 int32_t* __restrict__ d_status) {
     extern __shared__ uint8_t smem_dyn[];
-    pdl_early<4>();
     pdl_wait();
     const int chunk = blockIdx.x, head = blockIdx.y, seq = blockIdx.z / n_groups;
     const int first = ar.lo + (int)(blockIdx.z % n_groups) * ar.group;        // the group's rows: row r of it sits at position len + r
@@ -122,6 +121,7 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_early<4>();                                    // not before the tensor memory is held: a successor takes its own ahead of its wait
     const uint32_t tmem = *tmem_slot;
     bool ok = true;
 

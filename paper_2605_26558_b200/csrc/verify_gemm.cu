@@ -91,8 +91,8 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
             tma_load_2d(sA + kb * kTcABytes, &map_w, (kb0 + kb) * kTcBK, m0, &full[kb]);
         }
     }
-    pdl_early<5>();
     pdl_wait();
+    pdl_early<5>();
 
     if (warp == 0 && lane == 0) {
         // ---- producer: TMA loads into the ring ----
