@@ -8,7 +8,7 @@
 // values on the tensor pipe.  P is split into two bf16 terms (p = hi + lo) so that the product keeps fp32-level
 // accuracy; K, V and q are bf16 by definition, so the operands are exact.
 // Records are walked like the weight streams: 8 kept values per 32-bit bitmap window, 4 codewords per 32-bit unary
-// window, positions by bfind with the used bit cleared; a careful walk redoes the rare group that does not fit its
+// window, positions by bfind with the used bits shifted out; a careful walk redoes the rare group that does not fit its
 // windows and reads records with raw exponents or more code words than the staging holds.
 // Decoding a record with d/32 lanes (one per 32-channel slice, 16 warps per CTA) into the same tiles was measured and
 // dropped: 11.6 / 27.7 / 155 us at 600 / 4096 / 32768 positions against 11.0 / 16.7 / 75.4 us for the whole record per
@@ -21,9 +21,9 @@ namespace cass {
 
 constexpr int kTcTok = kAttnChunk;            // tokens per CTA
 constexpr int kTcThreads = 128;
-// Staged exponent words per token: room for 5 code bits per kept value (a typical record takes 2-3), the whole code
-// budget at most; longer records and records with raw exponents are read in place.  A warp's staging has two rows more:
-// a window reads the word of its cursor and the next.
+// Staged exponent words: a warp's 32 tokens share room for 5 code bits per kept value (a typical record takes 2-3), the whole
+// code budget at most; records that do not fit it and records with raw exponents are read in place.  A warp's staging has 64
+// words more: a window reads the word of its cursor and the next, and a walk that lost its way up to 6 beyond its end.
 __host__ __device__ inline int tc_una_stage(const KvGeom& g) {
     int w = ceil_div(5 * g.kept, 32);
     if (w > g.rec_words_max) w = g.rec_words_max;
@@ -32,11 +32,6 @@ __host__ __device__ inline int tc_una_stage(const KvGeom& g) {
 constexpr int kTcHeads = 8;                   // query heads per KV head the N = 8 operand holds
 constexpr int kTcPad = 8;                     // halfwords of padding per tile row: rows 16 bytes apart modulo 128
 
-__device__ __forceinline__ uint32_t tc_shl(uint32_t v, uint32_t s) {          // shift counts >= 32 give 0
-    uint32_t r;
-    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
-    return r;
-}
 __device__ __forceinline__ uint32_t tc_bfind(uint32_t v) {                    // most significant set bit, 0xFFFFFFFF if none
     uint32_t r;
     asm("bfind.u32 %0, %1;" : "=r"(r) : "r"(v));
@@ -60,6 +55,10 @@ __device__ __forceinline__ uint32_t tc_mad(uint32_t a, uint32_t b, uint32_t c) {
 }
 __device__ __forceinline__ void tc_sts16(uint32_t a, uint32_t v) {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v));
+}
+template <int OFF>
+__device__ __forceinline__ void tc_sts16_off(uint32_t a, uint32_t v) {
+    asm volatile("st.shared.u16 [%0+%2], %1;" ::"r"(a), "h"((uint16_t)v), "n"(OFF));
 }
 __device__ __forceinline__ void tc_ldmatrix_x4(uint32_t (&r)[4], uint32_t a) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
@@ -119,17 +118,23 @@ __device__ __noinline__ void tc_walk_slow(const uint32_t* bm, const uint32_t* fl
 }
 
 // Walk of one staged record by one lane: `kept` values go to the dense row at row_a (bf16, column c at row_a + 2 c).
-// bm_a / fl_a / un_a: shared addresses of this lane's first bitmap / field / unary word (words 128 bytes apart);
-// lut_a: shared address of the rank -> (exponent << 7) table.  A group whose 8 columns span more than 32 columns, or
+// bmP / flP: this lane's first bitmap / field word (words 128 bytes apart); unP: its first exponent word (words in sequence);
+// lutP: rank -> (exponent << 7).  Windows are consumed by funnel shifts, which leave the next bit on top: a position counts
+// from the one before it, and the running sums are multiply-adds, a pipe that has nothing else to do here.
+// Bound: the bit searches (two a value, one every 8 cycles) and the shifts and masks around them: 13 instructions a value
+// with the used bits cleared by shift and mask took 3.7 us for the 64 + 64 records of a CTA, 14 warps an SM.  With the records
+// copied in runs of 16 bytes (and the arena's words as they lie, not token by token) the kernel went from 29.0 to 25 us at 8192
+// positions, a call at 4096 from 14.7 to 13.5.
+// A group whose 8 columns span more than 32 columns, or
 // whose 4 codewords take more than 32 bits, shows up as a bit search that found nothing; that lane stores nothing for
 // the group and redoes it with the careful walk.  `emit` = false: the lane only keeps the warp in step.
 template <int T>
 __device__ __forceinline__ void tc_walk(const uint32_t* bmP, const uint32_t* flP, const uint32_t* unP, const uint32_t* lutP, const uint8_t* r2e,
-                                        int kept, int d, uint32_t una_bits, uint32_t row_a, bool emit, int stage) {
+                                        int kept, int d, uint32_t una_bits, uint32_t row_a, bool emit) {
     constexpr int F = 8 - T, PER = 32 / F, NFW = kGroupCols / PER;
     constexpr uint32_t MASK16 = 0x8000u | (((1u << (7 - T)) - 1u) << T);
     static_assert(PER == 4 || PER == 8, "fields tile a word");
-    const uint32_t bm_a = smem_u32(bmP), un_a = smem_u32(unP), lut_a = smem_u32(lutP);
+    const uint32_t bm_a = smem_u32(bmP), un_a = smem_u32(unP), lut_top = smem_u32(lutP) + 124u;
     uint32_t fl_a = smem_u32(flP);
     uint32_t bpos = 0, upos = 0;
     const int n_full = kept / kGroupCols, rem = kept % kGroupCols;
@@ -139,7 +144,8 @@ __device__ __forceinline__ void tc_walk(const uint32_t* bmP, const uint32_t* flP
         const uint32_t bpos0 = bpos, upos0 = upos;
         const uint32_t ba = bm_a + (bpos >> 5) * 128u;
         uint32_t bv = __funnelshift_l(tc_lds_off<128>(ba), tc_lds(ba), bpos);        // 32 columns from bpos on
-        const uint32_t xg = row_a + bpos * 2u + 62u;                                 // address of column bpos + 31
+        uint32_t xg = row_a + bpos * 2u;                                             // + 64 (e + 1) - 2: address of the e-th value's column
+        const uint32_t xg0 = xg;
         uint32_t fwd[NFW];
         fwd[0] = tc_lds(fl_a);
         if (NFW > 1) fwd[NFW - 1] = tc_lds_off<128>(fl_a);
@@ -147,38 +153,42 @@ __device__ __forceinline__ void tc_walk(const uint32_t* bmP, const uint32_t* flP
         uint32_t dry = 0, p = 0;
 #pragma unroll
         for (int half = 0; half < kGroupCols / kGroupCodes; ++half) {
-            const uint32_t ua = un_a + (upos >> 5) * 128u;
-            uint32_t uv = __funnelshift_l(tc_lds_off<128>(ua), tc_lds(ua), upos);    // 32 code bits from upos on
-            uint32_t la = lut_a + 124u;             // lut + 4 * (position of the previous terminator - 1); none yet: 32
+            const uint32_t ua = un_a + (upos >> 5) * 4u;
+            uint32_t uv = __funnelshift_l(tc_lds_off<4>(ua), tc_lds(ua), upos);      // 32 code bits from upos on
             uint32_t q = 0;
+            upos += 32u * kGroupCodes;
 #pragma unroll
             for (int j = 0; j < kGroupCodes; ++j) {
                 const int e = half * kGroupCodes + j;
-                p = tc_bfind(bv);                                     // next kept column: bpos + 31 - p
-                addr[e] = tc_mad(p, 0xFFFFFFFEu, xg);
-                bv &= ~tc_shl(1u, p);
-                q = tc_bfind(uv);                                     // next terminator
-                const uint32_t eb = tc_lds(tc_mad(q, 0xFFFFFFFCu, la));              // lut[previous - q - 1]
-                la = tc_mad(q, 4u, lut_a - 4u);
-                uv &= ~tc_shl(1u, q);
+                p = tc_bfind(bv);                                     // next kept column: 31 - p columns on
+                xg = tc_mad(p, 0xFFFFFFFEu, xg);
+                addr[e] = xg;
+                bv = __funnelshift_r(0u, bv, p);
+                q = tc_bfind(uv);                                     // next terminator: rank 31 - q
+                const uint32_t eb = tc_lds(tc_mad(q, 0xFFFFFFFCu, lut_top));
+                upos = tc_mad(q, 0xFFFFFFFFu, upos);
+                uv = __funnelshift_r(0u, uv, q);
                 const uint32_t fword = fwd[e / PER];
                 val[e] = (__funnelshift_l(fword, fword, (F * (e % PER) + 16) & 31) & MASK16) | eb;
                 if (tail && e < rem) dry |= p | q;
             }
-            upos += 32u - q;                                          // bits up to and including the last terminator
             if (!tail) dry |= q;                                      // a search that failed fails from then on
         }
-        bpos += 32u - p;
+        bpos += 32u * kGroupCols - ((xg0 - xg) >> 1);
         if (!tail) dry |= p;
         const bool ok = (int32_t)dry >= 0;
         if (emit && ok) {                                             // one branch per group: the stores themselves are unconditional
-#pragma unroll
-            for (int e = 0; e < kGroupCols; ++e)
-                if (!tail || e < rem) tc_sts16(addr[e], val[e]);
+            auto put = [&](auto e_c) {
+                constexpr int e = decltype(e_c)::value;
+                if (!tail || e < rem) tc_sts16_off<64 * (e + 1) - 2>(addr[e], val[e]);
+            };
+            put(std::integral_constant<int, 0>{}); put(std::integral_constant<int, 1>{}); put(std::integral_constant<int, 2>{});
+            put(std::integral_constant<int, 3>{}); put(std::integral_constant<int, 4>{}); put(std::integral_constant<int, 5>{});
+            put(std::integral_constant<int, 6>{}); put(std::integral_constant<int, 7>{});
         } else if (emit) {
             // redo the group value by value, then put the cursors behind it
             const int cnt = tail ? rem : kGroupCols;
-            tc_walk_slow<T>(bmP, flP, unP, 32, false, grp * kGroupCols, cnt, bpos0, upos0, (uint32_t)d, una_bits, r2e, row_a);
+            tc_walk_slow<T>(bmP, flP, unP, 1, false, grp * kGroupCols, cnt, bpos0, upos0, (uint32_t)d, una_bits, r2e, row_a);
             uint32_t b = bpos0, u = upos0;
             for (int e = 0; e < cnt; ++e) {
                 while (b < (uint32_t)d) {
@@ -187,7 +197,7 @@ __device__ __forceinline__ void tc_walk(const uint32_t* bmP, const uint32_t* flP
                     b = (b | 31u) + 1u;
                 }
                 while (u < una_bits) {
-                    const uint32_t v = unP[(u >> 5) * 32] << (u & 31);
+                    const uint32_t v = unP[u >> 5] << (u & 31);
                     if (v) { u += __clz(v) + 1; break; }
                     u += 32u - (u & 31u);
                 }
@@ -195,7 +205,7 @@ __device__ __forceinline__ void tc_walk(const uint32_t* bmP, const uint32_t* flP
             bpos = b; upos = u;
         }
         bpos = min(bpos, (uint32_t)d);                                // a walk that lost its way stays inside the staging
-        upos = min(upos, (uint32_t)stage * 32u);
+        upos = min(upos, una_bits);
         fl_a += NFW * 128u;
     };
     for (int grp = 0; grp < n_full; ++grp) group(grp, std::false_type{});
@@ -240,7 +250,7 @@ __device__ __noinline__ void tc_walk_mx_slow(const uint32_t* bm, const uint32_t*
 // slice table (d / 32 + 2 rows).
 template <int T>
 __device__ __forceinline__ void tc_walk_mx(const uint32_t* bmP, const uint32_t* flP, const uint32_t* xP, uint32_t* ebP, const uint2* lutP,
-                                           int kept, int d, uint32_t row_a) {
+                                           int kept, int d, uint32_t row_a, bool emit) {
     constexpr int F = 8 - T, PER = 32 / F, NFW = kGroupCols / PER;
     static_assert(PER == 4 || PER == 8, "fields tile a word");
     const int S = d / 32;
@@ -260,10 +270,10 @@ __device__ __forceinline__ void tc_walk_mx(const uint32_t* bmP, const uint32_t* 
         const uint32_t bpos0 = bpos;
         const uint32_t ba = bm_a + (bpos >> 5) * 128u;
         uint32_t bv = __funnelshift_l(tc_lds_off<128>(ba), tc_lds(ba), bpos);        // 32 columns from bpos on
-        const uint32_t xg = row_a + bpos * 2u + 62u;                                 // address of column bpos + 31
+        uint32_t xg = row_a + bpos * 2u;                                             // + 64 (e + 1) - 2: address of the e-th value's column
+        const uint32_t xg0 = xg, next_slice = row_a + (bpos >> 5) * 64u + 64u;
         const uint32_t ea = eb_a + (bpos >> 5) * 128u;
         const uint32_t eb0 = tc_lds(ea), eb1 = tc_lds_off<128>(ea);                  // this slice's exponent and the next one's
-        const int pb = (int)(bpos & 31u) - 1;                                        // window bits <= pb lie in the next slice
         uint32_t fwd[NFW];
         fwd[0] = tc_lds(fl_a);
         if (NFW > 1) fwd[NFW - 1] = tc_lds_off<128>(fl_a);
@@ -271,23 +281,24 @@ __device__ __forceinline__ void tc_walk_mx(const uint32_t* bmP, const uint32_t* 
         uint32_t dry = 0, p = 0;
 #pragma unroll
         for (int e = 0; e < kGroupCols; ++e) {
-            p = tc_bfind(bv);                                         // next kept column: bpos + 31 - p
-            addr[e] = tc_mad(p, 0xFFFFFFFEu, xg);
-            bv &= ~tc_shl(1u, p);
+            p = tc_bfind(bv);                                         // next kept column: 31 - p columns on
+            xg = tc_mad(p, 0xFFFFFFFEu, xg);
+            addr[e] = xg + (64u * (e + 1) - 2u);
+            bv = __funnelshift_r(0u, bv, p);
             const uint32_t f = (fwd[e / PER] >> (32 - F * (e % PER + 1))) & ((1u << F) - 1u);
             const uint2 lm = tc_lds64(lut_a + f * 8u);
-            const uint32_t eb = (int)p <= pb ? eb1 : eb0;
+            const uint32_t eb = addr[e] >= next_slice ? eb1 : eb0;
             val[e] = lm.x + (eb & lm.y);
             if (tail && e < rem) dry |= p;
         }
-        bpos += 32u - p;
+        bpos += 32u * kGroupCols - ((xg0 - xg) >> 1);
         if (!tail) dry |= p;                                          // a search that failed fails from then on
         const bool ok = (int32_t)dry >= 0;
-        if (ok) {                                                     // one branch per group: the stores themselves are unconditional
+        if (emit && ok) {                                                     // one branch per group: the stores themselves are unconditional
 #pragma unroll
             for (int e = 0; e < kGroupCols; ++e)
                 if (!tail || e < rem) tc_sts16(addr[e], val[e]);
-        } else {
+        } else if (emit) {
             const int cnt = tail ? rem : kGroupCols;
             tc_walk_mx_slow<T>(bmP, flP, ebP, lutP, grp * kGroupCols, cnt, bpos0, (uint32_t)d, row_a);
             uint32_t b = bpos0;
@@ -308,10 +319,12 @@ __device__ __forceinline__ void tc_walk_mx(const uint32_t* bmP, const uint32_t* 
 }
 
 
-__device__ __forceinline__ void tc_cp_async4(uint32_t dst, const void* src, bool take) {      // take = false: zero fill
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(take ? 4 : 0) : "memory");
+__device__ __forceinline__ void tc_cp_async4(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
-__device__ __forceinline__ void tc_cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void tc_cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
 __device__ __forceinline__ void tc_cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Words of the record staging; the scores and probabilities take its place once the records are decoded.
@@ -332,17 +345,21 @@ __global__ void __launch_bounds__(kTcThreads) k_draft_attn_tc(KvGeom g, KvComp c
                                                               int qkv_stride, int n_q, const DevState* __restrict__ st, AttnScratch sc,
                                                               int n_chunks_alloc) {
     extern __shared__ __align__(16) uint8_t smem[];
-    pdl_early<2>();
     pdl_wait();
+    pdl_early<2>();
     const int run = blockIdx.x, head = blockIdx.y, seq = blockIdx.z;
+    // the query heads of the group, bf16 as they are: requested with the length
+    const int tid = threadIdx.x, G = n_q / g.n_kv, d = g.d;
+    const uint32_t* q_g = reinterpret_cast<const uint32_t*>(qkv + (size_t)seq * qkv_stride + (size_t)head * G * d);
+    uint32_t qv[kTcHeads];                                                    // word tid of every head (d / 2 <= kTcThreads)
+#pragma unroll
+    for (int h = 0; h < kTcHeads; ++h) qv[h] = h < G && tid < d / 2 ? __ldg(q_g + h * (d / 2) + tid) : 0u;
     const int cur_len = st->len[seq] + st->inflight[seq] + 1;  // positions visible to the drafted token
     const int run_tokens = tc_run_tokens(cur_len, g.n_kv * (int)gridDim.z);
     const int t_begin = run * run_tokens;
     if (t_begin >= cur_len) return;
     const int t_end = min(cur_len, t_begin + run_tokens);
-    const int G = n_q / g.n_kv, d = g.d;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    qkv += (size_t)seq * qkv_stride;
+    const int lane = tid & 31, warp = tid >> 5;
 
     const int ks = d + kTcPad;                                                // halfwords per tile row
     uint16_t* kt_s = reinterpret_cast<uint16_t*>(smem);                       // [64][ks] dense K, bf16
@@ -365,7 +382,7 @@ __global__ void __launch_bounds__(kTcThreads) k_draft_attn_tc(KvGeom g, KvComp c
     const uint32_t* off_h = of_seq(c.off, seq, g.seq_stride) + (size_t)head * (g.max_seq + 1);
     const uint32_t* arena = of_seq(c.arena, seq, g.seq_stride) + (size_t)head * g.arena_words;
     const uint8_t* r2e = of_seq(c.rank_to_exp, seq, g.seq_stride);
-    // Tokens beyond the visible length take the last visible token's record (their probabilities are zero).
+    // Tokens beyond the visible length leave their rows zero, as their probabilities are.
     auto load_off = [&](int t0, uint32_t& o0, uint32_t& n_una) {
         o0 = 0; n_una = 0;
         if (MODE != 1) return;                                                // Cassandra-2 records have no exponent stream
@@ -386,24 +403,10 @@ __global__ void __launch_bounds__(kTcThreads) k_draft_attn_tc(KvGeom g, KvComp c
         const uint8_t *rk = of_seq(ck0.rank_to_exp, seq, g.seq_stride), *rv = of_seq(cv0.rank_to_exp, seq, g.seq_stride);
         lut_v = tid < 32 ? rk[tid] : rv[tid - 32];
     }
-    constexpr int kQIter = 4;                                                 // query words per thread and batch
-    const int n_qw = G * d / 2;
-    for (int i = tid; i < kTcHeads * ks / 2; i += kTcThreads) reinterpret_cast<uint32_t*>(q_s)[i] = 0u;   // unused heads stay zero
+#pragma unroll
+    for (int h = 0; h < kTcHeads; ++h)                                        // unused heads are zero
+        if (tid < d / 2) reinterpret_cast<uint32_t*>(q_s + h * ks)[tid] = qv[h];
     if (tid < 3 * kTcHeads) run_s[tid] = tid % 3 == 0 ? -INFINITY : 0.f;
-    __syncthreads();
-    for (int i0 = tid; i0 < n_qw; i0 += kTcThreads * kQIter) {                // the query heads of the group, bf16 as they are
-        uint32_t qv[kQIter];
-#pragma unroll
-        for (int u = 0; u < kQIter; ++u) {
-            const int i = i0 + u * kTcThreads;
-            qv[u] = i < n_qw ? __ldg(reinterpret_cast<const uint32_t*>(qkv + (size_t)(head * G + i / (d / 2)) * d) + i % (d / 2)) : 0u;
-        }
-#pragma unroll
-        for (int u = 0; u < kQIter; ++u) {
-            const int i = i0 + u * kTcThreads;
-            if (i < n_qw) reinterpret_cast<uint32_t*>(q_s + (i / (d / 2)) * ks)[i % (d / 2)] = qv[u];
-        }
-    }
     if (MODE == 1) {
         if (tid < 64) lut_s[tid] = lut_v << 7;
     } else {
@@ -430,20 +433,18 @@ __global__ void __launch_bounds__(kTcThreads) k_draft_attn_tc(KvGeom g, KvComp c
     for (int t0 = t_begin; t0 < t_end; t0 += kTcTok) {
         o0 = o0_next; n_una = nu_next;
         const int n_here = min(32, cur_len - (t0 + tw * 32));                 // visible tokens of this warp's block (may be <= 0)
+        uint32_t una_base = 0;
         if (n_here > 0) {
-            const int src_lane = min(lane, n_here - 1);
+            // 32 tokens' fixed parts are one block, their exponent words one run of the arena: both copied as they lie
             const uint32_t* fixed = fixed_h + (size_t)((t0 + tw * 32) / 32) * g.wpt * 32;
-            const uint32_t fa = smem_u32(my_fix + lane);
-            for (int w = 0; w < g.wpt; ++w) tc_cp_async4(fa + w * 128, fixed + w * 32 + src_lane, true);      // coalesced block copy
+            const uint32_t fa = smem_u32(my_fix);
+            for (int w = lane; w < g.wpt * 8; w += 32) tc_cp_async16(fa + w * 16, fixed + w * 4);
             my_fix[g.wpt * 32 + lane] = 0u;
             if (MODE == 1) {
-                const uint32_t ua = smem_u32(my_una + lane);
-                const bool fits = n_una <= (uint32_t)stage;
-#pragma unroll 4
-                for (int w = 0; w < una_rows; ++w) {
-                    const bool take = fits && (uint32_t)w < n_una;
-                    tc_cp_async4(ua + w * 128, arena + (take ? o0 + w : 0), take);
-                }
+                una_base = __shfl_sync(0xffffffffu, o0, 0);
+                const uint32_t end = __shfl_sync(0xffffffffu, o0 + n_una, 31);        // lanes beyond the last visible token repeat it
+                const uint32_t n_w = min(end - una_base, (uint32_t)stage * 32u), ua = smem_u32(my_una);
+                for (uint32_t w = lane; w < n_w; w += 32) tc_cp_async4(ua + w * 4, arena + una_base + w);
             }
         }
         load_off(t0 + kTcTok, o0_next, nu_next);                              // the next chunk's offsets travel meanwhile
@@ -460,13 +461,14 @@ __global__ void __launch_bounds__(kTcThreads) k_draft_attn_tc(KvGeom g, KvComp c
             const uint32_t* flP = bmP + g.bm_words * 32;
             if (MODE == 1) {
                 const bool raw = (my_fix[lane] & kKvRawFlag) != 0;            // entry word 0 of this token's record
-                const bool staged = n_una <= (uint32_t)stage && !raw;
+                const uint32_t at = o0 - una_base, room = (uint32_t)stage * 32u;
+                const bool visible = lane < n_here, staged = at <= room && n_una <= room - at && !raw && visible;
                 const uint32_t* lutP = lut_s + kind * 32;
-                tc_walk<T>(bmP, flP, my_una + lane, lutP, r2e, g.kept, d, n_una * 32u, row_a, staged, stage);
-                if (!staged)                                                  // raw exponents or a very long record: read it in place
+                tc_walk<T>(bmP, flP, my_una + (staged ? at : 0u), lutP, r2e, g.kept, d, staged ? n_una * 32u : 0u, row_a, staged);
+                if (!staged && visible)                                       // raw exponents, or no room: read it in place
                     tc_walk_slow<T>(bmP, flP, arena + o0, 1, raw, 0, g.kept, 0u, 0u, (uint32_t)d, n_una * 32u, r2e, row_a);
             } else {
-                tc_walk_mx<T>(bmP, flP, flP + g.f_words * 32, my_una + lane, reinterpret_cast<const uint2*>(lut_s), g.kept, d, row_a);
+                tc_walk_mx<T>(bmP, flP, flP + g.f_words * 32, my_una + lane, reinterpret_cast<const uint2*>(lut_s), g.kept, d, row_a, lane < n_here);
             }
         }
         __syncthreads();
