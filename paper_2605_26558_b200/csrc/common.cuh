@@ -52,7 +52,7 @@ constexpr int kGroupCodes = 4;             // codewords per unary-walk group
 constexpr int kMaxVerifyRows = 16;         // rows of one sequence in one verification call; also the margin kept at the end of a cache
 constexpr int kMaxBatch = 8;               // sequences per session
 constexpr int kMaxRows = 64;               // rows of all sequences in one call
-constexpr int kPrefillRows = 128;          // rows of all sequences in one pass of a prefill
+constexpr int kPrefillRows = 256;          // rows of all sequences in one pass of a prefill
 
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 __host__ __device__ inline size_t align_up(size_t a, size_t b) { return (a + b - 1) / b * b; }

@@ -254,10 +254,10 @@ int launch_attn_merge(const AttnScratch& sc, int chunk_tokens, int n_seq, const 
                       int draft_mode, int draft_units, uint16_t* out, cudaStream_t s);
 
 // ---- verification GEMM (verify_gemm.cu): Y[r][n] = sum_k W[n][k] X[r][k], bf16 in, fp32 accumulate (tcgen05) ----
-// X is a buffer of `bn` rows of k values (bn = 16, 32, 64 or 128 token columns of the MMA; the first `rows` are used);
+// X is a buffer of `bn` rows of k values (bn = 16, 32, 64, 128 or 256 token columns of the MMA; the first `rows` are used);
 // partial: fp32 scratch of verify_gemm_partial_floats.
 // With both outputs null only the partial sums are produced: [splits][bn][n], see verify_gemm_partials().
-inline int verify_gemm_bn(int rows) { return rows <= 16 ? 16 : rows <= 32 ? 32 : rows <= 64 ? 64 : 128; }
+inline int verify_gemm_bn(int rows) { return rows <= 16 ? 16 : rows <= 32 ? 32 : rows <= 64 ? 64 : rows <= 128 ? 128 : 256; }
 size_t verify_gemm_partial_floats(int n, int k, int bn);
 Partials verify_gemm_partials(const float* partial, int n, int k, int bn);
 // w_static: kWeightsStatic: W is not the output of a kernel that may still be running when this one is scheduled (the bf16

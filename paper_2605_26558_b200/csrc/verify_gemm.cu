@@ -2,7 +2,7 @@
 // memory-bound on the bf16 weights): Y[r][n] = sum_k W[n][k] X[r][k], bf16 operands, fp32 accumulation.
 //
 // tcgen05 version, "swap-AB": the weights are the M operand (128 output features per CTA), the token rows the N
-// operand (padded to BN = 16, 32, 64 or, in a prefill, 128 columns), the accumulator lives in tensor memory.  One CTA = one 128-feature tile x
+// operand (padded to BN = 16, 32, 64 or, in a prefill, 128 or 256 columns), the accumulator lives in tensor memory.  One CTA = one 128-feature tile x
 // one K range (split-K so that small matrices still fill the GPU); warp 0 streams 128x64 weight tiles and the
 // BNx64 activation tile through a ring of TMA loads (128-byte swizzle), warp 1 issues the MMAs, warps 2-5 read the
 // accumulator back and store fp32 partial sums; a second kernel adds the K ranges in fixed order.
@@ -15,7 +15,7 @@
 namespace cass {
 
 constexpr int kTcBM = 128, kTcBK = 64;
-constexpr int tc_stages(int bn) { return bn <= 16 ? 6 : bn <= 32 ? 5 : bn <= 64 ? 4 : 3; }      // two CTAs per SM at every bn
+constexpr int tc_stages(int bn) { return bn <= 16 ? 6 : bn <= 32 ? 5 : bn <= 64 ? 4 : bn <= 128 ? 3 : 2; }      // two CTAs per SM at every bn (shared memory; tensor memory too)
 constexpr int kTcABytes = kTcBM * kTcBK * 2;
 constexpr int kTcThreads = 192;
 constexpr int tc_b_bytes(int bn) { return bn * kTcBK * 2; }
@@ -220,7 +220,7 @@ static int launch_tc(const CUtensorMap& mw, const CUtensorMap& mx, float* partia
 
 int launch_verify_gemm(const uint16_t* W, const uint16_t* X, int rows, int bn, int n, int k, float* partial, uint16_t* y_bf16,
                        float* y_f32, int32_t* d_status, cudaStream_t s, int w_static) {
-    if (rows < 1 || rows > bn || (bn != 16 && bn != 32 && bn != 64 && bn != 128) || (k % 8) || n < 1 || !partial || !d_status)
+    if (rows < 1 || rows > bn || (bn != 16 && bn != 32 && bn != 64 && bn != 128 && bn != 256) || (k % 8) || n < 1 || !partial || !d_status)
         return CASS_ERR_INVALID_ARG;
     if (((uintptr_t)W & 15) || ((uintptr_t)X & 15)) return CASS_ERR_INVALID_ARG;
     CUtensorMap mw, mx;
@@ -232,6 +232,7 @@ int launch_verify_gemm(const uint16_t* W, const uint16_t* X, int rows, int bn, i
     split_plan(n, k, &kbt, &kbs, &ns);
     if (bn == 16) rc = launch_tc<16>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
     else if (bn == 32) rc = launch_tc<32>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
+    else if (bn == 256) rc = launch_tc<256>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
     else if (bn == 128) rc = launch_tc<128>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
     else rc = launch_tc<64>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
     if (rc) return rc;
