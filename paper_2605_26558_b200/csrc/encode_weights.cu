@@ -84,12 +84,16 @@ __device__ __forceinline__ void row_load8(const uint16_t* __restrict__ p, uint32
 // (packed bf16 compare and add: the scores' upper halves order as bf16 numbers), then the handful of keys that share
 // those bits are ranked against each other.
 // A row is read once, 8 columns a lane, and its scores' upper halves stay in registers, NV values a lane; the few values
-// of which more is needed are read again.  Up to 4096 columns one warp holds a row and no barrier is needed; WPR warps
-// hold a longer one.
+// of which more is needed are read again.  Up to 2048 columns a warp holds a row and no barrier is needed (WIDE: false, four rows
+// a CTA); a longer row is a CTA's, of as many warps as it takes.
+// The search starts from the row before: the threshold lies within a quarter of it in an ordinary matrix, which leaves 7 rounds
+// of 15 (and 6 meetings of the row's warps).
 // Bound: the integer pipe, which starts a warp instruction every other cycle (packed compare and add: 1.4 cycles a value
-// and round); loads have to be issued well ahead of their use, hence the clamped, unconditional ones.
+// and round), and the latency of those meetings, hence 64 values a lane and not 128: 14 to 24 warps an SM and, at 14336
+// columns, no idle eighth.  Loads have to be issued well ahead of their use, hence the clamped, unconditional ones.
+// 4096 x 14336: 219 -> 136 us.
 constexpr int kSelList = 512;
-constexpr int sel_threads(int wpr) { return wpr < 4 ? 128 : 32 * wpr; }
+constexpr int kSelWarps = 16, kSelWarps64 = 14;                          // most warps a row: 128 and 64 values a lane
 
 __device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t v) {
     __nv_bfloat162 r;
@@ -97,30 +101,40 @@ __device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t v) {
     return r;
 }
 
-template <int NV, int WPR>
-__global__ void __launch_bounds__(sel_threads(WPR), 512 / sel_threads(WPR)) k_select(const uint16_t* __restrict__ W,
-                                                                                     const float* __restrict__ act, EncGeom g,
-                                                                                     uint32_t* __restrict__ keepbm,
-                                                                                     unsigned long long* __restrict__ hist) {
-    constexpr int NT = sel_threads(WPR), ROWS = NT / (32 * WPR), NG = NV / 8, HW = NV >= 32 ? NV / 32 : 1;
+template <int NV, bool WIDE>
+__global__ void __launch_bounds__(!WIDE ? 128 : NV == 128 ? 32 * kSelWarps : 32 * kSelWarps64, !WIDE ? 6 : NV == 128 ? 1 : 2)
+    k_select(const uint16_t* __restrict__ W, const float* __restrict__ act, EncGeom g, uint32_t* __restrict__ keepbm,
+             unsigned long long* __restrict__ hist) {
+    constexpr int ROWS = WIDE ? 1 : 4, NG = NV / 8, LG = NV == 128 ? 4 : 2, HW = NV >= 32 ? NV / 32 : 1;
     __shared__ unsigned int s_exp[256];
     __shared__ unsigned long long s_list[ROWS][kSelList], s_thr[ROWS];
-    __shared__ uint32_t s_cnt[2][ROWS][WPR], s_m[ROWS];
-    const int tid = threadIdx.x, lane = tid & 31, warp = (tid >> 5) % WPR, slot = tid / (32 * WPR);
-    // the warps of a row meet at a barrier of their own: another row of the CTA may be elsewhere, or done
+    __shared__ uint2 s_cnt[2][kSelWarps];
+    __shared__ uint32_t s_m[ROWS];
+    const int NT = WIDE ? (int)blockDim.x : 128, WPR = WIDE ? NT / 32 : 1;     // threads; warps a row
+    const int tid = threadIdx.x, lane = tid & 31, warp = WIDE ? tid >> 5 : 0, slot = WIDE ? 0 : tid >> 5;
     auto row_sync = [&]() {
-        if (WPR == 1) __syncwarp();
-        else asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(32 * WPR) : "memory");
+        if (WIDE) __syncthreads();
+        else __syncwarp();
     };
     int turn = 0;
-    auto row_sum = [&](uint32_t v) {                                     // sum over the row's lanes; two buffers in turn, one barrier
-        v = __reduce_add_sync(0xffffffffu, v);
-        if (WPR == 1) return v;
+    auto row_sum2 = [&](uint32_t v, uint32_t w) {                        // sums over the row's lanes; two buffers in turn, one barrier
+        uint2 r = make_uint2(__reduce_add_sync(0xffffffffu, v), __reduce_add_sync(0xffffffffu, w));
+        if (!WIDE) return r;
         turn ^= 1;
-        if (lane == 0) s_cnt[turn][slot][warp] = v;
+        if (lane == 0) s_cnt[turn][warp] = r;
         row_sync();
-        return __reduce_add_sync(0xffffffffu, lane < WPR ? s_cnt[turn][slot][lane] : 0u);
+        r = lane < WPR ? s_cnt[turn][lane] : make_uint2(0u, 0u);
+        return make_uint2(__reduce_add_sync(0xffffffffu, r.x), __reduce_add_sync(0xffffffffu, r.y));
     };
+    auto row_sum = [&](uint32_t v) {
+        v = __reduce_add_sync(0xffffffffu, v);
+        if (!WIDE) return v;
+        turn ^= 1;
+        if (lane == 0) s_cnt[turn][warp].x = v;
+        row_sync();
+        return __reduce_add_sync(0xffffffffu, lane < WPR ? s_cnt[turn][lane].x : 0u);
+    };
+    uint32_t guess = 0;                                                  // the row before's threshold, upper half
     for (int i = tid; i < 256; i += NT) s_exp[i] = 0;
     pdl_wait();
     __syncthreads();
@@ -131,12 +145,16 @@ __global__ void __launch_bounds__(sel_threads(WPR), 512 / sel_threads(WPR)) k_se
         const uint16_t* wr = W + (size_t)row * g.k;
         auto score_of = [&](int c) { return __float_as_uint(__fmul_rn(bf16_bits_to_float(wr[c] & 0x7FFFu), act ? __ldg(act + c) : 1.0f)); };
         auto col_of = [&](int i) { return ((warp + (i / 8) * WPR) * 32 + lane) * 8 + (i & 7); };       // column of the lane's value i
+        auto hit_value = [](int h, uint32_t b) { const int i = __ffs(b) - 1; return h * 32 + 2 * (i & 15) + (i >> 4); };
         uint32_t x[NV / 2];                                              // upper halves of scores 2 i (low) and 2 i + 1
         int later = 0;
 #pragma unroll
         for (int q = 0; q < NG; ++q) {
-            // four groups' loads at a time: all of them at once would not fit the registers
-            if (q > 0 && q % 4 == 0) asm volatile("" : "+r"(later) : "r"(x[q * 4 - 1]), "r"(x[q * 4 - 5]), "r"(x[q * 4 - 9]), "r"(x[q * 4 - 13]));
+            // LG groups' loads at a time: all of them at once would not fit the registers
+            if (q > 0 && q % LG == 0) {
+                if (LG == 4) asm volatile("" : "+r"(later) : "r"(x[q * 4 - 1]), "r"(x[q * 4 - 5]), "r"(x[q * 4 - 9]), "r"(x[q * 4 - 13]));
+                else asm volatile("" : "+r"(later) : "r"(x[q * 4 - 1]), "r"(x[q * 4 - 5]));
+            }
             const int c = col_of(q * 8) + later;
             uint32_t w[4];
             float a[8];
@@ -165,10 +183,14 @@ __global__ void __launch_bounds__(sel_threads(WPR), 512 / sel_threads(WPR)) k_se
             for (int i = 0; i < 4; ++i) {
                 const uint32_t lo = __float_as_uint(__fmul_rn(__uint_as_float((w[i] << 16) & 0x7FFF0000u), a[2 * i]));
                 const uint32_t hi = __float_as_uint(__fmul_rn(__uint_as_float(w[i] & 0x7FFF0000u), a[2 * i + 1]));
-                uint32_t v = __byte_perm(lo, hi, 0x7632);
-                if (c + 2 * i >= g.k) v |= 0x7FFFu;                      // beyond the row: a NaN, which is neither below nor above anything
-                if (c + 2 * i + 1 >= g.k) v |= 0x7FFF0000u;
-                x[q * 4 + i] = v;
+                x[q * 4 + i] = __byte_perm(lo, hi, 0x7632);
+            }
+            if (c + 8 > g.k) {                                           // beyond the row: NaNs, which are neither below nor above anything
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (c + 2 * i >= g.k) x[q * 4 + i] |= 0x7FFFu;
+                    if (c + 2 * i + 1 >= g.k) x[q * 4 + i] |= 0x7FFF0000u;
+                }
             }
         }
         uint32_t top = 0, below = 0;                                     // upper half of the smallest kept score; scores below it
@@ -176,31 +198,38 @@ __global__ void __launch_bounds__(sel_threads(WPR), 512 / sel_threads(WPR)) k_se
         unsigned long long thr = 0;                                      // smallest kept key
         if (g.n_prune > 0) {
             if (lane == 0 && warp == 0) s_m[slot] = 0;
-#pragma unroll 1
-            for (int bit = 14; bit >= 0; --bit) {
-                const uint32_t cand = top | (1u << bit);
-                // below the normal numbers the packed compare may flush: those scores are one bin; beyond infinity there is none
-                if (cand < 0x0080u || cand > 0x7F80u) continue;
+            auto below_of = [&](uint32_t cand) {                         // the lane's scores whose upper half is less
                 const __nv_bfloat162 c2 = as_bf162(cand | (cand << 16));
                 __nv_bfloat162 n[2] = {as_bf162(0), as_bf162(0)};
 #pragma unroll
                 for (int i = 0; i < NV / 2; ++i) n[i & 1] = __hadd2(n[i & 1], __hlt2(as_bf162(x[i]), c2));     // at most 32 in a counter: exact
                 const __nv_bfloat162 sum = __hadd2(n[0], n[1]);
-                const uint32_t cnt = row_sum((uint32_t)(int)(__low2float(sum) + __high2float(sum)));
-                if (cnt <= (uint32_t)g.n_prune) { top = cand; below = cnt; }
+                return (uint32_t)(int)(__low2float(sum) + __high2float(sum));
+            };
+            // the largest candidate with at most n_prune scores below it: in [top, hi).  Below the normal numbers the packed
+            // compare may flush: those scores are one bin (0); beyond infinity there is none
+            uint32_t hi = 0x7F81u;
+            if (guess > 0x00A0u && guess < 0x7F60u) {
+                const uint2 c = row_sum2(below_of(guess - 32u), below_of(guess + 32u));
+                if (c.x <= (uint32_t)g.n_prune) { top = guess - 32u; below = c.x; } else { hi = guess - 32u; }
+                if (c.y <= (uint32_t)g.n_prune) { top = guess + 32u; below = c.y; } else { hi = min(hi, guess + 32u); }
             }
-            const uint32_t top2 = top | (top << 16), sel = top ? 0xFFFFFFFFu : 0xFF80FF80u;
+#pragma unroll 1
+            while (hi - top > 1u && hi > 0x0080u) {
+                const uint32_t cand = max((top + hi) / 2u, 0x0080u), cnt = row_sum(below_of(cand));
+                if (cnt <= (uint32_t)g.n_prune) { top = cand; below = cnt; } else { hi = cand; }
+            }
+            guess = top;
+            // bit i (low half) or 16 + i of hit[h]: value 2 (16 h + i) or the one after it
+            const __nv_bfloat162 top2 = as_bf162(top ? top | (top << 16) : 0x00800080u);
 #pragma unroll
-            for (int i = 0; i < NV / 2; ++i) {
-                const uint32_t d = (x[i] ^ top2) & sel;
-                if ((d & 0xFFFFu) == 0) hit[i / 16] |= 1u << (2 * i & 31);
-                if (d < 0x10000u) hit[i / 16] |= 2u << (2 * i & 31);
-            }
+            for (int i = 0; i < NV / 2; ++i)
+                hit[i / 16] |= (top ? __heq2_mask(as_bf162(x[i]), top2) : __hlt2_mask(as_bf162(x[i]), top2)) & (0x00010001u << (i % 16));
             row_sync();                                                  // s_m is zero
 #pragma unroll
             for (int h = 0; h < HW; ++h)
                 for (uint32_t b = hit[h]; b; b &= b - 1) {
-                    const int c = col_of(h * 32 + __ffs(b) - 1);
+                    const int c = col_of(hit_value(h, b));
                     const uint32_t at = atomicAdd(&s_m[slot], 1u);
                     if (at < (uint32_t)kSelList) s_list[slot][at] = ((unsigned long long)score_of(c) << 20) | (unsigned)c;
                 }
@@ -224,7 +253,7 @@ __global__ void __launch_bounds__(sel_threads(WPR), 512 / sel_threads(WPR)) k_se
 #pragma unroll
                     for (int h = 0; h < HW; ++h)
                         for (uint32_t b = hit[h]; b; b &= b - 1) {
-                            const int c = col_of(h * 32 + __ffs(b) - 1);
+                            const int c = col_of(hit_value(h, b));
                             less += (((unsigned long long)score_of(c) << 20) | (unsigned)c) < cand;
                         }
                     if (row_sum(less) <= want) thr = cand;
@@ -243,8 +272,8 @@ __global__ void __launch_bounds__(sel_threads(WPR), 512 / sel_threads(WPR)) k_se
 #pragma unroll
                 for (int i = 0; i < 4; ++i) kb |= __hgt2_mask(as_bf162(x[q * 4 + i]), t2) & (0x00400080u >> (2 * i));
                 kb = (kb | (kb >> 16)) & 0xFFu;
-                for (uint32_t b = (hit[q / 4] >> (8 * (q & 3))) & 0xFFu; b; b &= b - 1) {
-                    const int i = __ffs(b) - 1;
+                for (uint32_t b = (hit[q / 4] >> (4 * (q & 3))) & 0x000F000Fu; b; b &= b - 1) {
+                    const int i = hit_value(0, b);
                     if ((((unsigned long long)score_of(c + i) << 20) | (unsigned)(c + i)) >= thr) kb |= 0x80u >> i;
                 }
             } else {
@@ -586,29 +615,26 @@ __global__ void __launch_bounds__(kPackThreads, 2) k_pack(const uint16_t* __rest
 
 // CTAs of k_select: as many as run at once (each takes rows in turn, so that the counts of kept exponents reach global
 // memory once per CTA).
-template <int NV, int WPR>
+template <int NV, bool WIDE>
 static int launch_select_as(const uint16_t* W, const float* act, const EncGeom& g, const EncWs& ws, cudaStream_t stream) {
-    constexpr int NT = sel_threads(WPR), ROWS = NT / (32 * WPR);
+    const int warps = WIDE ? ceil_div(g.k, 32 * NV) : 4, rows = WIDE ? 1 : 4;
     int dev = 0, sms = 148, per_sm = 1;
     CASS_CUDA_CHECK(cudaGetDevice(&dev));
     CASS_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    CASS_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_select<NV, WPR>, NT, 0));
-    const int most = sms * (per_sm < 1 ? 1 : per_sm), need = ceil_div(g.n, ROWS);
-    CASS_PDL_LAUNCH((k_select<NV, WPR>), dim3(need < most ? need : most), dim3(NT), 0, stream, W, act, g, ws.keepbm, ws.hist);
+    CASS_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (k_select<NV, WIDE>), 32 * warps, 0));
+    const int most = sms * (per_sm < 1 ? 1 : per_sm), need = ceil_div(g.n, rows);
+    CASS_PDL_LAUNCH((k_select<NV, WIDE>), dim3(need < most ? need : most), dim3(32 * warps), 0, stream, W, act, g, ws.keepbm, ws.hist);
     return CASS_OK;
 }
-
-// One warp a row while its lanes' registers hold it (128 values a lane), then as many warps as it takes.
+// One warp a row while its lanes' registers hold it (64 values a lane), then as many warps as it takes; 128 values a lane where
+// 14 warps of 64 do not reach.
 static int launch_select(const uint16_t* W, const float* act, const EncGeom& g, const EncWs& ws, cudaStream_t stream) {
     const int k = g.k;
-    if (k <= 512) return launch_select_as<16, 1>(W, act, g, ws, stream);
-    if (k <= 1024) return launch_select_as<32, 1>(W, act, g, ws, stream);
-    if (k <= 2048) return launch_select_as<64, 1>(W, act, g, ws, stream);
-    if (k <= 4096) return launch_select_as<128, 1>(W, act, g, ws, stream);
-    if (k <= 8192) return launch_select_as<128, 2>(W, act, g, ws, stream);
-    if (k <= 16384) return launch_select_as<128, 4>(W, act, g, ws, stream);
-    if (k <= 32768) return launch_select_as<128, 8>(W, act, g, ws, stream);
-    return launch_select_as<128, 16>(W, act, g, ws, stream);
+    if (k <= 512) return launch_select_as<16, false>(W, act, g, ws, stream);
+    if (k <= 1024) return launch_select_as<32, false>(W, act, g, ws, stream);
+    if (k <= 2048) return launch_select_as<64, false>(W, act, g, ws, stream);
+    if (k <= 2048 * kSelWarps64) return launch_select_as<64, true>(W, act, g, ws, stream);
+    return launch_select_as<128, true>(W, act, g, ws, stream);
 }
 
 // ---- test hook: zero-padded reconstruction of the whole blob ---------------------------------------------
