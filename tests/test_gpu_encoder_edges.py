@@ -50,6 +50,31 @@ def test_rows_around_the_splits(cass, cols, mode):
     assert np.array_equal(got, enc(_bits(w), act, 400, 4)[0])
 
 
+@pytest.mark.parametrize("rows,cols", [(4736, 40), (4737, 40), (4800, 520), (4500, 2056), (1200, 9000), (1100, 29000)])
+def test_rows_in_turn(cass, rows, cols):
+    """More rows than CTAs at once, so that a search starts from another row's threshold: rows like it, rows of another scale,
+    rows of one value."""
+    g = torch.Generator(device="cuda").manual_seed(cols)
+    w = torch.randn(rows, cols, generator=g, device="cuda") + 0.0
+    scale = torch.randint(-3, 4, (rows, 1), generator=g, device="cuda") * (torch.rand(rows, 1, generator=g, device="cuda") < 0.3)
+    w = (w.abs() + 1e-3) * w.sign() * torch.exp2(scale.float())
+    w[::7] = 0.5
+    w = torch.where(w == 0, 1e-3, w).to(torch.bfloat16)
+    act = torch.rand(cols, generator=g, device="cuda") + 0.05
+    fmt = cass.default_format()
+    bound, ws_bytes = cass.cass_encoded_weight_bytes(fmt, rows, cols)
+    blob = torch.zeros(bound, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    cass.cass_encode_weights(fmt, w, act, blob, torch.zeros(ws_bytes, dtype=torch.uint8, device="cuda"), status)
+    dec = torch.empty_like(w)
+    cass.cass_decode_weights(blob, cass.cass_weight_blob_info(blob), dec)
+    order = torch.sort(w.float().abs() * act, dim=1, stable=True).indices
+    keep = torch.ones_like(w, dtype=torch.bool).scatter_(1, order[:, : cols * 400 // 1000], False)
+    trunc = (w.view(torch.int16) & -16).view(torch.bfloat16)
+    assert int(status.item()) == 0
+    assert torch.equal(dec, torch.where(keep, trunc, torch.zeros_like(w)))
+
+
 def test_constant_rows_and_no_pruning(cass):
     w = torch.full((40, 3000), 0.5, dtype=torch.bfloat16)
     w[7] = 0.0
