@@ -177,11 +177,11 @@ int launch_qkv_rope(uint16_t* qkv, Partials pp, const float* cos_t, const float*
                     const DevState* st, int use_inflight, int rows, int rps, int n_q, int n_kv, int d, cudaStream_t s);
 int launch_swiglu(const uint16_t* gu_bf16, Partials pp, uint16_t* act, int rows,
                   int ffn, cudaStream_t s);
-// logits (fp32 [rows][vocab], or formed from partials) -> lowest-index argmax per row; optional copy
+// logits (fp32, formed from partials) -> lowest-index argmax per row; optional copy
 // of the logits; bump_inflight adds 1 to the draft counter of sequence r (one row per sequence) afterwards.
 // tmp_v / tmp_i: scratch of kMaxRows x 128 entries each.
 // Row r's token goes to out[r * out_stride].
-int launch_argmax(const float* logits, Partials pp, int rows, int vocab, int32_t* out, int out_stride,
+int launch_argmax(Partials pp, int rows, int vocab, int32_t* out, int out_stride,
                   float* logits_copy, float* tmp_v, int32_t* tmp_i, DevState* st, int bump_inflight, cudaStream_t s);
 int launch_set_len(DevState* st, int len, cudaStream_t s);
 int launch_last_rows(const uint16_t* src, int n_seq, int rps, int take, int cols, uint16_t* dst, cudaStream_t s);

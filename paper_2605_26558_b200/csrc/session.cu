@@ -515,7 +515,7 @@ extern "C" int cass_verify(void* session, const int32_t* toks, int g, int32_t* t
     }
     if (calib) RC(launch_calib_accum(s->xn, rows, d.hidden, s->calib_lm, s->st, st));
     RC(launch_verify_gemm(weight(s->lm_head, s->lm_blob, s->lm_bi, s->lm_vdata), s->xn, rows, bn, d.vocab, d.hidden, s->vg_partial, nullptr, nullptr, status, st, s->from_parts ? 0 : 1));
-    RC(launch_argmax(nullptr, vparts(d.vocab, d.hidden), rows, d.vocab, target_argmax, 1, logits_opt,
+    RC(launch_argmax(vparts(d.vocab, d.hidden), rows, d.vocab, target_argmax, 1, logits_opt,
                      s->argmax_val, s->argmax_tmp, s->st, 0, st));
     return w_rc;
 }
@@ -604,7 +604,7 @@ extern "C" int cass_prefill(void* session, const int32_t* toks, int n, int32_t* 
     RC(launch_last_rows(s->pattn, B, w, last, qd, s->attn, st));
     RC(launch_last_rows(s->pxn, B, w, 1, d.hidden, s->xn, st));
     RC(launch_verify_gemm(weight(s->lm_head, s->lm_blob, s->lm_bi, s->lm_vdata), s->xn, B, s->R, d.vocab, d.hidden, s->vg_partial, nullptr, nullptr, status, st, w_static));
-    RC(launch_argmax(nullptr, verify_gemm_partials(s->vg_partial, d.vocab, d.hidden, s->R), B, d.vocab, target_argmax, 1, nullptr,
+    RC(launch_argmax(verify_gemm_partials(s->vg_partial, d.vocab, d.hidden, s->R), B, d.vocab, target_argmax, 1, nullptr,
                      s->argmax_val, s->argmax_tmp, s->st, 0, st));
     RC(launch_set_len(s->st, n, st));
     s->drafts_pending = 0;
@@ -650,7 +650,7 @@ extern "C" int cass_draft_step(void* session, const int32_t* tok_in, int32_t* to
         RC(launch_residual_rmsnorm(s->h, nullptr, draftp(L.bi[3]), next_gain, s->xn, B, d.hidden, d.rms_eps, st));
     }
     RC(launch_draft_gemv(s->lm_blob, s->lm_bi, s->xn, B, s->partial, status, st));
-    RC(launch_argmax(nullptr, draftp(s->lm_bi), B, d.vocab, tok_out, tok_stride, logits_opt, s->argmax_val, s->argmax_tmp, s->st, 1, st));
+    RC(launch_argmax(draftp(s->lm_bi), B, d.vocab, tok_out, tok_stride, logits_opt, s->argmax_val, s->argmax_tmp, s->st, 1, st));
     return CASS_OK;
 }
 
