@@ -65,8 +65,9 @@ class Engine:
         # toks[b][1..g] = its drafted tokens
         self.toks = torch.zeros(64, dtype=torch.int32, device=self.device)
         self.targ = torch.zeros(64, dtype=torch.int32, device=self.device)
-        self.out_tokens = torch.zeros(64, dtype=torch.int32, device=self.device)
-        self.n_acc = torch.zeros(8, dtype=torch.int32, device=self.device)
+        # a step's results side by side: one copy brings them to the host
+        self._results = torch.zeros(8 + 64, dtype=torch.int32, device=self.device)
+        self.n_acc, self.out_tokens = self._results[:8], self._results[8:]
         self._stride = 1              # gamma + 1 of the layout the token buffers are in
         self._graphs = {}
 
@@ -241,10 +242,9 @@ class Engine:
 
     def _collect(self, out, stats):
         s = self._stride
-        acc = self.n_acc[: self.batch].tolist()
-        toks = self.out_tokens[: self.batch * s].view(self.batch, s).tolist()
-        for b, a in enumerate(acc):
-            out[b].extend(toks[b][: a + 1])
+        got = self._results[: 8 + self.batch * s].tolist()
+        for b, a in enumerate(got[: self.batch]):
+            out[b].extend(got[8 + b * s: 8 + b * s + a + 1])
             stats.accepted += a
             stats.emitted += a + 1
         stats.steps += 1
