@@ -207,23 +207,7 @@ __global__ void __launch_bounds__(32 * kKvWarps) k_kv_append(KvGeom g, KvComp ck
                         k0 += __popc(bm[j]);
                     }
                 } else {
-                    // the codewords' terminating ones: a slice has at most 1023 code bits here, two slices' scans share a word
-                    uint32_t ubase = 0;
-#pragma unroll
-                    for (int j = 0; j < NJ; j += 2) {
-                        if (j >= nj) break;
-                        uint32_t incl = len[j] | (len[j + 1] << 16);
-#pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-                            if (lane >= o) incl += v;
-                        }
-                        const uint32_t all = __shfl_sync(0xffffffffu, incl, 31);
-                        const uint32_t p = ubase + (incl & 0xFFFFu) - 1u, q = ubase + (all & 0xFFFFu) + (incl >> 16) - 1u;
-                        if (len[j]) atomicOr(&una[(p >> 5) & 63u], 0x80000000u >> (p & 31));
-                        if (len[j + 1]) atomicOr(&una[(q >> 5) & 63u], 0x80000000u >> (q & 31));
-                        ubase += (all & 0xFFFFu) + (all >> 16);
-                    }
+                    kv_code_bits<NJ>(len, nj, lane, una);
                 }
             }
             __syncwarp();

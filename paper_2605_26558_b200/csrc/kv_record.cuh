@@ -76,6 +76,28 @@ __device__ __forceinline__ uint32_t kv_entries(const KvGeom& g, const uint32_t (
     return (ub + 31) / 32;
 }
 
+// The codewords' terminating ones into una (64 words, zero): a slice has at most 1023 code bits where codes are stored, so the
+// scans of two slices share a word.
+template <int NJ>
+__device__ __forceinline__ void kv_code_bits(const uint32_t (&len)[NJ], int nj, int lane, uint32_t* una) {
+    uint32_t base = 0;
+#pragma unroll
+    for (int j = 0; j < NJ; j += 2) {
+        if (j >= nj) break;
+        uint32_t incl = len[j] | (len[j + 1] << 16);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const uint32_t all = __shfl_sync(0xffffffffu, incl, 31);
+        const uint32_t p = base + (incl & 0xFFFFu) - 1u, q = base + (all & 0xFFFFu) + (incl >> 16) - 1u;
+        if (len[j]) atomicOr(&una[(p >> 5) & 63u], 0x80000000u >> (p & 31));
+        if (len[j + 1]) atomicOr(&una[(q >> 5) & 63u], 0x80000000u >> (q & 31));
+        base += (all & 0xFFFFu) + (all >> 16);
+    }
+}
+
 // Sign and kept mantissa bits of one value; MX (Cassandra-2): sign and magnitude in the unit of its 32-channel slice, whose shared
 // exponent is E (0 otherwise).
 template <int T>

@@ -226,29 +226,20 @@ __global__ void __launch_bounds__(32 * kSpanWarps) k_kv_codes(KvGeom g, KvComp c
         una[lane] = 0;
         una[lane + 32] = 0;
         __syncwarp();
-        uint32_t base = 0;                                              // code bits, or kept values, of the slices before
-        const bool raw = (first & kKvRawFlag) != 0;
+        if (first & kKvRawFlag) {                                       // the kept exponents as bytes
+            uint32_t base = 0;                                          // kept values of the slices before
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            if (j >= nj) break;
-            const bool keep = (bm[j] << lane) >> 31;
-            const uint32_t e = (bits[j] >> 7) & 0xFFu;
-            if (raw) {
+            for (int j = 0; j < NJ; ++j) {
+                if (j >= nj) break;
                 const uint32_t k = base + (lane ? __popc(bm[j] >> (32 - lane)) : 0u);
-                if (keep) atomicOr(&una[(k >> 2) & 63u], e << (24 - 8 * (k & 3)));
+                if ((bm[j] << lane) >> 31) atomicOr(&una[(k >> 2) & 63u], ((bits[j] >> 7) & 0xFFu) << (24 - 8 * (k & 3)));
                 base += __popc(bm[j]);
-            } else {
-                const uint32_t len = keep ? s_len[e] : 0u;
-                uint32_t incl = len;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += v;
-                }
-                const uint32_t p = base + incl - 1;                     // the codeword's terminating one
-                if (keep) atomicOr(&una[(p >> 5) & 63u], 0x80000000u >> (p & 31));
-                base += __shfl_sync(0xffffffffu, incl, 31);
             }
+        } else {
+            uint32_t len[NJ];
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) len[j] = (bm[j] << lane) >> 31 ? s_len[(bits[j] >> 7) & 0xFFu] : 0u;
+            kv_code_bits<NJ>(len, nj, lane, una);
         }
         __syncwarp();
         for (uint32_t w = lane; w < nw && w < 64u; w += 32) arena[o0 + w] = una[w];
