@@ -667,18 +667,21 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
     // superblocks beside SMs with 4 x 3: 56.7 instead of 54.4 us on the 28672 x 4096 matrix).  Several vectors: the x
     // slice a CTA stages is nb times larger, so CTAs keep theirs and loop (one CTA per superblock: 52.3 instead of
     // 48.6 ms per step with 8 sequences).
-    int g = bi.n_rowblocks;
+    int g = bi.n_rowblocks, per_sm = (int)((228 * 1024) / (smem + 1024));                 // CTAs an SM holds
+    if (per_sm > 2048 / threads) per_sm = 2048 / threads;
+    if (per_sm < 1) per_sm = 1;
     if (nb > 1) {
-        int per_sm = (int)((228 * 1024) / (smem + 1024));
-        if (per_sm > 2048 / threads) per_sm = 2048 / threads;
-        if (per_sm < 1) per_sm = 1;
         g = ceil_div(gemv_sm_count() * per_sm, bi.n_seg);
         if (g > bi.n_rowblocks) g = bi.n_rowblocks;
     }
     if (g < 1) g = 1;
-    // results inside the kernel where the segments of a row block are one CTA, or a cluster of CTAs with one tile each
+    // Results inside the kernel where the segments of a row block are one CTA, or a cluster of CTAs with one tile each and the
+    // grid fills at most three quarters of the chip: a cluster starts only when all of its CTAs have room, which leaves SMs
+    // idle where CTAs queue (12613 x 5686 at t = 0: 57.4 us, 47.0 with the finishing kernel; 4096 x 14336: 31.5 and 28.7;
+    // against that 1000 x 3000: 8.6 and 8.9, 2000 x 11000: 17.9 and 18.4).
     const bool want = y_bf16 || y_f32;
-    const int out = !want ? 0 : bi.n_seg == 1 ? 1 : (bi.n_seg <= 8 && g == bi.n_rowblocks) ? 2 : 0;
+    const bool room = 4ll * bi.n_seg * g <= 3ll * gemv_sm_count() * per_sm;
+    const int out = !want ? 0 : bi.n_seg == 1 ? 1 : (bi.n_seg <= 8 && g == bi.n_rowblocks && room) ? 2 : 0;
     // with q = 1 - p kept, 8 kept columns span 8 / q columns, give or take sqrt(8 p) / q: more than 32 about once in 10^4 groups
     // of a lane at p = 50 %, once in 40 at 60 %, and one lane's long gap costs its warp a careful walk (359 x 1467 at p = 60 %:
     // 26 us without the second window, 12.8 with it)

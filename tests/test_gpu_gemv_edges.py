@@ -23,7 +23,7 @@ def _bits(t):
 @pytest.mark.parametrize("mode,t", [(1, 4), (1, 0), (1, 3), (2, 4)])
 @pytest.mark.parametrize("rows,cols,p,seg", [
     (1, 1, 0, 0), (33, 31, 520, 0), (40, 2048, 530, 0), (65, 2049, 400, 0), (70, 700, 700, 256), (37, 2304, 600, 256),
-    (64, 2300, 900, 256), (31, 16400, 400, 0), (2000, 513, 800, 256)])
+    (64, 2300, 900, 256), (31, 16400, 400, 0), (2000, 513, 800, 256), (9000, 2100, 400, 0)])
 def test_walk_and_results(cass, mode, t, rows, cols, p, seg):
     w = synth.student_t_weight(rows, cols, 8, f"gemv/{rows}x{cols}").float()
     if rows > 30 and cols > 600:
