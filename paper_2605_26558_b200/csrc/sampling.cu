@@ -110,6 +110,8 @@ __global__ void __launch_bounds__(1024) k_softmax_rows_long(const float* __restr
 // summing threads then never share a bank).  Returns the index to every thread (vocab - 1 when the total is not positive).
 // Bound: the chain of additions (`per` of a segment, then the 256 sums); reading each segment from global memory as it was
 // summed took a dependent round trip for every few values, 350 us over a vocabulary of 128256.
+// The kernel arrives at the cluster's barrier when it starts (barrier_arrive), and the first draw waits for it here before it
+// stores into rank 0's memory: a CTA's shared memory may be touched only once that CTA is known to run.
 struct DrawShared {
     float seg[kSampleThreads + 1];         // this CTA's copy of all sums, then the sums before each segment; last: the total
     float all[kSampleThreads];             // rank 0: where the CTAs leave their sums
@@ -119,8 +121,10 @@ struct DrawShared {
 __host__ __device__ inline int draw_stride(int vocab) { return ceil_div(vocab, kSampleThreads) | 1; }
 
 // STAGED = false: a vocabulary whose segments do not fit shared memory is read where it is.
+// first: the kernel's first draw.
 template <bool STAGED, class W>
-__device__ int cluster_inverse_cdf(cg::cluster_group& cluster, W weight, int vocab, float u, DrawShared& sh, float* w_s, float* total_out) {
+__device__ int cluster_inverse_cdf(cg::cluster_group& cluster, bool first, W weight, int vocab, float u, DrawShared& sh, float* w_s,
+                                   float* total_out) {
     const int cs = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
     const int per = ceil_div(vocab, kSampleThreads), stride = draw_stride(vocab), n_seg = kSampleThreads / cs, seg0 = rank * n_seg;
@@ -154,6 +158,7 @@ __device__ int cluster_inverse_cdf(cg::cluster_group& cluster, W weight, int voc
 #pragma unroll
         for (int k = 0; k < 8; ++k) { sum += x[k]; x[k] = nx[k]; }         // adding 0 at the end changes nothing
     }
+    if (first) cluster.barrier_wait();
     if (tid < n_seg) *cluster.map_shared_rank(&sh.all[seg0 + tid], 0) = sum;
     cluster.sync();
     sh.seg[tid] = *cluster.map_shared_rank(&sh.all[tid], 0);
@@ -207,10 +212,11 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(const float* __r
     extern __shared__ float w_s[];
     __shared__ DrawShared sh;
     cg::cluster_group cluster = cg::this_cluster();
+    cluster.barrier_arrive();
     pdl_wait();
     const int row = blockIdx.x / (int)cluster.num_blocks();
     const float* p = probs + (size_t)row * vocab;
-    const int pick = cluster_inverse_cdf<STAGED>(cluster, [&](int v) { return __ldg(p + v); }, vocab, u[row], sh, w_s, nullptr);
+    const int pick = cluster_inverse_cdf<STAGED>(cluster, true, [&](int v) { return __ldg(p + v); }, vocab, u[row], sh, w_s, nullptr);
     if (cluster.block_rank() == 0 && threadIdx.x == 0) tokens[(size_t)row * tok_stride] = pick;
 }
 
@@ -226,6 +232,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_accept_sampling(DevState* st
     __shared__ DrawShared sh;
     __shared__ int s_n;
     cg::cluster_group cluster = cg::this_cluster();
+    cluster.barrier_arrive();
     pdl_wait();
     const int b = blockIdx.x / (int)cluster.num_blocks();
     draft += (size_t)b * draft_stride;
@@ -246,8 +253,9 @@ __global__ void __launch_bounds__(kSampleThreads) k_accept_sampling(DevState* st
     const float* qn = q + (size_t)n * vocab;                               // read only when n < g
     float total = 0.f;
     int extra = 0;
-    if (n < g) extra = cluster_inverse_cdf<STAGED>(cluster, [&](int v) { return fmaxf(__ldg(pn + v) - __ldg(qn + v), 0.f); }, vocab, u[b], sh, w_s, &total);
-    if (!(total > 0.f)) extra = cluster_inverse_cdf<STAGED>(cluster, [&](int v) { return __ldg(pn + v); }, vocab, u[b], sh, w_s, nullptr);
+    if (n < g)
+        extra = cluster_inverse_cdf<STAGED>(cluster, true, [&](int v) { return fmaxf(__ldg(pn + v) - __ldg(qn + v), 0.f); }, vocab, u[b], sh, w_s, &total);
+    if (!(total > 0.f)) extra = cluster_inverse_cdf<STAGED>(cluster, n == g, [&](int v) { return __ldg(pn + v); }, vocab, u[b], sh, w_s, nullptr);
     if (cluster.block_rank() != 0 || threadIdx.x != 0) return;
     out_tokens += (size_t)b * (g + 1);
     for (int i = 0; i < n; ++i) out_tokens[i] = draft[i];
