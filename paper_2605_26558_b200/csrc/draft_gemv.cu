@@ -383,8 +383,14 @@ __device__ __forceinline__ void chunk_dot_mx4(const uint32_t* __restrict__ sb, c
 // out = 1: the matrix is one segment wide, a sum is the result.  out = 2: the n_seg CTAs of a row block are a cluster with one
 // tile each, and the first adds the others' sums in segment order.  (A kernel of its own for these additions costs a launch,
 // 2 us of the 10 us that a small matrix takes.)  out = 0: only `partial` is written.
+// A thread whose wait for a copy runs out leaves the kernel: threads that have left hold up neither __syncthreads nor their
+// warp's exchanges, and the others run out of their own waits in turn.  With out = 2 it must still meet its CTA and the cluster:
+// its warp goes on through the one tile as one of no values (the results are then void, as the status says).
+// Launch bounds: a blob may have chunks for 1024 threads, and the compiler then likes to fit two such CTAs, 32 registers a thread.
+// Told that one is enough it takes 48 to 55 for two Cassandra-2 vectors, whose walk does not fit 32 without a spill (5120 x 13824:
+// 37 to 39 us at 32 registers, as the rest of the kernel falls, 34.7 so).
 template <int T, int NB, bool WIDE>
-__global__ void __launch_bounds__(1024) k_draft_gemv(const uint32_t* __restrict__ blob, const uint16_t* __restrict__ x,
+__global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gemv(const uint32_t* __restrict__ blob, const uint16_t* __restrict__ x,
                                                      float* __restrict__ partial, int32_t* __restrict__ d_status,
                                                      int stage_bytes, int max_sb, int n, int k, int t, int seg_cols,
                                                      int chunk_cols, int n_seg, int n_rb, unsigned long long blob_bytes,
@@ -539,13 +545,16 @@ __global__ void __launch_bounds__(1024) k_draft_gemv(const uint32_t* __restrict_
         for (int i = 0; i < n_tiles; ++i) {
             const int s = i % kGemvStages;
             const int rb = rb0 + i * rb_step;
+            bool lost = false;
             if (!mbar_wait_bounded(&bar[s], (uint32_t)(i / kGemvStages) & 1u)) {
                 // give up: flag the error, let the copies still in flight into this CTA's buffers land (bounded), leave
                 if (d_status) atomicExch(d_status, CASS_ERR_TIMEOUT);
                 for (int j = i; j < n_tiles && j < i + kGemvStages; ++j)
                     mbar_wait_bounded(&bar[j % kGemvStages], (uint32_t)(j / kGemvStages) & 1u);
-                return false;
+                if (out != 2) return false;
+                lost = true;
             }
+            lost = __any_sync(0xffffffffu, lost);
             const uint32_t* sb = reinterpret_cast<const uint32_t*>(smem_raw + (size_t)s * stage_bytes);
             float acc[NB];
 #pragma unroll
@@ -553,18 +562,19 @@ __global__ void __launch_bounds__(1024) k_draft_gemv(const uint32_t* __restrict_
             if (warp < n_ch && !s_skip[s]) {
                 const uint32_t* dir = s_dir[s] - 1;                   // written before the copy was started; its arrival orders the read
                 const SbGeom g = SbGeom::make(n_ch, scols, (int)dir[1], (int)dir[2]);
+                const int elems = lost ? 0 : dir_chunk_elems(dir[3]);
                 if (T == 104) {
-                    chunk_dot_mx4<NB, WIDE>(sb, g, warp, lane, dir_chunk_elems(dir[3]), xs, reinterpret_cast<const float*>(lut), acc);
+                    chunk_dot_mx4<NB, WIDE>(sb, g, warp, lane, elems, xs, reinterpret_cast<const float*>(lut), acc);
                 } else if (T == -2) {
                     const uint32_t xs_a = smem_u32(xs);
-                    decode_chunk_generic_mx(sb, g, dir_chunk_elems(dir[3]), warp, lane, t, [&](int col, uint16_t bits) {
+                    decode_chunk_generic_mx(sb, g, elems, warp, lane, t, [&](int col, uint16_t bits) {
                         x_fma<NB>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
                     });
                 } else if (T >= 0) {
-                    chunk_dot_fast<(T >= 0 && T <= 5 ? T : 0), NB, WIDE>(sb, g, warp, lane, dir_chunk_elems(dir[3]), xs, lut, acc);
+                    chunk_dot_fast<(T >= 0 && T <= 5 ? T : 0), NB, WIDE>(sb, g, warp, lane, elems, xs, lut, acc);
                 } else {
                     const uint32_t xs_a = smem_u32(xs);
-                    decode_chunk_generic(sb, g, dir_chunk_elems(dir[3]), warp, lane, t, cb, [&](int col, uint16_t bits) {
+                    decode_chunk_generic(sb, g, elems, warp, lane, t, cb, [&](int col, uint16_t bits) {
                         x_fma<NB>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
                     });
                 }

@@ -21,3 +21,13 @@ def test_distributed_shared_memory_is_touched_behind_a_cluster_barrier(name):
         first = body.find("map_shared_rank")
         if first >= 0:
             assert re.search(r"cluster\.(sync|barrier_wait)\(\)", body[:first]), body[:200]
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_who_gives_up_still_meets_the_cluster(name):
+    """A thread that gives up a bounded wait and goes straight to the cluster's barrier leaves the others of its CTA at
+    __syncthreads, and the cluster waits for them for good: its warp decides as one and stays on the way that all take."""
+    for body in _functions(name):
+        if "mbar_wait_bounded(" in body and re.search(r"cluster\.(sync|barrier_arrive|barrier_wait)\(\)", body):
+            gives_up = re.search(r"\n( +)if \(!mbar_wait_bounded\([^;{]*\{(.*?)\n\1\}\n +lost = __any_sync\(0xffffffffu, lost\);", body, re.S)
+            assert gives_up and re.findall(r"\n *(.*)return", gives_up[2]) == ["if (out != 2) "], body[:200]
