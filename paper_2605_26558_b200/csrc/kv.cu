@@ -73,11 +73,15 @@ __global__ void __launch_bounds__(32 * kKvWarps) k_kv_append(KvGeom g, KvComp ck
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nj = FUSED ? NJ : g.d / 32;
     const bool coded = (flags & CASS_KV_COMPRESSED) != 0;
-    // The codebook tables were written when the codebook was frozen, long before this launch's predecessor: they may be
-    // read ahead of the wait, which hides their latency.
-    if (coded && (!FUSED || head < g.n_kv)) s_len[threadIdx.x] = of_seq((kind ? cv : ck).exp_to_rank, seq, g.seq_stride)[threadIdx.x] + 1u;
+    auto code_lengths = [&]() {
+        if (coded && (!FUSED || head < g.n_kv)) s_len[threadIdx.x] = of_seq((kind ? cv : ck).exp_to_rank, seq, g.seq_stride)[threadIdx.x] + 1u;
+    };
+    // FUSED: the predecessor is a projection, and the codebook tables were written before that: read ahead of the wait, they cost
+    // no time.  A stand-alone append may follow their writer (k_kv_rank ends a codebook of no tokens).
+    if (FUSED) code_lengths();
     pdl_wait();
     pdl_early<1>();
+    if (!FUSED) code_lengths();
     int start_pos = start_pos_arg;
     if (FUSED || start_pos < 0) start_pos = st->len[seq] + (use_inflight ? st->inflight[seq] : 0);
     if (FUSED && head >= g.n_kv) {

@@ -139,3 +139,29 @@ def test_span_of_tokens_equals_tokens_in_turn(cass, d, kv_p, kv_t, kv_mode, n_ne
     for e in engs:
         assert e.status()[0] == 0
         e.close()
+
+
+def test_append_right_behind_a_codebook_of_no_tokens(cass):
+    """The last kernel of such a codebook writes the tables that the append reads."""
+    d, n0 = 128, 24
+    shape = synth.ModelShape(n_layers=1, hidden=256, n_q_heads=4, n_kv_heads=2, head_dim=d, ffn=256, vocab=256)
+    wt = synth.model_weights(shape, 0, device="cuda")
+    gw = {"layers": [cass.engine.fuse_layer_weights(lw) for lw in wt["layers"]], "embed": wt["embed"], "lm_head": wt["lm_head"],
+          "norm_final": wt["norm_final"]}
+    k, v = (x.cuda() for x in synth.kv_fill(n0 + 4, 2, d, 3, "edge/kv"))
+    engs = [cass.engine.Engine(shape, gw, max_seq=384, gamma_max=4) for _ in range(2)]
+    for e in engs:
+        cass.cass_kv_append(e.session, 0, k[:n0].contiguous(), v[:n0].contiguous(), 0, n0, cass.KV_BF16)
+    a, b = k[n0:].contiguous(), v[n0:].contiguous()
+    for tokens in [n0, 0] * 20:                          # another codebook each time
+        for e in engs:
+            cass.cass_kv_build_codebook(e.session, tokens)
+            if e is engs[1]:
+                torch.cuda.synchronize()
+            cass.cass_kv_append(e.session, 0, a, b, n0, 4, cass.KV_COMPRESSED)
+        torch.cuda.synchronize()
+        for i, (x, y) in enumerate(zip(_records(cass, engs[0], 0, 0), _records(cass, engs[1], 0, 0))):
+            assert torch.equal(x, y), (tokens, i)
+    for e in engs:
+        assert e.status()[0] == 0
+        e.close()
