@@ -159,7 +159,8 @@ int cass_decode_full(const void* blob, const cass_blob_info* h_info, const void*
  * x: bf16 [cols].  partial: fp32 scratch [n_seg][n_rowblocks*32], which receives the per-segment sums.  Either
  * output pointer may be NULL; with both NULL only `partial` is produced.
  * h_info is what cass_weight_blob_info returned for this blob (that call synchronises, so the blob is complete: the
- * kernel starts reading the blob before earlier work on the stream has finished).  The blob buffer holds at least
+ * kernel starts reading the blob before earlier work on the stream has finished; a caller who fills the buffer with a
+ * kernel of its own synchronises likewise before the first call).  The blob buffer holds at least
  * h_info->total_bytes bytes; nothing beyond them is read, and a directory entry that points outside, like a header
  * that differs from h_info, is refused through d_status (CASS_ERR_INVALID_ARG) instead of being followed.
  * ---------------------------------------------------------------------------------------------------- */

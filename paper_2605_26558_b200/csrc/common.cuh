@@ -20,7 +20,10 @@
 
 // Launch with programmatic stream serialisation: the grid may be scheduled while its predecessor in the stream is
 // still running; every kernel launched this way calls pdl_wait() before it touches global memory, which returns
-// once the predecessor has completed and its writes are visible.
+// once the predecessor has completed and its writes are visible.  Four read something ahead of it that was there before the
+// predecessor began: the draft GEMV its blob (written by k_directory and k_pack, whose caller synchronises before the blob is
+// used), the verification projection a session's matrix, the norm its gains (both behind the embedding or a projection), the
+// fused KV encoder its codebook (written by k_kv_rank, behind a projection).  k_pack and k_kv_rank release nobody early.
 #define CASS_PDL_LAUNCH(kernel_, grid_, block_, smem_, stream_, ...)                                              \
     do {                                                                                                    \
         cudaLaunchConfig_t _cfg = {};                                                                       \
@@ -179,7 +182,8 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 // 0 small operators, 1 KV encoder, 2 draft attention, 3 attention merge, 4 verification attention, 5 verification
 // GEMM, 6 draft GEMV).  A kernel outside the mask releases its successor when it exits.  The release always comes after the
 // kernel's own griddepcontrol.wait, so that whoever starts finds everything before its predecessor complete, and after its
-// tensor-memory allocation.  The successor's set-up (barriers, tables, its first weight copies) then runs while the last CTAs
+// tensor-memory allocation.  (The two kernels that only add a stand-alone projection's parts release before it: whoever starts
+// then finds everything before that projection complete.)  The successor's set-up (barriers, tables, its first weight copies) then runs while the last CTAs
 // finish: decode step of the 8B shape 6.73 -> 6.54 ms, smallest draft GEMV 6.3 -> 5.3 us a call, projection 12.2 -> 10.6.
 // (Released before the wait, waiting CTAs took the predecessor's place: 25.5 -> 27.1 ms on the full model.)
 // Draft attention and the merge keep their successors out: 14.3 -> 13.5 us a stand-alone attention, the step the same.

@@ -488,8 +488,10 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
             for (int i = 0; i < 9; ++i) bad = bad || hw[i] != want[i];
             s_bad = bad;
         }
-        // Everything above touches only the blob, which no kernel writes.  When the launch allows this grid to start
-        // before its predecessor in the stream has finished, wait here: x and the scratch `partial` are the predecessor's.
+        // Everything above reads only the blob, ahead of the wait for the predecessor: a blob is complete before it is multiplied
+        // with.  Its writers are the encoder (k_directory and k_pack; its caller then asks for the blob's description, a call that
+        // synchronises) and a caller's copy of it, which in a session lies behind the embedding and the norm before the first
+        // projection.  x and the scratch `partial` are the predecessor's.
         pdl_wait();
         pdl_early<6>();
         // x of this segment (fp32), zero beyond the matrix
