@@ -82,7 +82,9 @@ __device__ __forceinline__ void row_load8(const uint16_t* __restrict__ p, uint32
 // "prune the n_prune smallest keys" is the rule "lowest score first, lower column first among equals".  The smallest
 // kept key is found in two steps: the top 16 bits of its score by a bitwise search that counts smaller ones two at a time
 // (packed bf16 compare and add: the scores' upper halves order as bf16 numbers), then the handful of keys that share
-// those bits are ranked against each other.
+// those bits are ranked against each other.  A score that is no number (a NaN weight, an infinite one times a norm of 0) counts
+// as infinite in the first step, which compares numbers, and as its bits in the second: it ranks above all others, as in an
+// integer order, and every row keeps the same count, on which the layout of the verification data rests.
 // A row is read once, 8 columns a lane, and its scores' upper halves stay in registers, NV values a lane; the few values
 // of which more is needed are read again.  Up to 2048 columns a warp holds a row and no barrier is needed (WIDE: false, four rows
 // a CTA); a longer row is a CTA's, of as many warps as it takes.
@@ -183,7 +185,7 @@ __global__ void __launch_bounds__(!WIDE ? 128 : NV == 128 ? 32 * kSelWarps : 32 
             for (int i = 0; i < 4; ++i) {
                 const uint32_t lo = __float_as_uint(__fmul_rn(__uint_as_float((w[i] << 16) & 0x7FFF0000u), a[2 * i]));
                 const uint32_t hi = __float_as_uint(__fmul_rn(__uint_as_float(w[i] & 0x7FFF0000u), a[2 * i + 1]));
-                x[q * 4 + i] = __byte_perm(lo, hi, 0x7632);
+                x[q * 4 + i] = __vminu2(__byte_perm(lo, hi, 0x7632), 0x7F807F80u);
             }
             if (c + 8 > g.k) {                                           // beyond the row: NaNs, which are neither below nor above anything
 #pragma unroll

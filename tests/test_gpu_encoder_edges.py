@@ -84,6 +84,44 @@ def test_constant_rows_and_no_pruning(cass):
         assert np.array_equal(got, layout.encode_weight_blob(_bits(w), act, p, t)[0]), (p, t)
 
 
+@pytest.mark.parametrize("rows,cols", [(8, 40), (37, 700), (37, 2048), (9, 2056), (8, 14336)])
+def test_scores_that_are_no_numbers_rank_highest(cass, rows, cols):
+    """NaN and infinite weights and norms: every row keeps its count, and the matrix comes back from its two parts."""
+    p = 400
+    rng = np.random.default_rng(cols)
+    w = _bits(synth.student_t_weight(rows, cols, 9, f"nan/{cols}"))
+    w[1, ::3] = 0x7FC1                                   # a third NaN
+    w[2, ::2], w[2, 1] = 0xFFC0, 0x7F80                  # half of the row -NaN, an infinity
+    w[3] = 0x7FFF
+    w[4, : cols - 5] = 0x7F80                            # more infinities than are kept
+    w[5, 3] = 0xFF80
+    w[6, cols // 3:] = 0x7F81                            # two thirds: among equals the lower columns go
+    act = (np.abs(rng.standard_normal(cols)) + 0.05).astype(np.float32)
+    act[7::11], act[8::13] = 0.0, np.inf                 # inf x 0 either way round
+    w[7, ::2] = 0
+    with np.errstate(invalid="ignore", over="ignore"):
+        score = (((w & 0x7FFF).astype(np.uint32) << 16).view(np.float32) * act).astype(np.float32)
+    key = np.where(np.isnan(score), np.uint32(0x7FFFFFFF), score.view(np.uint32))
+    keep = np.ones((rows, cols), dtype=bool)
+    np.put_along_axis(keep, np.argsort(key, axis=1, kind="stable")[:, : cols * p // 1000], False, axis=1)
+    wd = torch.from_numpy(w.view(np.int16)).cuda().view(torch.bfloat16)
+    fmt = cass.default_format(w_p=p)
+    bound, ws_bytes = cass.cass_encoded_weight_bytes(fmt, rows, cols)
+    blob = torch.zeros(bound, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    cass.cass_encode_weights(fmt, wd, torch.from_numpy(act).cuda(), blob, torch.zeros(ws_bytes, dtype=torch.uint8, device="cuda"), status)
+    info = cass.cass_weight_blob_info(blob)
+    assert int(status.item()) == 0
+    dec = torch.empty_like(wd)
+    cass.cass_decode_weights(blob, info, dec)
+    assert np.array_equal(_bits(dec), np.where(keep, w & 0xFFF0, 0))
+    vdata = torch.zeros(cass.cass_verification_data_bytes(info), dtype=torch.uint8, device="cuda")
+    cass.cass_encode_verification_data(blob, info, wd, vdata)
+    full = torch.empty_like(wd)
+    cass.cass_decode_full(blob, info, vdata, full)
+    assert np.array_equal(_bits(full), w)
+
+
 def _records(cass, eng, layer, seq):
     base, mem, out = eng.mem.data_ptr(), eng.mem.view(torch.int32), []
     for kind in (0, 1):
