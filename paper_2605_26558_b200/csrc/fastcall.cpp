@@ -2,10 +2,12 @@
 // ctypes and the Python expressions around it (one object per pointer, three attribute look-ups per tensor, shapes) took 1.5 to
 // 2.5 us of host time a call beside a launch of about 4 us: 6.0 -> 4.5 us for a draft GEMV, 16.3 -> 9.1 for a sampled step.
 // Every wrapper is generated from its C prototype: a tensor or None or an int (address) for a pointer, the ctypes structure for a
-// description, None for the current stream.  The interpreter lock is released around the call, as ctypes does.
+// description, None for the current stream.  The interpreter lock is released around the call, as ctypes does.  What torch throws
+// on the way (a tensor without storage, as under vmap; a CUDA that does not come up) becomes a Python exception.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <tuple>
@@ -113,13 +115,16 @@ struct Entry<F> {
         return PyLong_FromLong(rc);
     }
     static PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t n) {
+        HANDLE_TH_ERRORS
         if (n != (Py_ssize_t)N) return PyErr_Format(PyExc_TypeError, "%zd arguments where %zu are wanted", n, N);
         return run(args, std::make_index_sequence<N>{});
+        END_HANDLE_TH_ERRORS
     }
 };
 
 // (w, x, rows, scratch, y_bf16, y_f32, status, stream): sizes come from the tensors
 PyObject* verify_gemm(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
     if (n != 8) return PyErr_Format(PyExc_TypeError, "%zd arguments where 8 are wanted", n);
     for (int i : {0, 1, 3})
         if (!THPVariable_Check(a[i])) return PyErr_Format(PyExc_TypeError, "expected a CUDA tensor");
@@ -141,6 +146,7 @@ PyObject* verify_gemm(PyObject*, PyObject* const* a, Py_ssize_t n) {
     rc = cass_verify_gemm(wp, xp, (int)rows, nn, kk, sp, bytes, y16, static_cast<float*>(y32), static_cast<int32_t*>(st), stream);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
+    END_HANDLE_TH_ERRORS
 }
 
 #define CASS_ENTRY(NAME) {#NAME, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&Entry<&NAME>::call)), METH_FASTCALL, nullptr}

@@ -59,6 +59,34 @@ def test_host_only_queries_and_argument_checks():
     assert cass.cass_calib_norms_count(desc) == 2 * 4 * 688 + 256
 
 
+_STORAGELESS = """
+import types
+import torch
+from torch._subclasses import FakeTensorMode
+from paper_2605_26558_b200 import binding as B
+seen, stream = [], types.SimpleNamespace(cuda_stream=0)
+def raises(fn, *args):
+    try:
+        fn(*args, stream=stream)
+    except RuntimeError as e:
+        seen.append(not isinstance(e, B.CassError))
+def batched(x):
+    raises(B.cass_softmax, x, 1, 8, 1.0, x)
+    raises(B.cass_verify_gemm, x.new_empty(8, 8), x.expand(16, 8), 1, x, None, x, x)
+    return x
+with FakeTensorMode():
+    torch.func.vmap(batched)(torch.empty(2, 8, device="cuda"))
+assert seen == [True, True], seen
+"""
+
+
+def test_a_tensor_without_storage_is_an_exception_not_the_end_of_the_process():
+    """Under vmap a tensor has no address, and asking for it throws in C++; in a process of its own, which must live on."""
+    import subprocess
+    r = subprocess.run([sys.executable, "-c", _STORAGELESS], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, (r.returncode, r.stderr[-800:])
+
+
 def _replica_worker(rank, world, port, q):
     import torch.distributed as dist
     sys.path.insert(0, ROOT)
