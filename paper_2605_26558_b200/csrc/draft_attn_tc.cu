@@ -579,7 +579,7 @@ int launch_draft_attn_tc(const KvGeom& g, const KvComp& ck, const KvComp& cv, co
     if (!draft_attn_tc_supported(g, n_q)) return CASS_ERR_UNSUPPORTED;
     const int n_chunks = ceil_div(g.max_seq, kTcTok);
     const size_t smem = draft_attn_tc_smem_bytes(g);
-    if (smem > 227 * 1024) return CASS_ERR_UNSUPPORTED;
+    if (smem > kSmemPerBlock) return CASS_ERR_UNSUPPORTED;
     dim3 grid(n_chunks, g.n_kv, n_seq);
 #define CASS_TC_LAUNCH(MM, TT)                                                                                           \
     do {                                                                                                             \

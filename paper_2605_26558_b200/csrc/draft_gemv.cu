@@ -27,11 +27,14 @@ static size_t gemv_stage_bytes(const cass_blob_info& bi) { return align_up((size
 // Bytes per column of the x slice in shared memory: one vector is kept as fp32, several as packed bf16 [col][nb].
 __host__ __device__ constexpr int x_col_bytes(int nb) { return nb == 1 ? 4 : 2 * nb; }
 
-size_t gemv_smem_bytes(const cass_blob_info& bi, int nb) {
+static size_t gemv_smem_bytes(const cass_blob_info& bi, int nb) {
     const int n_ch = ceil_div(bi.seg_cols, bi.chunk_cols);
     return kGemvStages * gemv_stage_bytes(bi) + (size_t)(bi.seg_cols + kXSlack) * x_col_bytes(nb) + 256 * 4 +
            (size_t)(nb < 2 ? 2 : nb) * n_ch * 32 * 4 + 64;
 }
+
+// With what the kernel declares itself: a segment's sums, the tile's sizes and flags, up to where the dynamic part may begin.
+size_t gemv_smem_total(const cass_blob_info& bi, int nb) { return gemv_smem_bytes(bi, nb) + align_up((size_t)nb * 32 * 4 + 32, 512); }
 
 __device__ __forceinline__ uint32_t shl_sat(uint32_t v, uint32_t s) {      // shift counts >= 32 give 0
     uint32_t r;
@@ -671,15 +674,15 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
     const int n_ch = ceil_div(bi.seg_cols, bi.chunk_cols);
     if (n_ch > 32) return CASS_ERR_UNSUPPORTED;
     if (nb != 1 && nb != 2 && nb != 4 && nb != 8) return CASS_ERR_UNSUPPORTED;
-    const size_t smem = gemv_smem_bytes(bi, nb);
-    if (smem > 227 * 1024) return CASS_ERR_CAPACITY;
+    const size_t smem = gemv_smem_bytes(bi, nb), total = gemv_smem_total(bi, nb);
+    if (total > kSmemPerBlock) return CASS_ERR_CAPACITY;
     const int threads = 32 * n_ch;
     // One vector: one CTA per superblock -- the hardware hands out CTAs as shared memory frees, which balances the SMs to
     // within one superblock (a grid of as many CTAs as fit at once, each looping over its share, left SMs with 4 x 4
     // superblocks beside SMs with 4 x 3: 56.7 instead of 54.4 us on the 28672 x 4096 matrix).  Several vectors: the x
     // slice a CTA stages is nb times larger, so CTAs keep theirs and loop (one CTA per superblock: 52.3 instead of
     // 48.6 ms per step with 8 sequences).
-    int g = bi.n_rowblocks, per_sm = (int)((228 * 1024) / (smem + 1024));                 // CTAs an SM holds
+    int g = bi.n_rowblocks, per_sm = (int)((228 * 1024) / (total + 1024));                 // CTAs an SM holds
     if (per_sm > 2048 / threads) per_sm = 2048 / threads;
     if (per_sm < 1) per_sm = 1;
     if (nb > 1) {

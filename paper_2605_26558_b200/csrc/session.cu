@@ -208,7 +208,7 @@ static int read_blob_infos(Session* s, const cass_model_blobs* blobs, cudaStream
             int rc = cass_weight_blob_info(ptr[i], &s->layers[l].bi[i], stream);
             if (rc) return rc;
             if (s->layers[l].bi[i].rows != rows[i] || s->layers[l].bi[i].cols != cols[i]) return CASS_ERR_INVALID_ARG;
-            if (gemv_smem_bytes(s->layers[l].bi[i], s->B) > 227 * 1024) return CASS_ERR_CAPACITY;
+            if (gemv_smem_total(s->layers[l].bi[i], s->B) > kSmemPerBlock) return CASS_ERR_CAPACITY;
             if ((size_t)s->layers[l].bi[i].n_seg * s->layers[l].bi[i].n_rowblocks * 32 > s->partial_floats) return CASS_ERR_CAPACITY;
             s->layers[l].blob[i] = ptr[i];
         }
@@ -217,6 +217,7 @@ static int read_blob_infos(Session* s, const cass_model_blobs* blobs, cudaStream
     int rc = cass_weight_blob_info(blobs->lm_head, &s->lm_bi, stream);
     if (rc) return rc;
     if (s->lm_bi.rows != s->d.vocab || s->lm_bi.cols != s->d.hidden) return CASS_ERR_INVALID_ARG;
+    if (gemv_smem_total(s->lm_bi, s->B) > kSmemPerBlock) return CASS_ERR_CAPACITY;
     if ((size_t)s->lm_bi.n_seg * s->lm_bi.n_rowblocks * 32 > s->partial_floats) return CASS_ERR_CAPACITY;
     s->lm_blob = blobs->lm_head;
     s->have_blobs = true;

@@ -59,6 +59,25 @@ def test_host_only_queries_and_argument_checks():
     assert cass.cass_calib_norms_count(desc) == 2 * 4 * 688 + 256
 
 
+@pytest.mark.parametrize("n_vec,static", [(1, 512), (8, 1536)])
+def test_gemv_counts_all_of_its_shared_memory_against_the_limit(n_vec, static):
+    """A superblock that fits only without the kernel's own arrays is refused like a larger one, before anything is launched."""
+    import types
+
+    import paper_2605_26558_b200 as cass
+    stage = 512
+    rest = (2048 + 288) * (4 if n_vec == 1 else 2 * n_vec) + 1024 + max(n_vec, 2) * 8 * 32 * 4 + 64
+    while stage + 512 + rest <= 227 * 1024:
+        stage += 512
+    assert stage + rest + static > 227 * 1024
+    info = cass.binding.BlobInfo(rows=32, cols=2048, prune_permille=400, trunc_bits=4, seg_cols=2048, chunk_cols=256, n_seg=1, n_rowblocks=1,
+                                 kept_per_row=1229, max_superblock_bytes=stage - 384, mode=1, total_bytes=1 << 20)
+    for info.max_superblock_bytes in (stage - 384, 1 << 18):
+        with pytest.raises(cass.CassError) as e:
+            cass.cass_draft_gemv_batch(4096, info, 4096, n_vec, 4096, None, 4096, None, stream=types.SimpleNamespace(cuda_stream=0))
+        assert e.value.code == cass.ERR_CAPACITY
+
+
 _STORAGELESS = """
 import types
 import torch
