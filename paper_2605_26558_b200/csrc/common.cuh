@@ -35,6 +35,7 @@
         if (cudaLaunchKernelEx(&_cfg, kernel_, __VA_ARGS__) != cudaSuccess) return CASS_ERR_CUDA;            \
     } while (0)
 
+#include <atomic>
 #include <cstdlib>
 
 namespace cass {
@@ -60,6 +61,28 @@ constexpr int kPrefillRows = 256;          // rows of all sequences in one pass 
 
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 __host__ __device__ inline size_t align_up(size_t a, size_t b) { return (a + b - 1) / b * b; }
+
+// Dynamic shared memory beyond 48 KB is allowed per kernel and device and stays as it was last set.  All that a kernel can take is
+// allowed ahead of its first launch on a device: a limit that follows the calls' sizes could be lowered by one thread between
+// another's setting and its launch.
+template <auto Kernel>
+inline int allow_smem() {
+    static std::atomic<unsigned long long> done{0};                       // a bit per device
+    int dev = 0;
+    CASS_CUDA_CHECK(cudaGetDevice(&dev));
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_relaxed) & bit) return CASS_OK;
+    cudaFuncAttributes own;
+    CASS_CUDA_CHECK(cudaFuncGetAttributes(&own, Kernel));
+    CASS_CUDA_CHECK(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemPerBlock - own.sharedSizeBytes)));
+    done.fetch_or(bit, std::memory_order_relaxed);
+    return CASS_OK;
+}
+#define CASS_ALLOW_SMEM(...)                                              \
+    do {                                                                  \
+        const int _rc = cass::allow_smem<__VA_ARGS__>();                  \
+        if (_rc) return _rc;                                              \
+    } while (0)
 
 // ---- sign + mantissa fields of the speculation data ----------------------------------------------------
 // A field is the sign bit followed by the 7-t kept mantissa bits (F = 8-t bits); a 32-bit word holds 32/F

@@ -168,11 +168,7 @@ int launch_attn_merge(const AttnScratch& sc, int chunk_tokens, int n_seq, const 
 #undef CASS_MERGE_FEW
     const size_t smem = ((size_t)((ar.chunks + 3) & ~3) + (size_t)kMergeWarps * d) * 4;
     if (smem > 200 * 1024) return CASS_ERR_CAPACITY;
-    static size_t attr = 48 * 1024;
-    if (smem > attr) {
-        CASS_CUDA_CHECK(cudaFuncSetAttribute(k_attn_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr = smem;
-    }
+    CASS_ALLOW_SMEM(k_attn_merge);
     CASS_PDL_LAUNCH(k_attn_merge, grid, dim3(kMergeThreads), smem, s, sc, chunk_tokens, ar, n_q, d, st, draft_mode,
                     draft_units, out);
     return CASS_OK;

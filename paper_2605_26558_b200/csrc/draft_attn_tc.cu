@@ -583,11 +583,7 @@ int launch_draft_attn_tc(const KvGeom& g, const KvComp& ck, const KvComp& cv, co
     dim3 grid(n_chunks, g.n_kv, n_seq);
 #define CASS_TC_LAUNCH(MM, TT)                                                                                           \
     do {                                                                                                             \
-        static size_t attr = 0;                                                                                      \
-        if (smem > attr) {                                                                                           \
-            CASS_CUDA_CHECK(cudaFuncSetAttribute((k_draft_attn_tc<MM, TT>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-            attr = smem;                                                                                             \
-        }                                                                                                            \
+        CASS_ALLOW_SMEM(k_draft_attn_tc<MM, TT>);                                                                    \
         CASS_PDL_LAUNCH((k_draft_attn_tc<MM, TT>), grid, dim3(kTcThreads), smem, s, g, ck, cv, qkv, qkv_stride, n_q, st, sc, n_chunks);      \
     } while (0)
     if (g.mode == 1 && g.t == 4) CASS_TC_LAUNCH(1, 4);

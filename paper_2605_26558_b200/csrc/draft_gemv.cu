@@ -707,12 +707,7 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
     const int stage = (int)gemv_stage_bytes(bi);
 #define CASS_GEMV_LAUNCH(TT, NN, WW)                                                                             \
     do {                                                                                                       \
-        static int attr_smem = 0;      /* largest size already granted to this instantiation */              \
-        if ((int)smem > attr_smem) {                                                                           \
-            CASS_CUDA_CHECK(cudaFuncSetAttribute((k_draft_gemv<TT, NN, WW>), cudaFuncAttributeMaxDynamicSharedMemorySize,\
-                                                 (int)smem));                                                  \
-            attr_smem = (int)smem;                                                                             \
-        }                                                                                                      \
+        CASS_ALLOW_SMEM(k_draft_gemv<TT, NN, WW>);                                                             \
         cudaLaunchConfig_t cfg = {};                                                                           \
         cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;            \
         cudaLaunchAttribute at[2];                                                                             \

@@ -311,7 +311,7 @@ int launch_sample(const float* probs, int rows, int vocab, const float* u, int32
     int cs;
     const size_t smem = draw_plan(vocab, &cs);
     if (!smem) return launch_clusters(k_sample_rows<false>, rows, cs, kSampleThreads, 0, s, probs, vocab, u, tokens, tok_stride);
-    CASS_CUDA_CHECK(cudaFuncSetAttribute(k_sample_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CASS_ALLOW_SMEM(k_sample_rows<true>);
     return launch_clusters(k_sample_rows<true>, rows, cs, kSampleThreads, smem, s, probs, vocab, u, tokens, tok_stride);
 }
 
@@ -321,7 +321,7 @@ int launch_accept_sampling(DevState* st, int n_seq, const int32_t* draft, int dr
     int cs;
     const size_t smem = draw_plan(vocab, &cs);
     auto kernel = smem ? k_accept_sampling<true> : k_accept_sampling<false>;
-    CASS_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CASS_ALLOW_SMEM(k_accept_sampling<true>);
     return launch_clusters(kernel, n_seq, cs, kSampleThreads, smem, s, st, draft, draft_stride, p, q, vocab, r, u, g, n_acc, out_tokens,
                            next_tok, next_stride);
 }

@@ -140,11 +140,7 @@ int launch_verify_attn(const KvGeom& g, const uint16_t* k_cache, const uint16_t*
     const int n_groups = ceil_div(ar.hi - ar.lo, ar.group);
     size_t smem = (size_t)kAttnChunk * (g.d + 8) * 2 + (size_t)kAttnChunk * g.d * 2 + (size_t)kVaMaxPairs * g.d * 4 +
                   (size_t)kVaMaxPairs * kAttnChunk * 4;
-    static size_t attr = 0;
-    if (smem > attr) {
-        CASS_CUDA_CHECK(cudaFuncSetAttribute(k_verify_attn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr = smem;
-    }
+    CASS_ALLOW_SMEM(k_verify_attn);
     dim3 grid(ar.chunks, g.n_kv, n_seq * n_groups);
     CASS_PDL_LAUNCH(k_verify_attn, grid, dim3(kVaThreads), smem, s, g, k_cache, v_cache, qkv, ar, n_groups, n_q, st, sc);
     return launch_attn_merge(sc, kAttnChunk, n_seq, ar, n_q, g.d, st, 0, 0, out, s);

@@ -260,19 +260,11 @@ int launch_verify_attn_tc(const KvGeom& g, const uint16_t* k_cache, const uint16
     const int n_groups = ceil_div(ar.hi - ar.lo, ar.group);
     dim3 grid(ar.chunks, g.n_kv, n_seq * n_groups);
     if (np_cols == 32) {
-        static bool attr = false;
-        if (!attr) {
-            CASS_CUDA_CHECK(cudaFuncSetAttribute(k_verify_attn_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, vt_smem(32)));
-            attr = true;
-        }
+        CASS_ALLOW_SMEM(k_verify_attn_tc<32>);
         CASS_PDL_LAUNCH(k_verify_attn_tc<32>, grid, dim3(kVtThreads), (size_t)vt_smem(32), s, mk, mv, qkv, ar, n_groups, fine, n_q,
                         g.n_kv, st, sc, d_status);
     } else {
-        static bool attr = false;
-        if (!attr) {
-            CASS_CUDA_CHECK(cudaFuncSetAttribute(k_verify_attn_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, vt_smem(64)));
-            attr = true;
-        }
+        CASS_ALLOW_SMEM(k_verify_attn_tc<64>);
         CASS_PDL_LAUNCH(k_verify_attn_tc<64>, grid, dim3(kVtThreads), (size_t)vt_smem(64), s, mk, mv, qkv, ar, n_groups, fine, n_q,
                         g.n_kv, st, sc, d_status);
     }

@@ -208,11 +208,7 @@ size_t verify_gemm_partial_floats(int n, int k, int bn) {
 template <int BN>
 static int launch_tc(const CUtensorMap& mw, const CUtensorMap& mx, float* partial, int rows, int n, int kbt, int kbs, int ns,
                      int32_t* d_status, int w_static, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) {
-        CASS_CUDA_CHECK(cudaFuncSetAttribute(k_verify_gemm_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem(BN)));
-        attr = true;
-    }
+    CASS_ALLOW_SMEM(k_verify_gemm_tc<BN>);
     dim3 grid(ceil_div(n, kTcBM), ns);
     CASS_PDL_LAUNCH(k_verify_gemm_tc<BN>, grid, dim3(kTcThreads), (size_t)tc_smem(BN), s, mw, mx, partial, rows, n, kbt, kbs, d_status, w_static);
     return CASS_OK;

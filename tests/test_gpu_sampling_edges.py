@@ -59,3 +59,31 @@ def test_acceptance_draws_from_the_residual_or_the_target(cass, vocab):
                               torch.full((3,), 0.5, device="cuda"), g, n_acc, out, nxt)
     assert n_acc.tolist() == [0, 2, 0]
     assert out.view(3, 3).tolist() == [[7, -1, -1], [5, 5, vocab - 1], [9, -1, -1]] and nxt.tolist() == [7, vocab - 1, 9]
+
+
+def test_threads_with_different_vocabularies(cass):
+    """Calls of two threads, each on its own stream, whose draws need different amounts of shared memory."""
+    import threading
+    sizes, errors = (1000, 200000), []
+    probs = [torch.full((1, n), 1.0 / n, device="cuda") for n in sizes]
+    u = torch.full((1,), 0.5, device="cuda")
+    start = threading.Barrier(len(sizes))
+
+    def calls(i):
+        stream, tok = torch.cuda.Stream(), torch.zeros(1, dtype=torch.int32, device="cuda")
+        start.wait()
+        try:
+            for _ in range(3000):
+                cass.cass_sample(probs[i], 1, sizes[i], u, tok, stream=stream)
+            stream.synchronize()
+            assert abs(int(tok.item()) - sizes[i] // 2) <= 1 + sizes[i] // 10000
+        except Exception as e:                              # noqa: BLE001
+            errors.append((sizes[i], repr(e)))
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=calls, args=(i,)) for i in range(len(sizes))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
