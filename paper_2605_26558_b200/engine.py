@@ -69,7 +69,7 @@ class Engine:
         self._results = torch.zeros(8 + 64, dtype=torch.int32, device=self.device)
         self.n_acc, self.out_tokens = self._results[:8], self._results[8:]
         self._stride = 1              # gamma + 1 of the layout the token buffers are in
-        self._graphs = {}
+        self._graphs = {}             # captured steps by gamma; they hold the addresses of the parts they read
 
     def close(self):
         if self.session is not None:
@@ -147,6 +147,7 @@ class Engine:
                 setattr(self._lb[i], nm, d[nm].data_ptr())
         self._mb = B.ModelBlobs(self._lb, blobs["lm_head"].data_ptr())
         B.cass_session_set_blobs(self.session, self._mb)
+        self._graphs.clear()
 
     def verify_from_parts(self, drop_bf16: bool = False) -> int:
         """Encodes the verification data of every matrix and makes the session verify from speculation + verification
@@ -175,6 +176,7 @@ class Engine:
         self.vscratch = torch.empty(B.cass_verify_from_parts_scratch_bytes(self.desc), dtype=torch.uint8, device=self.device)
         torch.cuda.synchronize(self.device)
         B.cass_session_verify_from_parts(self.session, self._mv, self.vscratch)
+        self._graphs.clear()
         if drop_bf16:
             for lw in self.w["layers"]:
                 for nm in ("wqkv", "wo", "wgu", "wd"):

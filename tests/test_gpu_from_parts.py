@@ -77,3 +77,32 @@ def test_from_parts_equals_the_bf16_copy(cass, shape, n_prompt, gamma):
     assert torch.equal(l16a, l16b)
     for e in (ref, par):
         e.close()
+
+
+def test_captured_steps_follow_a_change_of_what_they_read(cass):
+    """A step captured with one set of speculation data, or with the bf16 matrices, is not replayed once the engine was given
+    another set or verifies from the parts: tokens and acceptance are those of an engine that never captured one."""
+    shape, gamma = synth.TINY, 4
+    gw = _weights(cass, shape, 0)
+    prompt = synth.random_prompt(40, shape.vocab, 0)
+
+    def decode(captured):
+        w = {"layers": [dict(lw) for lw in gw["layers"]], "embed": gw["embed"], "lm_head": gw["lm_head"], "norm_final": gw["norm_final"]}
+        eng = cass.engine.Engine(shape, w, max_seq=256, gamma_max=8)
+        out = []
+        for p in (400, 900, None):                           # two sets of speculation data (the second accepts fewer drafts); the parts
+            eng.prefill(prompt, calibrate=not out)
+            if p:
+                eng.fmt = cass.default_format(w_p=p)
+                eng.encode_weights(eng.calib_norms())
+            else:
+                eng.verify_from_parts(drop_bf16=True)
+            eng.build_kv_codebook()
+            toks, stats = eng.generate(24, gamma, use_graph=captured)
+            out.append((toks, stats.accepted, stats.steps))
+        assert eng.status()[0] == 0
+        eng.close()
+        return out
+
+    a, b = decode(True), decode(False)
+    assert a == b and a[0] != a[1]
