@@ -382,7 +382,8 @@ __global__ void __launch_bounds__(kTcThreads) k_draft_attn_tc(KvGeom g, KvComp c
     const uint32_t* off_h = of_seq(c.off, seq, g.seq_stride) + (size_t)head * (g.max_seq + 1);
     const uint32_t* arena = of_seq(c.arena, seq, g.seq_stride) + (size_t)head * g.arena_words;
     const uint8_t* r2e = of_seq(c.rank_to_exp, seq, g.seq_stride);
-    // Tokens beyond the visible length leave their rows zero, as their probabilities are.
+    // Tokens beyond the visible length leave their rows zero, as their probabilities are.  A position that was never encoded (tokens
+    // generated before the codebooks were there) has whatever offsets: no record is read further than one can be long.
     auto load_off = [&](int t0, uint32_t& o0, uint32_t& n_una) {
         o0 = 0; n_una = 0;
         if (MODE != 1) return;                                                // Cassandra-2 records have no exponent stream
@@ -390,7 +391,7 @@ __global__ void __launch_bounds__(kTcThreads) k_draft_attn_tc(KvGeom g, KvComp c
         if (t0 < t_end && n_here > 0) {
             const int tok = t0 + tw * 32 + min(lane, n_here - 1);
             o0 = __ldg(off_h + tok);
-            n_una = __ldg(off_h + tok + 1) - o0;
+            n_una = min(__ldg(off_h + tok + 1) - o0, (uint32_t)g.rec_words_max);
         }
     };
 

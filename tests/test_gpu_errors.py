@@ -173,3 +173,19 @@ def test_sequence_full_is_reported_not_overrun(cass):
     with pytest.raises(cass.CassError):
         cass.cass_set_len(eng.session, 120)               # would leave no room for the next call's rows
     eng.close()
+
+
+def test_tokens_generated_before_the_codebooks_are_read_within_bounds(cass):
+    """Plain decoding before the codebooks leaves positions without a record; drafts over them are poor, nothing more."""
+    a, b = _tiny_engine(cass, max_seq=256), _tiny_engine(cass, max_seq=256)
+    for eng in (a, b):
+        eng.prefill(synth.random_prompt(60, synth.TINY.vocab, 5), calibrate=True)
+        eng.generate(70, 0)
+        eng.encode_weights(eng.calib_norms())
+    a.build_kv_codebook()
+    spec, _ = a.generate(40, 4)
+    plain, _ = b.generate(40, 0)
+    n = min(len(spec), len(plain))
+    assert n >= 40 and spec[:n] == plain[:n] and a.status()[0] == 0
+    a.close()
+    b.close()
