@@ -140,6 +140,10 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
         } else {
             atomicExch(d_status, CASS_ERR_TIMEOUT); ok = false;
         }
+        if (!ok) {                                     // what is in flight lands before the CTA ends (bounded)
+            mbar_wait_bounded(bar_k, 0);
+            mbar_wait_bounded(bar_v, 0);
+        }
         tc_commit(bar_s);
         // ---- out^T = V^T . P^T: A = V tile as stored (rows = tokens: M-contiguous), B = P (K-major over tokens) ----
         if (ok && mbar_wait_bounded(bar_v, 0) && mbar_wait_bounded(bar_p, 0)) {
@@ -157,6 +161,7 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
             }
         } else if (ok) {
             atomicExch(d_status, CASS_ERR_TIMEOUT);
+            mbar_wait_bounded(bar_v, 0);
         }
         tc_commit(bar_o);
     }

@@ -117,7 +117,13 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
         for (int kb = 0; kb < nkb && ok; ++kb) {
             const int s = kb % kTcStages;
             const uint32_t ph = (uint32_t)(kb / kTcStages) & 1u;
-            if (!mbar_wait_bounded(&full[s], ph)) { atomicExch(d_status, CASS_ERR_TIMEOUT); ok = false; break; }
+            if (!mbar_wait_bounded(&full[s], ph)) {
+                atomicExch(d_status, CASS_ERR_TIMEOUT);
+                ok = false;
+                for (int j = kb; j < nkb && j < kb + kTcStages; ++j)          // what is in flight lands before the CTA ends (bounded)
+                    mbar_wait_bounded(&full[j % kTcStages], (uint32_t)(j / kTcStages) & 1u);
+                break;
+            }
             tc_fence_after();
             const uint64_t ad = tc_smem_desc(sA + s * kTcABytes), bd = tc_smem_desc(sB + s * kTcBBytes);
 #pragma unroll

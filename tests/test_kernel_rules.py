@@ -31,3 +31,12 @@ def test_who_gives_up_still_meets_the_cluster(name):
         if "mbar_wait_bounded(" in body and re.search(r"cluster\.(sync|barrier_arrive|barrier_wait)\(\)", body):
             gives_up = re.search(r"\n( +)if \(!mbar_wait_bounded\([^;{]*\{(.*?)\n\1\}\n +lost = __any_sync\(0xffffffffu, lost\);", body, re.S)
             assert gives_up and re.findall(r"\n *(.*)return", gives_up[2]) == ["if (out != 2) "], body[:200]
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_copies_in_flight_land_before_their_block_ends(name):
+    """A kernel that gives up a wait for a copy waits (again with a limit, whatever the outcome) for the copies it has started: they
+    would land in the shared memory of the block after it."""
+    for body in _functions(name):
+        if "__global__" in body and re.search(r"\b(tma_load_\dd|bulk_g2s)\(", body):
+            assert re.search(r"\n +mbar_wait_bounded\(", body), body[:200]
