@@ -289,7 +289,9 @@ int cass_verify(void* session, const int32_t* toks, int g, int32_t* target_argma
  * (all sequences equally long, n <= max_seq - 16).  Writes K/V of those positions into the bf16 cache, and into the compressed
  * one if the codebooks are built; the greedy token after each prompt goes to target_argmax[b]; every length becomes n and no
  * draft is in flight.  While calibration is on, the statistics of every row are accumulated.  The passes are wider than those
- * of cass_verify and the results the same.  toks: device [max_batch][n]; target_argmax: device [max_batch]. */
+ * of cass_verify.  A row has the bits that cass_verify gives it where both take the same attention kernel; with head size 128
+ * and more than four query heads a KV head, cass_verify takes 16 rows to the fp32 pipes and the wide pass stays on the tensor
+ * cores, as accurate (probabilities in two bf16 terms) but in another order of additions.  toks: device [max_batch][n]; target_argmax: device [max_batch]. */
 int cass_prefill(void* session, const int32_t* toks, int n, int32_t* target_argmax, void* stream);
 
 /* Stand-alone draft attention of one layer (Sec. 4.1 draft inference over the KV speculation data of Sec. 4.2):

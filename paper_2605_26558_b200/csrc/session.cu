@@ -545,8 +545,9 @@ static int prefill_attention(Session* s, const LayerDev& L, int pos, int w, int 
 
 // The prompt in passes of kPrefillRows rows over all sequences: every pass reads the weights once for its rows (16 rows a
 // pass, as verification takes them, read them 16 times as often: 51.8 ms instead of 4.3 ms, and 128 rows a pass 5.5 ms, for 1000 tokens of four
-// 8B-shaped layers), and lm_head runs once.  A row's result is what cass_verify gives for it: the same K ranges, added in
-// the same order.
+// 8B-shaped layers), and lm_head runs once.  A row's projections are what cass_verify gives for it: the same K ranges, added in
+// the same order.  So is its attention, except where cass_verify takes 16 rows to the fp32 pipes (head size 128, more than four query
+// heads a KV head): those rows stay on the tensor cores here, as accurate but in another order of additions.
 extern "C" int cass_prefill(void* session, const int32_t* toks, int n, int32_t* target_argmax, void* stream_) {
     if (!session || !toks || !target_argmax) return CASS_ERR_INVALID_ARG;
     Session* s = (Session*)session;
