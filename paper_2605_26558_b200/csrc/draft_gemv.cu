@@ -36,12 +36,6 @@ static size_t gemv_smem_bytes(const cass_blob_info& bi, int nb) {
 // With what the kernel declares itself: a segment's sums, the tile's sizes and flags, up to where the dynamic part may begin.
 size_t gemv_smem_total(const cass_blob_info& bi, int nb) { return gemv_smem_bytes(bi, nb) + align_up((size_t)nb * 32 * 4 + 32, 512); }
 
-__device__ __forceinline__ uint32_t shl_sat(uint32_t v, uint32_t s) {      // shift counts >= 32 give 0
-    uint32_t r;
-    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
-    return r;
-}
-
 __device__ __forceinline__ uint32_t bfind_u32(uint32_t v) {         // index of the most significant one, -1 if none
     uint32_t r;
     asm("bfind.u32 %0, %1;" : "=r"(r) : "r"(v));

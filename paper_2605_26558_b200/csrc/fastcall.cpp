@@ -149,12 +149,22 @@ PyObject* verify_gemm(PyObject*, PyObject* const* a, Py_ssize_t n) {
     END_HANDLE_TH_ERRORS
 }
 
+// (stream) -> its handle as an int; None: the current stream's
+PyObject* stream_address(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    void* stream;
+    if (n != 1) return PyErr_Format(PyExc_TypeError, "%zd arguments where 1 is wanted", n);
+    return stream_handle(a[0], &stream) ? PyLong_FromVoidPtr(stream) : nullptr;
+    END_HANDLE_TH_ERRORS
+}
+
 #define CASS_ENTRY(NAME) {#NAME, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&Entry<&NAME>::call)), METH_FASTCALL, nullptr}
 PyMethodDef kMethods[] = {
     CASS_ENTRY(cass_draft_gemv), CASS_ENTRY(cass_draft_gemv_batch), CASS_ENTRY(cass_draft_gemv_static), CASS_ENTRY(cass_kv_append),
     CASS_ENTRY(cass_set_len), CASS_ENTRY(cass_draft_step), CASS_ENTRY(cass_verify), CASS_ENTRY(cass_draft_attention), CASS_ENTRY(cass_accept),
     CASS_ENTRY(cass_accept_sampling), CASS_ENTRY(cass_softmax), CASS_ENTRY(cass_sample),
     {"cass_verify_gemm", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&verify_gemm)), METH_FASTCALL, nullptr},
+    {"stream_address", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&stream_address)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_fastcall", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
 

@@ -128,26 +128,6 @@ __device__ __forceinline__ void parts_sum4_pair(const Partials& pp, size_t off_a
             }
     }
 }
-// The same for N offsets at once: all loads of a batch of parts travel together.
-template <int N>
-__device__ __forceinline__ void parts_sum_n(const Partials& pp, const size_t (&off)[N], const bool (&on)[N], float (&acc)[N]) {
-    constexpr int B = N >= 8 ? 2 : (N >= 4 ? 4 : 8);                  // parts per batch: at most 16-32 loads in flight per thread
-#pragma unroll
-    for (int j = 0; j < N; ++j) acc[j] = 0.f;
-    for (int s0 = 0; s0 < pp.n_seg; s0 += B) {
-        float v[N][B];
-#pragma unroll
-        for (int j = 0; j < N; ++j)
-#pragma unroll
-            for (int i = 0; i < B; ++i)
-                v[j][i] = (on[j] && s0 + i < pp.n_seg) ? __ldcg(pp.p + (size_t)(s0 + i) * pp.seg_stride + off[j]) : 0.f;
-#pragma unroll
-        for (int j = 0; j < N; ++j)
-#pragma unroll
-            for (int i = 0; i < B; ++i)
-                if (on[j] && s0 + i < pp.n_seg) acc[j] += v[j][i];
-    }
-}
 
 constexpr int kAttnChunk = 64;       // split-K granularity over the sequence (fixed absolute boundaries)
 

@@ -138,11 +138,7 @@ static size_t layout(Session* s, uint8_t* base) {
     s->pattn = (uint16_t*)at(p.take(W * d.n_q_heads * d.head_dim * 2));
     s->pact = (uint16_t*)at(p.take(W * d.ffn * 2));
     s->logits = (float*)at(p.take((size_t)R * d.vocab * 4));
-    // split-K partials of the draft GEMVs: segments (<= ceil(K/256)) x padded rows
-    size_t nmax = (size_t)d.vocab;
-    if ((size_t)2 * d.ffn > nmax) nmax = 2 * (size_t)d.ffn;
-    if ((size_t)s->qkv_dim > nmax) nmax = s->qkv_dim;
-    size_t segmax = (size_t)ceil_div(s->kmax, 256) + 1;
+    // split-K partials of the draft GEMVs: segments x padded rows
     size_t pf = 0;
     {   // exact bound: max over the five matrix shapes of ceil(K/256) * pad32(N) (smallest legal segment is one chunk)
         auto need = [&](size_t n, size_t k) { return (size_t)ceil_div((int)k, 256) * align_up(n, 32); };
@@ -150,7 +146,6 @@ static size_t layout(Session* s, uint8_t* base) {
                        need(d.hidden, d.ffn), need(d.vocab, d.hidden)};
         for (size_t v : c) if (v > pf) pf = v;
     }
-    (void)segmax; (void)nmax;
     s->partial_floats = pf;                                   // per vector of a draft GEMV
     s->partial = (float*)at(p.take(pf * 4 * s->B));
     {   // split-K scratch of the verification GEMMs
