@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import concurrent.futures
+import importlib.metadata
 import os
 import subprocess
 import sys
@@ -10,6 +11,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcass.so")
 FASTCALL = os.path.join(HERE, "_fastcall.so")          # CPython entry points of the library (csrc/fastcall.cpp)
+FASTCALL_FOR = os.path.join(HERE, "_build", "_fastcall.txt")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
          "--expt-relaxed-constexpr"]
@@ -26,9 +28,21 @@ def _stale(target: str, deps: list[str]) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _fastcall_for() -> str:
+    """What the entry points are compiled against: another torch or interpreter may lay its objects out otherwise."""
+    return f"torch {importlib.metadata.version('torch')} {sys.implementation.cache_tag}"
+
+
+def _fastcall_current(src: str, header: str) -> bool:
+    if _stale(FASTCALL, [src, header]) or not os.path.exists(FASTCALL_FOR):
+        return False
+    with open(FASTCALL_FOR) as f:
+        return f.read() == _fastcall_for()
+
+
 def _build_fastcall(header: str, force: bool) -> None:
     src = os.path.join(CSRC, "fastcall.cpp")
-    if not force and not _stale(FASTCALL, [src, header]):
+    if not force and _fastcall_current(src, header):
         return
     import sysconfig
 
@@ -43,6 +57,8 @@ def _build_fastcall(header: str, force: bool) -> None:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed for {src}:\n{r.stdout}\n{r.stderr}")
+    with open(FASTCALL_FOR, "w") as f:
+        f.write(_fastcall_for())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

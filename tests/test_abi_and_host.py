@@ -30,6 +30,16 @@ def test_library_exports_every_declared_symbol():
     assert "sm_100a" in cass.cass_version()
 
 
+def test_entry_points_are_rebuilt_for_another_torch(monkeypatch):
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2605_26558_b200 import build
+    at = [os.path.join(build.CSRC, "fastcall.cpp"), os.path.join(ROOT, "include", "cass.h")]
+    assert build._fastcall_current(*at)
+    monkeypatch.setattr(build.importlib.metadata, "version", lambda name: "0.0")
+    assert not build._fastcall_current(*at)
+
+
 def test_host_only_queries_and_argument_checks():
     import paper_2605_26558_b200 as cass
     fmt = cass.default_format()
