@@ -56,6 +56,7 @@ constexpr int kGroupCodes = 4;             // codewords per unary-walk group
 constexpr int kMaxVerifyRows = 16;         // rows of one sequence in one verification call; also the margin kept at the end of a cache
 constexpr int kMaxBatch = 8;               // sequences per session
 constexpr int kMaxRows = 64;               // rows of all sequences in one call
+constexpr int kSms = 148;                  // of a B200: what grids and the rules between kernels are sized by
 constexpr size_t kSmemPerBlock = 227 * 1024;      // shared memory a CTA may have, its own arrays included
 constexpr int kPrefillRows = 256;          // rows of all sequences in one pass of a prefill
 

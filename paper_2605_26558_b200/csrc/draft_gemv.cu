@@ -652,16 +652,6 @@ __global__ void k_gemv_finish(const float* __restrict__ partial, int n, int n_pa
     if (y_bf16) y_bf16[(size_t)b * n + r] = float_to_bf16_bits(acc);
 }
 
-static int gemv_sm_count() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-            n = 148;
-    }
-    return n;
-}
-
 // y_bf16 / y_f32 (either may be null): [nb][rows] results.  Both null: only `partial`, which the caller's next kernel adds.
 static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x_bf16, int nb, float* partial, uint16_t* y_bf16,
                        float* y_f32, int32_t* d_status, cudaStream_t stream) {
@@ -680,7 +670,7 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
     if (per_sm > 2048 / threads) per_sm = 2048 / threads;
     if (per_sm < 1) per_sm = 1;
     if (nb > 1) {
-        g = ceil_div(gemv_sm_count() * per_sm, bi.n_seg);
+        g = ceil_div(kSms * per_sm, bi.n_seg);
         if (g > bi.n_rowblocks) g = bi.n_rowblocks;
     }
     if (g < 1) g = 1;
@@ -689,7 +679,7 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
     // idle where CTAs queue (12613 x 5686 at t = 0: 57.4 us, 47.0 with the finishing kernel; 4096 x 14336: 31.5 and 28.7;
     // against that 1000 x 3000: 8.6 and 8.9, 2000 x 11000: 17.9 and 18.4).
     const bool want = y_bf16 || y_f32;
-    const bool room = 4ll * bi.n_seg * g <= 3ll * gemv_sm_count() * per_sm;
+    const bool room = 4ll * bi.n_seg * g <= 3ll * kSms * per_sm;
     const int out = !want ? 0 : bi.n_seg == 1 ? 1 : (bi.n_seg <= 8 && g == bi.n_rowblocks && room) ? 2 : 0;
     // with q = 1 - p kept, 8 kept columns span 8 / q columns, give or take sqrt(8 p) / q: more than 32 about once in 10^4 groups
     // of a lane at p = 50 %, once in 40 at 60 %, and one lane's long gap costs its warp a careful walk (359 x 1467 at p = 60 %:

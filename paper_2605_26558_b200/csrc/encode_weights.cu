@@ -619,11 +619,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_pack(const uint16_t* __restri
 template <int NV, bool WIDE>
 static int launch_select_as(const uint16_t* W, const float* act, const EncGeom& g, const EncWs& ws, cudaStream_t stream) {
     const int warps = WIDE ? ceil_div(g.k, 32 * NV) : 4, rows = WIDE ? 1 : 4;
-    int dev = 0, sms = 148, per_sm = 1;
-    CASS_CUDA_CHECK(cudaGetDevice(&dev));
-    CASS_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int per_sm = 1;
     CASS_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (k_select<NV, WIDE>), 32 * warps, 0));
-    const int most = sms * (per_sm < 1 ? 1 : per_sm), need = ceil_div(g.n, rows);
+    const int most = kSms * (per_sm < 1 ? 1 : per_sm), need = ceil_div(g.n, rows);
     CASS_PDL_LAUNCH((k_select<NV, WIDE>), dim3(need < most ? need : most), dim3(32 * warps), 0, stream, W, act, g, ws.keepbm, ws.hist);
     return CASS_OK;
 }
@@ -751,7 +749,7 @@ extern "C" int cass_encode_weights(const cass_format* fmt, const void* W_bf16, c
                         (const uint8_t*)ws.exp_to_rank, b32, (const uint32_t*)ws.abort_flag);
         return CASS_OK;
     };
-    if (n_sb <= 148) rc = g.mx ? (g.t == 4 ? launch_pack(k_pack<true, 4, 1024>, 1024) : launch_pack(k_pack<true, -1, 1024>, 1024))
+    if (n_sb <= kSms) rc = g.mx ? (g.t == 4 ? launch_pack(k_pack<true, 4, 1024>, 1024) : launch_pack(k_pack<true, -1, 1024>, 1024))
                                : (g.t == 4 ? launch_pack(k_pack<false, 4, 1024>, 1024) : launch_pack(k_pack<false, -1, 1024>, 1024));
     else rc = g.mx ? (g.t == 4 ? launch_pack(k_pack<true, 4, 512>, 512) : launch_pack(k_pack<true, -1, 512>, 512))
                    : (g.t == 4 ? launch_pack(k_pack<false, 4, 512>, 512) : launch_pack(k_pack<false, -1, 512>, 512));

@@ -59,7 +59,7 @@ __host__ __device__ inline int kv_code_budget(int kept) { return 8 * kept < 1023
 // CTAs per SM.  The kernel and its merge compute it from the same visible length, so they agree without host involvement.
 __host__ __device__ inline int tc_run_tokens(int visible, int heads_x_seqs) {
     int t = 64;
-    while (t < 2048 && ceil_div(visible, t) * heads_x_seqs > 592) t *= 2;
+    while (t < 2048 && ceil_div(visible, t) * heads_x_seqs > 4 * kSms) t *= 2;
     return t;
 }
 __host__ __device__ __forceinline__ KvComp of_seq(const KvComp& c, int b, size_t seq_stride) {

@@ -181,7 +181,7 @@ __global__ void k_verify_gemm_finish(const float* __restrict__ partial, int rows
 // needs a few CTAs more than the 296 that run at once pays a second, nearly empty wave for them (320 CTAs for the
 // 4096 x 4096 matrix: 12.5 us; 256: see the microbenchmark summary), so such a plan gives up ranges until it fits.
 static void split_plan(int n, int k, int* kb_total, int* kb_per_split, int* n_split) {
-    constexpr int kSlots = 296;
+    constexpr int kSlots = 2 * kSms;
     const int tiles = ceil_div(n, kTcBM);
     *kb_total = ceil_div(k, kTcBK);
     int want = ceil_div(kSlots, tiles);
