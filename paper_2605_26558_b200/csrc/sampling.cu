@@ -24,10 +24,11 @@ __device__ __forceinline__ float block_reduce(float v, bool is_max, float* s_red
     return r;
 }
 
-// probs[r][v] = exp((logits[r][v] - max) / T) / sum.  A cluster of CTAs holds a row in registers (NV values a thread), so
-// that it is read and written once and only the two reductions cross CTAs, through distributed shared memory.
-// Bound: latency (one round trip to memory, two cluster barriers); one CTA a row was 501 dependent rounds over a
-// vocabulary of 128256, 200 us.
+// probs[r][v] = exp((logits[r][v] - max) / T) / sum.  A cluster of CTAs holds a row (NV values a thread, in registers up to 16; of
+// 32 and 40, which vocabularies of 128256 and 152064 take, the compiler spills 27 and 52: two CTAs
+// an SM leave 64 registers a thread), so that it is read and written once and only the two reductions cross CTAs, through distributed shared
+// memory.  Bound: latency (one round trip to memory, two cluster barriers): 13.5 us for 20 rows of 128256, 18.2 for 20 of 152064;
+// one CTA a row was 501 dependent rounds over a vocabulary of 128256, 200 us.
 constexpr int kSoftmaxThreads = 512;
 
 template <int NV>
@@ -109,7 +110,8 @@ __global__ void __launch_bounds__(1024) k_softmax_rows_long(const float* __restr
 // A CTA brings its segments into shared memory with contiguous reads first (segments an odd number of floats apart: the
 // summing threads then never share a bank).  Returns the index to every thread (vocab - 1 when the total is not positive).
 // Bound: the chain of additions (`per` of a segment, then the 256 sums); reading each segment from global memory as it was
-// summed took a dependent round trip for every few values, 350 us over a vocabulary of 128256.
+// summed took a dependent round trip for every few values, 350 us over a vocabulary of 128256; four draws now take 12.7 us, an
+// acceptance of four sequences 14.1.
 // The kernel arrives at the cluster's barrier when it starts (barrier_arrive), and the first draw waits for it here before it
 // stores into rank 0's memory: a CTA's shared memory may be touched only once that CTA is known to run.
 struct DrawShared {

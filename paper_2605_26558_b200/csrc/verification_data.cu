@@ -128,7 +128,11 @@ __global__ void __launch_bounds__(32 * kSplitWarps) k_split(const uint32_t* __re
 // and filling the gaps in a second pass over the output took 255 us for a 6144 x 4096 matrix; four warps for the second step
 // of one chunk, three of them waiting for the first, 145 us; this, 131 us.
 constexpr int kJoinWarps = 4;
-constexpr int kJoinCap = 168;                                           // values of a row in hand; longer chunks take several turns
+// Values of a row in hand: the most with five CTAs an SM, and what a chunk of 256 columns holds from 40 % pruning on.  Longer chunks
+// take a second turn over every row for their last few values: 113 us for 6144 x 4096 at 40 %, 219 at 35 %, 215 at 30 %.  With room
+// for 184 values and four CTAs it was 113, 116 and 165, but 250 instead of 221 for 4096 x 14336 at 40 % and 440 instead of 379 for
+// 28672 x 4096.
+constexpr int kJoinCap = 168;
 constexpr int kJoinStride = kJoinCap + 2;                               // halfwords: an odd number of words, rows in different banks
 constexpr int kJoinSpan = 5;                                            // pairs of bitmap words (64 columns) of a row at a time
 static_assert(kJoinCap % 8 == 0 && (kJoinStride / 2) % 2 == 1, "groups of 8; odd row stride in words");
@@ -369,7 +373,7 @@ extern "C" int cass_decode_full(const void* blob, const cass_blob_info* bi, cons
     const JoinGeom jg{bi->rows, bi->cols, ceil_div(bi->cols, 32) * 32, bi->trunc_bits, bi->seg_cols, bi->n_seg, n_ch,
                       bi->n_rowblocks * bi->n_seg * n_ch, vdata_lo_words(bi->kept_per_row, bi->trunc_bits),
                       vdata_row_words(bi->cols, bi->kept_per_row, bi->trunc_bits), bi->cols - bi->kept_per_row};
-    // below about half of the 2960 warps that run at once, teams: 24 instead of 46 us for 986 x 1289 (186 chunks), 54 instead of
+    // below about half of the 20 kSms = 2960 warps that run at once, teams: 24 instead of 46 us for 986 x 1289 (186 chunks), 54 instead of
     // 62 for 4096 x 2048 (1024 chunks), but 99 instead of 76 for 4096 x 4096 (2048)
     const bool team = jg.n_tasks < 1536;
 #define CASS_JOIN(T_)                                                                                                               \
