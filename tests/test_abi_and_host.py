@@ -150,5 +150,5 @@ def test_launch_count_formula():
     # the count depends neither on the cache length nor on the KV format
     assert bench.launches_per_step(32, 4, max_seq=4096) == bench.launches_per_step(32, 4)
     assert bench.launches_per_step(32, 4, kv_mode=2) == bench.launches_per_step(32, 4)
-    # verification from the two parts: two reconstruction launches per matrix
-    assert bench.launches_per_step(2, 1, from_parts=True) - bench.launches_per_step(2, 1) == 2 * (2 * 4 + 1)
+    # verification from the two parts: one reconstruction launch per matrix
+    assert bench.launches_per_step(2, 1, from_parts=True) - bench.launches_per_step(2, 1) == 2 * 4 + 1
