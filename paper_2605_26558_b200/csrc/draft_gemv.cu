@@ -139,9 +139,9 @@ __device__ __forceinline__ uint32_t lds_u32_off(uint32_t addr) {
 // A group whose 8 kept columns span more than 32 columns (wide: four of them), or four of whose codewords take more than 32
 // bits, shows up as a window that ran dry (nothing left to find); that lane then redoes the group with the careful walk while
 // the others wait.
-// Bound: about 16 warp instructions a kept value and lane, of which 7 on the integer pipe (one every other cycle), two bit
-// searches (one every 8 cycles) and 3 shared-memory loads (the gather of x meets a bank two to three times): issue slots 76 %,
-// shared memory 61 %, integer pipe 58 %, searches 55 % busy.  Clearing the used bit with a shift and a mask, positions kept
+// Bound: 17.5 warp instructions a kept value and lane with the kernel around them, of which 7 on the integer pipe (one every other
+// cycle), two bit searches (one every 8 cycles) and 3 shared-memory loads (the gather of x meets a bank two to three times): issue
+// slots 73 %, searches 70 %, shared memory 64 %, integer pipe 55 % busy.  Clearing the used bit with a shift and a mask, positions kept
 // absolute and a code window for every 4 values took 19: 58.6 -> 53.0 us on 28672 x 4096 with the results added in the kernel.
 // Finding some terminators by a conversion to float instead of a search: 54.5 to 56 us.
 template <int T, int NB, bool WIDE>
