@@ -74,10 +74,11 @@ __global__ void __launch_bounds__(32 * kKvWarps) k_kv_append(KvGeom g, KvComp ck
     const int nj = FUSED ? NJ : g.d / 32;
     const bool coded = (flags & CASS_KV_COMPRESSED) != 0;
     auto code_lengths = [&]() {
-        if (coded && (!FUSED || head < g.n_kv)) s_len[threadIdx.x] = of_seq((kind ? cv : ck).exp_to_rank, seq, g.seq_stride)[threadIdx.x] + 1u;
+        if (coded && g.mode == 1 && (!FUSED || head < g.n_kv)) s_len[threadIdx.x] = of_seq((kind ? cv : ck).exp_to_rank, seq, g.seq_stride)[threadIdx.x] + 1u;
     };
     // FUSED: the predecessor is a projection, and the codebook tables were written before that: read ahead of the wait, they cost
-    // no time.  A stand-alone append may follow their writer (k_kv_rank ends a codebook of no tokens).
+    // no time.  A stand-alone append may follow their writer (k_kv_rank ends a codebook of no tokens).  Cassandra-2 records have no
+    // codes, and what is looked up for them is not used.
     if (FUSED) code_lengths();
     pdl_wait();
     pdl_early<1>();
