@@ -58,7 +58,8 @@ constexpr int kMaxBatch = 8;               // sequences per session
 constexpr int kMaxRows = 64;               // rows of all sequences in one call
 constexpr int kSms = 148;                  // of a B200: what grids and the rules between kernels are sized by
 constexpr size_t kSmemPerBlock = 227 * 1024;      // shared memory a CTA may have, its own arrays included
-constexpr int kPrefillRows = 256;          // rows of all sequences in one pass of a prefill
+constexpr int kSplitRows = 256;            // most rows of the split-K projection
+constexpr int kPrefillRows = 1024;         // most rows of all sequences in one pass of a prefill; a session of fewer positions has room for those
 
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 __host__ __device__ inline size_t align_up(size_t a, size_t b) { return (a + b - 1) / b * b; }

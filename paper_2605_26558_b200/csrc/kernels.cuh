@@ -240,10 +240,17 @@ int launch_attn_merge(const AttnScratch& sc, int chunk_tokens, int n_seq, const 
 inline int verify_gemm_bn(int rows) { return rows <= 16 ? 16 : rows <= 32 ? 32 : rows <= 64 ? 64 : rows <= 128 ? 128 : 256; }
 size_t verify_gemm_partial_floats(int n, int k, int bn);
 Partials verify_gemm_partials(const float* partial, int n, int k, int bn);
+void verify_gemm_split(int n, int k, int* kb_total, int* kb_per_split, int* n_split);      // its K ranges, in blocks of 64
 // w_static: kWeightsStatic: W is not the output of a kernel that may still be running when this one is scheduled (the bf16
 // matrices of a session); its first tiles are then requested before the wait for the predecessor.
 enum { kWeightsRebuilt = 0, kWeightsStatic = 1, kWeightsInput = 2 };
 int launch_verify_gemm(const uint16_t* W, const uint16_t* X, int rows, int bn, int n, int k, float* partial, uint16_t* y_bf16,
                        float* y_f32, int32_t* d_status, cudaStream_t s, int w_static = kWeightsRebuilt);
+
+// Many rows (wide_gemm.cu): out[r][i] = bf16 of the same sums, without parts.  X: a buffer of x_rows rows.  wide_gemm_pays: whether a
+// call should take it, which above kSplitRows rows it has to.
+bool wide_gemm_pays(int rows, int n, int k);
+int launch_wide_gemm(const uint16_t* W, const uint16_t* X, int x_rows, int rows, int n, int k, uint16_t* out, int32_t* d_status, cudaStream_t s,
+                     int w_static);
 
 }  // namespace cass

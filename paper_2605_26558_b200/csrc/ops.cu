@@ -126,6 +126,11 @@ __global__ void __launch_bounds__(1024) k_residual_rmsnorm(uint16_t* __restrict_
     }
 }
 
+__device__ __forceinline__ void unpack4(uint2 v, float (&x)[4]) {
+    x[0] = __uint_as_float(v.x << 16); x[1] = __uint_as_float(v.x & 0xFFFF0000u);
+    x[2] = __uint_as_float(v.y << 16); x[3] = __uint_as_float(v.y & 0xFFFF0000u);
+}
+
 // Four rotated pairs, or eight plain v elements, a thread (head sizes are multiples of 32): 16-byte loads of the parts.
 __global__ void __launch_bounds__(128) k_qkv_rope(uint16_t* __restrict__ qkv, Partials pp,
                                                   const float* __restrict__ cos_t, const float* __restrict__ sin_t,
@@ -146,8 +151,8 @@ __global__ void __launch_bounds__(128) k_qkv_rope(uint16_t* __restrict__ qkv, Pa
             x[0] = round_bf16(s.x); x[1] = round_bf16(s.y); x[2] = round_bf16(s.z); x[3] = round_bf16(s.w);
             y[0] = round_bf16(t.x); y[1] = round_bf16(t.y); y[2] = round_bf16(t.z); y[3] = round_bf16(t.w);
         } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) { x[q] = bf16_bits_to_float(row[ia + q]); y[q] = bf16_bits_to_float(row[ib + q]); }
+            unpack4(*reinterpret_cast<const uint2*>(row + ia), x);
+            unpack4(*reinterpret_cast<const uint2*>(row + ib), y);
         }
     };
     auto store4 = [&](int i, const float (&x)[4]) {
@@ -192,11 +197,8 @@ __global__ void __launch_bounds__(128) k_swiglu(const uint16_t* __restrict__ gu,
             g[0] = round_bf16(gs.x); g[1] = round_bf16(gs.y); g[2] = round_bf16(gs.z); g[3] = round_bf16(gs.w);
             u[0] = round_bf16(us.x); u[1] = round_bf16(us.y); u[2] = round_bf16(us.z); u[3] = round_bf16(us.w);
         } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                g[q] = bf16_bits_to_float(gu[(size_t)r * 2 * ffn + i + q]);
-                u[q] = bf16_bits_to_float(gu[(size_t)r * 2 * ffn + ffn + i + q]);
-            }
+            unpack4(*reinterpret_cast<const uint2*>(gu + (size_t)r * 2 * ffn + i), g);
+            unpack4(*reinterpret_cast<const uint2*>(gu + (size_t)r * 2 * ffn + ffn + i), u);
         }
         uint32_t o[4];
 #pragma unroll

@@ -38,7 +38,9 @@ struct Session {
     int B, R;                // sequences; row capacity of one call (16, 32 or 64 = token columns of the verification MMA)
     // activations (R rows)
     uint16_t *h, *xn, *qkv, *attn, *y, *gu, *act;
-    uint16_t *ph, *pxn, *pqkv, *pattn, *pact;      // the same of a prefill pass (kPrefillRows rows)
+    uint16_t *ph, *pxn, *pqkv, *pattn, *pact;      // the same of a prefill pass (W rows)
+    uint16_t* pproj;                               // its projections' results, before the kernels that consume them
+    int W;
     float *logits, *partial, *vg_partial;
     size_t partial_floats;
     AttnScratch asc;
@@ -131,12 +133,17 @@ static size_t layout(Session* s, uint8_t* base) {
     s->y = (uint16_t*)at(p.take((size_t)R * d.hidden * 2));
     s->gu = (uint16_t*)at(p.take((size_t)R * 2 * d.ffn * 2));
     s->act = (uint16_t*)at(p.take((size_t)R * d.ffn * 2));
-    const size_t W = kPrefillRows;
+    {   // rows of a prefill pass: a multiple of 16 for each of up to 8 sequences
+        const size_t all = align_up((size_t)s->B * d.max_seq, 256);
+        s->W = all < (size_t)kPrefillRows ? (int)all : kPrefillRows;
+    }
+    const size_t W = s->W;
     s->ph = (uint16_t*)at(p.take(W * d.hidden * 2));
     s->pxn = (uint16_t*)at(p.take(W * d.hidden * 2));
     s->pqkv = (uint16_t*)at(p.take(W * s->qkv_dim * 2));
     s->pattn = (uint16_t*)at(p.take(W * d.n_q_heads * d.head_dim * 2));
     s->pact = (uint16_t*)at(p.take(W * d.ffn * 2));
+    s->pproj = (uint16_t*)at(p.take(W * (size_t)(2 * d.ffn > d.hidden ? 2 * d.ffn : d.hidden) * 2));
     s->logits = (float*)at(p.take((size_t)R * d.vocab * 4));
     // split-K partials of the draft GEMVs: segments x padded rows
     size_t pf = 0;
@@ -149,8 +156,8 @@ static size_t layout(Session* s, uint8_t* base) {
     s->partial_floats = pf;                                   // per vector of a draft GEMV
     s->partial = (float*)at(p.take(pf * 4 * s->B));
     {   // split-K scratch of the verification GEMMs
-        size_t c[5] = {verify_gemm_partial_floats(s->qkv_dim, d.hidden, kPrefillRows), verify_gemm_partial_floats(d.hidden, d.n_q_heads * d.head_dim, kPrefillRows),
-                       verify_gemm_partial_floats(2 * d.ffn, d.hidden, kPrefillRows), verify_gemm_partial_floats(d.hidden, d.ffn, kPrefillRows),
+        size_t c[5] = {verify_gemm_partial_floats(s->qkv_dim, d.hidden, kSplitRows), verify_gemm_partial_floats(d.hidden, d.n_q_heads * d.head_dim, kSplitRows),
+                       verify_gemm_partial_floats(2 * d.ffn, d.hidden, kSplitRows), verify_gemm_partial_floats(d.hidden, d.ffn, kSplitRows),
                        verify_gemm_partial_floats(d.vocab, d.hidden, R)};
         size_t m = 0;
         for (size_t v : c) if (v > m) m = v;
@@ -159,7 +166,7 @@ static size_t layout(Session* s, uint8_t* base) {
     // attention scratch: what the rows of one verification call can need and, up to 64 MB, those of a prefill pass
     const int n_chunks = ceil_div(d.max_seq, kAttnChunk);
     size_t parts = (size_t)R * d.n_q_heads * n_chunks;
-    size_t wide = (size_t)kPrefillRows * d.n_q_heads * ceil_div(n_chunks, 2);
+    size_t wide = W * d.n_q_heads * ceil_div(n_chunks, 2);
     if (wide > ((size_t)16 << 20) / d.head_dim) wide = ((size_t)16 << 20) / d.head_dim;
     if (wide > parts) parts = wide;
     s->attn_parts = parts;
@@ -538,9 +545,9 @@ static int prefill_attention(Session* s, const LayerDev& L, int pos, int w, int 
     return CASS_OK;
 }
 
-// The prompt in passes of kPrefillRows rows over all sequences: every pass reads the weights once for its rows (16 rows a
-// pass, as verification takes them, read them 16 times as often: 51.8 ms instead of 4.3 ms, and 128 rows a pass 5.5 ms, for 1000 tokens of four
-// 8B-shaped layers), and lm_head runs once.  A row's projections are what cass_verify gives for it: the same K ranges, added in
+// The prompt in passes of up to kPrefillRows rows over all sequences: every pass reads the weights once for its rows (16 rows a
+// pass, as verification takes them, read them 16 times as often: 51.8 ms for 1000 tokens of four 8B-shaped layers, 4.3 ms with
+// passes of 256 rows), and lm_head runs once.  A row's projections are what cass_verify gives for it: the same K ranges, added in
 // the same order.  So is its attention, except where cass_verify takes 16 rows to the fp32 pipes (head size 128, more than four query
 // heads a KV head): those rows stay on the tensor cores here, as accurate but in another order of additions.
 extern "C" int cass_prefill(void* session, const int32_t* toks, int n, int32_t* target_argmax, void* stream_) {
@@ -551,7 +558,7 @@ extern "C" int cass_prefill(void* session, const int32_t* toks, int n, int32_t* 
     if (n < 1 || n + kMaxVerifyRows > d.max_seq) return CASS_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream_;
     int32_t* status = &s->st->status;
-    const int w_max = kPrefillRows / B, chunk = kMaxVerifyRows < s->R / B ? kMaxVerifyRows : s->R / B;
+    const int w_max = s->W / B, chunk = kMaxVerifyRows < s->R / B ? kMaxVerifyRows : s->R / B;
     // rows that calls of `chunk` rows would give to the fp32-pipe attention keep its accuracy
     auto tc_rows = [&](int rps) { return verify_attn_tc_usable(s->kg, rps <= d.gamma_max + 1 ? d.gamma_max + 1 : rps, d.n_q_heads); };
     const int rest = n % chunk;
@@ -566,31 +573,40 @@ extern "C" int cass_prefill(void* session, const int32_t* toks, int n, int32_t* 
         return s->vscratch;
     };
     const int w_static = s->from_parts ? 0 : 1;
+    // passes of about the same size (a multiple of 16 rows a sequence, so that a pass begins where a call of `chunk` rows would)
+    const int w_each = (int)align_up(ceil_div(n, ceil_div(n, w_max)), 16);
     int w = 0;
     for (int pos = 0; pos < n; pos += w) {
-        w = n - pos < w_max ? n - pos : w_max;
+        w = n - pos < w_each ? n - pos : w_each;
         const int rows = B * w, bn = verify_gemm_bn(rows);
-        auto parts = [&](int nn, int k) { return verify_gemm_partials(s->vg_partial, nn, k, bn); };
+        // a projection's results: bf16 at `out`, or parts that the next kernel adds
+        auto project = [&](const uint16_t* W, const uint16_t* X, int nn, int k, uint16_t* out, Partials* pp) {
+            const bool wide = wide_gemm_pays(rows, nn, k);
+            *pp = wide ? Partials{nullptr, 0, 0, 0} : verify_gemm_partials(s->vg_partial, nn, k, bn);
+            return wide ? launch_wide_gemm(W, X, s->W, rows, nn, k, out, status, st, w_static)
+                        : launch_verify_gemm(W, X, rows, bn, nn, k, s->vg_partial, nullptr, nullptr, status, st, w_static);
+        };
+        Partials pp;
         RC(launch_set_len(s->st, pos, st));
         RC(launch_embed(toks + pos, w, n, (const uint16_t*)s->embed, s->ph, rows, d.hidden, st));
         RC(launch_rmsnorm(s->ph, (const uint16_t*)s->layers[0].w.norm_attn, s->pxn, rows, d.hidden, d.rms_eps, st));
         for (int l = 0; l < d.n_layers; ++l) {
             LayerDev& L = s->layers[l];
             if (calib) RC(launch_calib_accum(s->pxn, rows, d.hidden, L.calib[0], s->st, st));
-            RC(launch_verify_gemm(weight(L.w.wqkv, L.blob[0], L.bi[0], L.vdata[0]), s->pxn, rows, bn, s->qkv_dim, d.hidden, s->vg_partial, nullptr, nullptr, status, st, w_static));
-            RC(launch_qkv_rope(s->pqkv, parts(s->qkv_dim, d.hidden), s->cos_t, s->sin_t, s->st, 0, rows, w, d.n_q_heads, d.n_kv_heads, d.head_dim, st));
+            RC(project(weight(L.w.wqkv, L.blob[0], L.bi[0], L.vdata[0]), s->pxn, s->qkv_dim, d.hidden, s->pqkv, &pp));
+            RC(launch_qkv_rope(s->pqkv, pp, s->cos_t, s->sin_t, s->st, 0, rows, w, d.n_q_heads, d.n_kv_heads, d.head_dim, st));
             RC(launch_kv_span(s->kg, L.ck, L.cv, L.kc, L.vc, s->pqkv + qd, s->pqkv + qd + kvd, s->qkv_dim, pos, w, kv_flags, s->st, 0, B, st));
             RC(prefill_attention(s, L, pos, w, fine - pos, st));
             if (calib) RC(launch_calib_accum(s->pattn, rows, qd, L.calib[1], s->st, st));
-            RC(launch_verify_gemm(weight(L.w.wo, L.blob[1], L.bi[1], L.vdata[1]), s->pattn, rows, bn, d.hidden, qd, s->vg_partial, nullptr, nullptr, status, st, w_static));
-            RC(launch_residual_rmsnorm(s->ph, nullptr, parts(d.hidden, qd), (const uint16_t*)L.w.norm_ffn, s->pxn, rows, d.hidden, d.rms_eps, st));
+            RC(project(weight(L.w.wo, L.blob[1], L.bi[1], L.vdata[1]), s->pattn, d.hidden, qd, s->pproj, &pp));
+            RC(launch_residual_rmsnorm(s->ph, s->pproj, pp, (const uint16_t*)L.w.norm_ffn, s->pxn, rows, d.hidden, d.rms_eps, st));
             if (calib) RC(launch_calib_accum(s->pxn, rows, d.hidden, L.calib[2], s->st, st));
-            RC(launch_verify_gemm(weight(L.w.wgu, L.blob[2], L.bi[2], L.vdata[2]), s->pxn, rows, bn, 2 * d.ffn, d.hidden, s->vg_partial, nullptr, nullptr, status, st, w_static));
-            RC(launch_swiglu(nullptr, parts(2 * d.ffn, d.hidden), s->pact, rows, d.ffn, st));
+            RC(project(weight(L.w.wgu, L.blob[2], L.bi[2], L.vdata[2]), s->pxn, 2 * d.ffn, d.hidden, s->pproj, &pp));
+            RC(launch_swiglu(s->pproj, pp, s->pact, rows, d.ffn, st));
             if (calib) RC(launch_calib_accum(s->pact, rows, d.ffn, L.calib[3], s->st, st));
-            RC(launch_verify_gemm(weight(L.w.wd, L.blob[3], L.bi[3], L.vdata[3]), s->pact, rows, bn, d.hidden, d.ffn, s->vg_partial, nullptr, nullptr, status, st, w_static));
+            RC(project(weight(L.w.wd, L.blob[3], L.bi[3], L.vdata[3]), s->pact, d.hidden, d.ffn, s->pproj, &pp));
             const uint16_t* next_gain = (const uint16_t*)(l + 1 < d.n_layers ? s->layers[l + 1].w.norm_attn : s->norm_final);
-            RC(launch_residual_rmsnorm(s->ph, nullptr, parts(d.hidden, d.ffn), next_gain, s->pxn, rows, d.hidden, d.rms_eps, st));
+            RC(launch_residual_rmsnorm(s->ph, s->pproj, pp, next_gain, s->pxn, rows, d.hidden, d.rms_eps, st));
         }
         if (calib) RC(launch_calib_accum(s->pxn, rows, d.hidden, s->calib_lm, s->st, st));
     }

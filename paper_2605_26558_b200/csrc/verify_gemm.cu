@@ -22,20 +22,6 @@ constexpr int tc_b_bytes(int bn) { return bn * kTcBK * 2; }
 constexpr int tc_smem(int bn) { return tc_stages(bn) * (kTcABytes + tc_b_bytes(bn)) + 256 + 1024; }     // + barriers + alignment slack
 constexpr int tc_tmem_cols(int bn) { return bn <= 32 ? 32 : bn; }                                   // a power of two >= 32
 
-// bf16 matrix [rows][cols] row-major -> map with a (box_rows x 64)-element box, 128-byte swizzle, zero fill outside.
-static int make_map(CUtensorMap* m, const void* ptr, int rows, int cols, int box_rows) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return CASS_ERR_CUDA;
-    cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t gstride[1] = {(cuuint64_t)cols * 2};
-    cuuint32_t box[2] = {(cuuint32_t)kTcBK, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), gdim, gstride, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? CASS_OK : CASS_ERR_INVALID_ARG;
-}
-
 // Instruction descriptor of kind::f16: D fp32, A and B bf16, both K-major, M = 128, N = bn.
 constexpr uint32_t tc_idesc(int bn) { return tc_idesc_mn(kTcBM, bn, false); }
 
@@ -142,12 +128,7 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
 #pragma unroll
             for (int c0 = 0; c0 < BN; c0 += 16) {          // 16 accumulator columns (token rows) at a time
                 uint32_t v[16];
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-                      "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                    : "r"(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
                 if (feat < n && nkb > 0) {
 #pragma unroll
                     for (int r = 0; r < 16; ++r)
@@ -180,7 +161,7 @@ __global__ void k_verify_gemm_finish(const float* __restrict__ partial, int rows
 // K ranges: a function of (n, k) only.  Enough CTAs for about two per SM, at least 4 k-blocks per range.  A plan that
 // needs a few CTAs more than the 296 that run at once pays a second, nearly empty wave for them (320 CTAs for the
 // 4096 x 4096 matrix: 12.5 us; 256: see the microbenchmark summary), so such a plan gives up ranges until it fits.
-static void split_plan(int n, int k, int* kb_total, int* kb_per_split, int* n_split) {
+void verify_gemm_split(int n, int k, int* kb_total, int* kb_per_split, int* n_split) {
     constexpr int kSlots = 2 * kSms;
     const int tiles = ceil_div(n, kTcBM);
     *kb_total = ceil_div(k, kTcBK);
@@ -201,13 +182,13 @@ static void split_plan(int n, int k, int* kb_total, int* kb_per_split, int* n_sp
 
 Partials verify_gemm_partials(const float* partial, int n, int k, int bn) {
     int kbt, kbs, ns;
-    split_plan(n, k, &kbt, &kbs, &ns);
+    verify_gemm_split(n, k, &kbt, &kbs, &ns);
     return Partials{partial, ns, (size_t)bn * n, (size_t)n};
 }
 
 size_t verify_gemm_partial_floats(int n, int k, int bn) {
     int kbt, kbs, ns;
-    split_plan(n, k, &kbt, &kbs, &ns);
+    verify_gemm_split(n, k, &kbt, &kbs, &ns);
     return (size_t)ns * bn * n;
 }
 
@@ -226,12 +207,12 @@ int launch_verify_gemm(const uint16_t* W, const uint16_t* X, int rows, int bn, i
         return CASS_ERR_INVALID_ARG;
     if (((uintptr_t)W & 15) || ((uintptr_t)X & 15)) return CASS_ERR_INVALID_ARG;
     CUtensorMap mw, mx;
-    int rc = make_map(&mw, W, n, k, kTcBM);
+    int rc = tc_matrix_map(&mw, W, n, k, kTcBM);
     if (rc) return rc;
-    rc = make_map(&mx, X, bn, k, bn);      // the activation buffer always has bn rows
+    rc = tc_matrix_map(&mx, X, bn, k, bn);      // the activation buffer always has bn rows
     if (rc) return rc;
     int kbt, kbs, ns;
-    split_plan(n, k, &kbt, &kbs, &ns);
+    verify_gemm_split(n, k, &kbt, &kbs, &ns);
     if (bn == 16) rc = launch_tc<16>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
     else if (bn == 32) rc = launch_tc<32>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);
     else if (bn == 256) rc = launch_tc<256>(mw, mx, partial, rows, n, kbt, kbs, ns, d_status, w_static, s);

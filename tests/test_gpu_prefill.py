@@ -107,6 +107,27 @@ def test_long_prompts_equal_verification_calls(cass, heads, kv, d):
     b.close()
 
 
+@pytest.mark.parametrize("batch,n", [(1, 33), (1, 127), (1, 128), (1, 192), (1, 193), (1, 257), (1, 385), (1, 1024), (1, 1030), (2, 520), (4, 259)])
+def test_wide_projections_equal_verification_calls(cass, batch, n):
+    """Edges of the wide projection's tiles (128, 192 and 256 rows, 256 features), several K ranges a tile with a block left over,
+    K and features off the tiles' multiples, one pass more than its rows hold."""
+    shape = synth.ModelShape(n_layers=1, hidden=1288, n_q_heads=4, n_kv_heads=2, head_dim=64, ffn=1032, vocab=512)
+    wt = synth.model_weights(shape, 4, device="cuda")
+    gw = {"layers": [cass.engine.fuse_layer_weights(lw) for lw in wt["layers"]], "embed": wt["embed"], "lm_head": wt["lm_head"],
+          "norm_final": wt["norm_final"]}
+    prompt = torch.stack([synth.random_prompt(n, shape.vocab, 50 + b) for b in range(batch)])
+    a, b = (cass.engine.Engine(shape, gw, max_seq=1056, gamma_max=4, batch=batch) for _ in range(2))
+    first = a.prefill(prompt)
+    want, rows = _chunked(cass, b, prompt)
+    assert ([first] if batch == 1 else first) == want
+    assert a.status()[0] == b.status()[0] == 0
+    assert all(torch.equal(x, y) for x, y in zip(_cache(cass, a, n), _cache(cass, b, n)))
+    for w in (0, 1, 2):
+        assert torch.equal(_activation(cass, a, w, batch * rows), _activation(cass, b, w, batch * rows)), w
+    a.close()
+    b.close()
+
+
 def test_two_bf16_terms_are_as_accurate_as_the_fp32_pipes(cass):
     """Five query heads a KV head at head size 128: verification takes 16 rows to the fp32 pipes, the wide pass to the tensor
     cores with P in two bf16 terms.  On the same queries and caches both differ from 64 bits by the rounding of the output alone
