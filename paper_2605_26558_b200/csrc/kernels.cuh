@@ -229,6 +229,13 @@ bool verify_attn_tc_usable(const KvGeom& g, int rps, int n_q);
 int launch_verify_attn_tc(const KvGeom& g, const uint16_t* k_cache, const uint16_t* v_cache, const uint16_t* qkv, int n_seq,
                           const AttnRows& ar, int fine, int n_q, int np_cols, const DevState* st, const AttnScratch& sc, uint16_t* out,
                           int32_t* d_status, cudaStream_t s);
+// All rps rows of a prefill pass at positions pos .. pos + rps - 1 at once, no merge (prefill_attn.cu): head_dim 128 and up to 256 chunks
+// of 128 positions.  sc.m and sc.l hold prefill_attn_stats numbers each, sc.o (beyond 8 chunks) 128 for every 128 (row, head) pairs.
+constexpr int kPrefillChunk = 128;
+bool prefill_attn_usable(const KvGeom& g, int n_q);
+size_t prefill_attn_stats(const KvGeom& g, int n_q, int n_seq, int rps, int positions);
+int launch_prefill_attn(const KvGeom& g, const uint16_t* k_cache, const uint16_t* v_cache, const uint16_t* qkv, int n_seq, int rps, int pos, int fine,
+                        int n_q, const DevState* st, const AttnScratch& sc, uint16_t* out, int32_t* d_status, cudaStream_t s);
 // Combines the partial results of rows lo .. hi - 1 (draft attention: ar.rps = 1, draft_units < 0, see draft_attn.cu).
 int launch_attn_merge(const AttnScratch& sc, int chunk_tokens, int n_seq, const AttnRows& ar, int n_q, int d, const DevState* st,
                       int draft_mode, int draft_units, uint16_t* out, cudaStream_t s);

@@ -168,11 +168,17 @@ static size_t layout(Session* s, uint8_t* base) {
     size_t parts = (size_t)R * d.n_q_heads * n_chunks;
     size_t wide = W * d.n_q_heads * ceil_div(n_chunks, 2);
     if (wide > ((size_t)16 << 20) / d.head_dim) wide = ((size_t)16 << 20) / d.head_dim;
+    size_t stats = 0;
+    if (prefill_attn_usable(g, d.n_q_heads)) {         // its passes leave statistics and, for long prompts, one output a pair
+        wide = prefill_attn_stats(g, d.n_q_heads, s->B, W / s->B, kPrefillChunk);
+        stats = prefill_attn_stats(g, d.n_q_heads, s->B, W / s->B, d.max_seq);
+    }
     if (wide > parts) parts = wide;
+    if (parts > stats) stats = parts;
     s->attn_parts = parts;
     s->asc.o = (float*)at(p.take(parts * d.head_dim * 4));
-    s->asc.m = (float*)at(p.take(parts * 4));
-    s->asc.l = (float*)at(p.take(parts * 4));
+    s->asc.m = (float*)at(p.take(stats * 4));
+    s->asc.l = (float*)at(p.take(stats * 4));
     s->argmax_tmp = (int32_t*)at(p.take((size_t)R * 128 * 4));
     s->argmax_val = (float*)at(p.take((size_t)R * 128 * 4));
     s->layers.resize(d.n_layers);
@@ -528,6 +534,8 @@ extern "C" int cass_verify(void* session, const int32_t* toks, int g, int32_t* t
 static int prefill_attention(Session* s, const LayerDev& L, int pos, int w, int fine, cudaStream_t st) {
     const cass_model_desc& d = s->d;
     const bool tc = !simt_verify_attn() && verify_attn_tc_usable(s->kg, 1, d.n_q_heads);
+    if (tc && prefill_attn_usable(s->kg, d.n_q_heads))
+        return launch_prefill_attn(s->kg, L.kc, L.vc, s->pqkv, s->B, w, pos, fine, d.n_q_heads, s->st, s->asc, s->pattn, &s->st->status, st);
     const int tok = tc ? 2 * kAttnChunk : kAttnChunk, grp = d.n_q_heads / d.n_kv_heads;
     // rows a CTA: what 64 pair columns hold, 16 at most (more would leave the long passes of few heads without CTAs)
     int group = 16;

@@ -3,7 +3,7 @@
 
 #include <cuda.h>
 
-#include "common.cuh"
+#include "kernels.cuh"
 
 namespace cass {
 
@@ -39,6 +39,19 @@ inline int tc_matrix_map(CUtensorMap* m, const void* ptr, int rows, int cols, in
     return r == CUDA_SUCCESS ? CASS_OK : CASS_ERR_INVALID_ARG;
 }
 
+// Sequence 0's bf16 K or V cache of one layer ([max_seq][n_kv][128]; the other sequences lie seq_stride bytes apart) -> map over
+// [dim, position, sequence] with a box of 64 dims x 128 positions.
+inline int tc_cache_map(CUtensorMap* m, const KvGeom& g, const uint16_t* cache, int n_seq) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return CASS_ERR_CUDA;
+    const cuuint64_t gdim[3] = {(cuuint64_t)g.n_kv * g.d, (cuuint64_t)g.max_seq, (cuuint64_t)n_seq};
+    const cuuint64_t gstride[2] = {(cuuint64_t)g.n_kv * g.d * 2, (cuuint64_t)(n_seq > 1 ? g.seq_stride : (size_t)g.max_seq * g.n_kv * g.d * 2)};
+    const cuuint32_t box[3] = {64, 128, 1}, estr[3] = {1, 1, 1};
+    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<uint16_t*>(cache), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? CASS_OK : CASS_ERR_INVALID_ARG;
+}
+
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
                      smem_u32(smem_dst)),
@@ -56,6 +69,11 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m
                  : "memory");
 }
 
+__device__ __forceinline__ bool tc_elect() {                                  // one lane of a converged warp
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 

@@ -230,25 +230,15 @@ bool verify_attn_tc_usable(const KvGeom& g, int rps, int n_q) {
     return g.d == kVtD && rps * (n_q / g.n_kv) <= kVtMaxPairs && (g.seq_stride % 16) == 0;
 }
 
-// caches: sequence 0's bf16 K and V of one layer ([max_seq][n_kv][128]); the other sequences lie seq_stride bytes apart.
 int launch_verify_attn_tc(const KvGeom& g, const uint16_t* k_cache, const uint16_t* v_cache, const uint16_t* qkv, int n_seq,
                           const AttnRows& ar, int fine, int n_q, int np_cols, const DevState* st, const AttnScratch& sc, uint16_t* out,
                           int32_t* d_status, cudaStream_t s) {
     if (!verify_attn_tc_usable(g, ar.group, n_q) || (np_cols != 32 && np_cols != 64) || ar.group * (n_q / g.n_kv) > np_cols)
         return CASS_ERR_UNSUPPORTED;
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return CASS_ERR_CUDA;
     CUtensorMap mk, mv;
-    const cuuint64_t gdim[3] = {(cuuint64_t)g.n_kv * g.d, (cuuint64_t)g.max_seq, (cuuint64_t)n_seq};
-    const cuuint64_t gstride[2] = {(cuuint64_t)g.n_kv * g.d * 2, (cuuint64_t)(n_seq > 1 ? g.seq_stride : (size_t)g.max_seq * g.n_kv * g.d * 2)};
-    const cuuint32_t box[3] = {64, (cuuint32_t)kVtTok, 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    for (int i = 0; i < 2; ++i) {
-        CUresult r = fn(i ? &mv : &mk, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<uint16_t*>(i ? v_cache : k_cache), gdim, gstride,
-                        box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return CASS_ERR_INVALID_ARG;
-    }
+    int rc = tc_cache_map(&mk, g, k_cache, n_seq);
+    if (!rc) rc = tc_cache_map(&mv, g, v_cache, n_seq);
+    if (rc) return rc;
     const int n_groups = ceil_div(ar.hi - ar.lo, ar.group);
     dim3 grid(ar.chunks, g.n_kv, n_seq * n_groups);
     if (np_cols == 32) {

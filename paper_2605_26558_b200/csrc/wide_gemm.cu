@@ -38,11 +38,6 @@ __device__ __forceinline__ uint32_t wg_leader_addr(const void* p) {          // 
     asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(p)));
     return r;
 }
-__device__ __forceinline__ bool wg_elect() {                                  // one lane of a converged warp
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-    return p != 0;
-}
 __device__ __forceinline__ void wg_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
@@ -144,15 +139,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kWgThreads, 1)
             }
         }
     };
-    if (warp == 0 && w_static == kWeightsStatic && wg_elect()) produce(true);
+    if (warp == 0 && w_static == kWeightsStatic && tc_elect()) produce(true);
     __syncwarp();
     pdl_wait();
     pdl_early<5>();
 
     if (warp == 0) {
-        if (wg_elect()) produce(false);                                      // this CTA's half of every stage
+        if (tc_elect()) produce(false);                                      // this CTA's half of every stage
     } else if (warp == 1) {
-        if (rank == 0 && wg_elect()) {                                       // the MMAs of both CTAs
+        if (rank == 0 && tc_elect()) {                                       // the MMAs of both CTAs
             int it = 0, rng = 0;
             bool ok = true;
             for (int i = 0; i < my_tiles && ok; ++i)

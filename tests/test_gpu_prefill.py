@@ -128,6 +128,29 @@ def test_wide_projections_equal_verification_calls(cass, batch, n):
     b.close()
 
 
+@pytest.mark.parametrize("heads,kv,batch,n", [(2, 2, 1, 127), (2, 2, 1, 257), (2, 1, 1, 1025), (3, 1, 2, 129), (3, 1, 1, 1190), (4, 1, 4, 300), (8, 1, 1, 300), (7, 1, 1, 1100)])
+def test_prefill_attention_of_every_group(cass, heads, kv, batch, n):
+    """Head size 128: groups that leave lanes of a CTA without a pair, ends of chunks and of CTAs, more than eight chunks (chains of
+    the merge's order).  With more than four query heads a KV head verification takes 16 rows to the fp32 pipes; both round the
+    output to bf16 (2^-9 of it each), and a flipped bit of an activation travels on: 5e-3, as above."""
+    shape = synth.ModelShape(n_layers=1, hidden=256, n_q_heads=heads, n_kv_heads=kv, head_dim=128, ffn=256, vocab=512)
+    wt = synth.model_weights(shape, 5, device="cuda")
+    gw = {"layers": [cass.engine.fuse_layer_weights(lw) for lw in wt["layers"]], "embed": wt["embed"], "lm_head": wt["lm_head"],
+          "norm_final": wt["norm_final"]}
+    prompt = torch.stack([synth.random_prompt(n, shape.vocab, 60 + b) for b in range(batch)])
+    a, b = (cass.engine.Engine(shape, gw, max_seq=1216, gamma_max=4, batch=batch) for _ in range(2))
+    a.prefill(prompt)
+    _, rows = _chunked(cass, b, prompt)
+    assert a.status()[0] == b.status()[0] == 0
+    x, y = (_activation(cass, e, 1, batch * rows) for e in (a, b))
+    if heads // kv <= 4:
+        assert torch.equal(x, y)
+    else:
+        assert (x.float() - y.float()).norm() / y.float().norm() <= 5e-3
+    a.close()
+    b.close()
+
+
 def test_two_bf16_terms_are_as_accurate_as_the_fp32_pipes(cass):
     """Five query heads a KV head at head size 128: verification takes 16 rows to the fp32 pipes, the wide pass to the tensor
     cores with P in two bf16 terms.  On the same queries and caches both differ from 64 bits by the rounding of the output alone
