@@ -7,6 +7,8 @@
 // ceil(kept*t/32) words of t-bit groups (kept values in column order, MSB first), then the pruned values in column
 // order as 16-bit halfwords (little endian, padded to a word).  Every row has the same kept count, so rows are
 // equally long.  The bitmap is the one in the speculation data.
+#include <type_traits>
+
 #include "wblob.cuh"
 
 namespace cass {
@@ -117,36 +119,44 @@ __global__ void __launch_bounds__(32 * kSplitWarps) k_split(const uint32_t* __re
 }
 
 // Exact reconstruction (Sec. 4.1 target inference: speculation and verification data are loaded and the original values
-// rebuilt; Sec. 5.1 mantissa concatenator).  One warp takes one (superblock, chunk) in two steps:
-//   lane = row: the chunk's codewords, fields and low mantissa bits become complete bf16 values in a list in shared memory,
-//     8 at a time as in the draft GEMV (the bitmap is not needed for this, so there is no search for columns); the words of
-//     the next group are requested before a group is decoded;
-//   lane = two neighbouring columns, one row after the other: a prefix count of the bitmap says which list entry, or which
-//     pruned value of the verification data, each column takes, and the row leaves as contiguous stores.  A row's loads are
-//     all under way before its first store.
-// Every output value is written once.  Bound: instruction issue.  Storing kept values at their columns from the decoding lanes
-// and filling the gaps in a second pass over the output took 255 us for a 6144 x 4096 matrix; four warps for the second step
-// of one chunk, three of them waiting for the first, 145 us; this, 131 us.
+// rebuilt; Sec. 5.1 mantissa concatenator).  One warp takes one (superblock, chunk), 64 columns (two bitmap words) of its 32 rows at a
+// time, in two steps over a buffer in shared memory:
+//   lane = row: the codewords, fields and low mantissa bits of the window's kept values become complete bf16 values, 8 at a time
+//     as in the draft GEMV, in a list; groups of 8 do not end where windows do, so up to 7 values stay for the next window.  Behind
+//     the list the window's pruned values, copied from the verification data meanwhile, half a warp a row;
+//   lane = 8 columns, four rows at a time: a prefix count of the bitmap says where in the list and among the pruned values the
+//     columns begin; each then takes the next of either, and the eight leave in one store.
+// Kept and pruned values of a window are 64 together, so the buffer is 82 halfwords a row, whatever the matrix looks like, and 28 warps
+// fit an SM (by registers).  Bound: instruction issue (59 %) and the latency of a window's steps: 34 M warp instructions for 6144 x 4096
+// (49 M with a list of a whole chunk's values, which 20 warps an SM had room for, and one row after the other with its loads), of
+// which decoding 13, writing 12, copying 5.  6144 x 4096 at 40 % pruning 115 -> 61 us, at 30 % 217 -> 64 (a chunk took a second turn), at
+// 60 % 109 -> 57; 28672 x 4096 374 -> 219.
 constexpr int kJoinWarps = 4;
-// Values of a row in hand: the most with five CTAs an SM, and what a chunk of 256 columns holds from 40 % pruning on.  Longer chunks
-// take a second turn over every row for their last few values: 113 us for 6144 x 4096 at 40 %, 219 at 35 %, 215 at 30 %.  With room
-// for 184 values and four CTAs it was 113, 116 and 165, but 250 instead of 221 for 4096 x 14336 at 40 % and 440 instead of 379 for
-// 28672 x 4096.
-constexpr int kJoinCap = 168;
-constexpr int kJoinStride = kJoinCap + 2;                               // halfwords: an odd number of words, rows in different banks
-constexpr int kJoinSpan = 5;                                            // pairs of bitmap words (64 columns) of a row at a time
-static_assert(kJoinCap % 8 == 0 && (kJoinStride / 2) % 2 == 1, "groups of 8; odd row stride in words");
+// Chunks up to which teams: 22 and 29 us with and without for 986 x 1289 (186 chunks), 27 and 33 for 4096 x 2048 (1024), but 63 and 51 for
+// 2000 x 5000 (1260, t = 3) and 89 and 61 for 6144 x 4096 (3072).
+constexpr int kJoinTeamMax = 8 * kSms;
+constexpr int kJoinRow = 82;                                            // halfwords: 7 + 64 + 7 + 2 for odd places; an odd number of words, rows in different banks
 
 struct JoinGeom {
     int n, k, k_pad, t, seg_cols, n_seg, n_ch, n_tasks, lo_words, row_words, n_raw;
 };
 
-// TEAM: the CTA's four warps share one chunk, the first decoding and each writing a quarter of the rows: the latency of a small
-// matrix; in a large one three warps would wait while the first decodes.
-template <int TT, bool TEAM>                                            // TT: truncated bits (0..5), or -1: any (from the geometry)
-__global__ void __launch_bounds__(32 * kJoinWarps, 5) k_join(const uint32_t* __restrict__ blob, const uint32_t* __restrict__ vdata,
-                                                             uint16_t* __restrict__ out, JoinGeom jg) {
-    __shared__ uint16_t s_lists[kJoinWarps * 32 * kJoinStride + 64 * kJoinSpan + 2];      // a look past the last list reads what no column takes
+__device__ __forceinline__ uint32_t join_lds16(uint32_t a) {
+    uint16_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+    return v;
+}
+
+// TT: truncated bits (0..5), or -1: any (from the geometry).  TEAM: the CTA's four warps share one chunk, the first decoding and all of them
+// copying and writing: the latency of a small matrix.
+template <int TT, bool TEAM>
+__global__ void __launch_bounds__(32 * kJoinWarps) k_join(const uint32_t* __restrict__ blob, const uint32_t* __restrict__ vdata,
+                                                          uint16_t* __restrict__ out, JoinGeom jg) {
+    // a window's first and last eight columns may reach up to 7 beyond it: what they read there is not stored
+    constexpr int kTasks = TEAM ? 1 : kJoinWarps, kSteps = TEAM ? kJoinWarps : 1;      // chunks a CTA; warps a chunk
+    __shared__ __align__(16) uint16_t s_buf[8 + kTasks * 32 * kJoinRow + 8];
+    __shared__ uint4 s_row[kTasks][32];                                 // a row's window: bitmap words, places and ends, first word | kept values in it
+    __shared__ uint2 s_copy[kTasks][32];                                // its pruned values: words from, how many | to
     __shared__ uint16_t s_lut[256];                                     // rank -> exponent at its bf16 position
     const int t = TT >= 0 ? TT : jg.t, F = 8 - t, PER = 32 / F;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -154,7 +164,11 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 5) k_join(const uint32_t* __r
     pdl_wait();
     for (int i = threadIdx.x; i < 256; i += 32 * kJoinWarps) s_lut[i] = (uint16_t)cb[i] << 7;
     __syncthreads();
-    const int task = TEAM ? (int)blockIdx.x : (int)blockIdx.x * kJoinWarps + warp;
+    const int slot = TEAM ? 0 : warp, share = TEAM ? warp : 0, task = (int)blockIdx.x * kTasks + slot;
+    auto sync = [&]() {
+        if (TEAM) __syncthreads();
+        else __syncwarp();
+    };
     if (task >= jg.n_tasks) return;
     const int sb = task / jg.n_ch, ch = task % jg.n_ch, rb = sb / jg.n_seg, seg = sb % jg.n_seg;
     const uint4 dir = __ldg(reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4) + sb);
@@ -162,15 +176,18 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 5) k_join(const uint32_t* __r
     if (ch >= n_ch) return;                                             // a shorter last segment
     const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir.y, (int)dir.z);
     const uint32_t* body = blob + (size_t)dir.x * 4;
-    const int c_base = seg * jg.seg_cols;
+    const int c_base = seg * jg.seg_cols, row = rb * kRowsPerBlock + lane;
     const uint32_t* un = body + sg.un + lane;
     const uint32_t* fl = body + sg.fl + lane;
-    const uint32_t* lo = vdata + kVdataHeaderWords + (size_t)min(rb * kRowsPerBlock + lane, jg.n - 1) * jg.row_words;
+    const uint32_t* bmr = body + sg.bm + lane;
+    const uint32_t vrow = kVdataHeaderWords + (uint32_t)min(row, jg.n - 1) * (uint32_t)jg.row_words;     // the row's words of the verification data
+    const uint32_t* lo = vdata + vrow;
     const int wu_last = max(sg.w_u - 1, 0), wf_last = max(sg.w_f - 1, 0), lo_last = max(jg.lo_words - 1, 0);
     const uint32_t ulimit = (uint32_t)sg.w_u * 32u, low_mask = (1u << t) - 1u, keep_bits = 0x8000u | (0x7Fu & ~low_mask);
     const uint32_t e0 = __ldg(body + sg.tab + ch * 32 + lane), total = __ldg(body + sg.tab + n_ch * 32 + lane);
-    const int col_end = ch + 1 < n_ch ? (int)(__ldg(body + sg.tab + (ch + 1) * 32 + lane) >> 20) : scols;
     int col = ch == 0 ? 0 : (int)(e0 >> 20);                            // this lane's row: first column not yet written
+    int col_end = ch + 1 < n_ch ? (int)(__ldg(body + sg.tab + (ch + 1) * 32 + lane) >> 20) : scols;
+    col_end = row < jg.n ? min(col_end, jg.k - c_base) : col;
     const int cnt = max(0, min(E, (int)(total >> 20) - ch * E));        // its kept values in this chunk
     uint32_t upos = e0 & 0xFFFFFu;
     int k_row = ch * E;                                                 // kept values of the row before this chunk
@@ -178,163 +195,205 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 5) k_join(const uint32_t* __r
         const uint4 dp = __ldg(reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4) + rb * jg.n_seg + i);
         k_row += (int)(__ldg(blob + (size_t)dp.x * 4 + dir_n_ch(dp.w) * 32 + lane) >> 20);
     }
-    const int n_max = __reduce_max_sync(0xffffffffu, cnt);
     constexpr int NFW = TT == 4 ? 1 : TT == 0 ? 2 : 4, NLW = TT == 0 ? 0 : TT > 0 && TT <= 4 ? 2 : 3;       // words a group of 8 can touch
-    uint16_t* s_list = s_lists + (TEAM ? 0 : warp * 32 * kJoinStride);
-    uint16_t* mine = s_list + lane * kJoinStride;
+    constexpr int LW = NLW > 0 ? NLW : 1;
+    uint16_t* buf = s_buf + 8 + slot * 32 * kJoinRow;
+    uint16_t* mine = buf + lane * kJoinRow;
+    const uint32_t buf_a = smem_u32(buf), lut_top = smem_u32(s_lut) + 62u;
+    const bool vec16 = jg.k % 8 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0, vec4 = jg.k % 2 == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0;
 
-    for (int p0 = 0; p0 == 0 || p0 < n_max; p0 += kJoinCap) {
-        const int n_here = min(kJoinCap, n_max - p0);
-        if (!TEAM || warp == 0) {
-            // ---- lane = row: values p0 .. p0 + n_here - 1 of the chunk ----
-            uint32_t fw[NFW], lw[NLW > 0 ? NLW : 1], fn[NFW], ln[NLW > 0 ? NLW : 1];
-            auto fetch = [&](int g) {                                   // field and low words of the group that starts at value g
-                const int fi = (ch * E + p0 + g) / PER;
+    // field and low words of the group of 8 that starts at value g of the chunk, asked for a group ahead
+    uint32_t fn[NFW], ln[LW];
+    auto fetch = [&](int g, bool first) {
+        const int fi = (ch * E + g) / PER;
 #pragma unroll
-                for (int i = 0; i < NFW; ++i) fn[i] = __ldg(fl + min(fi + i, wf_last) * 32);
-                if (NLW > 0) {
-                    const int li = (int)((uint32_t)(k_row + p0 + g) * (uint32_t)t >> 5);
+        for (int i = 0; i < NFW; ++i) fn[i] = __ldg(fl + min(fi + i, wf_last) * 32);
+        if (NLW > 0) {
+            const int li = (int)((uint32_t)(k_row + g) * (uint32_t)t >> 5);
+            if (TT == 4 && !first) {                                    // one word a group
+                ln[0] = ln[LW - 1];
+                ln[LW - 1] = __ldg(lo + min(li + 1, lo_last));
+            } else {
 #pragma unroll
-                    for (int i = 0; i < NLW; ++i) ln[i] = __ldg(lo + min(li + i, lo_last));
+                for (int i = 0; i < LW; ++i) ln[i] = __ldg(lo + min(li + i, lo_last));
+            }
+        }
+    };
+    int at = (int)(upos >> 5);                                          // u0, u1, u2: code words at, at + 1, at + 2
+    uint32_t u0 = __ldg(un + min(at, wu_last) * 32), u1 = __ldg(un + min(at + 1, wu_last) * 32), u2 = __ldg(un + min(at + 2, wu_last) * 32);
+    fetch(0, true);
+    int j0 = col >> 5, ks = 0, dec = 0;                                 // first bitmap word of the window; values taken; values decoded
+    auto bm_word = [&](int j) { return j < sg.bm_words ? __ldg(bmr + j * 32) : 0u; };
+    uint32_t wn0 = bm_word(j0), wn1 = bm_word(j0 + 1);
+
+#pragma unroll 1
+    while (__any_sync(0xffffffffu, col < col_end)) {
+        // ---- the window: columns col .. hi - 1 of this lane's row, bits of others cleared ----
+        const bool more = col < col_end;
+        const int off = more ? col - j0 * 32 : 64, hi = more ? min(64, col_end - j0 * 32) : 64;      // from the first word's first column on
+        uint32_t w0 = wn0, w1 = wn1;
+        wn0 = bm_word(j0 + 2);
+        wn1 = bm_word(j0 + 3);
+        {
+            unsigned long long m = off < 64 ? ~0ull >> off : 0ull;
+            if (hi < 64) m &= ~(~0ull >> hi);
+            w0 &= (uint32_t)(m >> 32);
+            w1 &= (uint32_t)m;
+        }
+        const int n0 = __popc(w0), kw = n0 + __popc(w1), base8 = ks & ~7, ke = ks + kw, dec_end = (ke + 7) & ~7;
+        // ---- its pruned values, behind the list ----
+        const int s0 = c_base + col - (k_row + ks), n_raw = hi - off - kw;
+        const uint32_t rw = vrow + (uint32_t)jg.lo_words + (uint32_t)(s0 >> 1);
+        const int n_w = n_raw > 0 ? ((s0 & 1) + n_raw + 1) >> 1 : 0, to_w = (lane * kJoinRow + dec_end - base8) >> 1;
+        const uint32_t place = (uint32_t)(ks - base8) | ((uint32_t)(dec_end - base8 + (s0 & 1)) << 8) | ((uint32_t)off << 16) | ((uint32_t)hi << 24);
+        if (share == 0) {
+            s_copy[slot][lane] = make_uint2(rw, (uint32_t)n_w | ((uint32_t)to_w << 16));
+            s_row[slot][lane] = make_uint4(w0, w1, place, (uint32_t)j0 | ((uint32_t)n0 << 16));
+        }
+        const bool whole = __all_sync(0xffffffffu, off == 0 && hi == 64);
+        sync();
+        auto copy = [&](uint32_t to, uint32_t from) {
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(vdata + from) : "memory");
+        };
+#pragma unroll 4
+        for (int r = share * 2 + (lane >> 4); r < kRowsPerBlock; r += 2 * kSteps) {        // half a warp a row
+            const uint2 cp = s_copy[slot][r];
+            const uint32_t n = cp.y & 0xFFFFu, to = buf_a + (cp.y >> 16) * 4u + (uint32_t)(lane & 15) * 4u, from = cp.x + (uint32_t)(lane & 15);
+            if ((uint32_t)(lane & 15) < n) copy(to, from);
+            if (n > 16u)                                                // up to 33 words
+                for (uint32_t w = 16; w + (uint32_t)(lane & 15) < n; w += 16) copy(to + w * 4u, from + w);
+        }
+        // ---- lane = row: values up to ke, whole groups ----
+        while (share == 0 && dec < dec_end) {
+            uint32_t fw[NFW], lw[LW];
+#pragma unroll
+            for (int i = 0; i < NFW; ++i) fw[i] = fn[i];
+#pragma unroll
+            for (int i = 0; i < LW; ++i) lw[i] = ln[i];
+            fetch(dec + 8, false);
+            uint32_t uv = __funnelshift_l(u1, u0, upos), used = 8u * 32u, q = 0, v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {                               // shifting the found one out leaves the next code at the top
+                asm("bfind.u32 %0, %1;" : "=r"(q) : "r"(uv));
+                uint32_t a;
+                asm("mad.lo.u32 %0, %1, 0xFFFFFFFE, %2;" : "=r"(a) : "r"(q), "r"(lut_top));
+                v[i] = join_lds16(a);
+                used -= q;
+                uv = __funnelshift_r(0u, uv, q);
+            }
+            if ((int32_t)q < 0) {                                       // the codes did not fit the window: one by one
+                uint32_t ub = upos;
+#pragma unroll 1
+                for (int i = 0; i < 8; ++i) {
+                    uint32_t x = 0;
+                    if (dec + i < cnt) x = s_lut[read_unary(un, ub, ulimit) & 255];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[j] = i == j ? x : v[j];
                 }
-            };
-            int at = (int)(upos >> 5);                                  // u0, u1, u2: code words at, at + 1, at + 2
-            uint32_t u0 = __ldg(un + min(at, wu_last) * 32), u1 = __ldg(un + min(at + 1, wu_last) * 32), u2 = __ldg(un + min(at + 2, wu_last) * 32);
-            fetch(0);
-            for (int g = 0; g < n_here; g += 8) {
+                used = ub - upos;
+            }
+            upos += used;
+            const int step = (int)(upos >> 5) - at;
+            if (step == 1) {
+                u0 = u1; u1 = u2;
+                u2 = __ldg(un + min(at + 3, wu_last) * 32);
+            } else if (step > 1) {
+                u0 = __ldg(un + min(at + step, wu_last) * 32);
+                u1 = __ldg(un + min(at + step + 1, wu_last) * 32);
+                u2 = __ldg(un + min(at + step + 2, wu_last) * 32);
+            }
+            at += step;
+            const int k = ch * E + dec;                                 // of the segment: fields are numbered through it
+            const uint32_t bit0 = ((uint32_t)(k_row + dec) * (uint32_t)t) & 31u;
+            const uint32_t l8 = TT == 4 ? __funnelshift_l(lw[LW - 1], lw[0], bit0) : 0u;
 #pragma unroll
-                for (int i = 0; i < NFW; ++i) fw[i] = fn[i];
-#pragma unroll
-                for (int i = 0; i < NLW; ++i) lw[i] = ln[i];
-                if (g + 8 < n_here) fetch(g + 8);
-                uint32_t uv = __funnelshift_l(u1, u0, upos), used = 0, q = 0, v[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {                           // shifting the found one out leaves the next code at the top
-                    asm("bfind.u32 %0, %1;" : "=r"(q) : "r"(uv));
-                    v[i] = s_lut[(31u - q) & 255u];
-                    used += 32u - q;
-                    uv = __funnelshift_r(0u, uv, q);
+            for (int i = 0; i < 8; ++i) {
+                uint32_t sm;
+                if (TT == 4) {
+                    sm = __funnelshift_l(fw[0], fw[0], (4 * i + 16) & 31);
+                } else if (TT == 0) {
+                    sm = __funnelshift_l(fw[i / 4 % NFW], fw[i / 4 % NFW], (8 * (i & 3) + 16) & 31);
+                } else {
+                    const int j = k % PER + i, wi = j / PER;            // up to three words on
+                    sm = field_sign_mant_bf16(wi == 0 ? fw[0] : wi == 1 ? fw[1 % NFW] : wi == 2 ? fw[2 % NFW] : fw[3 % NFW], j - wi * PER, t);
                 }
-                if ((int32_t)q < 0) {                                   // the codes did not fit the window: one by one
-                    uint32_t ub = upos;
+                v[i] |= sm & keep_bits;
+                if (TT == 4) {
+                    v[i] |= (l8 >> (28 - 4 * i)) & 15u;
+                } else if (NLW > 0 && t > 0) {
+                    const uint32_t b = bit0 + (uint32_t)(i * t), wi = b >> 5;
+                    const uint32_t hi_w = wi == 0 ? lw[0] : wi == 1 || NLW == 2 ? lw[LW > 1 ? 1 : 0] : lw[LW > 2 ? 2 : 0];
+                    const uint32_t nx = wi == 0 || NLW == 2 ? lw[LW > 1 ? 1 : 0] : lw[LW > 2 ? 2 : 0];
+                    v[i] |= (__funnelshift_l(nx, hi_w, b) >> (32 - t)) & low_mask;
+                }
+            }
+            uint32_t* to = reinterpret_cast<uint32_t*>(mine + dec - base8);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (p0 + g + i < cnt) v[i] = s_lut[read_unary(un, ub, ulimit) & 255];
-                    used = ub - upos;
-                }
-                upos += used;
-                const int step = (int)(upos >> 5) - at;
-                if (step == 1) {
-                    u0 = u1; u1 = u2;
-                    u2 = __ldg(un + min(at + 3, wu_last) * 32);
-                } else if (step > 1) {
-                    u0 = __ldg(un + min(at + step, wu_last) * 32);
-                    u1 = __ldg(un + min(at + step + 1, wu_last) * 32);
-                    u2 = __ldg(un + min(at + step + 2, wu_last) * 32);
-                }
-                at += step;
-                const int k = ch * E + p0 + g;                          // of the segment: fields are numbered through it
-                const uint32_t bit0 = ((uint32_t)(k_row + p0 + g) * (uint32_t)t) & 31u;
+            for (int i = 0; i < 4; ++i) to[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x5410);
+            dec += 8;
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        sync();
+        // ---- lane = 8 columns of one of four rows ----
+        auto write = [&](auto whole_c, auto vec_c) {
+            constexpr bool W = decltype(whole_c)::value;                // every row has the whole window: nothing to leave out
+            constexpr int V = decltype(vec_c)::value;                   // bytes a store
+            const int o = lane & 7, c = o * 8, r_first = share * 4 + (lane >> 3);
+            const uint32_t sh = 8u * (uint32_t)(o & 3);
+            uint16_t* to_row = out + (size_t)(rb * kRowsPerBlock + r_first) * jg.k + (c_base + c);
+            uint32_t row_a = buf_a + (uint32_t)(r_first * kJoinRow) * 2u;
+#pragma unroll 1
+            for (int r = r_first; r < kRowsPerBlock; r += 4 * kSteps, to_row += (size_t)(4 * kSteps) * jg.k, row_a += 4 * kSteps * kJoinRow * 2) {
+                const uint4 p = s_row[slot][r];
+                const int r_off = W ? 0 : (int)((p.z >> 16) & 0xFFu), r_hi = W ? 64 : (int)(p.z >> 24);
+                if (!W && (c + 8 <= r_off || c >= r_hi)) continue;      // none of the window's columns
+                const uint32_t w = o < 4 ? p.x : p.y, b = w << sh;
+                const uint32_t before = (uint32_t)__popc(__funnelshift_rc(w, 0u, 32u - sh)) + (o < 4 ? 0u : p.w >> 16);      // kept values of the window before these columns
+                uint32_t ak = row_a + ((p.z & 0xFFu) + before) * 2u;
+                uint32_t ar = row_a + (((p.z >> 8) & 0xFFu) + (uint32_t)(c - r_off) - before) * 2u;
+                uint32_t x[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    uint32_t sm;
-                    if (TT == 4) {
-                        sm = __funnelshift_l(fw[0], fw[0], (4 * i + 16) & 31);
-                    } else if (TT == 0) {
-                        sm = __funnelshift_l(fw[i / 4 % NFW], fw[i / 4 % NFW], (8 * (i & 3) + 16) & 31);
+                    const bool keep = b & (0x80000000u >> i);
+                    x[i] = join_lds16(keep ? ak : ar);
+                    ak += keep ? 2u : 0u;
+                    ar += keep ? 0u : 2u;
+                }
+                uint16_t* to = to_row + (p.w & 0xFFFFu) * 32u;
+                if (V >= 4 && (W || (c >= r_off && c + 8 <= r_hi))) {
+                    const uint4 y = make_uint4(x[0] | (x[1] << 16), x[2] | (x[3] << 16), x[4] | (x[5] << 16), x[6] | (x[7] << 16));
+                    if (V == 16) {
+                        *reinterpret_cast<uint4*>(to) = y;
                     } else {
-                        const int j = k % PER + i, wi = j / PER;        // up to three words on
-                        sm = field_sign_mant_bf16(wi == 0 ? fw[0] : wi == 1 ? fw[1 % NFW] : wi == 2 ? fw[2 % NFW] : fw[3 % NFW], j - wi * PER, t);
+                        reinterpret_cast<uint32_t*>(to)[0] = y.x; reinterpret_cast<uint32_t*>(to)[1] = y.y;
+                        reinterpret_cast<uint32_t*>(to)[2] = y.z; reinterpret_cast<uint32_t*>(to)[3] = y.w;
                     }
-                    v[i] |= sm & keep_bits;
-                    if (NLW > 0 && t > 0) {
-                        const uint32_t b = bit0 + (uint32_t)(i * t), wi = b >> 5;
-                        const uint32_t hi = wi == 0 ? lw[0] : wi == 1 || NLW == 2 ? lw[NLW > 1 ? 1 : 0] : lw[NLW > 2 ? 2 : 0];
-                        const uint32_t nx = wi == 0 || NLW == 2 ? lw[NLW > 1 ? 1 : 0] : lw[NLW > 2 ? 2 : 0];
-                        v[i] |= (__funnelshift_l(nx, hi, b) >> (32 - t)) & low_mask;
-                    }
-                    mine[g + i] = (uint16_t)v[i];
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (W || (c + i >= r_off && c + i < r_hi)) to[i] = (uint16_t)x[i];
                 }
             }
-        }
-        if (TEAM) __syncthreads(); else __syncwarp();
-        // ---- lane = two columns: one row after the other ----
-        constexpr int kRowStep = TEAM ? kJoinWarps : 1;
-        uint32_t bm_next = 0;                                           // the row's bitmap words, one a lane, fetched a row ahead
-        auto words = [&](int r) {
-            const int c0 = __shfl_sync(0xffffffffu, col, r), j = (c0 >> 5) + lane;
-            return lane < 2 * kJoinSpan && j < sg.bm_words ? __ldg(body + sg.bm + j * 32 + r) : 0u;
         };
-        bm_next = words(TEAM ? warp : 0);
-#pragma unroll 1
-        for (int r = TEAM ? warp : 0; r < kRowsPerBlock; r += kRowStep) {
-            uint32_t bmv = bm_next;
-            if (r + kRowStep < kRowsPerBlock) bm_next = words(r + kRowStep);
-            const int row = rb * kRowsPerBlock + r;
-            if (row >= jg.n) break;
-            const int c0 = __shfl_sync(0xffffffffu, col, r), c_row = __shfl_sync(0xffffffffu, col_end, r);
-            const int n_row = __shfl_sync(0xffffffffu, cnt, r), kr = __shfl_sync(0xffffffffu, k_row, r);
-            if (c0 >= c_row) continue;
-            const int k_end = min(p0 + n_here, n_row);                  // list entries of this turn: chunk values p0 .. k_end - 1
-            const bool last = k_end == n_row;                           // else the row goes up to the value k_end, exclusive
-            const uint16_t* list = s_list + r * kJoinStride - p0;
-            const uint16_t* raw = reinterpret_cast<const uint16_t*>(vdata + (jg.n_raw > 0 ? kVdataHeaderWords + (size_t)row * jg.row_words + jg.lo_words : 0));
-            uint16_t* orow = out + (size_t)row * jg.k + c_base;
-            const bool pairs = (((size_t)row * jg.k) & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0;
-            const int lim = min(last ? c_row : scols, jg.k - c_base), j_end = (lim + 31) / 32;
-            int kpos = p0, stop = c_row;
-            const uint32_t r_last = (uint32_t)max(jg.n_raw - 1, 0), left = ~(0xFFFFFFFFu >> (2 * (lane & 15)));
-            for (int j0 = c0 >> 5;;) {
-                if (j0 * 32 < c0 && lane == 0) bmv &= 0xFFFFFFFFu >> (c0 & 31);      // values before belong to an earlier turn
-                int pre = __popc(bmv), here = pre;                      // kept values before each word
+        auto write_v = [&](auto whole_c) {
+            if (vec16) write(whole_c, std::integral_constant<int, 16>{});
+            else if (vec4) write(whole_c, std::integral_constant<int, 4>{});
+            else write(whole_c, std::integral_constant<int, 2>{});
+        };
+        if (whole) write_v(std::true_type{});
+        else write_v(std::false_type{});
+        sync();
+        // ---- values decoded ahead move to the front ----
+        if (share == 0 && (ke & 7) && (ke & ~7) != base8) {
+            const uint32_t* from = reinterpret_cast<const uint32_t*>(mine + (ke & ~7) - base8);
+            const uint32_t m[4] = {from[0], from[1], from[2], from[3]};
+            uint32_t* to = reinterpret_cast<uint32_t*>(mine);
 #pragma unroll
-                for (int o = 1; o < 16; o <<= 1) {
-                    const int v = __shfl_up_sync(0xffffffffu, pre, o);
-                    if (lane >= o) pre += v;
-                }
-                const int all = __shfl_sync(0xffffffffu, pre, 15);
-                pre += kpos - here;
-                // both candidates of every column are loaded, without a condition, before any is used: a choice between the
-                // loads is a divergent branch that waits for each in turn
-                uint32_t lx[kJoinSpan][2], rx[kJoinSpan][2], two[kJoinSpan];
-                int bf[kJoinSpan];
-                const int q0 = c_base + lane * 2 - kr;
-#pragma unroll
-                for (int i = 0; i < kJoinSpan; ++i) {
-                    const uint32_t b = __shfl_sync(0xffffffffu, bmv, 2 * i + (lane >> 4));
-                    bf[i] = __shfl_sync(0xffffffffu, pre, 2 * i + (lane >> 4)) + __popc(b & left);      // kept values before the first column
-                    two[i] = b << (2 * (lane & 15));                    // kept? this lane's columns at the top
-                    const uint32_t p_at = (uint32_t)(q0 + (j0 + 2 * i) * 32 - bf[i]);                   // pruned ones = columns - kept
-                    lx[i][0] = list[bf[i]];
-                    lx[i][1] = list[bf[i] + 1];
-                    rx[i][0] = __ldg(raw + min(p_at, r_last));
-                    rx[i][1] = __ldg(raw + min(p_at + 1u, r_last));
-                }
-#pragma unroll
-                for (int i = 0; i < kJoinSpan; ++i) {
-                    const int j = j0 + 2 * i, c = j * 32 + lane * 2;
-                    const bool k0 = two[i] >> 31, k1 = (two[i] >> 30) & 1u;
-                    const uint32_t x0 = k0 ? lx[i][0] : rx[i][0];
-                    const uint32_t xl = k0 ? lx[i][1] : lx[i][0], xr = k0 ? rx[i][0] : rx[i][1], x1 = k1 ? xl : xr;
-                    if (pairs && last && j * 32 >= c0 && (j + 2) * 32 <= lim) {
-                        *reinterpret_cast<uint32_t*>(orow + c) = x0 | (x1 << 16);
-                    } else if (j < j_end) {                             // the row's ends, and rows off 4-byte boundaries
-                        if (c >= c0 && c < lim && (last || bf[i] + k0 <= k_end)) orow[c] = (uint16_t)x0;
-                        if (c + 1 >= c0 && c + 1 < lim && (last || bf[i] + k0 + k1 <= k_end)) orow[c + 1] = (uint16_t)x1;
-                        if (!last && kpos + all > k_end && stop == c_row) {      // the value k_end is in these words: its column begins the next turn
-                            const uint32_t at = __reduce_min_sync(0xffffffffu, k0 && bf[i] == k_end ? (uint32_t)c : k1 && bf[i] + k0 == k_end ? (uint32_t)(c + 1) : 0xFFFFFFFFu);
-                            if (at != 0xFFFFFFFFu) stop = (int)at;
-                        }
-                    }
-                }
-                j0 += 2 * kJoinSpan;
-                if (j0 >= j_end || stop != c_row) break;
-                kpos += all;
-                bmv = lane < 2 * kJoinSpan && j0 + lane < sg.bm_words ? __ldg(body + sg.bm + (j0 + lane) * 32 + r) : 0u;
-            }
-            if (lane == r) col = last ? c_row : stop;
+            for (int i = 0; i < 4; ++i) to[i] = m[i];
         }
-        if (TEAM) __syncthreads(); else __syncwarp();
+        ks = ke;
+        if (more) col = j0 * 32 + hi;
+        j0 += 2;
     }
 }
 
@@ -373,9 +432,7 @@ extern "C" int cass_decode_full(const void* blob, const cass_blob_info* bi, cons
     const JoinGeom jg{bi->rows, bi->cols, ceil_div(bi->cols, 32) * 32, bi->trunc_bits, bi->seg_cols, bi->n_seg, n_ch,
                       bi->n_rowblocks * bi->n_seg * n_ch, vdata_lo_words(bi->kept_per_row, bi->trunc_bits),
                       vdata_row_words(bi->cols, bi->kept_per_row, bi->trunc_bits), bi->cols - bi->kept_per_row};
-    // below about half of the 20 kSms = 2960 warps that run at once, teams: 24 instead of 46 us for 986 x 1289 (186 chunks), 54 instead of
-    // 62 for 4096 x 2048 (1024 chunks), but 99 instead of 76 for 4096 x 4096 (2048)
-    const bool team = jg.n_tasks < 1536;
+    const bool team = jg.n_tasks < kJoinTeamMax;
 #define CASS_JOIN(T_)                                                                                                               \
     do {                                                                                                                            \
         if (team) CASS_PDL_LAUNCH((k_join<T_, true>), dim3(jg.n_tasks), dim3(32 * kJoinWarps), 0, stream, b32, v32, o16, jg);        \
