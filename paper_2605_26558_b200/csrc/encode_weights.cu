@@ -1,16 +1,19 @@
 // Offline weight encoder: Wanda-scored per-row pruning, mantissa truncation, unary exponent coding,
 // superblock packing (Sec. 4.2, 5.1, 5.3).  Bit-exact counterpart of the CPU oracle's blob.
+#include <type_traits>
+
 #include "wblob.cuh"
 
 namespace cass {
 
 // Workspace carve-up (all offsets 256-byte aligned).
 struct EncWs {
-    uint32_t* keepbm;        // [n][k_pad/32]
+    uint32_t* keepbm;        // [n][k_pad/32], or (by lanes) [n_rb][k_pad/32][32]
     uint2* sb_size;          // [n_rb * n_seg]  of each superblock's rows: most kept values, most code words
     unsigned long long* hist;   // [256] exponents of the kept values; zeroed by the caller, as is abort_flag behind it
     uint32_t* abort_flag;    // [1]
     uint8_t* exp_to_rank;    // [256]
+    uint32_t* blk_size;      // [n_rb * n_seg][16][32]  code bits | kept values << 16 of a superblock's rows in each 128 columns
     size_t zero_bytes;       // hist and abort_flag
     size_t bytes;
 };
@@ -25,6 +28,7 @@ static EncWs carve(void* base, int n_pad, int k_pad, int n_seg) {
     w.exp_to_rank = (uint8_t*)take(256);
     w.keepbm = (uint32_t*)take((size_t)n_pad * (k_pad / 32) * 4);
     w.sb_size = (uint2*)take((size_t)(n_pad / kRowsPerBlock) * n_seg * 8);
+    w.blk_size = (uint32_t*)take((size_t)(n_pad / kRowsPerBlock) * n_seg * 16 * 32 * 4);
     w.bytes = off;
     return w;
 }
@@ -32,6 +36,7 @@ static EncWs carve(void* base, int n_pad, int k_pad, int n_seg) {
 struct EncGeom {
     int n, k, k_pad, n_pad, n_rb, n_seg, seg_cols, chunk_cols, p, t, n_prune;
     int mx;          // 1: Cassandra-2 (shared exponents), 0: Cassandra-1 (unary code)
+    int lanes;       // sizes and packing by lanes: the bitmaps' words lie 32 rows side by side
 };
 
 static int make_geom(const cass_format* fmt, int rows, int cols, EncGeom* g) {
@@ -53,6 +58,11 @@ static int make_geom(const cass_format* fmt, int rows, int cols, EncGeom* g) {
     g->n_rb = ceil_div(rows, kRowsPerBlock);
     g->n_pad = g->n_rb * kRowsPerBlock;
     g->n_prune = (int)(((long long)cols * p) / 1000);
+    // Sizes and packing by lanes (a warp's chain is long) or by warps, by the blocks of 128 columns of 32 rows there are: 113 -> 85 us by
+    // lanes for 3000 x 2050 (1598 blocks), 79 -> 73 for 5000 x 1027 (1413), but 34 and 34 for 1000 x 1000 (256).  Rows of few columns take
+    // a warp little: 40 -> 52 for 5000 x 512 (628), 42 -> 54 for 9000 x 400 (1124), 88 -> 93 for 20000 x 501 (2500), 120 -> 103 for 30000 x 301 (2814).
+    const long long blocks = (long long)g->n_rb * ceil_div(g->k_pad, 128);
+    g->lanes = !g->mx && t == 4 && blocks >= (g->seg_cols > 512 ? 1400 : 2600);
     return CASS_OK;
 }
 
@@ -265,7 +275,9 @@ __global__ void __launch_bounds__(!WIDE ? 128 : NV == 128 ? 32 * kSelWarps : 32 
         }
         // kept: the values above the shared upper half, and those of the list from the threshold on
         const __nv_bfloat162 t2 = as_bf162(top ? top | (top << 16) : 0x007F007Fu);
-        uint8_t* keep_row = reinterpret_cast<uint8_t*>(keepbm) + (size_t)row * row_bytes;
+        const size_t row_at = g.lanes ? (size_t)(row / kRowsPerBlock) * kRowsPerBlock * row_bytes + (size_t)(row % kRowsPerBlock) * 4 : (size_t)row * row_bytes;
+        uint8_t* keep_row = reinterpret_cast<uint8_t*>(keepbm) + row_at;
+        const int word_at = g.lanes ? 4 * kRowsPerBlock : 4;             // bytes between a row's words
 #pragma unroll
         for (int q = 0; q < NG; ++q) {
             const int c = col_of(q * 8);
@@ -282,7 +294,7 @@ __global__ void __launch_bounds__(!WIDE ? 128 : NV == 128 ? 32 * kSelWarps : 32 
                 kb = c + 8 <= g.k ? 0xFFu : c < g.k ? (0xFF00u >> (g.k - c)) & 0xFFu : 0u;
             }
             // byte of column c in its word: the first column at the most significant end
-            if (c / 8 < row_bytes) keep_row[(c / 8) ^ 3] = (uint8_t)kb;
+            if (c / 8 < row_bytes) keep_row[(size_t)(c / 32) * word_at + ((c / 8 & 3) ^ 3)] = (uint8_t)kb;
             if (!g.mx) {
                 uint32_t v[4];
                 row_load8(wr + c, kb, vec, v);
@@ -350,6 +362,290 @@ __global__ void __launch_bounds__(1024) k_sizes(const uint16_t* __restrict__ W, 
         const uint32_t mk = __reduce_max_sync(0xffffffffu, s_kept[lane]), mw = __reduce_max_sync(0xffffffffu, s_words[lane]);
         if (lane == 0) sb_size[blockIdx.x] = make_uint2(mk, mw);
     }
+}
+
+// ---- E4 and E6 for unary blobs by lanes: a warp takes 32 rows of some columns, a lane a row -------------------------------
+// The weights come 64 columns of 32 rows at a time into shared memory with whole-line reads (rows 16 bytes beyond a multiple of
+// 32 apart: lanes read 16 bytes of their own rows without conflicts); from there on a lane works on its own row, with no scans,
+// shuffles or ballots.  Blocks of 128 columns are the unit of sizes and splits: k_sizes_lanes leaves the code bits and kept values of
+// every row and block, so that k_pack_lanes can start anywhere.
+// Bound: memory latency and issue.  4096 x 14336, t = 4: packing 154 -> 83 us (111 M -> 45 M warp instructions), sizes 39 -> 33 (HBM alone: 18),
+// the whole encoder 332 -> 258.  Bitmaps in rows (each lane's word in a line of its own): packing 125, sizes 52; tiles of 128 columns, three
+// CTAs an SM for two and a bit rounds: 97 and 43; sizes without the next tile's loads under way 43.
+constexpr int kBlkCols = 128, kSegBlks = 2048 / kBlkCols;
+constexpr int kTileCols = 64, kTileWords = kTileCols / 32, kBlkTiles = kBlkCols / kTileCols;
+constexpr int kLaneRow = 16 + 2 * kTileCols;             // bytes of a row: up to 7 values left of the tile before, and the tile's
+constexpr int kLaneTile = 32 * kLaneRow;
+
+// Columns c0 .. c0 + 63 of rows row0 .. row0 + 31 on their way to s + 16, in pieces of the size that the rows' boundaries allow (V); zero
+// beyond the matrix.  ask: the loads, ahead of work on the tile before; put: into shared memory.
+template <class V>
+struct LanesTile {
+    static constexpr int NB = (int)sizeof(V), LR = kTileCols * 2 / NB < 32 ? kTileCols * 2 / NB : 32, RS = 32 / LR;      // bytes, lanes a row, rows at a time
+    static constexpr int NC = kTileCols * 2 / NB / LR, N = 32 / RS * NC;                                       // pieces a lane and row; in all
+    V v[N];
+    __device__ __forceinline__ void ask(const uint16_t* __restrict__ W, int n, int k, int row0, int c0, int lane) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const int r = row0 + i / NC * RS + lane / LR, c = c0 + (lane % LR + i % NC * LR) * (NB / 2);
+            v[i] = r < n && c < k ? __ldg(reinterpret_cast<const V*>(W + (size_t)r * k + c)) : V{};
+        }
+    }
+    __device__ __forceinline__ void put(int lane, uint8_t* s) {
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            *reinterpret_cast<V*>(s + (i / NC * RS + lane / LR) * kLaneRow + 16 + (lane % LR + i % NC * LR) * NB) = v[i];
+        __syncwarp();
+    }
+};
+// Two bytes a load would take 64 registers: the values are read when they are put, 8 rows at a time.
+template <>
+struct LanesTile<uint16_t> {
+    const uint16_t* from;
+    int rows, cols, pitch;
+    __device__ __forceinline__ void ask(const uint16_t* __restrict__ W, int n, int k, int row0, int c0, int lane) {
+        from = W + (size_t)row0 * k + c0 + lane;
+        rows = n - row0;
+        cols = k - c0 - lane;
+        pitch = k;
+    }
+    __device__ __forceinline__ void put(int lane, uint8_t* s) {
+#pragma unroll 1
+        for (int r0 = 0; r0 < 32; r0 += 8) {
+            uint16_t h[8][kTileWords];
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int i = 0; i < kTileWords; ++i) h[r][i] = r0 + r < rows && i * 32 < cols ? __ldg(from + (size_t)(r0 + r) * pitch + i * 32) : (uint16_t)0;
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                for (int i = 0; i < kTileWords; ++i) *reinterpret_cast<uint16_t*>(s + (r0 + r) * kLaneRow + 16 + (i * 32 + lane) * 2) = h[r][i];
+        }
+        __syncwarp();
+    }
+};
+// Sign and exponent of value i of eight (words of two, the lower column in the lower half): index of the rank table.
+__device__ __forceinline__ uint32_t lanes_code(const uint32_t (&x)[4], int i) { return (i & 1) ? x[i / 2] >> 23 : (x[i / 2] >> 7) & 0x1FFu; }
+__device__ __forceinline__ void lanes_get8(const uint8_t* p, uint32_t (&x)[4]) {
+    const uint4 v = *reinterpret_cast<const uint4*>(p);
+    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+}
+
+// One CTA a superblock: its sizes, and those of its blocks.
+constexpr int kSizeWarps = 8;
+template <class V>
+__global__ void __launch_bounds__(32 * kSizeWarps) k_sizes_lanes(const uint16_t* __restrict__ W, EncGeom g, const uint32_t* __restrict__ keepbm,
+                                                                 const uint8_t* __restrict__ exp_to_rank, uint2* __restrict__ sb_size,
+                                                                 uint32_t* __restrict__ blk_size) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ uint8_t s_rank[512];
+    __shared__ uint32_t s_kept[32], s_bits[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int sb = blockIdx.x, rb = sb / g.n_seg, seg = sb % g.n_seg, row0 = rb * kRowsPerBlock, row = row0 + lane;
+    pdl_wait();
+    const int nw = seg_cols_of(g.k_pad, g.seg_cols, seg) / 32, w0 = seg * (g.seg_cols / 32);
+    uint8_t* s = smem + warp * kLaneTile;
+    // the warp's tiles: of block `warp`, then of block warp + kSizeWarps
+    LanesTile<V> t;
+    uint32_t bm[kTileWords];
+    auto ask = [&](int w) {
+        t.ask(W, g.n, g.k, row0, (w0 + w) * 32, lane);
+#pragma unroll
+        for (int j = 0; j < kTileWords; ++j)
+            bm[j] = row < g.n && w + j < nw ? __ldg(keepbm + ((size_t)rb * (g.k_pad / 32) + w0 + w + j) * 32 + lane) : 0u;
+    };
+    constexpr int kBlk = kBlkCols / 32;                                  // words of a block
+    uint32_t bits = 0, kept = 0;
+    int w = warp * kBlk;
+    if (w < nw) ask(w);
+    // (the rank table is filled and the sums are zero behind the first loads)
+    for (int i = tid; i < 512; i += 32 * kSizeWarps) s_rank[i] = exp_to_rank[i & 255];
+    if (tid < 32) s_kept[tid] = s_bits[tid] = 0;
+    __syncthreads();
+#pragma unroll 1
+    while (w < nw) {
+        t.put(lane, s);
+        uint32_t now[kTileWords];
+#pragma unroll
+        for (int j = 0; j < kTileWords; ++j) now[j] = bm[j];
+        const int b = w / kBlk;
+        int next = w + kTileWords;
+        const bool block_end = next % kBlk == 0 || next >= nw;
+        if (block_end) next = (b + kSizeWarps) * kBlk;
+        if (next < nw) ask(next);
+#pragma unroll
+        for (int j = 0; j < kTileWords; ++j) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t x[4];
+                lanes_get8(s + lane * kLaneRow + 16 + j * 64 + q * 16, x);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t rank = s_rank[lanes_code(x, i)];
+                    bits += now[j] & (0x80000000u >> (q * 8 + i)) ? rank : 0u;
+                }
+            }
+            kept += __popc(now[j]);
+        }
+        if (block_end) {
+            bits += kept;                                                // a code is as long as its rank and one
+            blk_size[((size_t)sb * kSegBlks + b) * 32 + lane] = bits | (kept << 16);
+            atomicAdd(&s_kept[lane], kept);
+            atomicAdd(&s_bits[lane], bits);
+            bits = kept = 0;
+        }
+        __syncwarp();
+        w = next;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t mk = __reduce_max_sync(0xffffffffu, s_kept[lane]), mw = __reduce_max_sync(0xffffffffu, (s_bits[lane] + 31u) / 32u);
+        if (lane == 0) sb_size[sb] = make_uint2(mk, mw);
+    }
+}
+
+// One CTA a superblock of t = 4, NW warps of kSegBlks / NW blocks each.  A block's kept values move to the front of the row, behind those
+// that were left over (no branches: every value is stored, the next one takes its place if it is pruned), and leave as groups of 8: a field word,
+// and code bits in one word that goes to the row's code stream.  A word that two warps fill is zero before either adds to it.
+template <int NW, class V>
+__global__ void __launch_bounds__(32 * NW) k_pack_lanes(const uint16_t* __restrict__ W, EncGeom g, const uint32_t* __restrict__ keepbm,
+                                                        const uint8_t* __restrict__ exp_to_rank, const uint32_t* __restrict__ blk_size,
+                                                        uint32_t* __restrict__ blob, const uint32_t* __restrict__ abort_flag) {
+    constexpr uint32_t kMask = 0x80700000u;                              // sign and kept mantissa bits of a binary32
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ uint8_t s_rank[512];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    pdl_wait();
+    if (*abort_flag) return;
+    const int sb = blockIdx.x, rb = sb / g.n_seg, seg = sb % g.n_seg, row0 = rb * kRowsPerBlock, row = row0 + lane;
+    const uint4 dir = reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4)[sb];
+    const int scols = seg_cols_of(g.k_pad, g.seg_cols, seg), n_ch = dir_n_ch(dir.w), nw = scols / 32, w0 = seg * (g.seg_cols / 32);
+    const uint32_t E = (uint32_t)dir_chunk_elems(dir.w);
+    const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir.y, (int)dir.z);
+    uint32_t* body = blob + (size_t)dir.x * 4 + lane;                    // this row's words, 32 apart
+    uint32_t *tab = body + sg.tab, *bmo = body + sg.bm, *fl = body + sg.fl, *un = body + sg.un;
+    for (int i = tid; i < 512; i += 32 * NW) s_rank[i] = exp_to_rank[i & 255];
+    const uint32_t* bmr = keepbm + ((size_t)rb * (g.k_pad / 32) + w0) * 32 + lane;
+    auto bm_word = [&](int j) { return row < g.n && j < nw ? __ldg(bmr + j * 32) : 0u; };
+    // where the warp's blocks begin: kept values and code bits of the row before them
+    const int b0 = warp * (kSegBlks / NW), b1 = b0 + kSegBlks / NW;
+    uint32_t k = 0, pos = 0, all_k = 0, all_bits = 0;
+#pragma unroll
+    for (int b = 0; b < kSegBlks; ++b) {
+        const uint32_t v = b * (kBlkCols / 32) < nw ? __ldg(blk_size + ((size_t)sb * kSegBlks + b) * 32 + lane) : 0u;
+        all_k += v >> 16;
+        all_bits += v & 0xFFFFu;
+        k += b < b0 ? v >> 16 : 0u;
+        pos += b < b0 ? v & 0xFFFFu : 0u;
+    }
+    // words that more than one warp may add to, and what a row leaves of its sections
+    if ((int)(k >> 3) < sg.w_f) fl[(k >> 3) * 32] = 0;
+    if ((int)(pos >> 5) < sg.w_u) un[(pos >> 5) * 32] = 0;
+    if (warp == NW - 1) {
+        for (int j = (int)(all_k >> 3); j < sg.w_f; ++j) fl[j * 32] = 0;
+        for (int j = (int)(all_bits >> 5); j < sg.w_u; ++j) un[j * 32] = 0;
+        for (int c = 0; c <= n_ch; ++c)                                  // the totals, and chunks the row has no value for
+            if (c == n_ch) tab[c * 32] = (all_k << 20) | all_bits;
+            else if ((uint32_t)c * E >= all_k) tab[c * 32] = ((uint32_t)scols << 20) | all_bits;
+    }
+    __syncthreads();
+    uint8_t* tile = smem + warp * kLaneTile;
+    uint8_t* mine = tile + lane * kLaneRow;
+    uint32_t skip = k & 7u, acc = 0;                                     // of the first group: values of the warp before; the code word in hand
+    uint32_t k_grp = k & ~7u, k_next = (k + E - 1) / E * E;              // first value of the next group; of the next chunk
+    bool un_shared = true, fl_shared = true;
+    auto flush = [&]() {                                                 // the code word in hand is full
+        if (un_shared) atomicOr(&un[(pos >> 5) * 32], acc);
+        else un[(pos >> 5) * 32] = acc;
+        un_shared = false;
+    };
+    auto append = [&](uint32_t bits, uint32_t len) {                     // len <= 32 bits from the top of `bits`
+        const uint32_t s = pos & 31u;
+        acc |= bits >> s;
+        if (s + len >= 32u) {
+            flush();
+            acc = s ? bits << (32u - s) : 0u;
+        }
+        pos += len;
+    };
+    auto group = [&](uint32_t at, uint32_t first, uint32_t last, auto whole_c) {      // values first .. last - 1 of the eight at `at`
+        constexpr bool whole = decltype(whole_c)::value;
+        uint32_t x[4], f = 0, off = 0, bits = 0;
+        lanes_get8(mine + at, x);
+        if (first == 0 && k_grp % E == 0) atomicOr(&tab[k_grp / E * 32], pos);          // a chunk's first code bit
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const bool in = whole || ((uint32_t)i >= first && (uint32_t)i < last);
+            const uint32_t canon = ((i & 1) ? x[i / 2] : x[i / 2] << 16) & kMask, rank = s_rank[lanes_code(x, i)];
+            f = __funnelshift_l(f, f, 4) | (in ? canon : 0u);
+            off += in ? rank + 1u : 0u;
+            bits |= in && off <= 32u ? 0x80000000u >> (off - 1u) : 0u;
+        }
+        f = __funnelshift_l(f, f, 4);
+        if (!whole || fl_shared) atomicOr(&fl[(k_grp >> 3) * 32], f);
+        else fl[(k_grp >> 3) * 32] = f;
+        fl_shared = false;
+        if (off <= 32u) {
+            append(bits, off);
+        } else {
+#pragma unroll 1
+            for (uint32_t i = first; i < last; ++i) {
+                uint32_t len = s_rank[(uint32_t)(*reinterpret_cast<const uint16_t*>(mine + at + i * 2)) >> 7] + 1u;
+                for (; len > 32u; len -= 32u) append(0u, 32u);
+                append(0x80000000u >> (len - 1u), len);
+            }
+        }
+        k_grp += 8;
+    };
+    const int w_end = min(nw, b1 * (kBlkCols / 32));
+    LanesTile<V> t;
+#pragma unroll 1
+    for (int w = b0 * (kBlkCols / 32); w < w_end; w += kTileWords) {
+        uint32_t bm[kTileWords];
+#pragma unroll
+        for (int j = 0; j < kTileWords; ++j) {
+            bm[j] = bm_word(w + j);
+            if (w + j < nw) bmo[(w + j) * 32] = bm[j];
+        }
+        t.ask(W, g.n, g.k, row0, (w0 + w) * 32, lane);      // (a tile ahead: 88 registers instead of 60, 83 -> 88 us)
+        t.put(lane, tile);
+        uint32_t to = k - k_grp;                                         // place in the list: behind the values left (or skipped)
+        uint8_t* p = mine + to * 2;
+#pragma unroll
+        for (int j = 0; j < kTileWords; ++j) {
+            const uint32_t pc = __popc(bm[j]);
+            while (k_next < k + pc) {                                    // a chunk begins in these columns
+                uint32_t m = bm[j];
+                for (uint32_t i = k_next - k; i > 0; --i) m &= ~(0x80000000u >> __clz(m));
+                tab[k_next / E * 32] = (uint32_t)((w + j) * 32 + __clz(m)) << 20;
+                k_next += E;
+            }
+            k += pc;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t x[4];
+                lanes_get8(mine + 16 + j * 64 + q * 16, x);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    *reinterpret_cast<uint16_t*>(p) = (uint16_t)((i & 1) ? x[i / 2] >> 16 : x[i / 2]);
+                    p += bm[j] & (0x80000000u >> (q * 8 + i)) ? 2 : 0;
+                }
+            }
+        }
+        __syncwarp();
+        uint32_t at = 0;
+        if (skip > 0 && k - k_grp >= 8u) {                               // the group that the warp before began
+            group(0, skip, 8, std::false_type{});
+            skip = 0;
+            at = 16;
+        }
+        for (; skip == 0 && k - k_grp >= 8u; at += 16) group(at, 0, 8, std::true_type{});
+        if (at > 0) *reinterpret_cast<uint4*>(mine) = *reinterpret_cast<const uint4*>(mine + at);      // up to 7 values left
+        __syncwarp();
+    }
+    if (k > k_grp + skip) group(0, skip, k - k_grp, std::false_type{});
+    if (pos & 31u) atomicOr(&un[(pos >> 5) * 32], acc);
 }
 
 // ---- E5: directory (exclusive scan of superblock sizes) and header -------------------------------------
@@ -738,8 +1034,22 @@ extern "C" int cass_encode_weights(const cass_format* fmt, const void* W_bf16, c
         CASS_PDL_LAUNCH(k_codebook, dim3(1), dim3(256), 0, stream, (const unsigned long long*)ws.hist, (uint8_t*)blob + kBlobHeaderBytes,
                         ws.exp_to_rank);
     }
-    CASS_PDL_LAUNCH(k_sizes, dim3((unsigned)n_sb), dim3(1024), 0, stream, W, g, (const uint32_t*)ws.keepbm, (const uint8_t*)ws.exp_to_rank,
-                    ws.sb_size);
+    // rows on 16-byte, 4-byte or 2-byte boundaries
+    const uintptr_t ends = (uintptr_t)W | ((uintptr_t)g.k * 2);
+    if (g.lanes) {
+        auto sizes = [&](auto piece) -> int {
+            using V = decltype(piece);
+            CASS_ALLOW_SMEM(k_sizes_lanes<V>);
+            CASS_PDL_LAUNCH(k_sizes_lanes<V>, dim3((unsigned)n_sb), dim3(32 * kSizeWarps), (size_t)(kSizeWarps * kLaneTile), stream, W, g,
+                            (const uint32_t*)ws.keepbm, (const uint8_t*)ws.exp_to_rank, ws.sb_size, ws.blk_size);
+            return CASS_OK;
+        };
+        rc = ends % 16 == 0 ? sizes(uint4{}) : ends % 4 == 0 ? sizes(uint32_t{}) : sizes(uint16_t{});
+        if (rc) return rc;
+    } else {
+        CASS_PDL_LAUNCH(k_sizes, dim3((unsigned)n_sb), dim3(1024), 0, stream, W, g, (const uint32_t*)ws.keepbm, (const uint8_t*)ws.exp_to_rank,
+                        ws.sb_size);
+    }
     CASS_PDL_LAUNCH(k_directory, dim3(1), dim3(1024), 0, stream, g, (const uint2*)ws.sb_size, b32, (unsigned long long)blob_cap,
                     ws.abort_flag, d_status);
     auto launch_pack = [&](auto pack, int threads) -> int {
@@ -749,10 +1059,27 @@ extern "C" int cass_encode_weights(const cass_format* fmt, const void* W_bf16, c
                         (const uint8_t*)ws.exp_to_rank, b32, (const uint32_t*)ws.abort_flag);
         return CASS_OK;
     };
+    if (g.lanes) {
+        // warps a superblock: some 3000 of them in all, no more than it has blocks
+        const int blks = ceil_div(g.seg_cols, kBlkCols), nw = blks <= 2 ? 2 : blks <= 4 || n_sb >= 750 ? 4 : blks <= 8 || n_sb >= 375 ? 8 : 16;
+        auto pack_as = [&](auto warps, auto piece) -> int {
+            constexpr int NW = decltype(warps)::value;
+            using V = decltype(piece);
+            CASS_ALLOW_SMEM(k_pack_lanes<NW, V>);
+            CASS_PDL_LAUNCH((k_pack_lanes<NW, V>), dim3((unsigned)n_sb), dim3(32 * NW), (size_t)(NW * kLaneTile), stream, W, g, (const uint32_t*)ws.keepbm,
+                            (const uint8_t*)ws.exp_to_rank, (const uint32_t*)ws.blk_size, b32, (const uint32_t*)ws.abort_flag);
+            return CASS_OK;
+        };
+        auto pack = [&](auto piece) {
+            return nw == 2 ? pack_as(std::integral_constant<int, 2>{}, piece) : nw == 4 ? pack_as(std::integral_constant<int, 4>{}, piece)
+                   : nw == 8 ? pack_as(std::integral_constant<int, 8>{}, piece) : pack_as(std::integral_constant<int, 16>{}, piece);
+        };
+        return ends % 16 == 0 ? pack(uint4{}) : ends % 4 == 0 ? pack(uint32_t{}) : pack(uint16_t{});
+    }
     if (n_sb <= kSms) rc = g.mx ? (g.t == 4 ? launch_pack(k_pack<true, 4, 1024>, 1024) : launch_pack(k_pack<true, -1, 1024>, 1024))
                                : (g.t == 4 ? launch_pack(k_pack<false, 4, 1024>, 1024) : launch_pack(k_pack<false, -1, 1024>, 1024));
     else rc = g.mx ? (g.t == 4 ? launch_pack(k_pack<true, 4, 512>, 512) : launch_pack(k_pack<true, -1, 512>, 512))
-                   : (g.t == 4 ? launch_pack(k_pack<false, 4, 512>, 512) : launch_pack(k_pack<false, -1, 512>, 512));
+                   : launch_pack(k_pack<false, -1, 512>, 512);      // t = 4: by lanes
     if (rc) return rc;
     return CASS_OK;
 }

@@ -75,6 +75,23 @@ def test_rows_in_turn(cass, rows, cols):
     assert torch.equal(dec, torch.where(keep, trunc, torch.zeros_like(w)))
 
 
+@pytest.mark.parametrize("rows,cols,p,seg,chunk", [(9000, 520, 400, 0, 0), (41601, 200, 400, 0, 0), (21000, 470, 300, 0, 0), (2310, 2569, 400, 0, 0),
+                                                    (2310, 2570, 600, 0, 0), (1100, 5300, 0, 0, 0), (3000, 2056, 400, 1024, 32), (1480, 4100, 990, 0, 0)])
+def test_blobs_by_lanes(cass, rows, cols, p, seg, chunk):
+    """Matrices of so many blocks that sizes and packing go by lanes: 2 to 16 warps a superblock, rows on 16-, 4- and 2-byte
+    boundaries, chunks of few values, a last row block that is not full; rows of one value, of none, and with codes longer than a word."""
+    w = synth.student_t_weight(rows, cols, 2, f"lanes/{rows}x{cols}").float()
+    w[1] = 0.25
+    w[2] = 0.0
+    w[3, ::7] *= torch.exp2(torch.arange(len(w[3, ::7]), dtype=torch.float32) % 120 - 60)
+    w[5, : cols // 2] = 0.0
+    w[-1] *= 2.0 ** 20
+    w = w.to(torch.bfloat16)
+    act = (np.abs(np.random.default_rng(cols).standard_normal(cols)) + 0.05).astype(np.float32)
+    got = _blob(cass, w, act, cass.default_format(w_p=p, seg_cols=seg, chunk_cols=chunk))
+    assert np.array_equal(got, layout.encode_weight_blob(_bits(w), act, p, 4, *((seg, chunk) if seg else ()))[0])
+
+
 def test_constant_rows_and_no_pruning(cass):
     w = torch.full((40, 3000), 0.5, dtype=torch.bfloat16)
     w[7] = 0.0
