@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
     __shared__ __align__(16) int s_lim[NP];
     __shared__ __align__(16) uint32_t s_at[NP];
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int G = n_q / n_kv, P = rows * G;
     const int qkv_dim = (n_q + 2 * n_kv) * kVtD;
     if (tid == 0) {
@@ -112,47 +112,48 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
     const uint32_t tmem = *tmem_slot;
     bool ok = true;
 
-    if (warp == 1 && lane == 0) {
-        // ---- scores^T = K . Q^T: A = K tile (K-major over d), B = Q (K-major over d) ----
-        if (mbar_wait_bounded(bar_k, 0)) {
-            tc_fence_after();
-            constexpr uint32_t idesc1 = tc_idesc_mn(kVtTok, kVtPairs, false);
+    if (warp == 1) {
+        if (tc_elect()) {
+            // ---- scores^T = K . Q^T: A = K tile (K-major over d), B = Q (K-major over d) ----
+            if (mbar_wait_bounded(bar_k, 0)) {
+                tc_fence_after();
+                constexpr uint32_t idesc1 = tc_idesc_mn(kVtTok, kVtPairs, false);
 #pragma unroll
-            for (int kb = 0; kb < 2; ++kb) {
-                const uint64_t ad = tc_smem_desc(sK + kb * kVtTileBytes), bd = tc_smem_desc(sQ + kb * kVtQBytes);
+                for (int kb = 0; kb < 2; ++kb) {
+                    const uint64_t ad = tc_smem_desc(sK + kb * kVtTileBytes), bd = tc_smem_desc(sQ + kb * kVtQBytes);
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    tc_mma(tmem, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc1, (uint32_t)((kb | kk) != 0));
+                    for (int kk = 0; kk < 4; ++kk)
+                        tc_mma(tmem, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), idesc1, (uint32_t)((kb | kk) != 0));
+                }
+            } else {
+                atomicExch(d_status, CASS_ERR_TIMEOUT); ok = false;
             }
-        } else {
-            atomicExch(d_status, CASS_ERR_TIMEOUT); ok = false;
-        }
-        if (!ok) {                                     // what is in flight lands before the CTA ends (bounded)
-            mbar_wait_bounded(bar_k, 0);
-            mbar_wait_bounded(bar_v, 0);
-        }
-        tc_commit(bar_s);
-        // ---- out^T = V^T . P^T: A = V tile as stored (rows = tokens: M-contiguous), B = P (K-major over tokens) ----
-        if (ok && mbar_wait_bounded(bar_v, 0) && mbar_wait_bounded(bar_p, 0)) {
-            tc_fence_after();
-            constexpr uint32_t idesc2 = tc_idesc_mn(kVtD, kVtPairs, true);
-#pragma unroll
-            for (int kk = 0; kk < kVtTok / 16; ++kk) {                   // 16 tokens per MMA
-                // A: 16 token rows of 128 bytes = 2048 bytes further per step; the second 64-dim block is the other box
-                const uint64_t ad = tc_smem_desc(sV + kk * 2048, kVtTileBytes);
-                // B: block kk / 4 of P (64 tokens each), 32 bytes per 16 tokens inside the swizzled row
-                const uint64_t bd = tc_smem_desc(sP + (kk >> 2) * kVtQBytes) + (uint64_t)((kk & 3) * 2);
-                tc_mma(tmem + (uint32_t)NP, ad, bd, idesc2, (uint32_t)(kk != 0));
-                if (two_terms)
-                    tc_mma(tmem + (uint32_t)NP, ad, tc_smem_desc(sQ + (kk >> 2) * kVtQBytes) + (uint64_t)((kk & 3) * 2), idesc2, 1u);
+            if (!ok) {                                     // what is in flight lands before the CTA ends (bounded)
+                mbar_wait_bounded(bar_k, 0);
+                mbar_wait_bounded(bar_v, 0);
             }
-        } else if (ok) {
-            atomicExch(d_status, CASS_ERR_TIMEOUT);
-            mbar_wait_bounded(bar_v, 0);
+            tc_commit(bar_s);
+            // ---- out^T = V^T . P^T: A = V tile as stored (rows = tokens: M-contiguous), B = P (K-major over tokens) ----
+            if (ok && mbar_wait_bounded(bar_v, 0) && mbar_wait_bounded(bar_p, 0)) {
+                tc_fence_after();
+                constexpr uint32_t idesc2 = tc_idesc_mn(kVtD, kVtPairs, true);
+#pragma unroll
+                for (int kk = 0; kk < kVtTok / 16; ++kk) {                   // 16 tokens per MMA
+                    // A: 16 token rows of 128 bytes = 2048 bytes further per step; the second 64-dim block is the other box
+                    const uint64_t ad = tc_smem_desc(sV + kk * 2048, kVtTileBytes);
+                    // B: block kk / 4 of P (64 tokens each), 32 bytes per 16 tokens inside the swizzled row
+                    const uint64_t bd = tc_smem_desc(sP + (kk >> 2) * kVtQBytes) + (uint64_t)((kk & 3) * 2);
+                    tc_mma(tmem + (uint32_t)NP, ad, bd, idesc2, (uint32_t)(kk != 0));
+                    if (two_terms)
+                        tc_mma(tmem + (uint32_t)NP, ad, tc_smem_desc(sQ + (kk >> 2) * kVtQBytes) + (uint64_t)((kk & 3) * 2), idesc2, 1u);
+                }
+            } else if (ok) {
+                atomicExch(d_status, CASS_ERR_TIMEOUT);
+                mbar_wait_bounded(bar_v, 0);
+            }
+            tc_commit(bar_o);
         }
-        tc_commit(bar_o);
-    }
-    else if (warp >= 2) {
+    } else if (warp >= 2) {
         const int q = warp & 3;                       // the tensor-memory lane quarter this warp may read
         const int et = q * 32 + lane;                 // this thread's token (scores) and dim (output)
         const float scale = rsqrtf((float)kVtD);
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(kVtThreads) k_verify_attn_tc(const __grid_cons
             atomicExch(d_status, CASS_ERR_TIMEOUT);
         }
     }
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {

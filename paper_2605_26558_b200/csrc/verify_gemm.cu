@@ -7,6 +7,9 @@
 // BNx64 activation tile through a ring of TMA loads (128-byte swizzle), warp 1 issues the MMAs, warps 2-5 read the
 // accumulator back and store fp32 partial sums; a second kernel adds the K ranges in fixed order.
 //
+// The issuing threads are found by elect.sync: of a thread found by its lane the compiler does not know that it is alone, and wraps
+// every issue in a loop (20 rows of two Qwen-shaped layers 558 -> 549 us).
+//
 // Row-count invariance: an accumulator column belongs to one token row, the tile shape, the K ranges and the order
 // of the MMAs depend on (n, k) only, so a row gives the same bits whether it is verified alone or with others.
 #include "tc.cuh"
@@ -43,7 +46,7 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
     uint64_t* acc_ready = empty + kTcStages;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_ready + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int m0 = blockIdx.x * kTcBM, ks = blockIdx.y;
     const int kb0 = ks * kb_per_split;
     const int nkb = min(kb_per_split, kb_total - kb0);
@@ -68,10 +71,10 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
     // (kWeightsInput: a caller's matrix, which a preceding kernel may be writing: its first tiles are asked for as far as L2,
     // where a later write still finds them; memory is then busy while the previous call's parts are added: 12.1 instead of
     // 13.1 us a call on 6144 x 4096)
-    if (warp == 0 && lane == 0 && w_static == kWeightsInput) {
+    if (warp == 0 && w_static == kWeightsInput && tc_elect()) {
         for (int kb = 0; kb < n_pre; ++kb) tma_prefetch_2d(&map_w, (kb0 + kb) * kTcBK, m0);
     }
-    if (warp == 0 && lane == 0 && w_static == kWeightsStatic) {
+    if (warp == 0 && w_static == kWeightsStatic && tc_elect()) {
         for (int kb = 0; kb < n_pre; ++kb) {                 // stages are empty at the start: nothing to wait for
             mbar_expect_tx(&full[kb], kTcABytes + kTcBBytes);
             tma_load_2d(sA + kb * kTcABytes, &map_w, (kb0 + kb) * kTcBK, m0, &full[kb]);
@@ -80,45 +83,49 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
     pdl_wait();
     pdl_early<5>();
 
-    if (warp == 0 && lane == 0) {
-        // ---- producer: TMA loads into the ring ----
-        for (int kb = 0; kb < n_pre; ++kb) {
-            if (w_static != kWeightsStatic) {
-                mbar_expect_tx(&full[kb], kTcABytes + kTcBBytes);
-                tma_load_2d(sA + kb * kTcABytes, &map_w, (kb0 + kb) * kTcBK, m0, &full[kb]);
+    if (warp == 0) {
+        if (tc_elect()) {
+            // ---- producer: TMA loads into the ring ----
+            for (int kb = 0; kb < n_pre; ++kb) {
+                if (w_static != kWeightsStatic) {
+                    mbar_expect_tx(&full[kb], kTcABytes + kTcBBytes);
+                    tma_load_2d(sA + kb * kTcABytes, &map_w, (kb0 + kb) * kTcBK, m0, &full[kb]);
+                }
+                tma_load_2d(sB + kb * kTcBBytes, &map_x, (kb0 + kb) * kTcBK, 0, &full[kb]);
             }
-            tma_load_2d(sB + kb * kTcBBytes, &map_x, (kb0 + kb) * kTcBK, 0, &full[kb]);
-        }
-        for (int kb = n_pre; kb < nkb; ++kb) {
-            const int s = kb % kTcStages;
-            const uint32_t ph = (uint32_t)(kb / kTcStages) & 1u;
-            if (!mbar_wait_bounded(&empty[s], ph ^ 1u)) { atomicExch(d_status, CASS_ERR_TIMEOUT); break; }
-            mbar_expect_tx(&full[s], kTcABytes + kTcBBytes);
-            tma_load_2d(sA + s * kTcABytes, &map_w, (kb0 + kb) * kTcBK, m0, &full[s]);
-            tma_load_2d(sB + s * kTcBBytes, &map_x, (kb0 + kb) * kTcBK, 0, &full[s]);
-        }
-    } else if (warp == 1 && lane == 0) {
-        // ---- MMA issuer ----
-        bool ok = true;
-        for (int kb = 0; kb < nkb && ok; ++kb) {
-            const int s = kb % kTcStages;
-            const uint32_t ph = (uint32_t)(kb / kTcStages) & 1u;
-            if (!mbar_wait_bounded(&full[s], ph)) {
-                atomicExch(d_status, CASS_ERR_TIMEOUT);
-                ok = false;
-                for (int j = kb; j < nkb && j < kb + kTcStages; ++j)          // what is in flight lands before the CTA ends (bounded)
-                    mbar_wait_bounded(&full[j % kTcStages], (uint32_t)(j / kTcStages) & 1u);
-                break;
+            for (int kb = n_pre; kb < nkb; ++kb) {
+                const int s = kb % kTcStages;
+                const uint32_t ph = (uint32_t)(kb / kTcStages) & 1u;
+                if (!mbar_wait_bounded(&empty[s], ph ^ 1u)) { atomicExch(d_status, CASS_ERR_TIMEOUT); break; }
+                mbar_expect_tx(&full[s], kTcABytes + kTcBBytes);
+                tma_load_2d(sA + s * kTcABytes, &map_w, (kb0 + kb) * kTcBK, m0, &full[s]);
+                tma_load_2d(sB + s * kTcBBytes, &map_x, (kb0 + kb) * kTcBK, 0, &full[s]);
             }
-            tc_fence_after();
-            const uint64_t ad = tc_smem_desc(sA + s * kTcABytes), bd = tc_smem_desc(sB + s * kTcBBytes);
+        }
+    } else if (warp == 1) {
+        if (tc_elect()) {
+            // ---- MMA issuer ----
+            bool ok = true;
+            for (int kb = 0; kb < nkb && ok; ++kb) {
+                const int s = kb % kTcStages;
+                const uint32_t ph = (uint32_t)(kb / kTcStages) & 1u;
+                if (!mbar_wait_bounded(&full[s], ph)) {
+                    atomicExch(d_status, CASS_ERR_TIMEOUT);
+                    ok = false;
+                    for (int j = kb; j < nkb && j < kb + kTcStages; ++j)          // what is in flight lands before the CTA ends (bounded)
+                        mbar_wait_bounded(&full[j % kTcStages], (uint32_t)(j / kTcStages) & 1u);
+                    break;
+                }
+                tc_fence_after();
+                const uint64_t ad = tc_smem_desc(sA + s * kTcABytes), bd = tc_smem_desc(sB + s * kTcBBytes);
 #pragma unroll
-            for (int kk = 0; kk < kTcBK / 16; ++kk)      // 16 bf16 = 32 bytes along K inside the swizzle row: +2 in the address field
-                tc_mma(tmem, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), kIdesc, (uint32_t)((kb | kk) != 0));
-            tc_commit(&empty[s]);                        // frees the stage once these MMAs have read it
+                for (int kk = 0; kk < kTcBK / 16; ++kk)      // 16 bf16 = 32 bytes along K inside the swizzle row: +2 in the address field
+                    tc_mma(tmem, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 2), kIdesc, (uint32_t)((kb | kk) != 0));
+                tc_commit(&empty[s]);                        // frees the stage once these MMAs have read it
+            }
+            tc_commit(acc_ready);                            // accumulator complete (or abandoned after a time-out)
         }
-        tc_commit(acc_ready);                            // accumulator complete (or abandoned after a time-out)
-    } else if (warp >= 2) {
+    } else {
         // ---- epilogue: warp w may read the 32 accumulator lanes of quarter w % 4 ----
         if (mbar_wait_bounded(acc_ready, 0)) {
             __syncwarp();
@@ -139,6 +146,7 @@ __global__ void __launch_bounds__(kTcThreads) k_verify_gemm_tc(const __grid_cons
             atomicExch(d_status, CASS_ERR_TIMEOUT);
         }
     }
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
