@@ -20,17 +20,25 @@ namespace cg = cooperative_groups;
 namespace cass {
 
 constexpr int kGemvStages = 1;         // stages of the copy ring per CTA; several CTAs share an SM, so their copies and decodes overlap
-constexpr int kXSlack = 288;           // readable floats after the x slice: a window walk may run up to 8 x 32 + 8 columns past its start
-
-static size_t gemv_stage_bytes(const cass_blob_info& bi) { return align_up((size_t)bi.max_superblock_bytes + 384, 512); }
+constexpr int kXSlack = 288;           // a window walk may look up to 8 x 32 + 8 columns past its start: what lies behind the x slice there is not used
 
 // Bytes per column of the x slice in shared memory: one vector is kept as fp32, several as packed bf16 [col][nb].
 __host__ __device__ constexpr int x_col_bytes(int nb) { return nb == 1 ? 4 : 2 * nb; }
+__host__ __device__ constexpr uint32_t x_slice_bytes(int seg_cols, int nb) { return (uint32_t)(seg_cols * x_col_bytes(nb) + 511) / 512 * 512; }
 
+// Shared memory, up to two vectors: superblock, x slice and slack, table, the chunks' sums (twice).  More: x slice, superblock, table; the
+// slack is the superblock, and the sums take its place once it has been read: slack and sums (4.6 and 8 KB of 8 vectors) are the room of a
+// third CTA on an SM (5120 x 13824, eight Cassandra-2 vectors: 96 -> 82 us with it and the paired multiply-adds).
+__host__ __device__ constexpr bool gemv_compact(int nb) { return nb >= 4; }
+static size_t gemv_stage_bytes(const cass_blob_info& bi, int nb) {
+    const size_t sums = !gemv_compact(nb) ? 0 : (size_t)nb * ceil_div(bi.seg_cols, bi.chunk_cols) * 32 * 4, body = (size_t)bi.max_superblock_bytes + 384;
+    return align_up(body > sums ? body : sums, 512);
+}
 static size_t gemv_smem_bytes(const cass_blob_info& bi, int nb) {
     const int n_ch = ceil_div(bi.seg_cols, bi.chunk_cols);
-    return kGemvStages * gemv_stage_bytes(bi) + (size_t)(bi.seg_cols + kXSlack) * x_col_bytes(nb) + 256 * 4 +
-           (size_t)(nb < 2 ? 2 : nb) * n_ch * 32 * 4 + 64;
+    const size_t stage = kGemvStages * gemv_stage_bytes(bi, nb), table = 256 * 4 + 64, slack = (size_t)kXSlack * x_col_bytes(nb);
+    if (!gemv_compact(nb)) return stage + (size_t)bi.seg_cols * x_col_bytes(nb) + slack + table + (size_t)2 * n_ch * 32 * 4;
+    return x_slice_bytes(bi.seg_cols, nb) + (stage + table > slack ? stage + table : slack);
 }
 
 // With what the kernel declares itself: a segment's sums, the tile's sizes and flags, up to where the dynamic part may begin.
@@ -75,24 +83,35 @@ __device__ __forceinline__ XRaw<NB> x_load(uint32_t addr) {
     return r;
 }
 
-template <int NB>
+// PAIRS: two multiply-adds an instruction, each rounded as one by itself.  28672 x 4096: four vectors 77 -> 69 us, two 60 -> 57, but two
+// Cassandra-2 vectors, whose CTAs then take more registers than five an SM leave, 46.7 -> 49.5; and where latency is all, two vectors
+// 7.1 -> 8.0 for 1376 x 256 and 10.4 -> 11.4 for 700 x 3000.
+template <int NB, bool PAIRS>
 __device__ __forceinline__ void x_fma(const XRaw<NB>& r, uint32_t wb, float (&acc)[NB]) {
-    const float w = __uint_as_float(wb);
     if constexpr (NB == 1) {
-        acc[0] = fmaf(w, __uint_as_float(r.w[0]), acc[0]);
-    } else {
+        acc[0] = fmaf(__uint_as_float(wb), __uint_as_float(r.w[0]), acc[0]);
+    } else if constexpr (!PAIRS) {
+        const float w = __uint_as_float(wb);
 #pragma unroll
         for (int i = 0; i < NB / 2; ++i) {
             acc[2 * i] = fmaf(w, __uint_as_float(r.w[i] << 16), acc[2 * i]);
             acc[2 * i + 1] = fmaf(w, __uint_as_float(r.w[i] & 0xFFFF0000u), acc[2 * i + 1]);
         }
+    } else {
+        unsigned long long ww;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(ww) : "r"(wb));
+#pragma unroll
+        for (int i = 0; i < NB / 2; ++i)
+            asm("{\n\t.reg .b64 a, x;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 x, {%3, %4};\n\tfma.rn.f32x2 a, %2, x, a;\n\tmov.b64 {%0, %1}, a;\n\t}"
+                : "+f"(acc[2 * i]), "+f"(acc[2 * i + 1])
+                : "l"(ww), "r"(r.w[i] << 16), "r"(r.w[i] & 0xFFFF0000u));
     }
 }
 
 // Careful walk of `count` (<= 8) kept values of one row from column bpos / code bit upos on: any gap between
 // kept columns, any codeword length.  Used for the rare groups that do not fit the 32-bit windows.
 // flC: the segment's first field word of this row; k0: index (inside the segment) of the group's first value.
-template <int T, int NB>
+template <int T, int NB, bool PAIRS>
 __device__ __noinline__ WalkState<NB> group_slow(const uint32_t* bmS, const uint32_t* unS, const uint32_t* flC, uint32_t k0, int count,
                                                  WalkState<NB> st, uint32_t bpos_lim, uint32_t upos_lim, const float* xs,
                                                  const uint32_t* lut) {
@@ -114,7 +133,7 @@ __device__ __noinline__ WalkState<NB> group_slow(const uint32_t* bmS, const uint
         uint32_t a;
         if constexpr (32 % F == 0) a = __funnelshift_l(fword, fword, (F * (k % PER)) & 31) & MASK;
         else a = packed_field_f32<T>(fword, k % PER);
-        x_fma<NB>(xv, a | lut[rank & 255], st.acc);
+        x_fma<NB, PAIRS>(xv, a | lut[rank & 255], st.acc);
     }
     return st;
 }
@@ -144,7 +163,7 @@ __device__ __forceinline__ uint32_t lds_u32_off(uint32_t addr) {
 // slots 73 %, searches 70 %, shared memory 64 %, integer pipe 55 % busy.  Clearing the used bit with a shift and a mask, positions kept
 // absolute and a code window for every 4 values took 19: 58.6 -> 53.0 us on 28672 x 4096 with the results added in the kernel.
 // Finding some terminators by a conversion to float instead of a search: 54.5 to 56 us.
-template <int T, int NB, bool WIDE>
+template <int T, int NB, bool WIDE, bool PAIRS>
 __device__ __forceinline__ void chunk_dot_fast(const uint32_t* __restrict__ sb, const SbGeom& g, int ch, int lane,
                                                int chunk_elems, const float* __restrict__ xs,
                                                const uint32_t* __restrict__ lut, float (&acc)[NB]) {
@@ -218,10 +237,10 @@ __device__ __forceinline__ void chunk_dot_fast(const uint32_t* __restrict__ sb, 
                 wb = packed_field_f32<T>(fword, jj - wsel * PER) | eb;
             }
             if constexpr (!tail) {
-                x_fma<NB>(xv, wb, acc);
+                x_fma<NB, PAIRS>(xv, wb, acc);
                 if (j == kGroupCodes - 1) dry |= WIDE ? p | q : q;
             } else if (e < rem) {
-                x_fma<NB>(xv, wb, acc);
+                x_fma<NB, PAIRS>(xv, wb, acc);
                 dry |= p | q;
             }
         };
@@ -245,7 +264,7 @@ __device__ __forceinline__ void chunk_dot_fast(const uint32_t* __restrict__ sb, 
         }
         if ((int32_t)dry < 0) {
             st0.bpos = (xc0 - xs_a) >> XL;
-            const WalkState<NB> r = group_slow<T, NB>(bmS, unS, flS, (uint32_t)(ch * chunk_elems + grp * kGroupCols), min(rem, kGroupCols),
+            const WalkState<NB> r = group_slow<T, NB, PAIRS>(bmS, unS, flS, (uint32_t)(ch * chunk_elems + grp * kGroupCols), min(rem, kGroupCols),
                                                       st0, (xc_lim - xs_a) >> XL, upos_lim, xs, lut);
 #pragma unroll
             for (int b = 0; b < NB; ++b) acc[b] = r.acc[b];
@@ -270,7 +289,7 @@ __device__ __forceinline__ void chunk_dot_fast(const uint32_t* __restrict__ sb, 
 // Same bitmap walk as above; the unary parse is replaced by a 16-entry table look-up of the signed magnitude, and a
 // block's 32 products are summed first and scaled by the block's power of two once (Sec. 5.1, MX decoder: the shared
 // exponent is broadcast to the elements of its block).
-template <int NB>
+template <int NB, bool PAIRS>
 __device__ __noinline__ WalkState<NB> group_slow_mx(const uint32_t* bmS, uint32_t fword, int count, WalkState<NB> st,
                                                     uint32_t bpos_lim, const float* xs, const float* nlut) {
     for (int e = 0; e < count; ++e) {
@@ -283,12 +302,12 @@ __device__ __noinline__ WalkState<NB> group_slow_mx(const uint32_t* bmS, uint32_
         if (!found) break;
         const XRaw<NB> xv = x_load<NB>(smem_u32(xs) + st.bpos * (uint32_t)x_col_bytes(NB));
         st.bpos += 1;
-        x_fma<NB>(xv, __float_as_uint(nlut[(fword >> (28 - 4 * e)) & 15u]), st.acc);
+        x_fma<NB, PAIRS>(xv, __float_as_uint(nlut[(fword >> (28 - 4 * e)) & 15u]), st.acc);
     }
     return st;
 }
 
-template <int NB, bool WIDE>
+template <int NB, bool WIDE, bool PAIRS>
 __device__ __forceinline__ void chunk_dot_mx4(const uint32_t* __restrict__ sb, const SbGeom& g, int ch, int lane,
                                               int chunk_elems, const float* __restrict__ xs,
                                               const float* __restrict__ nlut, float (&acc)[NB]) {
@@ -333,9 +352,9 @@ __device__ __forceinline__ void chunk_dot_mx4(const uint32_t* __restrict__ sb, c
             const uint32_t off = e < 7 ? (fword >> (26 - 4 * e)) : (fword << 2);
             const uint32_t wb = lds_u32((off & 0x3Cu) | nl_a);                         // +-(magnitude << 4) as a float
             if constexpr (!tail) {
-                x_fma<NB>(xv, wb, blk);
+                x_fma<NB, PAIRS>(xv, wb, blk);
             } else if (e < rem) {
-                x_fma<NB>(xv, wb, blk);
+                x_fma<NB, PAIRS>(xv, wb, blk);
                 dry |= p;
             }
         };
@@ -353,7 +372,7 @@ __device__ __forceinline__ void chunk_dot_mx4(const uint32_t* __restrict__ sb, c
         else dry |= p;
         if ((int32_t)dry < 0) {
             st0.bpos = (xc0 - xs_a) >> XL;
-            const WalkState<NB> r = group_slow_mx<NB>(bmS, fword, min(rem, kGroupCols), st0, (xc_lim - xs_a) >> XL, xs, nlut);
+            const WalkState<NB> r = group_slow_mx<NB, PAIRS>(bmS, fword, min(rem, kGroupCols), st0, (xc_lim - xs_a) >> XL, xs, nlut);
 #pragma unroll
             for (int b = 0; b < NB; ++b) blk[b] = r.acc[b];
             xc = xs_a + (r.bpos << XL);
@@ -386,7 +405,7 @@ __device__ __forceinline__ void chunk_dot_mx4(const uint32_t* __restrict__ sb, c
 // Launch bounds: a blob may have chunks for 1024 threads, and the compiler then likes to fit two such CTAs, 32 registers a thread.
 // Told that one is enough it takes 48 to 55 for two Cassandra-2 vectors, whose walk does not fit 32 without a spill (5120 x 13824:
 // 37 to 39 us at 32 registers, as the rest of the kernel falls, 34.7 so).
-template <int T, int NB, bool WIDE>
+template <int T, int NB, bool WIDE, bool PAIRS>
 __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gemv(const uint32_t* __restrict__ blob, const uint16_t* __restrict__ x,
                                                      float* __restrict__ partial, int32_t* __restrict__ d_status,
                                                      int stage_bytes, int max_sb, int n, int k, int t, int seg_cols,
@@ -420,10 +439,14 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
         const int seg = blockIdx.x, rb0 = blockIdx.y, rb_step = gridDim.y;
         const int tid = threadIdx.x, warp = tid >> 5, n_warps = blockDim.x >> 5;
 
-        float* xs = reinterpret_cast<float*>(smem_raw + (size_t)kGemvStages * stage_bytes);
-        uint32_t* lut = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(xs) + (size_t)(seg_cols + kXSlack) * x_col_bytes(NB));
-        float* red = reinterpret_cast<float*>(lut + 256);                       // NB = 1: [2][n_warps][32], else [NB][n_warps][32]
-        uint64_t* bar = reinterpret_cast<uint64_t*>(red + (NB < 2 ? 2 : NB) * n_warps * 32);    // [kGemvStages]
+        constexpr bool kCompact = gemv_compact(NB);
+        uint8_t* stage0 = smem_raw + (kCompact ? x_slice_bytes(seg_cols, NB) : 0u);
+        float* xs = reinterpret_cast<float*>(kCompact ? smem_raw : smem_raw + (size_t)kGemvStages * stage_bytes);
+        uint32_t* lut = reinterpret_cast<uint32_t*>(kCompact ? stage0 + (size_t)kGemvStages * stage_bytes
+                                                             : reinterpret_cast<uint8_t*>(xs) + (size_t)(seg_cols + kXSlack) * x_col_bytes(NB));
+        float* red = kCompact ? reinterpret_cast<float*>(stage0) : reinterpret_cast<float*>(lut + 256);      // NB = 1: [2][n_warps][32], else [NB][n_warps][32]
+        uint64_t* bar = reinterpret_cast<uint64_t*>(lut + 256 + (kCompact ? 0 : 2 * n_warps * 32));    // [kGemvStages]
+        const int x_cols = kCompact ? seg_cols : seg_cols + kXSlack;
         __shared__ int s_skip[kGemvStages], s_bad;
         __shared__ uint32_t s_dir[kGemvStages][3];          // sizes of the tile in each stage
 
@@ -464,7 +487,7 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
             s_skip[s] = 0;
             s_dir[s][0] = d1; s_dir[s][1] = d2; s_dir[s][2] = d3;
             const uint8_t* src = reinterpret_cast<const uint8_t*>(blob) + (size_t)d0 * 16;
-            uint8_t* dst = smem_raw + (size_t)s * stage_bytes;
+            uint8_t* dst = stage0 + (size_t)s * stage_bytes;
             mbar_expect_tx(&bar[s], bytes);
             for (uint32_t off = 0; off < bytes; off += 32768u) bulk_g2s(dst + off, src + off, min(32768u, bytes - off), &bar[s]);
         };
@@ -491,47 +514,59 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
         // projection.  x and the scratch `partial` are the predecessor's.
         pdl_wait();
         pdl_early<6>();
-        // x of this segment (fp32), zero beyond the matrix
-        const int c0 = seg * seg_cols;
-        if constexpr (NB > 1) {
-            // packed bf16 [col][NB]: all vectors' values of one column side by side
-            uint16_t* xs16 = reinterpret_cast<uint16_t*>(xs);
-            if ((k & 7) == 0 && ((uintptr_t)x & 15) == 0) {
-                const int n_oct = (seg_cols + kXSlack) / 8;
-                for (int it = tid; it < n_oct * NB; it += blockDim.x) {
-                    const int i = (it / NB) * 8, b = it % NB;
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (i < scols && c0 + i < k) v = *reinterpret_cast<const uint4*>(x + (size_t)b * k + c0 + i);
-                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        // x of this segment, zero beyond the matrix: eight columns of one vector a thread and turn.  (One value a turn where rows are off
+        // 16-byte boundaries, each turn a round trip: 17 us a call for 700 x 3000 and four vectors, 13 so; 28 and 17 for 2000 x 1500 and eight.)
+        const int c0 = seg * seg_cols, n_items = x_cols / 8 * NB;
+        auto put8 = [&](int it, const uint4& v) {
+            const int i = it / NB * 8;
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+            if constexpr (NB == 1) {                           // fp32
+                *reinterpret_cast<float4*>(xs + i) = make_float4(__uint_as_float(w[0] << 16), __uint_as_float(w[0] & 0xFFFF0000u),
+                                                                 __uint_as_float(w[1] << 16), __uint_as_float(w[1] & 0xFFFF0000u));
+                *reinterpret_cast<float4*>(xs + i + 4) = make_float4(__uint_as_float(w[2] << 16), __uint_as_float(w[2] & 0xFFFF0000u),
+                                                                     __uint_as_float(w[3] << 16), __uint_as_float(w[3] & 0xFFFF0000u));
+            } else {                                           // packed bf16 [col][NB]: all vectors' values of one column side by side
+                uint16_t* xs16 = reinterpret_cast<uint16_t*>(xs) + (size_t)i * NB + it % NB;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        xs16[(size_t)(i + 2 * q) * NB + b] = (uint16_t)(w[q] & 0xFFFFu);
-                        xs16[(size_t)(i + 2 * q + 1) * NB + b] = (uint16_t)(w[q] >> 16);
-                    }
-                }
-            } else {
-                for (int it = tid; it < (seg_cols + kXSlack) * NB; it += blockDim.x) {
-                    const int i = it / NB, b = it % NB, c = c0 + i;
-                    xs16[it] = (i < scols && c < k) ? x[(size_t)b * k + c] : (uint16_t)0;
+                for (int q = 0; q < 4; ++q) {
+                    xs16[2 * q * NB] = (uint16_t)(w[q] & 0xFFFFu);
+                    xs16[(2 * q + 1) * NB] = (uint16_t)(w[q] >> 16);
                 }
             }
-        } else if ((k & 7) == 0 && ((uintptr_t)x & 15) == 0) {
-            // eight values per 16-byte load: one round trip to L2 for the whole slice
-            for (int i = tid * 8; i < seg_cols + kXSlack; i += blockDim.x * 8) {
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (i < scols && c0 + i < k) v = *reinterpret_cast<const uint4*>(x + c0 + i);
-                float4 lo = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
-                                        __uint_as_float(v.y & 0xFFFF0000u));
-                float4 hi = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u), __uint_as_float(v.w << 16),
-                                        __uint_as_float(v.w & 0xFFFF0000u));
-                *reinterpret_cast<float4*>(xs + i) = lo;
-                *reinterpret_cast<float4*>(xs + i + 4) = hi;
+        };
+        const bool x_vec = (k & 7) == 0 && ((uintptr_t)x & 15) == 0;
+        auto get8 = [&](int it, bool vec) {
+            const int i = it / NB * 8, left = min(scols - i, k - c0 - i);
+            const uint16_t* p = x + (size_t)(it % NB) * k + c0 + i;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (vec) {
+                if (left > 0) v = __ldg(reinterpret_cast<const uint4*>(p));
+            } else {
+                uint32_t h[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) h[j] = j < left ? (uint32_t)__ldg(p + j) : 0u;
+                v = make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+            }
+            return v;
+        };
+        if constexpr (NB == 1) {
+            for (int it = tid; it < n_items; it += blockDim.x) put8(it, get8(it, x_vec));
+        } else if (x_vec) {                                    // two turns' loads under way
+            for (int it = tid; it < n_items; it += 2 * blockDim.x) {
+                uint4 v[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int at = it + u * blockDim.x, i = at / NB * 8;
+                    v[u] = make_uint4(0u, 0u, 0u, 0u);
+                    if (i < scols && c0 + i < k && at < n_items) v[u] = __ldg(reinterpret_cast<const uint4*>(x + (size_t)(at % NB) * k + c0 + i));
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (u == 0 || it + u * blockDim.x < n_items) put8(it + u * blockDim.x, v[u]);
             }
         } else {
-            for (int i = tid; i < seg_cols + kXSlack; i += blockDim.x) {
-                int c = c0 + i;
-                xs[i] = (i < scols && c < k) ? bf16_bits_to_float(x[c]) : 0.f;
-            }
+#pragma unroll 1
+            for (int it = tid; it < n_items; it += blockDim.x) put8(it, get8(it, false));
         }
         __syncthreads();
         if (s_bad) {
@@ -554,7 +589,7 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
                 lost = true;
             }
             lost = __any_sync(0xffffffffu, lost);
-            const uint32_t* sb = reinterpret_cast<const uint32_t*>(smem_raw + (size_t)s * stage_bytes);
+            const uint32_t* sb = reinterpret_cast<const uint32_t*>(stage0 + (size_t)s * stage_bytes);
             float acc[NB];
 #pragma unroll
             for (int b = 0; b < NB; ++b) acc[b] = 0.f;
@@ -563,18 +598,18 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
                 const SbGeom g = SbGeom::make(n_ch, scols, (int)dir[1], (int)dir[2]);
                 const int elems = lost ? 0 : dir_chunk_elems(dir[3]);
                 if (T == 104) {
-                    chunk_dot_mx4<NB, WIDE>(sb, g, warp, lane, elems, xs, reinterpret_cast<const float*>(lut), acc);
+                    chunk_dot_mx4<NB, WIDE, PAIRS>(sb, g, warp, lane, elems, xs, reinterpret_cast<const float*>(lut), acc);
                 } else if (T == -2) {
                     const uint32_t xs_a = smem_u32(xs);
                     decode_chunk_generic_mx(sb, g, elems, warp, lane, t, [&](int col, uint16_t bits) {
-                        x_fma<NB>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
+                        x_fma<NB, PAIRS>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
                     });
                 } else if (T >= 0) {
-                    chunk_dot_fast<(T >= 0 && T <= 5 ? T : 0), NB, WIDE>(sb, g, warp, lane, elems, xs, lut, acc);
+                    chunk_dot_fast<(T >= 0 && T <= 5 ? T : 0), NB, WIDE, PAIRS>(sb, g, warp, lane, elems, xs, lut, acc);
                 } else {
                     const uint32_t xs_a = smem_u32(xs);
                     decode_chunk_generic(sb, g, elems, warp, lane, t, cb, [&](int col, uint16_t bits) {
-                        x_fma<NB>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
+                        x_fma<NB, PAIRS>(x_load<NB>(xs_a + (uint32_t)col * (uint32_t)x_col_bytes(NB)), (uint32_t)bits << 16, acc);
                     });
                 }
             }
@@ -597,12 +632,14 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
                     }
                 }
             } else {
+                static_assert(kGemvStages == 1, "the sums take the place of the superblock that was read");
+                if (kCompact) __syncthreads();                // all reads of it are done
 #pragma unroll
                 for (int b = 0; b < NB; ++b) red[(b * n_warps + warp) * 32 + lane] = acc[b];
                 __syncthreads();
-                if (tid == 0 && i + kGemvStages < n_tiles) {
+                if (!kCompact && tid == 0 && i + 1 < n_tiles) {
                     fence_proxy_async();
-                    issue(i + kGemvStages);
+                    issue(i + 1);
                 }
                 for (int b = warp; b < NB; b += n_warps) {    // vector b's chunk sums, added in chunk order as with NB = 1
                     float sum = 0.f;
@@ -612,7 +649,13 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
                         result(b, row, sum);
                     }
                 }
-                __syncthreads();                              // the sums are read before the next tile overwrites them
+                if (i + 1 < n_tiles) {
+                    __syncthreads();                          // the sums are read before the next tile overwrites them
+                    if (kCompact && tid == 0) {
+                        fence_proxy_async();
+                        issue(i + 1);
+                    }
+                }
             }
         }
         return true;
@@ -621,9 +664,9 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
     if (out != 2) return;
     cg::cluster_group cluster = cg::this_cluster();
     cluster.sync();                                     // every CTA comes here, also one that gave up
-    if (done && cluster.block_rank() == 0 && threadIdx.x < 32) {
+    if (done && cluster.block_rank() == 0) {
         const int row = (int)blockIdx.y * kRowsPerBlock + lane;
-        for (int b = 0; b < NB; ++b) {
+        for (int b = threadIdx.x >> 5; b < NB; b += (int)blockDim.x >> 5) {
             float part[8];
 #pragma unroll
             for (int s = 0; s < 8; ++s) part[s] = *cluster.map_shared_rank(&s_sum[b][lane], min(s, n_seg - 1));
@@ -658,7 +701,8 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
     const int n_ch = ceil_div(bi.seg_cols, bi.chunk_cols);
     if (n_ch > 32) return CASS_ERR_UNSUPPORTED;
     if (nb != 1 && nb != 2 && nb != 4 && nb != 8) return CASS_ERR_UNSUPPORTED;
-    const size_t smem = gemv_smem_bytes(bi, nb), total = gemv_smem_total(bi, nb);
+    size_t smem = gemv_smem_bytes(bi, nb);
+    const size_t total = gemv_smem_total(bi, nb);
     if (total > kSmemPerBlock) return CASS_ERR_CAPACITY;
     const int threads = 32 * n_ch;
     // One vector: one CTA per superblock -- the hardware hands out CTAs as shared memory frees, which balances the SMs to
@@ -674,24 +718,27 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
         if (g > bi.n_rowblocks) g = bi.n_rowblocks;
     }
     if (g < 1) g = 1;
+    // three of these CTAs fit an SM; a grid of up to two an SM is kept from sitting three on some: 4096 x 4096, eight Cassandra-2 vectors 24 and 32 us
+    if (nb >= 4 && bi.n_seg * g > kSms && bi.n_seg * g <= 2 * kSms && smem < kSmemPerBlock / 3) smem = kSmemPerBlock / 3;
     // Results inside the kernel where the segments of a row block are one CTA, or a cluster of CTAs with one tile each and the
     // grid fills at most three quarters of the chip: a cluster starts only when all of its CTAs have room, which leaves SMs
     // idle where CTAs queue (12613 x 5686 at t = 0: 57.4 us, 47.0 with the finishing kernel; 4096 x 14336: 31.5 and 28.7;
     // against that 1000 x 3000: 8.6 and 8.9, 2000 x 11000: 17.9 and 18.4).
     const bool want = y_bf16 || y_f32;
-    const bool room = 4ll * bi.n_seg * g <= 3ll * kSms * per_sm;
+    const bool room = 4ll * bi.n_seg * g <= 3ll * kSms * (nb >= 4 && per_sm > 2 ? 2 : per_sm);
     const int out = !want ? 0 : bi.n_seg == 1 ? 1 : (bi.n_seg <= 8 && g == bi.n_rowblocks && room) ? 2 : 0;
     // with q = 1 - p kept, 8 kept columns span 8 / q columns, give or take sqrt(8 p) / q: more than 32 about once in 10^4 groups
     // of a lane at p = 50 %, once in 40 at 60 %, and one lane's long gap costs its warp a careful walk (359 x 1467 at p = 60 %:
     // 26 us without the second window, 12.8 with it)
     const bool wide = bi.prune_permille > 520;
+    const bool pairs2 = bi.n_seg * bi.n_rowblocks > 2 * kSms;
     dim3 grid(bi.n_seg, g), block(threads);
     const uint32_t* b = (const uint32_t*)blob;
     const uint16_t* x = (const uint16_t*)x_bf16;
-    const int stage = (int)gemv_stage_bytes(bi);
-#define CASS_GEMV_LAUNCH(TT, NN, WW)                                                                             \
+    const int stage = (int)gemv_stage_bytes(bi, nb);
+#define CASS_GEMV_LAUNCH(TT, NN, WW, PP)                                                                         \
     do {                                                                                                       \
-        CASS_ALLOW_SMEM(k_draft_gemv<TT, NN, WW>);                                                             \
+        CASS_ALLOW_SMEM(k_draft_gemv<TT, NN, WW, PP>);                                                             \
         cudaLaunchConfig_t cfg = {};                                                                           \
         cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;            \
         cudaLaunchAttribute at[2];                                                                             \
@@ -700,7 +747,7 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
         at[1].id = cudaLaunchAttributeClusterDimension;                                                        \
         at[1].val.clusterDim.x = bi.n_seg; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;             \
         cfg.attrs = at; cfg.numAttrs = out == 2 ? 2 : 1;                                                       \
-        CASS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, k_draft_gemv<TT, NN, WW>, b, x, partial, d_status, stage,         \
+        CASS_CUDA_CHECK(cudaLaunchKernelEx(&cfg, k_draft_gemv<TT, NN, WW, PP>, b, x, partial, d_status, stage,         \
                                            (int)bi.max_superblock_bytes, (int)bi.rows, (int)bi.cols,           \
                                            (int)bi.trunc_bits, (int)bi.seg_cols, (int)bi.chunk_cols,           \
                                            (int)bi.n_seg, (int)bi.n_rowblocks,                                 \
@@ -709,15 +756,18 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
 #define CASS_GEMV_LAUNCH_NB(TT)                                                                                \
     do {                                                                                                       \
         constexpr bool kHasWide = TT >= 0;          /* the generic decoders search any distance */               \
+        constexpr bool kPairs2 = TT == 4;           /* two vectors: pairs where superblocks abound */            \
         if (wide && kHasWide) {                                                                                \
-            if (nb == 1) CASS_GEMV_LAUNCH(TT, 1, kHasWide);                                                    \
-            else if (nb == 2) CASS_GEMV_LAUNCH(TT, 2, kHasWide);                                               \
-            else if (nb == 4) CASS_GEMV_LAUNCH(TT, 4, kHasWide);                                               \
-            else CASS_GEMV_LAUNCH(TT, 8, kHasWide);                                                            \
-        } else if (nb == 1) CASS_GEMV_LAUNCH(TT, 1, false);                                                    \
-        else if (nb == 2) CASS_GEMV_LAUNCH(TT, 2, false);                                                      \
-        else if (nb == 4) CASS_GEMV_LAUNCH(TT, 4, false);                                                      \
-        else CASS_GEMV_LAUNCH(TT, 8, false);                                                                   \
+            if (nb == 1) CASS_GEMV_LAUNCH(TT, 1, kHasWide, false);                                             \
+            else if (nb == 2 && pairs2 && kPairs2) CASS_GEMV_LAUNCH(TT, 2, kHasWide, kPairs2);                   \
+            else if (nb == 2) CASS_GEMV_LAUNCH(TT, 2, kHasWide, false);                                        \
+            else if (nb == 4) CASS_GEMV_LAUNCH(TT, 4, kHasWide, true);                                         \
+            else CASS_GEMV_LAUNCH(TT, 8, kHasWide, true);                                                      \
+        } else if (nb == 1) CASS_GEMV_LAUNCH(TT, 1, false, false);                                             \
+        else if (nb == 2 && pairs2 && kPairs2) CASS_GEMV_LAUNCH(TT, 2, false, kPairs2);                          \
+        else if (nb == 2) CASS_GEMV_LAUNCH(TT, 2, false, false);                                               \
+        else if (nb == 4) CASS_GEMV_LAUNCH(TT, 4, false, true);                                                \
+        else CASS_GEMV_LAUNCH(TT, 8, false, true);                                                             \
     } while (0)
     if (bi.mode == 2 && bi.trunc_bits == 4) CASS_GEMV_LAUNCH_NB(104);
     else if (bi.mode == 2) CASS_GEMV_LAUNCH_NB(-2);
