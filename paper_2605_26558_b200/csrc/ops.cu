@@ -131,6 +131,73 @@ __device__ __forceinline__ void unpack4(uint2 v, float (&x)[4]) {
     x[2] = __uint_as_float(v.y << 16); x[3] = __uint_as_float(v.y & 0xFFFF0000u);
 }
 
+// The same for many rows (a prefill pass) whose projections come as bf16: a quarter of the threads, each in the place of four whose
+// values lie `n_virt` / 4 warps apart, so that a row's sum is formed as above (lanes' sums of a warp by exchange, the warps' in order) and its bits
+// are the same.  A row of 1024 threads with one quadruple each waits, two rows an SM, for one round trip after the other: 18.5 -> 9.8 us for 1000 rows of 4096.
+template <int ITERS>
+__global__ void __launch_bounds__(256) k_residual_rmsnorm_rows(uint16_t* __restrict__ h, const uint16_t* __restrict__ y, const uint16_t* __restrict__ gain,
+                                                               uint16_t* __restrict__ out, int hidden, int n_virt, float eps) {
+    __shared__ float s_red[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, step = n_virt * 128;      // virtual warps warp + nw * v
+    pdl_wait();
+    pdl_early<0>();
+    uint16_t* hr = h + (size_t)blockIdx.x * hidden;
+    const uint16_t* yr = y + (size_t)blockIdx.x * hidden;
+    uint2 hv[4][ITERS], yv[4][ITERS];
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) {
+            const int w = warp + nw * v, i = (w * 32 + lane) * 4 + it * step;
+            const bool in = w < n_virt && i < hidden;
+            hv[v][it] = in ? *reinterpret_cast<const uint2*>(hr + i) : make_uint2(0u, 0u);
+            yv[v][it] = in ? *reinterpret_cast<const uint2*>(yr + i) : make_uint2(0u, 0u);
+        }
+    float vals[4][ITERS][4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        const int w = warp + nw * v;
+        float ss = 0.f;
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) {
+            const int i = (w * 32 + lane) * 4 + it * step;
+            float a[4], b[4];
+            unpack4(hv[v][it], a);
+            unpack4(yv[v][it], b);
+            if (w < n_virt && i < hidden) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) a[q] = round_bf16(a[q] + b[q]);
+                *reinterpret_cast<uint2*>(hr + i) = make_uint2((uint32_t)float_to_bf16_bits(a[0]) | ((uint32_t)float_to_bf16_bits(a[1]) << 16),
+                                                               (uint32_t)float_to_bf16_bits(a[2]) | ((uint32_t)float_to_bf16_bits(a[3]) << 16));
+#pragma unroll
+                for (int q = 0; q < 4; ++q) ss += a[q] * a[q];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) vals[v][it][q] = a[q];
+        }
+        ss = warp_sum(ss);
+        if (lane == 0 && w < n_virt) s_red[w] = ss;
+    }
+    __syncthreads();
+    float t = 0.f;
+    for (int w = 0; w < n_virt; ++w) t += s_red[w];
+    const float inv = 1.0f / sqrtf(t / (float)hidden + eps);
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+#pragma unroll
+        for (int it = 0; it < ITERS; ++it) {
+            const int w = warp + nw * v, i = (w * 32 + lane) * 4 + it * step;
+            if (w < n_virt && i < hidden) {
+                float g[4];
+                unpack4(__ldg(reinterpret_cast<const uint2*>(gain + i)), g);
+                uint32_t o[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) o[q] = float_to_bf16_bits(vals[v][it][q] * inv * g[q]);
+                *reinterpret_cast<uint2*>(out + (size_t)blockIdx.x * hidden + i) = make_uint2(o[0] | (o[1] << 16), o[2] | (o[3] << 16));
+            }
+        }
+}
+
 // Four rotated pairs, or eight plain v elements, a thread (head sizes are multiples of 32): 16-byte loads of the parts.
 __global__ void __launch_bounds__(128) k_qkv_rope(uint16_t* __restrict__ qkv, Partials pp,
                                                   const float* __restrict__ cos_t, const float* __restrict__ sin_t,
@@ -185,21 +252,16 @@ __global__ void __launch_bounds__(128) k_qkv_rope(uint16_t* __restrict__ qkv, Pa
 
 // Four features a thread: 16-byte loads of the parts, one address for four.  (One a thread was bound by instruction issue in a
 // prefill pass: 18.3 us for 128 rows of 14336, 29 MB of parts.)
-__global__ void __launch_bounds__(128) k_swiglu(const uint16_t* __restrict__ gu, Partials pp, uint16_t* __restrict__ act, int ffn) {
+__global__ void __launch_bounds__(128) k_swiglu(Partials pp, uint16_t* __restrict__ act, int ffn) {
     pdl_wait();
     pdl_early<0>();
     const int r = blockIdx.y;
     for (int i = (blockIdx.x * blockDim.x + threadIdx.x) * 4; i < ffn; i += gridDim.x * blockDim.x * 4) {
         float g[4], u[4];
-        if (pp.p) {
-            float4 gs, us;
-            parts_sum4_pair(pp, (size_t)r * pp.row_stride + i, (size_t)r * pp.row_stride + ffn + i, gs, us);
-            g[0] = round_bf16(gs.x); g[1] = round_bf16(gs.y); g[2] = round_bf16(gs.z); g[3] = round_bf16(gs.w);
-            u[0] = round_bf16(us.x); u[1] = round_bf16(us.y); u[2] = round_bf16(us.z); u[3] = round_bf16(us.w);
-        } else {
-            unpack4(*reinterpret_cast<const uint2*>(gu + (size_t)r * 2 * ffn + i), g);
-            unpack4(*reinterpret_cast<const uint2*>(gu + (size_t)r * 2 * ffn + ffn + i), u);
-        }
+        float4 gs, us;
+        parts_sum4_pair(pp, (size_t)r * pp.row_stride + i, (size_t)r * pp.row_stride + ffn + i, gs, us);
+        g[0] = round_bf16(gs.x); g[1] = round_bf16(gs.y); g[2] = round_bf16(gs.z); g[3] = round_bf16(gs.w);
+        u[0] = round_bf16(us.x); u[1] = round_bf16(us.y); u[2] = round_bf16(us.z); u[3] = round_bf16(us.w);
         uint32_t o[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -208,6 +270,27 @@ __global__ void __launch_bounds__(128) k_swiglu(const uint16_t* __restrict__ gu,
         }
         *reinterpret_cast<uint2*>(act + (size_t)r * ffn + i) = make_uint2(o[0] | (o[1] << 16), o[2] | (o[3] << 16));
     }
+}
+
+// The same of bf16 projections (a prefill pass), eight features a thread: two 16-byte loads under way and one store; rows of the grid are
+// taken in turn.  Four features a thread: 32 us for 1000 rows of 14336, 86 MB, 21 so.
+__global__ void __launch_bounds__(256) k_swiglu_rows(const uint16_t* __restrict__ gu, uint16_t* __restrict__ act, int ffn, int n_items) {
+    pdl_wait();
+    pdl_early<0>();
+    const int it = blockIdx.x * blockDim.x + threadIdx.x;
+    if (it >= n_items) return;
+    const int per = ffn / 8, r = it / per, i = (it - r * per) * 8;
+    const uint16_t* row = gu + (size_t)r * 2 * ffn + i;
+    const uint4 gv = __ldcs(reinterpret_cast<const uint4*>(row)), uv = __ldcs(reinterpret_cast<const uint4*>(row + ffn));
+    const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w}, uw[4] = {uv.x, uv.y, uv.z, uv.w};
+    uint32_t o[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float g0 = __uint_as_float(gw[q] << 16), g1 = __uint_as_float(gw[q] & 0xFFFF0000u);
+        const float s0 = g0 / (1.0f + expf(-g0)), s1 = g1 / (1.0f + expf(-g1));
+        o[q] = (uint32_t)float_to_bf16_bits(s0 * __uint_as_float(uw[q] << 16)) | ((uint32_t)float_to_bf16_bits(s1 * __uint_as_float(uw[q] & 0xFFFF0000u)) << 16);
+    }
+    *reinterpret_cast<uint4*>(act + (size_t)r * ffn + i) = make_uint4(o[0], o[1], o[2], o[3]);
 }
 
 // Greedy token of each row, lowest index on ties, in two levels: slices of the vocabulary, then the slices' winners.
@@ -372,6 +455,12 @@ int launch_residual_rmsnorm(uint16_t* h, const uint16_t* y_bf16, Partials pp,
                             const uint16_t* gain, uint16_t* out, int rows, int hidden, float eps, cudaStream_t s) {
     if (hidden % 4 || hidden > kNormMaxIter * 4 * 1024) return CASS_ERR_UNSUPPORTED;
     const int threads = norm_threads(hidden);
+    if (y_bf16 && !pp.p && out && rows > 2 * kSms && norm_iters(hidden, threads) <= 2) {
+        const int n_virt = threads / 32, quarter = ceil_div(n_virt, 4) * 32;
+        if (norm_iters(hidden, threads) == 1) CASS_PDL_LAUNCH(k_residual_rmsnorm_rows<1>, dim3(rows), dim3(quarter), 0, s, h, y_bf16, gain, out, hidden, n_virt, eps);
+        else CASS_PDL_LAUNCH(k_residual_rmsnorm_rows<2>, dim3(rows), dim3(quarter), 0, s, h, y_bf16, gain, out, hidden, n_virt, eps);
+        return CASS_OK;
+    }
     switch (norm_iters(hidden, threads)) {
         case 1: CASS_PDL_LAUNCH(k_residual_rmsnorm<1>, dim3(rows), dim3(threads), 0, s, h, y_bf16, pp, gain, out, hidden, eps); break;
         case 2: CASS_PDL_LAUNCH(k_residual_rmsnorm<2>, dim3(rows), dim3(threads), 0, s, h, y_bf16, pp, gain, out, hidden, eps); break;
@@ -394,8 +483,13 @@ int launch_qkv_rope(uint16_t* qkv, Partials pp, const float* cos_t, const float*
 
 int launch_swiglu(const uint16_t* gu_bf16, Partials pp, uint16_t* act, int rows, int ffn,
                   cudaStream_t s) {
-    dim3 grid(ceil_div(ffn, 512), rows);                     // ffn is a multiple of 8
-    CASS_PDL_LAUNCH(k_swiglu, grid, dim3(128), 0, s, gu_bf16, pp, act, ffn);
+    if (!pp.p) {                                             // ffn is a multiple of 8
+        const int items = rows * (ffn / 8);
+        CASS_PDL_LAUNCH(k_swiglu_rows, dim3(ceil_div(items, 256)), dim3(256), 0, s, gu_bf16, act, ffn, items);
+        return CASS_OK;
+    }
+    dim3 grid(ceil_div(ffn, 512), rows);
+    CASS_PDL_LAUNCH(k_swiglu, grid, dim3(128), 0, s, pp, act, ffn);
     return CASS_OK;
 }
 
