@@ -22,8 +22,8 @@
 // still running; every kernel launched this way calls pdl_wait() before it touches global memory, which returns
 // once the predecessor has completed and its writes are visible.  Four read something ahead of it that was there before the
 // predecessor began: the draft GEMV its blob (written by k_directory and k_pack, whose caller synchronises before the blob is
-// used), the verification projection a session's matrix, the norm its gains (both behind the embedding or a projection), the
-// fused KV encoder its codebook (written by k_kv_rank, behind a projection).  k_pack and k_kv_rank release nobody early.
+// used), the projections (of a verification and of a prefill) a session's matrix, the norm its gains (both behind the embedding or a
+// projection), the fused KV encoder its codebook (written by k_kv_rank, behind a projection).  k_pack and k_kv_rank release nobody early.
 #define CASS_PDL_LAUNCH(kernel_, grid_, block_, smem_, stream_, ...)                                              \
     do {                                                                                                    \
         cudaLaunchConfig_t _cfg = {};                                                                       \

@@ -101,8 +101,7 @@ __global__ void __launch_bounds__(kMergeThreads) k_attn_merge(AttnScratch sc, in
 
 // The same for at most MC chunks: one warp a (row, query head), lane = chunk for the statistics, then four dims a lane with all
 // chunks requested at once.  Every sum is formed in the order of k_attn_merge (eight interleaved chains, added in turn), so
-// the bits are the same.  A CTA of 8 warps and three barriers a pair, most of it idle, took 13.5 us for the 4096 pairs of a
-// prefill pass.
+// the bits are the same.  A CTA of 8 warps and three barriers a pair, most of it idle, took 13.5 us for 4096 pairs.
 template <int MC>
 __global__ void __launch_bounds__(kMergeThreads) k_attn_merge_few(AttnScratch sc, int chunk_tokens, AttnRows ar, int n_pairs, int n_q, int d,
                                                                   const DevState* __restrict__ st, int draft_mode, int draft_units,

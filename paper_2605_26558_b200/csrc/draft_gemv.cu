@@ -41,8 +41,15 @@ static size_t gemv_smem_bytes(const cass_blob_info& bi, int nb) {
     return x_slice_bytes(bi.seg_cols, nb) + (stage + table > slack ? stage + table : slack);
 }
 
-// With what the kernel declares itself: a segment's sums, the tile's sizes and flags, up to where the dynamic part may begin.
-size_t gemv_smem_total(const cass_blob_info& bi, int nb) { return gemv_smem_bytes(bi, nb) + align_up((size_t)nb * 32 * 4 + 32, 512); }
+// What the kernel declares itself: a segment's sums, the tile's sizes and flags, up to where the dynamic part may begin.
+static size_t gemv_smem_static(int nb) { return align_up((size_t)nb * 32 * 4 + 32, 512); }
+
+// What counts against a CTA's limit: every part side by side, whatever the layout, so that it does not decide which blobs are taken.
+size_t gemv_smem_total(const cass_blob_info& bi, int nb) {
+    const size_t stage = kGemvStages * align_up((size_t)bi.max_superblock_bytes + 384, 512);
+    const size_t sums = (size_t)(nb < 2 ? 2 : nb) * ceil_div(bi.seg_cols, bi.chunk_cols) * 32 * 4;
+    return stage + (size_t)(bi.seg_cols + kXSlack) * x_col_bytes(nb) + 256 * 4 + 64 + sums + gemv_smem_static(nb);
+}
 
 __device__ __forceinline__ uint32_t bfind_u32(uint32_t v) {         // index of the most significant one, -1 if none
     uint32_t r;
@@ -702,8 +709,8 @@ static int launch_gemv(const void* blob, const cass_blob_info& bi, const void* x
     if (n_ch > 32) return CASS_ERR_UNSUPPORTED;
     if (nb != 1 && nb != 2 && nb != 4 && nb != 8) return CASS_ERR_UNSUPPORTED;
     size_t smem = gemv_smem_bytes(bi, nb);
-    const size_t total = gemv_smem_total(bi, nb);
-    if (total > kSmemPerBlock) return CASS_ERR_CAPACITY;
+    const size_t total = smem + gemv_smem_static(nb);
+    if (gemv_smem_total(bi, nb) > kSmemPerBlock) return CASS_ERR_CAPACITY;
     const int threads = 32 * n_ch;
     // One vector: one CTA per superblock -- the hardware hands out CTAs as shared memory frees, which balances the SMs to
     // within one superblock (a grid of as many CTAs as fit at once, each looping over its share, left SMs with 4 x 4

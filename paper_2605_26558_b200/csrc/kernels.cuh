@@ -131,7 +131,7 @@ __device__ __forceinline__ void parts_sum4_pair(const Partials& pp, size_t off_a
 
 constexpr int kAttnChunk = 64;       // split-K granularity over the sequence (fixed absolute boundaries)
 
-size_t gemv_smem_total(const cass_blob_info& bi, int nb);       // shared memory a CTA takes; at most kSmemPerBlock
+size_t gemv_smem_total(const cass_blob_info& bi, int nb);       // what counts against kSmemPerBlock, a CTA takes at most that
 // x: bf16 [nb][cols], nb in {1, 2, 4, 8} vectors multiplied in one pass over the blob.
 // partial: fp32 [nb][n_seg][n_rowblocks*32]; the caller sums the segments (fixed order) afterwards.
 int launch_draft_gemv(const void* blob, const cass_blob_info& bi, const void* x_bf16, int nb, float* partial,

@@ -250,8 +250,8 @@ __global__ void __launch_bounds__(128) k_qkv_rope(uint16_t* __restrict__ qkv, Pa
     store4(ib, y);
 }
 
-// Four features a thread: 16-byte loads of the parts, one address for four.  (One a thread was bound by instruction issue in a
-// prefill pass: 18.3 us for 128 rows of 14336, 29 MB of parts.)
+// Four features a thread: 16-byte loads of the parts, one address for four.  (One a thread was bound by instruction issue:
+// 18.3 us for 128 rows of 14336, 29 MB of parts.)
 __global__ void __launch_bounds__(128) k_swiglu(Partials pp, uint16_t* __restrict__ act, int ffn) {
     pdl_wait();
     pdl_early<0>();

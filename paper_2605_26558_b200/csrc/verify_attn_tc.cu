@@ -8,9 +8,9 @@
 // swizzled layout.  The V tile is used as it lies in memory (rows = tokens), i.e. as an M-contiguous A operand.
 // Chunk results (o, running maximum m, sum l) go to the split-K scratch and k_attn_merge combines the chunks, as for
 // the SIMT kernel.  A (row, head) pair is one accumulator column, so its result does not depend on the other rows.
-// Needs head_dim = 128 and rows x group <= 64; other shapes use k_verify_attn.  More rows than that (prefill) are cut into
-// groups, one CTA each; where the fp32-pipe kernel would have taken them 16 at a time, P is kept as two bf16 terms and the
-// second product runs twice, so that the accuracy is that kernel's.
+// Needs head_dim = 128 and rows x group <= 64; other shapes use k_verify_attn.  More rows than that (a prefill over more chunks
+// than prefill_attn.cu takes) are cut into groups, one CTA each; where the fp32-pipe kernel would have taken them 16 at a time,
+// P is kept as two bf16 terms and the second product runs twice, so that the accuracy is that kernel's.
 #include "tc.cuh"
 #include "kernels.cuh"
 

@@ -2,7 +2,7 @@
 // memory-bound on the bf16 weights): Y[r][n] = sum_k W[n][k] X[r][k], bf16 operands, fp32 accumulation.
 //
 // tcgen05 version, "swap-AB": the weights are the M operand (128 output features per CTA), the token rows the N
-// operand (padded to BN = 16, 32, 64 or, in a prefill, 128 or 256 columns), the accumulator lives in tensor memory.  One CTA = one 128-feature tile x
+// operand (padded to BN = 16, 32, 64 or, in a short prefill, 128 or 256 columns), the accumulator lives in tensor memory.  One CTA = one 128-feature tile x
 // one K range (split-K so that small matrices still fill the GPU); warp 0 streams 128x64 weight tiles and the
 // BNx64 activation tile through a ring of TMA loads (128-byte swizzle), warp 1 issues the MMAs, warps 2-5 read the
 // accumulator back and store fp32 partial sums; a second kernel adds the K ranges in fixed order.
