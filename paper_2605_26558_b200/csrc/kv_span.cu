@@ -109,26 +109,29 @@ __global__ void __launch_bounds__(32 * kSpanWarps) k_kv_form(KvGeom g, KvComp ck
     }
 }
 
-// grid (K|V, layers * sequences): codebook from the histogram, which is left zero for the next time.  Four lanes an exponent.
-__global__ void __launch_bounds__(1024) k_kv_rank(KvGeom g, KvComp ck, KvComp cv, KvSpan sp) {
-    __shared__ unsigned long long s[256];
+// grid (K|V, layers * sequences): codebook from the histogram, which is left zero for the next time.  A count and its exponent are one
+// number, so that a comparison is one.  Lanes an exponent, us a call, 1 / 2 / 4 (and with two comparisons, one lane): 2000 tokens of two
+// 8B-shaped layers 52.7 / 52.6 / 53.6 (54.4 with four), three layers of two sequences of 234 tokens (head size 64) 16.4 / 16.3 / 17.3 (17.8).
+constexpr int kRankLanes = 2;
+__global__ void __launch_bounds__(256 * kRankLanes) k_kv_rank(KvGeom g, KvComp ck, KvComp cv, KvSpan sp) {
+    __shared__ __align__(16) unsigned long long s[256];
     const KvComp c = of_seq(blockIdx.x ? cv : ck, 1, span_shift(g, sp, blockIdx.y));
-    const int e = threadIdx.x >> 2, part = threadIdx.x & 3;
+    const int e = threadIdx.x / kRankLanes, part = threadIdx.x % kRankLanes;
     pdl_wait();
     if (threadIdx.x < 256) {
-        s[threadIdx.x] = c.hist[threadIdx.x];
+        s[threadIdx.x] = c.hist[threadIdx.x] << 8 | (255u - threadIdx.x);      // of equal counts the smaller exponent first
         c.hist[threadIdx.x] = 0;
     }
     __syncthreads();
     const unsigned long long mine = s[e];
     int rank = 0;
 #pragma unroll 16
-    for (int i = 0; i < 64; ++i) {
-        const int o = i * 4 + part;
-        rank += (s[o] > mine) || (s[o] == mine && o < e);
+    for (int i = 0; i < 128 / kRankLanes; ++i) {
+        const ulonglong2 o = reinterpret_cast<const ulonglong2*>(s)[i * kRankLanes + part];
+        rank += (o.x > mine ? 1 : 0) + (o.y > mine ? 1 : 0);
     }
-    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
-    rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+#pragma unroll
+    for (int i = 1; i < kRankLanes; i *= 2) rank += __shfl_xor_sync(0xffffffffu, rank, i);
     if (part == 0) {
         c.rank_to_exp[rank] = (uint8_t)e;
         c.exp_to_rank[e] = (uint8_t)rank;
@@ -263,7 +266,7 @@ __global__ void __launch_bounds__(32 * kSpanWarps) k_kv_codes(KvGeom g, KvComp c
 // fields and the code bits are then a lane's own work: no reductions, scans or ballots, which are most of what a warp on one record
 // of four values a lane executes.  Record words are 32 tokens side by side, so a warp's stores are whole lines.
 // Bound: the integer pipe (61 %) and latency, 235 instructions a record to form it (725 with a warp).  2000 tokens of two 8B-shaped layers
-// 104 -> 54 us (form 30, lengths 11, codes 20 under ncu), Cassandra-2 64 -> 41, four layers of four sequences of 1000 tokens 369 -> 160.
+// 104 -> 53 us (form 30, lengths 11, codes 20 under ncu), Cassandra-2 64 -> 41, four layers of four sequences of 1000 tokens 369 -> 160.
 // A warp's chain is long, 25 to 38 us for all the kernels whatever the size, against 8 to 20 where a warp a record leaves the chip idle:
 // 512 warps 36 (warps) and 38 us, 640 warps of head size 64 35 and 28.  Releasing the successors early: 54 -> 64 us, their waiting CTAs
 // take this one's place.
@@ -654,7 +657,7 @@ static int span_encode(const KvGeom& g, const KvComp& ck, const KvComp& cv, uint
         if (codebook) {
             CASS_PDL_LAUNCH((k_kv_form_lanes<NJ, T, true>), grid, lanes, 0, s, g, ck, cv, k_cache, v_cache, (const uint16_t*)nullptr,
                             (const uint16_t*)nullptr, 0, sp, flags);
-            CASS_PDL_LAUNCH(k_kv_rank, dim3(2, z), dim3(1024), 0, s, g, ck, cv, sp);
+            CASS_PDL_LAUNCH(k_kv_rank, dim3(2, z), dim3(256 * kRankLanes), 0, s, g, ck, cv, sp);
             if (g.mode == 1)
                 CASS_PDL_LAUNCH(k_kv_lengths_lanes<NJ>, grid, lanes, 0, s, g, ck, cv, (const uint16_t*)k_cache, (const uint16_t*)v_cache, sp);
         } else {
@@ -676,7 +679,7 @@ static int span_encode(const KvGeom& g, const KvComp& ck, const KvComp& cv, uint
         if (bx > 0)
             CASS_PDL_LAUNCH((k_kv_form<NJ, T, true>), dim3(bx, g.n_kv * 2, z), threads, 0, s, g, ck, cv, k_cache, v_cache,
                             (const uint16_t*)nullptr, (const uint16_t*)nullptr, 0, sp, flags);
-        CASS_PDL_LAUNCH(k_kv_rank, dim3(2, z), dim3(1024), 0, s, g, ck, cv, sp);
+        CASS_PDL_LAUNCH(k_kv_rank, dim3(2, z), dim3(256 * kRankLanes), 0, s, g, ck, cv, sp);
         if (bx == 0) return CASS_OK;
         if (g.mode == 1)
             CASS_PDL_LAUNCH(k_kv_lengths<NJ>, dim3(blocks, g.n_kv * 2, z), threads, 0, s, g, ck, cv, (const uint16_t*)k_cache,
