@@ -58,11 +58,14 @@ static int make_geom(const cass_format* fmt, int rows, int cols, EncGeom* g) {
     g->n_rb = ceil_div(rows, kRowsPerBlock);
     g->n_pad = g->n_rb * kRowsPerBlock;
     g->n_prune = (int)(((long long)cols * p) / 1000);
-    // Sizes and packing by lanes (a warp's chain is long) or by warps, by the blocks of 128 columns of 32 rows there are: 113 -> 85 us by
-    // lanes for 3000 x 2050 (1598 blocks), 79 -> 73 for 5000 x 1027 (1413), but 34 and 34 for 1000 x 1000 (256).  Rows of few columns take
-    // a warp little: 40 -> 52 for 5000 x 512 (628), 42 -> 54 for 9000 x 400 (1124), 88 -> 93 for 20000 x 501 (2500), 120 -> 103 for 30000 x 301 (2814).
-    const long long blocks = (long long)g->n_rb * ceil_div(g->k_pad, 128);
-    g->lanes = !g->mx && t == 4 && blocks >= (g->seg_cols > 512 ? 1400 : 2600);
+    // Sizes and packing by lanes (a warp's chain is long) or by warps, by the blocks of 128 columns of 32 rows there are: 104 -> 76 us by
+    // lanes for 2400 x 3000 (1800 blocks), 61 -> 56 for 900 x 8192 (1856), 79 -> 60 for 12000 x 520 (1875), but 34 and 34 for 1000 x 1000
+    // (256).  Rows of few columns take a warp little: 40 -> 52 for 5000 x 512 (628), 42 -> 54 for 9000 x 400 (1124), 88 -> 93 for
+    // 20000 x 501 (2500), 120 -> 103 for 30000 x 301 (2814).  Rows off 16-byte boundaries take lanes longer (4692 x 1184: 52, x 1185: 70), and
+    // they then lose to warps where those have a place on the chip for every superblock at once: 63 -> 70 for 4692 x 1185 (147
+    // superblocks), 75 -> 78 for 900 x 8191 (116), 65 -> 72 for 9000 x 641 (282), but 88 -> 79 for 4800 x 1185 (150), 89 -> 79 for 12000 x 513 (375).
+    const long long blocks = (long long)g->n_rb * ceil_div(g->k_pad, 128), places = kSms * (g->seg_cols > 768 ? 1 : 2);
+    g->lanes = !g->mx && t == 4 && blocks >= (g->seg_cols > 512 ? 1400 : 2600) && (cols % 8 == 0 || (long long)g->n_rb * g->n_seg > places);
     return CASS_OK;
 }
 
