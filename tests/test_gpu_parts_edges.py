@@ -24,7 +24,9 @@ def cass():
     (33, 1, 0, 4, 0, 0), (1, 31, 400, 4, 0, 0), (40, 257, 400, 1, 0, 0), (65, 2049, 300, 2, 0, 0), (31, 4097, 500, 3, 0, 0),
     (35, 1000, 400, 5, 0, 0), (34, 999, 400, 6, 256, 32), (33, 801, 200, 7, 0, 0), (37, 2048, 0, 4, 2048, 2048),
     (32, 4096, 990, 4, 2048, 2048), (70, 3001, 999, 4, 0, 0), (64, 1024, 100, 0, 1024, 512),
-    (1201, 1024, 400, 4, 1024, 32), (1190, 1031, 300, 2, 1024, 64), (1185, 1058, 600, 5, 1024, 32), (1216, 1040, 0, 4, 1024, 64)])
+    (1201, 1024, 400, 4, 1024, 32), (1470, 1031, 300, 2, 1024, 64), (1185, 1058, 600, 5, 1024, 32), (1480, 1040, 0, 4, 1024, 64),
+    (1500, 1055, 400, 4, 1024, 32), (401, 2049, 500, 3, 1024, 32), (400, 2050, 400, 0, 1024, 32), (390, 2049, 350, 6, 1024, 32),
+    (401, 2050, 450, 1, 1024, 32), (1181, 1025, 400, 4, 1024, 32)])
 def test_split_and_join(cass, rows, cols, p, t, seg, chunk):
     w = synth.student_t_weight(rows, cols, 6, f"parts/{rows}x{cols}").float()
     if rows > 20 and cols > 900:
