@@ -180,8 +180,9 @@ __global__ void __launch_bounds__(32 * kJoinWarps) k_join(const uint32_t* __rest
     const uint32_t* un = body + sg.un + lane;
     const uint32_t* fl = body + sg.fl + lane;
     const uint32_t* bmr = body + sg.bm + lane;
-    const uint32_t vrow = kVdataHeaderWords + (uint32_t)min(row, jg.n - 1) * (uint32_t)jg.row_words;     // the row's words of the verification data
-    const uint32_t* lo = vdata + vrow;
+    const uint32_t* vblock = vdata + kVdataHeaderWords + (size_t)rb * kRowsPerBlock * jg.row_words;      // these 32 rows' verification data
+    const uint32_t vrow = (uint32_t)(min(row, jg.n - 1) - rb * kRowsPerBlock) * (uint32_t)jg.row_words;      // the row's words in it (32 bits hold any block's)
+    const uint32_t* lo = vblock + vrow;
     const int wu_last = max(sg.w_u - 1, 0), wf_last = max(sg.w_f - 1, 0), lo_last = max(jg.lo_words - 1, 0);
     const uint32_t ulimit = (uint32_t)sg.w_u * 32u, low_mask = (1u << t) - 1u, keep_bits = 0x8000u | (0x7Fu & ~low_mask);
     const uint32_t e0 = __ldg(body + sg.tab + ch * 32 + lane), total = __ldg(body + sg.tab + n_ch * 32 + lane);
@@ -253,7 +254,7 @@ __global__ void __launch_bounds__(32 * kJoinWarps) k_join(const uint32_t* __rest
         const bool whole = __all_sync(0xffffffffu, off == 0 && hi == 64);
         sync();
         auto copy = [&](uint32_t to, uint32_t from) {
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(vdata + from) : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(vblock + from) : "memory");
         };
 #pragma unroll 4
         for (int r = share * 2 + (lane >> 4); r < kRowsPerBlock; r += 2 * kSteps) {        // half a warp a row

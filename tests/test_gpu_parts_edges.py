@@ -53,3 +53,27 @@ def test_split_and_join(cass, rows, cols, p, t, seg, chunk):
         cass.cass_decode_full(blob, info, vdata, out)
         assert np.array_equal(_bits(out), wb), shift
     assert torch.isnan(full[-1]).item()
+
+
+def test_join_of_more_verification_data_than_32_bits_count_words(cass):
+    """8.6 G values, 999 of 1000 pruned: the last 64 rows' words lie beyond 2^32."""
+    rows, cols, p, t = 524736, 16384, 999, 4
+    if torch.cuda.mem_get_info()[0] < 80e9:
+        pytest.skip("70 GB of the GPU's memory are not free")
+    w = torch.empty(rows, cols, dtype=torch.bfloat16, device="cuda")
+    w.view(torch.int16).random_(-2 ** 15, 2 ** 15, generator=torch.Generator(device="cuda").manual_seed(7))
+    fmt = cass.default_format(w_p=p, w_t=t)
+    bound, ws_bytes = cass.cass_encoded_weight_bytes(fmt, rows, cols)
+    blob = torch.empty(bound, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    cass.cass_encode_weights(fmt, w, None, blob, torch.empty(ws_bytes, dtype=torch.uint8, device="cuda"), status)
+    info = cass.cass_weight_blob_info(blob)
+    assert int(status.item()) == 0
+    n_bytes = cass.cass_verification_data_bytes(info)
+    assert n_bytes // 4 // rows * (rows - 64) > 2 ** 32
+    vdata = torch.empty(n_bytes // 4, dtype=torch.int32, device="cuda")
+    cass.cass_encode_verification_data(blob, info, w, vdata)
+    out = torch.full_like(w, float("nan"))
+    cass.cass_decode_full(blob, info, vdata, out)
+    for r in range(0, rows, 65536):
+        assert torch.equal(w[r: r + 65536].view(torch.int16), out[r: r + 65536].view(torch.int16)), r
