@@ -127,10 +127,10 @@ __global__ void __launch_bounds__(32 * kSplitWarps) k_split(const uint32_t* __re
 //   lane = 8 columns, four rows at a time: a prefix count of the bitmap says where in the list and among the pruned values the
 //     columns begin; each then takes the next of either, and the eight leave in one store.
 // Kept and pruned values of a window are 64 together, so the buffer is 82 halfwords a row, whatever the matrix looks like, and 28 warps
-// fit an SM (by registers).  Bound: instruction issue (59 %) and the latency of a window's steps: 34 M warp instructions for 6144 x 4096
-// (49 M with a list of a whole chunk's values, which 20 warps an SM had room for, and one row after the other with its loads), of
-// which decoding 13, writing 12, copying 5.  6144 x 4096 at 40 % pruning 115 -> 61 us, at 30 % 217 -> 64 (a chunk took a second turn), at
-// 60 % 109 -> 57; 28672 x 4096 374 -> 219.
+// fit an SM (72 registers; with 80 and 24 warps 20000 x 1528 takes 71 us instead of 64, with 64 and 32 28672 x 4096 258 instead of 217).
+// Bound: instruction issue (62 %) and the latency of a window's steps: 33 M warp instructions for 6144 x 4096 (49 M with a list of a
+// whole chunk's values, which 20 warps an SM had room for, and one row after the other with its loads).  6144 x 4096 at 40 %
+// pruning 109 -> 58 us, at 30 % 217 -> 61 (a chunk took a second turn), at 60 % 109 -> 54; 28672 x 4096 374 -> 209.
 constexpr int kJoinWarps = 4;
 // Chunks up to which teams: 31 and 37 us with and without for 9000 x 641 (846 chunks), 27 and 33 for 4096 x 2048 (1024), but 63 and 51 for
 // 2000 x 5000 (1260, t = 3) and 89 and 61 for 6144 x 4096 (3072).
@@ -138,7 +138,7 @@ constexpr int kJoinTeamMax = 8 * kSms;
 constexpr int kJoinRow = 82;                                            // halfwords: 7 + 64 + 7 + 2 for odd places; an odd number of words, rows in different banks
 
 struct JoinGeom {
-    int n, k, k_pad, t, seg_cols, n_seg, n_ch, n_tasks, lo_words, row_words, n_raw;
+    int n, k, k_pad, seg_cols, n_seg, n_ch, n_tasks, lo_words, row_words, n_raw;
 };
 
 __device__ __forceinline__ uint32_t join_lds16(uint32_t a) {
@@ -147,10 +147,157 @@ __device__ __forceinline__ uint32_t join_lds16(uint32_t a) {
     return v;
 }
 
-// TT: truncated bits (0..5), or -1: any (from the geometry).  TEAM: the CTA's four warps share one chunk, the first decoding and all of them
+// Decoder of one row's kept values in a chunk, 8 at a time and in order: code words by bit searches as in the draft GEMV, then fields and low
+// bits.  T, the truncated bits, is a constant, and with it every value's place: fields that do not fill a word (t = 2, 3, 5) are first
+// joined into one stream of 8 F bits, the low bits into one of 8 t.  With a place computed for every value 8987 x 4088 took 116 us at t = 2 and 117
+// at t = 5 instead of 93 and 95, 2171 x 4088 63 and 59 instead of 43 (t = 2, 5); fields and low bits of t = 4 by bytes: 6144 x 4096
+// 60.0 -> 57.8, 28672 x 4096 219 -> 210.
+template <int T>
+struct JoinGroups {
+    static constexpr int F = 8 - T, PER = 32 / F;
+    static constexpr int NFW = T == 4 || T >= 6 ? 1 : T == 2 || T == 3 ? 3 : 2, NLW = T == 0 ? 0 : T <= 4 ? 2 : 3;      // words a group can touch
+    static constexpr uint32_t kLow = (1u << T) - 1u, kKeep = 0x8000u | (0x7Fu & ~kLow);
+    const uint32_t* rows;                                               // the superblock's words of this row
+    int bm, un, last;                                                   // where in the superblock bitmap and codes begin, and its last words
+    int f_at, f_in, k_first;                                            // field word of the next group and its first field there; values of the segment before the chunk's
+    int row;                                                            // whose low bits
+    uint32_t lo_bit, upos, lut_top;                                     // next low bit of the row; next code bit; table of exponents
+    uint32_t u0, u1, u2, fn[NFW], ln[NLW > 0 ? NLW : 1];                // the word of bit upos and two more
+
+    __device__ __forceinline__ uint32_t word(int at) const { return __ldg(rows + min(at, last)); }
+    // field and low words of the next group, asked for a group ahead
+    __device__ __forceinline__ void fetch(const uint32_t* vdata, const JoinGeom& jg, bool first) {
+#pragma unroll
+        for (int i = 0; i < NFW; ++i) fn[i] = word(f_at + i * 32);
+        if constexpr (NLW > 0) {
+            const uint32_t* lo = vdata + kVdataHeaderWords + (size_t)row * jg.row_words;
+            const int li = (int)(lo_bit >> 5), lo_last = jg.lo_words - 1;
+            if (T == 4 && !first) {                                     // one word a group
+                ln[0] = ln[1];
+                ln[1] = __ldg(lo + min(li + 1, lo_last));
+            } else {
+#pragma unroll
+                for (int i = 0; i < NLW; ++i) ln[i] = __ldg(lo + min(li + i, lo_last));
+            }
+        }
+    }
+    // k: values of the segment, k_row: of the row, before the chunk's
+    __device__ __forceinline__ void begin(const uint32_t* body, const SbGeom& sg, int lane, int row_, int k, int k_row, uint32_t bit, const uint16_t* lut,
+                                          const uint32_t* vdata, const JoinGeom& jg) {
+        rows = body + lane;
+        bm = sg.bm;
+        un = sg.un;
+        last = sg.total - 32;
+        f_at = sg.fl + k / PER * 32;
+        f_in = k % PER;
+        k_first = k;
+        row = min(row_, jg.n - 1);
+        lo_bit = (uint32_t)k_row * (uint32_t)T;
+        upos = bit;
+        lut_top = smem_u32(lut) + 62u;
+        const int at = un + (int)(upos >> 5) * 32;
+        u0 = word(at);
+        u1 = word(at + 32);
+        u2 = word(at + 64);
+        fetch(vdata, jg, true);
+    }
+    // the values g .. g + 7 of the chunk, packed in pairs; those beyond its last are anything
+    __device__ __forceinline__ void next(int g, const uint16_t* lut, const uint32_t* vdata, const JoinGeom& jg, uint32_t (&out)[4]) {
+        // the group's fields from bit 31 of f0 on, its low bits from bit 31 of l0 on
+        uint32_t f0 = fn[0], f1 = fn[NFW > 1 ? 1 : 0], l0 = 0, l1 = 0;
+        if constexpr (T >= 6) {
+            f0 = __funnelshift_l(f0, f0, F * f_in);
+        } else if constexpr (T == 2 || T == 3 || T == 5) {              // a word's last two bits are none of a field's
+            const uint32_t s0 = fn[0] | (fn[1] >> 30), s1 = (fn[1] << 2) | (NFW > 2 ? fn[NFW - 1] >> 28 : 0u);
+            f0 = __funnelshift_l(s1, s0, F * f_in);
+            f1 = NFW > 2 ? __funnelshift_l(fn[NFW - 1] << 4, s1, F * f_in) : 0u;
+        }
+        if constexpr (NLW > 0) {
+            l0 = __funnelshift_l(ln[1], ln[0], lo_bit);
+            if constexpr (NLW > 2) l1 = __funnelshift_l(ln[2], ln[1], lo_bit);
+            lo_bit += 8 * T;
+        }
+        f_at += 8 / PER * 32;
+        if constexpr (8 % PER != 0) {
+            f_in += 8 % PER;
+            if (f_in >= PER) {
+                f_in -= PER;
+                f_at += 32;
+            }
+        }
+        fetch(vdata, jg, false);
+        uint32_t uv = __funnelshift_l(u1, u0, upos), used = 8u * 32u, q = 0, v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {                                   // shifting the found one out leaves the next code at the top
+            asm("bfind.u32 %0, %1;" : "=r"(q) : "r"(uv));
+            uint32_t a;
+            asm("mad.lo.u32 %0, %1, 0xFFFFFFFE, %2;" : "=r"(a) : "r"(q), "r"(lut_top));
+            v[i] = join_lds16(a);
+            used -= q;
+            uv = __funnelshift_r(0u, uv, q);
+        }
+        if ((int32_t)q < 0) {                                           // the codes did not fit the window: one by one
+            uint32_t ub = upos;
+            const int cnt = (int)(__ldg(rows + (bm - 32)) >> 20) - k_first;     // kept values of the segment from the chunk's first on
+#pragma unroll 1
+            for (int i = 0; i < 8; ++i) {
+                uint32_t x = 0;
+                if (g + i < cnt) x = lut[read_unary(rows + un, ub, (uint32_t)(last + 32 - un)) & 255];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = i == j ? x : v[j];
+            }
+            used = ub - upos;
+        }
+        const int was = (int)(upos >> 5);
+        upos += used;
+        const int now = (int)(upos >> 5), at = un + now * 32;
+        if (now == was + 1) {
+            u0 = u1; u1 = u2;
+            u2 = word(at + 64);
+        } else if (now > was) {
+            u0 = word(at);
+            u1 = word(at + 32);
+            u2 = word(at + 64);
+        }
+        // A pair of values: exponents | the rest.  F = 4: bytes 3 - j / 2 and 2 - j / 2 of the word have an even value's sign and mantissa (an odd one's
+        // once it is rotated by 4), and the low bits go beside the mantissa.
+        auto pair = [&](int i, uint32_t rest) { out[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x5410) | (rest & 0x807F807Fu); };
+        if constexpr (T == 4) {
+            const uint32_t fo = __funnelshift_l(f0, f0, 4), le = __funnelshift_r(l0, l0, 12), lo = __funnelshift_r(l0, l0, 8);
+            const uint32_t xe = (f0 & 0xF0F0F0F0u) | (le & 0x0F0F0F0Fu), xo = (fo & 0xF0F0F0F0u) | (lo & 0x0F0F0F0Fu);      // even, odd values
+            pair(0, __byte_perm(xe, xo, 0x7632));
+            pair(1, __byte_perm(xe, xo, 0x6521));
+            pair(2, __byte_perm(xe, xo, 0x5410));
+            pair(3, __byte_perm(xe, xo, 0x4703));
+        } else if constexpr (T == 0) {                                  // F = 8: bytes 3 - j and 2 - j
+            pair(0, __byte_perm(f0, 0u, 0x2132));
+            pair(1, __byte_perm(f0, 0u, 0x0310));
+            pair(2, __byte_perm(f1, 0u, 0x2132));
+            pair(3, __byte_perm(f1, 0u, 0x0310));
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if constexpr (32 % F == 0) {                            // rotated fields: one rotation puts both parts in place
+                    v[i] |= __funnelshift_l(f0, f0, (F * i + 16) & 31) & kKeep;
+                } else {                                                // packed ones: sign and mantissa both out of the top byte
+                    const int b = T == 1 ? F * (i & 3) : F * i;
+                    const uint32_t x = T == 1 ? (i < 4 ? f0 : f1) << b : b + F <= 32 ? f0 << b : b < 32 ? __funnelshift_l(f1, f0, b) : f1 << (b & 31);
+                    v[i] |= __byte_perm(x, 0u, 0x4433) & kKeep;
+                }
+                const int b = T * i;
+                const uint32_t x = b + T <= 32 ? l0 >> ((32 - b - T) & 31) : b < 32 ? __funnelshift_l(l1, l0, b) >> (32 - T) : l1 >> ((64 - b - T) & 31);
+                v[i] |= x & kLow;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) out[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x5410);
+        }
+    }
+};
+
+// T: truncated bits.  TEAM: the CTA's four warps share one chunk, the first decoding and all of them
 // copying and writing: the latency of a small matrix.
-template <int TT, bool TEAM>
-__global__ void __launch_bounds__(32 * kJoinWarps) k_join(const uint32_t* __restrict__ blob, const uint32_t* __restrict__ vdata,
+template <int T, bool TEAM>
+__global__ void __launch_bounds__(32 * kJoinWarps, 7) k_join(const uint32_t* __restrict__ blob, const uint32_t* __restrict__ vdata,
                                                           uint16_t* __restrict__ out, JoinGeom jg) {
     // a window's first and last eight columns may reach up to 7 beyond it: what they read there is not stored
     constexpr int kTasks = TEAM ? 1 : kJoinWarps, kSteps = TEAM ? kJoinWarps : 1;      // chunks a CTA; warps a chunk
@@ -158,7 +305,6 @@ __global__ void __launch_bounds__(32 * kJoinWarps) k_join(const uint32_t* __rest
     __shared__ uint4 s_row[kTasks][32];                                 // a row's window: bitmap words, places and ends, first word | kept values in it
     __shared__ uint2 s_copy[kTasks][32];                                // its pruned values: words from, how many | to
     __shared__ uint16_t s_lut[256];                                     // rank -> exponent at its bf16 position
-    const int t = TT >= 0 ? TT : jg.t, F = 8 - t, PER = 32 / F;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint8_t* cb = reinterpret_cast<const uint8_t*>(blob) + kBlobHeaderBytes;
     pdl_wait();
@@ -177,53 +323,24 @@ __global__ void __launch_bounds__(32 * kJoinWarps) k_join(const uint32_t* __rest
     const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir.y, (int)dir.z);
     const uint32_t* body = blob + (size_t)dir.x * 4;
     const int c_base = seg * jg.seg_cols, row = rb * kRowsPerBlock + lane;
-    const uint32_t* un = body + sg.un + lane;
-    const uint32_t* fl = body + sg.fl + lane;
     const uint32_t* bmr = body + sg.bm + lane;
-    const uint32_t* vblock = vdata + kVdataHeaderWords + (size_t)rb * kRowsPerBlock * jg.row_words;      // these 32 rows' verification data
-    const uint32_t vrow = (uint32_t)(min(row, jg.n - 1) - rb * kRowsPerBlock) * (uint32_t)jg.row_words;      // the row's words in it (32 bits hold any block's)
-    const uint32_t* lo = vblock + vrow;
-    const int wu_last = max(sg.w_u - 1, 0), wf_last = max(sg.w_f - 1, 0), lo_last = max(jg.lo_words - 1, 0);
-    const uint32_t ulimit = (uint32_t)sg.w_u * 32u, low_mask = (1u << t) - 1u, keep_bits = 0x8000u | (0x7Fu & ~low_mask);
-    const uint32_t e0 = __ldg(body + sg.tab + ch * 32 + lane), total = __ldg(body + sg.tab + n_ch * 32 + lane);
+    const uint32_t e0 = __ldg(body + sg.tab + ch * 32 + lane);
     int col = ch == 0 ? 0 : (int)(e0 >> 20);                            // this lane's row: first column not yet written
     int col_end = ch + 1 < n_ch ? (int)(__ldg(body + sg.tab + (ch + 1) * 32 + lane) >> 20) : scols;
     col_end = row < jg.n ? min(col_end, jg.k - c_base) : col;
-    const int cnt = max(0, min(E, (int)(total >> 20) - ch * E));        // its kept values in this chunk
-    uint32_t upos = e0 & 0xFFFFFu;
     int k_row = ch * E;                                                 // kept values of the row before this chunk
     for (int i = 0; i < seg; ++i) {
         const uint4 dp = __ldg(reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4) + rb * jg.n_seg + i);
         k_row += (int)(__ldg(blob + (size_t)dp.x * 4 + dir_n_ch(dp.w) * 32 + lane) >> 20);
     }
-    constexpr int NFW = TT == 4 ? 1 : TT == 0 ? 2 : 4, NLW = TT == 0 ? 0 : TT > 0 && TT <= 4 ? 2 : 3;       // words a group of 8 can touch
-    constexpr int LW = NLW > 0 ? NLW : 1;
+    JoinGroups<T> dec;
+    dec.begin(body, sg, lane, row, ch * E, k_row, e0 & 0xFFFFFu, s_lut, vdata, jg);
     uint16_t* buf = s_buf + 8 + slot * 32 * kJoinRow;
     uint16_t* mine = buf + lane * kJoinRow;
-    const uint32_t buf_a = smem_u32(buf), lut_top = smem_u32(s_lut) + 62u;
+    const uint32_t buf_a = smem_u32(buf);
     const bool vec16 = jg.k % 8 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0, vec4 = jg.k % 2 == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0;
 
-    // field and low words of the group of 8 that starts at value g of the chunk, asked for a group ahead
-    uint32_t fn[NFW], ln[LW];
-    auto fetch = [&](int g, bool first) {
-        const int fi = (ch * E + g) / PER;
-#pragma unroll
-        for (int i = 0; i < NFW; ++i) fn[i] = __ldg(fl + min(fi + i, wf_last) * 32);
-        if (NLW > 0) {
-            const int li = (int)((uint32_t)(k_row + g) * (uint32_t)t >> 5);
-            if (TT == 4 && !first) {                                    // one word a group
-                ln[0] = ln[LW - 1];
-                ln[LW - 1] = __ldg(lo + min(li + 1, lo_last));
-            } else {
-#pragma unroll
-                for (int i = 0; i < LW; ++i) ln[i] = __ldg(lo + min(li + i, lo_last));
-            }
-        }
-    };
-    int at = (int)(upos >> 5);                                          // u0, u1, u2: code words at, at + 1, at + 2
-    uint32_t u0 = __ldg(un + min(at, wu_last) * 32), u1 = __ldg(un + min(at + 1, wu_last) * 32), u2 = __ldg(un + min(at + 2, wu_last) * 32);
-    fetch(0, true);
-    int j0 = col >> 5, ks = 0, dec = 0;                                 // first bitmap word of the window; values taken; values decoded
+    int j0 = col >> 5, ks = 0, done = 0;                                // first bitmap word of the window; values taken; values decoded
     auto bm_word = [&](int j) { return j < sg.bm_words ? __ldg(bmr + j * 32) : 0u; };
     uint32_t wn0 = bm_word(j0), wn1 = bm_word(j0 + 1);
 
@@ -241,97 +358,36 @@ __global__ void __launch_bounds__(32 * kJoinWarps) k_join(const uint32_t* __rest
             w0 &= (uint32_t)(m >> 32);
             w1 &= (uint32_t)m;
         }
-        const int n0 = __popc(w0), kw = n0 + __popc(w1), base8 = ks & ~7, ke = ks + kw, dec_end = (ke + 7) & ~7;
+        const int n0 = __popc(w0), kw = n0 + __popc(w1), base8 = ks & ~7, ke = ks + kw, done_to = (ke + 7) & ~7;
         // ---- its pruned values, behind the list ----
         const int s0 = c_base + col - (k_row + ks), n_raw = hi - off - kw;
-        const uint32_t rw = vrow + (uint32_t)jg.lo_words + (uint32_t)(s0 >> 1);
-        const int n_w = n_raw > 0 ? ((s0 & 1) + n_raw + 1) >> 1 : 0, to_w = (lane * kJoinRow + dec_end - base8) >> 1;
-        const uint32_t place = (uint32_t)(ks - base8) | ((uint32_t)(dec_end - base8 + (s0 & 1)) << 8) | ((uint32_t)off << 16) | ((uint32_t)hi << 24);
+        const uint32_t rw = (uint32_t)(jg.lo_words + (s0 >> 1));
+        const int n_w = n_raw > 0 ? ((s0 & 1) + n_raw + 1) >> 1 : 0, to_w = (lane * kJoinRow + done_to - base8) >> 1;
+        const uint32_t place = (uint32_t)(ks - base8) | ((uint32_t)(done_to - base8 + (s0 & 1)) << 8) | ((uint32_t)off << 16) | ((uint32_t)hi << 24);
         if (share == 0) {
             s_copy[slot][lane] = make_uint2(rw, (uint32_t)n_w | ((uint32_t)to_w << 16));
             s_row[slot][lane] = make_uint4(w0, w1, place, (uint32_t)j0 | ((uint32_t)n0 << 16));
         }
         const bool whole = __all_sync(0xffffffffu, off == 0 && hi == 64);
         sync();
-        auto copy = [&](uint32_t to, uint32_t from) {
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(vblock + from) : "memory");
-        };
+        auto copy = [&](uint32_t to, const uint32_t* from) { asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(from) : "memory"); };
 #pragma unroll 4
         for (int r = share * 2 + (lane >> 4); r < kRowsPerBlock; r += 2 * kSteps) {        // half a warp a row
             const uint2 cp = s_copy[slot][r];
-            const uint32_t n = cp.y & 0xFFFFu, to = buf_a + (cp.y >> 16) * 4u + (uint32_t)(lane & 15) * 4u, from = cp.x + (uint32_t)(lane & 15);
+            const uint32_t n = cp.y & 0xFFFFu, to = buf_a + (cp.y >> 16) * 4u + (uint32_t)(lane & 15) * 4u;
+            const uint32_t* from = vdata + kVdataHeaderWords + (size_t)(rb * kRowsPerBlock + r) * jg.row_words + (cp.x + (uint32_t)(lane & 15));
             if ((uint32_t)(lane & 15) < n) copy(to, from);
             if (n > 16u)                                                // up to 33 words
                 for (uint32_t w = 16; w + (uint32_t)(lane & 15) < n; w += 16) copy(to + w * 4u, from + w);
         }
         // ---- lane = row: values up to ke, whole groups ----
-        while (share == 0 && dec < dec_end) {
-            uint32_t fw[NFW], lw[LW];
+        while (share == 0 && done < done_to) {
+            uint32_t v[4];
+            dec.next(done, s_lut, vdata, jg, v);
+            uint32_t* to = reinterpret_cast<uint32_t*>(mine + done - base8);
 #pragma unroll
-            for (int i = 0; i < NFW; ++i) fw[i] = fn[i];
-#pragma unroll
-            for (int i = 0; i < LW; ++i) lw[i] = ln[i];
-            fetch(dec + 8, false);
-            uint32_t uv = __funnelshift_l(u1, u0, upos), used = 8u * 32u, q = 0, v[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {                               // shifting the found one out leaves the next code at the top
-                asm("bfind.u32 %0, %1;" : "=r"(q) : "r"(uv));
-                uint32_t a;
-                asm("mad.lo.u32 %0, %1, 0xFFFFFFFE, %2;" : "=r"(a) : "r"(q), "r"(lut_top));
-                v[i] = join_lds16(a);
-                used -= q;
-                uv = __funnelshift_r(0u, uv, q);
-            }
-            if ((int32_t)q < 0) {                                       // the codes did not fit the window: one by one
-                uint32_t ub = upos;
-#pragma unroll 1
-                for (int i = 0; i < 8; ++i) {
-                    uint32_t x = 0;
-                    if (dec + i < cnt) x = s_lut[read_unary(un, ub, ulimit) & 255];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) v[j] = i == j ? x : v[j];
-                }
-                used = ub - upos;
-            }
-            upos += used;
-            const int step = (int)(upos >> 5) - at;
-            if (step == 1) {
-                u0 = u1; u1 = u2;
-                u2 = __ldg(un + min(at + 3, wu_last) * 32);
-            } else if (step > 1) {
-                u0 = __ldg(un + min(at + step, wu_last) * 32);
-                u1 = __ldg(un + min(at + step + 1, wu_last) * 32);
-                u2 = __ldg(un + min(at + step + 2, wu_last) * 32);
-            }
-            at += step;
-            const int k = ch * E + dec;                                 // of the segment: fields are numbered through it
-            const uint32_t bit0 = ((uint32_t)(k_row + dec) * (uint32_t)t) & 31u;
-            const uint32_t l8 = TT == 4 ? __funnelshift_l(lw[LW - 1], lw[0], bit0) : 0u;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                uint32_t sm;
-                if (TT == 4) {
-                    sm = __funnelshift_l(fw[0], fw[0], (4 * i + 16) & 31);
-                } else if (TT == 0) {
-                    sm = __funnelshift_l(fw[i / 4 % NFW], fw[i / 4 % NFW], (8 * (i & 3) + 16) & 31);
-                } else {
-                    const int j = k % PER + i, wi = j / PER;            // up to three words on
-                    sm = field_sign_mant_bf16(wi == 0 ? fw[0] : wi == 1 ? fw[1 % NFW] : wi == 2 ? fw[2 % NFW] : fw[3 % NFW], j - wi * PER, t);
-                }
-                v[i] |= sm & keep_bits;
-                if (TT == 4) {
-                    v[i] |= (l8 >> (28 - 4 * i)) & 15u;
-                } else if (NLW > 0 && t > 0) {
-                    const uint32_t b = bit0 + (uint32_t)(i * t), wi = b >> 5;
-                    const uint32_t hi_w = wi == 0 ? lw[0] : wi == 1 || NLW == 2 ? lw[LW > 1 ? 1 : 0] : lw[LW > 2 ? 2 : 0];
-                    const uint32_t nx = wi == 0 || NLW == 2 ? lw[LW > 1 ? 1 : 0] : lw[LW > 2 ? 2 : 0];
-                    v[i] |= (__funnelshift_l(nx, hi_w, b) >> (32 - t)) & low_mask;
-                }
-            }
-            uint32_t* to = reinterpret_cast<uint32_t*>(mine + dec - base8);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) to[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x5410);
-            dec += 8;
+            for (int i = 0; i < 4; ++i) to[i] = v[i];
+            done += 8;
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         sync();
@@ -410,12 +466,11 @@ static_assert(kJoinCap % 8 == 0 && (kJoinStride / 2) % 2 == 1, "groups of 8; odd
 // once more between the windows' teams and the end of a second wave: 7000 x 1529 (1314) 49 and 53.
 constexpr int kJoinRowsMax = 5 * kSms;
 
-template <int TT>                                                       // truncated bits (0..5), or -1: any (from the geometry)
+template <int T>                                                        // truncated bits
 __global__ void __launch_bounds__(32 * kJoinWarps, 5) k_join_rows(const uint32_t* __restrict__ blob, const uint32_t* __restrict__ vdata,
                                                                   uint16_t* __restrict__ out, JoinGeom jg) {
-    __shared__ uint16_t s_list[32 * kJoinStride + 64 * kJoinSpan + 2];      // a look past the last list reads what no column takes
+    __shared__ __align__(4) uint16_t s_list[32 * kJoinStride + 64 * kJoinSpan + 2];      // a look past the last list reads what no column takes
     __shared__ uint16_t s_lut[256];                                     // rank -> exponent at its bf16 position
-    const int t = TT >= 0 ? TT : jg.t, F = 8 - t, PER = 32 / F;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint8_t* cb = reinterpret_cast<const uint8_t*>(blob) + kBlobHeaderBytes;
     pdl_wait();
@@ -430,97 +485,33 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 5) k_join_rows(const uint32_t
     const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir.y, (int)dir.z);
     const uint32_t* body = blob + (size_t)dir.x * 4;
     const int c_base = seg * jg.seg_cols;
-    const uint32_t* un = body + sg.un + lane;
-    const uint32_t* fl = body + sg.fl + lane;
-    const uint32_t* lo = vdata + kVdataHeaderWords + (size_t)min(rb * kRowsPerBlock + lane, jg.n - 1) * jg.row_words;
-    const int wu_last = max(sg.w_u - 1, 0), wf_last = max(sg.w_f - 1, 0), lo_last = max(jg.lo_words - 1, 0);
-    const uint32_t ulimit = (uint32_t)sg.w_u * 32u, low_mask = (1u << t) - 1u, keep_bits = 0x8000u | (0x7Fu & ~low_mask);
     const uint32_t e0 = __ldg(body + sg.tab + ch * 32 + lane), total = __ldg(body + sg.tab + n_ch * 32 + lane);
     const int col_end = ch + 1 < n_ch ? (int)(__ldg(body + sg.tab + (ch + 1) * 32 + lane) >> 20) : scols;
     int col = ch == 0 ? 0 : (int)(e0 >> 20);                            // this lane's row: first column not yet written
     const int cnt = max(0, min(E, (int)(total >> 20) - ch * E));        // its kept values in this chunk
-    uint32_t upos = e0 & 0xFFFFFu;
     int k_row = ch * E;                                                 // kept values of the row before this chunk
     for (int i = 0; i < seg; ++i) {
         const uint4 dp = __ldg(reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4) + rb * jg.n_seg + i);
         k_row += (int)(__ldg(blob + (size_t)dp.x * 4 + dir_n_ch(dp.w) * 32 + lane) >> 20);
     }
     const int n_max = __reduce_max_sync(0xffffffffu, cnt);
-    constexpr int NFW = TT == 4 ? 1 : TT == 0 ? 2 : 4, NLW = TT == 0 ? 0 : TT > 0 && TT <= 4 ? 2 : 3;       // words a group of 8 can touch
+    JoinGroups<T> dec;
+    if (warp == 0) {
+        dec.begin(body, sg, lane, rb * kRowsPerBlock + lane, ch * E, k_row, e0 & 0xFFFFFu, s_lut, vdata, jg);
+    }
     uint16_t* mine = s_list + lane * kJoinStride;
 
     for (int p0 = 0; p0 == 0 || p0 < n_max; p0 += kJoinCap) {
         const int n_here = min(kJoinCap, n_max - p0);
         if (warp == 0) {
             // ---- lane = row: values p0 .. p0 + n_here - 1 of the chunk ----
-            uint32_t fw[NFW], lw[NLW > 0 ? NLW : 1], fn[NFW], ln[NLW > 0 ? NLW : 1];
-            auto fetch = [&](int g) {                                   // field and low words of the group that starts at value g
-                const int fi = (ch * E + p0 + g) / PER;
-#pragma unroll
-                for (int i = 0; i < NFW; ++i) fn[i] = __ldg(fl + min(fi + i, wf_last) * 32);
-                if (NLW > 0) {
-                    const int li = (int)((uint32_t)(k_row + p0 + g) * (uint32_t)t >> 5);
-#pragma unroll
-                    for (int i = 0; i < NLW; ++i) ln[i] = __ldg(lo + min(li + i, lo_last));
-                }
-            };
-            int at = (int)(upos >> 5);                                  // u0, u1, u2: code words at, at + 1, at + 2
-            uint32_t u0 = __ldg(un + min(at, wu_last) * 32), u1 = __ldg(un + min(at + 1, wu_last) * 32), u2 = __ldg(un + min(at + 2, wu_last) * 32);
-            fetch(0);
+#pragma unroll 1
             for (int g = 0; g < n_here; g += 8) {
+                uint32_t v[4];
+                dec.next(p0 + g, s_lut, vdata, jg, v);
+                uint32_t* to = reinterpret_cast<uint32_t*>(mine + g);
 #pragma unroll
-                for (int i = 0; i < NFW; ++i) fw[i] = fn[i];
-#pragma unroll
-                for (int i = 0; i < NLW; ++i) lw[i] = ln[i];
-                if (g + 8 < n_here) fetch(g + 8);
-                uint32_t uv = __funnelshift_l(u1, u0, upos), used = 0, q = 0, v[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {                           // shifting the found one out leaves the next code at the top
-                    asm("bfind.u32 %0, %1;" : "=r"(q) : "r"(uv));
-                    v[i] = s_lut[(31u - q) & 255u];
-                    used += 32u - q;
-                    uv = __funnelshift_r(0u, uv, q);
-                }
-                if ((int32_t)q < 0) {                                   // the codes did not fit the window: one by one
-                    uint32_t ub = upos;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        if (p0 + g + i < cnt) v[i] = s_lut[read_unary(un, ub, ulimit) & 255];
-                    used = ub - upos;
-                }
-                upos += used;
-                const int step = (int)(upos >> 5) - at;
-                if (step == 1) {
-                    u0 = u1; u1 = u2;
-                    u2 = __ldg(un + min(at + 3, wu_last) * 32);
-                } else if (step > 1) {
-                    u0 = __ldg(un + min(at + step, wu_last) * 32);
-                    u1 = __ldg(un + min(at + step + 1, wu_last) * 32);
-                    u2 = __ldg(un + min(at + step + 2, wu_last) * 32);
-                }
-                at += step;
-                const int k = ch * E + p0 + g;                          // of the segment: fields are numbered through it
-                const uint32_t bit0 = ((uint32_t)(k_row + p0 + g) * (uint32_t)t) & 31u;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    uint32_t sm;
-                    if (TT == 4) {
-                        sm = __funnelshift_l(fw[0], fw[0], (4 * i + 16) & 31);
-                    } else if (TT == 0) {
-                        sm = __funnelshift_l(fw[i / 4 % NFW], fw[i / 4 % NFW], (8 * (i & 3) + 16) & 31);
-                    } else {
-                        const int j = k % PER + i, wi = j / PER;        // up to three words on
-                        sm = field_sign_mant_bf16(wi == 0 ? fw[0] : wi == 1 ? fw[1 % NFW] : wi == 2 ? fw[2 % NFW] : fw[3 % NFW], j - wi * PER, t);
-                    }
-                    v[i] |= sm & keep_bits;
-                    if (NLW > 0 && t > 0) {
-                        const uint32_t b = bit0 + (uint32_t)(i * t), wi = b >> 5;
-                        const uint32_t hi = wi == 0 ? lw[0] : wi == 1 || NLW == 2 ? lw[NLW > 1 ? 1 : 0] : lw[NLW > 2 ? 2 : 0];
-                        const uint32_t nx = wi == 0 || NLW == 2 ? lw[NLW > 1 ? 1 : 0] : lw[NLW > 2 ? 2 : 0];
-                        v[i] |= (__funnelshift_l(nx, hi, b) >> (32 - t)) & low_mask;
-                    }
-                    mine[g + i] = (uint16_t)v[i];
-                }
+                for (int i = 0; i < 4; ++i) to[i] = v[i];
             }
         }
         __syncthreads();
@@ -636,7 +627,7 @@ extern "C" int cass_decode_full(const void* blob, const cass_blob_info* bi, cons
     cudaStream_t stream = (cudaStream_t)stream_;
     const uint32_t *b32 = (const uint32_t*)blob, *v32 = (const uint32_t*)vdata;
     uint16_t* o16 = (uint16_t*)W_bf16_out;
-    const JoinGeom jg{bi->rows, bi->cols, ceil_div(bi->cols, 32) * 32, bi->trunc_bits, bi->seg_cols, bi->n_seg, n_ch,
+    const JoinGeom jg{bi->rows, bi->cols, ceil_div(bi->cols, 32) * 32, bi->seg_cols, bi->n_seg, n_ch,
                       bi->n_rowblocks * bi->n_seg * n_ch, vdata_lo_words(bi->kept_per_row, bi->trunc_bits),
                       vdata_row_words(bi->cols, bi->kept_per_row, bi->trunc_bits), bi->cols - bi->kept_per_row};
     const bool team = jg.n_tasks < kJoinTeamMax;
@@ -654,7 +645,9 @@ extern "C" int cass_decode_full(const void* blob, const cass_blob_info* bi, cons
         case 3: CASS_JOIN(3); break;
         case 4: CASS_JOIN(4); break;
         case 5: CASS_JOIN(5); break;
-        default: CASS_JOIN(-1); break;
+        case 6: CASS_JOIN(6); break;
+        case 7: CASS_JOIN(7); break;
+        default: return CASS_ERR_INVALID_ARG;
     }
 #undef CASS_JOIN
     return CASS_OK;

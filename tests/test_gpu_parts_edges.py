@@ -26,7 +26,8 @@ def cass():
     (32, 4096, 990, 4, 2048, 2048), (70, 3001, 999, 4, 0, 0), (64, 1024, 100, 0, 1024, 512),
     (1201, 1024, 400, 4, 1024, 32), (1470, 1031, 300, 2, 1024, 64), (1185, 1058, 600, 5, 1024, 32), (1480, 1040, 0, 4, 1024, 64),
     (1500, 1055, 400, 4, 1024, 32), (401, 2049, 500, 3, 1024, 32), (400, 2050, 400, 0, 1024, 32), (390, 2049, 350, 6, 1024, 32),
-    (401, 2050, 450, 1, 1024, 32), (1181, 1025, 400, 4, 1024, 32)])
+    (401, 2050, 450, 1, 1024, 32), (1181, 1025, 400, 4, 1024, 32),
+    (8288, 512, 400, 4, 1024, 128), (8289, 511, 400, 3, 1024, 128)])                                     # the last chunks with a place at once, and one row block more
 def test_split_and_join(cass, rows, cols, p, t, seg, chunk):
     w = synth.student_t_weight(rows, cols, 6, f"parts/{rows}x{cols}").float()
     if rows > 20 and cols > 900:
@@ -47,12 +48,40 @@ def test_split_and_join(cass, rows, cols, p, t, seg, chunk):
     vdata = torch.full((cass.cass_verification_data_bytes(info) // 4,), -1, dtype=torch.int32, device="cuda")
     cass.cass_encode_verification_data(blob, info, wd, vdata)
     assert np.array_equal(vdata.cpu().numpy().view(np.uint32), want)
-    full = torch.full((rows * cols + 3,), float("nan"), dtype=torch.bfloat16, device="cuda")
-    for shift in (0, 1):                                     # output rows on and off 4-byte boundaries
-        out = full[shift: shift + rows * cols].view(rows, cols)
-        cass.cass_decode_full(blob, info, vdata, out)
-        assert np.array_equal(_bits(out), wb), shift
-    assert torch.isnan(full[-1]).item()
+    _join_at_every_phase(cass, blob, info, vdata, wb)
+
+
+def _join_at_every_phase(cass, blob, info, vdata, wb):
+    """The joined matrix against its bits, the output on 16-byte boundaries and off them, and nothing written around it."""
+    rows, cols = wb.shape
+    full = torch.empty(rows * cols + 16, dtype=torch.bfloat16, device="cuda")
+    for shift in (0, 1, 6):
+        full.fill_(float("nan"))
+        cass.cass_decode_full(blob, info, vdata, full[shift: shift + rows * cols].view(rows, cols))
+        assert np.array_equal(_bits(full[shift: shift + rows * cols].view(rows, cols)), wb), shift
+        assert torch.isnan(full[:shift]).all() and torch.isnan(full[shift + rows * cols:]).all()
+
+
+@pytest.mark.parametrize("t", range(8))
+@pytest.mark.parametrize("cols", [1000, 1002, 1001])
+@pytest.mark.parametrize("rows", [992, 1190])
+def test_join_of_every_truncation(cass, rows, cols, t):
+    """Teams on 992 chunks and a warp each on 1216, for every truncation and for rows on 16-byte, 4-byte and 2-byte boundaries."""
+    w = synth.student_t_weight(rows, cols, 8, f"join/{cols}").float()
+    w[7, ::5] *= 2.0 ** 40                                   # long codes
+    w[20, 50:700] = 0.0                                      # long runs of pruned values
+    w = w.to(torch.bfloat16)
+    fmt = cass.default_format(w_p=400, w_t=t, seg_cols=1024, chunk_cols=32)
+    bound, ws_bytes = cass.cass_encoded_weight_bytes(fmt, rows, cols)
+    blob = torch.zeros(bound, dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    wd = w.cuda()
+    cass.cass_encode_weights(fmt, wd, None, blob, torch.zeros(ws_bytes, dtype=torch.uint8, device="cuda"), status)
+    info = cass.cass_weight_blob_info(blob)
+    assert int(status.item()) == 0
+    vdata = torch.zeros(cass.cass_verification_data_bytes(info) // 4, dtype=torch.int32, device="cuda")
+    cass.cass_encode_verification_data(blob, info, wd, vdata)
+    _join_at_every_phase(cass, blob, info, vdata, _bits(w))
 
 
 def test_join_of_more_verification_data_than_32_bits_count_words(cass):
