@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(32 * kSplitWarps) k_split(const uint32_t* __re
 //     as in the draft GEMV, in a list; groups of 8 do not end where windows do, so up to 7 values stay for the next window.  Behind
 //     the list the window's pruned values, copied from the verification data meanwhile, half a warp a row;
 //   lane = 8 columns, four rows at a time: a prefix count of the bitmap says where in the list and among the pruned values the
-//     columns begin; each then takes the next of either, and the eight leave in one store.
+//     columns begin; each then takes the next of either, and the eight leave in one store, but for a chunk's first and last columns.
 // Kept and pruned values of a window are 64 together, so the buffer is 82 halfwords a row, whatever the matrix looks like, and 28 warps
 // fit an SM (72 registers; with 80 and 24 warps 20000 x 1528 takes 71 us instead of 64, with 64 and 32 28672 x 4096 258 instead of 217).
 // Bound: instruction issue (62 %) and the latency of a window's steps: 33 M warp instructions for 6144 x 4096 (49 M with a list of a
@@ -135,6 +135,10 @@ constexpr int kJoinWarps = 4;
 // Chunks up to which teams: 31 and 37 us with and without for 9000 x 641 (846 chunks), 27 and 33 for 4096 x 2048 (1024), but 63 and 51 for
 // 2000 x 5000 (1260, t = 3) and 89 and 61 for 6144 x 4096 (3072).
 constexpr int kJoinTeamMax = 8 * kSms;
+// Halfwords: a row's windows begin where its output is on a 16-byte boundary, so that whatever the width eight columns leave in one store.
+// With windows from bitmap words on and one store width for the whole matrix 8987 x 4089 took 139 us instead of 86, 19995 x 4090 171 instead of 160, and
+// 4096 x 13823 210 instead of 122.  On 32-, 64- and 128-byte boundaries a chunk takes more windows: 20000 x 1528 66.5, then 67.8, 68.7 and 73.7.
+constexpr int kJoinAlign = 8;
 constexpr int kJoinRow = 82;                                            // halfwords: 7 + 64 + 7 + 2 for odd places; an odd number of words, rows in different banks
 
 struct JoinGeom {
@@ -294,15 +298,15 @@ struct JoinGroups {
     }
 };
 
-// T: truncated bits.  TEAM: the CTA's four warps share one chunk, the first decoding and all of them
-// copying and writing: the latency of a small matrix.
+// T: truncated bits.  TEAM: the CTA's four warps share one chunk, the first decoding and all of them copying and writing: the latency of a small
+// matrix.
 template <int T, bool TEAM>
 __global__ void __launch_bounds__(32 * kJoinWarps, 7) k_join(const uint32_t* __restrict__ blob, const uint32_t* __restrict__ vdata,
                                                           uint16_t* __restrict__ out, JoinGeom jg) {
     // a window's first and last eight columns may reach up to 7 beyond it: what they read there is not stored
     constexpr int kTasks = TEAM ? 1 : kJoinWarps, kSteps = TEAM ? kJoinWarps : 1;      // chunks a CTA; warps a chunk
     __shared__ __align__(16) uint16_t s_buf[8 + kTasks * 32 * kJoinRow + 8];
-    __shared__ uint4 s_row[kTasks][32];                                 // a row's window: bitmap words, places and ends, first word | kept values in it
+    __shared__ uint4 s_row[kTasks][32];                                 // a row's window: its bits, places and ends, where it begins | kept values in the first half
     __shared__ uint2 s_copy[kTasks][32];                                // its pruned values: words from, how many | to
     __shared__ uint16_t s_lut[256];                                     // rank -> exponent at its bf16 position
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -323,7 +327,6 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 7) k_join(const uint32_t* __r
     const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir.y, (int)dir.z);
     const uint32_t* body = blob + (size_t)dir.x * 4;
     const int c_base = seg * jg.seg_cols, row = rb * kRowsPerBlock + lane;
-    const uint32_t* bmr = body + sg.bm + lane;
     const uint32_t e0 = __ldg(body + sg.tab + ch * 32 + lane);
     int col = ch == 0 ? 0 : (int)(e0 >> 20);                            // this lane's row: first column not yet written
     int col_end = ch + 1 < n_ch ? (int)(__ldg(body + sg.tab + (ch + 1) * 32 + lane) >> 20) : scols;
@@ -338,20 +341,23 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 7) k_join(const uint32_t* __r
     uint16_t* buf = s_buf + 8 + slot * 32 * kJoinRow;
     uint16_t* mine = buf + lane * kJoinRow;
     const uint32_t buf_a = smem_u32(buf);
-    const bool vec16 = jg.k % 8 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0, vec4 = jg.k % 2 == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0;
 
-    int j0 = col >> 5, ks = 0, done = 0;                                // first bitmap word of the window; values taken; values decoded
-    auto bm_word = [&](int j) { return j < sg.bm_words ? __ldg(bmr + j * 32) : 0u; };
-    uint32_t wn0 = bm_word(j0), wn1 = bm_word(j0 + 1);
+    // The row's windows begin where its output is on a 16-byte boundary, up to 7 columns before the chunk's first (and before the segment)
+    const uint32_t phase = (uint32_t)(reinterpret_cast<uintptr_t>(out) >> 1) + (uint32_t)row * (uint32_t)jg.k + (uint32_t)(c_base + col);
+    int b0 = col - (int)(phase & (uint32_t)(kJoinAlign - 1)), ks = 0;   // the window's first column; values taken (decoded: whole groups of them)
+    int raw_at = c_base + col - k_row;                                  // pruned values of the row before the window's
+    auto bm_word = [&](int j) { return (uint32_t)j < (uint32_t)sg.bm_words ? __ldg(dec.rows + (dec.bm + j * 32)) : 0u; };
+    uint32_t wa = bm_word(b0 >> 5), wb = bm_word((b0 >> 5) + 1), wc = bm_word((b0 >> 5) + 2);
 
 #pragma unroll 1
     while (__any_sync(0xffffffffu, col < col_end)) {
-        // ---- the window: columns col .. hi - 1 of this lane's row, bits of others cleared ----
+        // ---- the window: columns col .. b0 + hi - 1 of this lane's row, bits of others cleared ----
         const bool more = col < col_end;
-        const int off = more ? col - j0 * 32 : 64, hi = more ? min(64, col_end - j0 * 32) : 64;      // from the first word's first column on
-        uint32_t w0 = wn0, w1 = wn1;
-        wn0 = bm_word(j0 + 2);
-        wn1 = bm_word(j0 + 3);
+        const int off = more ? col - b0 : 64, hi = more ? min(64, col_end - b0) : 64;
+        uint32_t w0 = __funnelshift_l(wb, wa, b0), w1 = __funnelshift_l(wc, wb, b0);
+        wa = wc;
+        wb = bm_word((b0 >> 5) + 3);
+        wc = bm_word((b0 >> 5) + 4);
         {
             unsigned long long m = off < 64 ? ~0ull >> off : 0ull;
             if (hi < 64) m &= ~(~0ull >> hi);
@@ -360,13 +366,13 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 7) k_join(const uint32_t* __r
         }
         const int n0 = __popc(w0), kw = n0 + __popc(w1), base8 = ks & ~7, ke = ks + kw, done_to = (ke + 7) & ~7;
         // ---- its pruned values, behind the list ----
-        const int s0 = c_base + col - (k_row + ks), n_raw = hi - off - kw;
-        const uint32_t rw = (uint32_t)(jg.lo_words + (s0 >> 1));
-        const int n_w = n_raw > 0 ? ((s0 & 1) + n_raw + 1) >> 1 : 0, to_w = (lane * kJoinRow + done_to - base8) >> 1;
-        const uint32_t place = (uint32_t)(ks - base8) | ((uint32_t)(done_to - base8 + (s0 & 1)) << 8) | ((uint32_t)off << 16) | ((uint32_t)hi << 24);
+        const int n_raw = hi - off - kw;
+        const uint32_t rw = (uint32_t)(jg.lo_words + (raw_at >> 1));
+        const int n_w = n_raw > 0 ? ((raw_at & 1) + n_raw + 1) >> 1 : 0, to_w = (lane * kJoinRow + done_to - base8) >> 1;
+        const uint32_t place = (uint32_t)(ks - base8) | ((uint32_t)(done_to - base8 + (raw_at & 1)) << 8) | ((uint32_t)off << 16) | ((uint32_t)hi << 24);
         if (share == 0) {
             s_copy[slot][lane] = make_uint2(rw, (uint32_t)n_w | ((uint32_t)to_w << 16));
-            s_row[slot][lane] = make_uint4(w0, w1, place, (uint32_t)j0 | ((uint32_t)n0 << 16));
+            s_row[slot][lane] = make_uint4(w0, w1, place, (uint32_t)(b0 + kJoinAlign) | ((uint32_t)n0 << 16));
         }
         const bool whole = __all_sync(0xffffffffu, off == 0 && hi == 64);
         sync();
@@ -381,23 +387,21 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 7) k_join(const uint32_t* __r
                 for (uint32_t w = 16; w + (uint32_t)(lane & 15) < n; w += 16) copy(to + w * 4u, from + w);
         }
         // ---- lane = row: values up to ke, whole groups ----
-        while (share == 0 && done < done_to) {
+        for (int done = (ks + 7) & ~7; share == 0 && done < done_to; done += 8) {
             uint32_t v[4];
             dec.next(done, s_lut, vdata, jg, v);
             uint32_t* to = reinterpret_cast<uint32_t*>(mine + done - base8);
 #pragma unroll
             for (int i = 0; i < 4; ++i) to[i] = v[i];
-            done += 8;
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         sync();
         // ---- lane = 8 columns of one of four rows ----
-        auto write = [&](auto whole_c, auto vec_c) {
+        auto write = [&](auto whole_c) {
             constexpr bool W = decltype(whole_c)::value;                // every row has the whole window: nothing to leave out
-            constexpr int V = decltype(vec_c)::value;                   // bytes a store
             const int o = lane & 7, c = o * 8, r_first = share * 4 + (lane >> 3);
             const uint32_t sh = 8u * (uint32_t)(o & 3);
-            uint16_t* to_row = out + (size_t)(rb * kRowsPerBlock + r_first) * jg.k + (c_base + c);
+            uint16_t* to_row = out + (size_t)(rb * kRowsPerBlock + r_first) * jg.k + (c_base + c) - kJoinAlign;
             uint32_t row_a = buf_a + (uint32_t)(r_first * kJoinRow) * 2u;
 #pragma unroll 1
             for (int r = r_first; r < kRowsPerBlock; r += 4 * kSteps, to_row += (size_t)(4 * kSteps) * jg.k, row_a += 4 * kSteps * kJoinRow * 2) {
@@ -416,29 +420,18 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 7) k_join(const uint32_t* __r
                     ak += keep ? 2u : 0u;
                     ar += keep ? 0u : 2u;
                 }
-                uint16_t* to = to_row + (p.w & 0xFFFFu) * 32u;
-                if (V >= 4 && (W || (c >= r_off && c + 8 <= r_hi))) {
-                    const uint4 y = make_uint4(x[0] | (x[1] << 16), x[2] | (x[3] << 16), x[4] | (x[5] << 16), x[6] | (x[7] << 16));
-                    if (V == 16) {
-                        *reinterpret_cast<uint4*>(to) = y;
-                    } else {
-                        reinterpret_cast<uint32_t*>(to)[0] = y.x; reinterpret_cast<uint32_t*>(to)[1] = y.y;
-                        reinterpret_cast<uint32_t*>(to)[2] = y.z; reinterpret_cast<uint32_t*>(to)[3] = y.w;
-                    }
+                uint16_t* to = to_row + (p.w & 0xFFFFu);
+                if (W || (c >= r_off && c + 8 <= r_hi)) {
+                    *reinterpret_cast<uint4*>(to) = make_uint4(x[0] | (x[1] << 16), x[2] | (x[3] << 16), x[4] | (x[5] << 16), x[6] | (x[7] << 16));
                 } else {
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        if (W || (c + i >= r_off && c + i < r_hi)) to[i] = (uint16_t)x[i];
+                        if (c + i >= r_off && c + i < r_hi) to[i] = (uint16_t)x[i];
                 }
             }
         };
-        auto write_v = [&](auto whole_c) {
-            if (vec16) write(whole_c, std::integral_constant<int, 16>{});
-            else if (vec4) write(whole_c, std::integral_constant<int, 4>{});
-            else write(whole_c, std::integral_constant<int, 2>{});
-        };
-        if (whole) write_v(std::true_type{});
-        else write_v(std::false_type{});
+        if (whole) write(std::true_type{});
+        else write(std::false_type{});
         sync();
         // ---- values decoded ahead move to the front ----
         if (share == 0 && (ke & 7) && (ke & ~7) != base8) {
@@ -449,8 +442,9 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 7) k_join(const uint32_t* __r
             for (int i = 0; i < 4; ++i) to[i] = m[i];
         }
         ks = ke;
-        if (more) col = j0 * 32 + hi;
-        j0 += 2;
+        raw_at += n_raw;
+        if (more) col = b0 + hi;
+        b0 += 64;
     }
 }
 
