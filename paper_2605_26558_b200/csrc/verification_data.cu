@@ -132,9 +132,9 @@ __global__ void __launch_bounds__(32 * kSplitWarps) k_split(const uint32_t* __re
 // whole chunk's values, which 20 warps an SM had room for, and one row after the other with its loads).  6144 x 4096 at 40 %
 // pruning 109 -> 58 us, at 30 % 217 -> 61 (a chunk took a second turn), at 60 % 109 -> 54; 28672 x 4096 374 -> 209.
 constexpr int kJoinWarps = 4;
-// Chunks up to which teams: 31 and 37 us with and without for 9000 x 641 (846 chunks), 27 and 33 for 4096 x 2048 (1024), but 63 and 51 for
-// 2000 x 5000 (1260, t = 3) and 89 and 61 for 6144 x 4096 (3072).
-constexpr int kJoinTeamMax = 8 * kSms;
+// Chunks up to which teams: as long as all have a place at once, seven CTAs an SM.  23 and 32 us with and without for 3908 x 1528 (738 chunks), 20 and 27
+// for 9000 x 600 (846), but 43 and 41 for 640 x 14336 (1120), 40 and 37 for 2171 x 4088 (1088), 76 and 61 for 5979 x 4088 (2976).
+constexpr int kJoinTeamMax = 7 * kSms;
 // Halfwords: a row's windows begin where its output is on a 16-byte boundary, so that whatever the width eight columns leave in one store.
 // With windows from bitmap words on and one store width for the whole matrix 8987 x 4089 took 139 us instead of 86, 19995 x 4090 171 instead of 160, and
 // 4096 x 13823 210 instead of 122.  On 32-, 64- and 128-byte boundaries a chunk takes more windows: 20000 x 1528 66.5, then 67.8, 68.7 and 73.7.
@@ -448,147 +448,6 @@ __global__ void __launch_bounds__(32 * kJoinWarps, 7) k_join(const uint32_t* __r
     }
 }
 
-// The same for few chunks: a CTA's four warps share one, the first decoding a chunk's values into a list (kJoinCap of a row; longer chunks
-// take another turn), then each writing a quarter of the rows, lane = two neighbouring columns; a row's loads are all under way before
-// its first store.  Many more instructions, and less latency where all chunks have a place at once (kJoinRowsMax), above all with
-// odd columns, whose stores are halfwords: 3908 x 1529 27 us, by windows (teams) 33; with t = 3 27 and 43; 2000 x 1528 21 and 22.
-constexpr int kJoinCap = 168;
-constexpr int kJoinStride = kJoinCap + 2;                               // halfwords: an odd number of words, rows in different banks
-constexpr int kJoinSpan = 5;                                            // pairs of bitmap words (64 columns) of a row at a time
-static_assert(kJoinCap % 8 == 0 && (kJoinStride / 2) % 2 == 1, "groups of 8; odd row stride in words");
-// One wave of five CTAs an SM.  Beyond, 9000 x 641 (846 chunks) 39 us by rows, 31 by windows; 4096 x 2047 (1024) 45 and 37.  Odd columns
-// once more between the windows' teams and the end of a second wave: 7000 x 1529 (1314) 49 and 53.
-constexpr int kJoinRowsMax = 5 * kSms;
-
-template <int T>                                                        // truncated bits
-__global__ void __launch_bounds__(32 * kJoinWarps, 5) k_join_rows(const uint32_t* __restrict__ blob, const uint32_t* __restrict__ vdata,
-                                                                  uint16_t* __restrict__ out, JoinGeom jg) {
-    __shared__ __align__(4) uint16_t s_list[32 * kJoinStride + 64 * kJoinSpan + 2];      // a look past the last list reads what no column takes
-    __shared__ uint16_t s_lut[256];                                     // rank -> exponent at its bf16 position
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint8_t* cb = reinterpret_cast<const uint8_t*>(blob) + kBlobHeaderBytes;
-    pdl_wait();
-    for (int i = threadIdx.x; i < 256; i += 32 * kJoinWarps) s_lut[i] = (uint16_t)cb[i] << 7;
-    __syncthreads();
-    const int task = (int)blockIdx.x;
-    if (task >= jg.n_tasks) return;
-    const int sb = task / jg.n_ch, ch = task % jg.n_ch, rb = sb / jg.n_seg, seg = sb % jg.n_seg;
-    const uint4 dir = __ldg(reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4) + sb);
-    const int scols = seg_cols_of(jg.k_pad, jg.seg_cols, seg), n_ch = dir_n_ch(dir.w), E = dir_chunk_elems(dir.w);
-    if (ch >= n_ch) return;                                             // a shorter last segment
-    const SbGeom sg = SbGeom::make(n_ch, scols, (int)dir.y, (int)dir.z);
-    const uint32_t* body = blob + (size_t)dir.x * 4;
-    const int c_base = seg * jg.seg_cols;
-    const uint32_t e0 = __ldg(body + sg.tab + ch * 32 + lane), total = __ldg(body + sg.tab + n_ch * 32 + lane);
-    const int col_end = ch + 1 < n_ch ? (int)(__ldg(body + sg.tab + (ch + 1) * 32 + lane) >> 20) : scols;
-    int col = ch == 0 ? 0 : (int)(e0 >> 20);                            // this lane's row: first column not yet written
-    const int cnt = max(0, min(E, (int)(total >> 20) - ch * E));        // its kept values in this chunk
-    int k_row = ch * E;                                                 // kept values of the row before this chunk
-    for (int i = 0; i < seg; ++i) {
-        const uint4 dp = __ldg(reinterpret_cast<const uint4*>(blob + kBlobDirOffset / 4) + rb * jg.n_seg + i);
-        k_row += (int)(__ldg(blob + (size_t)dp.x * 4 + dir_n_ch(dp.w) * 32 + lane) >> 20);
-    }
-    const int n_max = __reduce_max_sync(0xffffffffu, cnt);
-    JoinGroups<T> dec;
-    if (warp == 0) {
-        dec.begin(body, sg, lane, rb * kRowsPerBlock + lane, ch * E, k_row, e0 & 0xFFFFFu, s_lut, vdata, jg);
-    }
-    uint16_t* mine = s_list + lane * kJoinStride;
-
-    for (int p0 = 0; p0 == 0 || p0 < n_max; p0 += kJoinCap) {
-        const int n_here = min(kJoinCap, n_max - p0);
-        if (warp == 0) {
-            // ---- lane = row: values p0 .. p0 + n_here - 1 of the chunk ----
-#pragma unroll 1
-            for (int g = 0; g < n_here; g += 8) {
-                uint32_t v[4];
-                dec.next(p0 + g, s_lut, vdata, jg, v);
-                uint32_t* to = reinterpret_cast<uint32_t*>(mine + g);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) to[i] = v[i];
-            }
-        }
-        __syncthreads();
-        // ---- lane = two columns: one row after the other ----
-        constexpr int kRowStep = kJoinWarps;
-        uint32_t bm_next = 0;                                           // the row's bitmap words, one a lane, fetched a row ahead
-        auto words = [&](int r) {
-            const int c0 = __shfl_sync(0xffffffffu, col, r), j = (c0 >> 5) + lane;
-            return lane < 2 * kJoinSpan && j < sg.bm_words ? __ldg(body + sg.bm + j * 32 + r) : 0u;
-        };
-        bm_next = words(warp);
-#pragma unroll 1
-        for (int r = warp; r < kRowsPerBlock; r += kRowStep) {
-            uint32_t bmv = bm_next;
-            if (r + kRowStep < kRowsPerBlock) bm_next = words(r + kRowStep);
-            const int row = rb * kRowsPerBlock + r;
-            if (row >= jg.n) break;
-            const int c0 = __shfl_sync(0xffffffffu, col, r), c_row = __shfl_sync(0xffffffffu, col_end, r);
-            const int n_row = __shfl_sync(0xffffffffu, cnt, r), kr = __shfl_sync(0xffffffffu, k_row, r);
-            if (c0 >= c_row) continue;
-            const int k_end = min(p0 + n_here, n_row);                  // list entries of this turn: chunk values p0 .. k_end - 1
-            const bool last = k_end == n_row;                           // else the row goes up to the value k_end, exclusive
-            const uint16_t* list = s_list + r * kJoinStride - p0;
-            const uint16_t* raw = reinterpret_cast<const uint16_t*>(vdata + (jg.n_raw > 0 ? kVdataHeaderWords + (size_t)row * jg.row_words + jg.lo_words : 0));
-            uint16_t* orow = out + (size_t)row * jg.k + c_base;
-            const bool pairs = (((size_t)row * jg.k) & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 3) == 0;
-            const int lim = min(last ? c_row : scols, jg.k - c_base), j_end = (lim + 31) / 32;
-            int kpos = p0, stop = c_row;
-            const uint32_t r_last = (uint32_t)max(jg.n_raw - 1, 0), left = ~(0xFFFFFFFFu >> (2 * (lane & 15)));
-            for (int j0 = c0 >> 5;;) {
-                if (j0 * 32 < c0 && lane == 0) bmv &= 0xFFFFFFFFu >> (c0 & 31);      // values before belong to an earlier turn
-                int pre = __popc(bmv), here = pre;                      // kept values before each word
-#pragma unroll
-                for (int o = 1; o < 16; o <<= 1) {
-                    const int v = __shfl_up_sync(0xffffffffu, pre, o);
-                    if (lane >= o) pre += v;
-                }
-                const int all = __shfl_sync(0xffffffffu, pre, 15);
-                pre += kpos - here;
-                // both candidates of every column are loaded, without a condition, before any is used: a choice between the
-                // loads is a divergent branch that waits for each in turn
-                uint32_t lx[kJoinSpan][2], rx[kJoinSpan][2], two[kJoinSpan];
-                int bf[kJoinSpan];
-                const int q0 = c_base + lane * 2 - kr;
-#pragma unroll
-                for (int i = 0; i < kJoinSpan; ++i) {
-                    const uint32_t b = __shfl_sync(0xffffffffu, bmv, 2 * i + (lane >> 4));
-                    bf[i] = __shfl_sync(0xffffffffu, pre, 2 * i + (lane >> 4)) + __popc(b & left);      // kept values before the first column
-                    two[i] = b << (2 * (lane & 15));                    // kept? this lane's columns at the top
-                    const uint32_t p_at = (uint32_t)(q0 + (j0 + 2 * i) * 32 - bf[i]);                   // pruned ones = columns - kept
-                    lx[i][0] = list[bf[i]];
-                    lx[i][1] = list[bf[i] + 1];
-                    rx[i][0] = __ldg(raw + min(p_at, r_last));
-                    rx[i][1] = __ldg(raw + min(p_at + 1u, r_last));
-                }
-#pragma unroll
-                for (int i = 0; i < kJoinSpan; ++i) {
-                    const int j = j0 + 2 * i, c = j * 32 + lane * 2;
-                    const bool k0 = two[i] >> 31, k1 = (two[i] >> 30) & 1u;
-                    const uint32_t x0 = k0 ? lx[i][0] : rx[i][0];
-                    const uint32_t xl = k0 ? lx[i][1] : lx[i][0], xr = k0 ? rx[i][0] : rx[i][1], x1 = k1 ? xl : xr;
-                    if (pairs && last && j * 32 >= c0 && (j + 2) * 32 <= lim) {
-                        *reinterpret_cast<uint32_t*>(orow + c) = x0 | (x1 << 16);
-                    } else if (j < j_end) {                             // the row's ends, and rows off 4-byte boundaries
-                        if (c >= c0 && c < lim && (last || bf[i] + k0 <= k_end)) orow[c] = (uint16_t)x0;
-                        if (c + 1 >= c0 && c + 1 < lim && (last || bf[i] + k0 + k1 <= k_end)) orow[c + 1] = (uint16_t)x1;
-                        if (!last && kpos + all > k_end && stop == c_row) {      // the value k_end is in these words: its column begins the next turn
-                            const uint32_t at = __reduce_min_sync(0xffffffffu, k0 && bf[i] == k_end ? (uint32_t)c : k1 && bf[i] + k0 == k_end ? (uint32_t)(c + 1) : 0xFFFFFFFFu);
-                            if (at != 0xFFFFFFFFu) stop = (int)at;
-                        }
-                    }
-                }
-                j0 += 2 * kJoinSpan;
-                if (j0 >= j_end || stop != c_row) break;
-                kpos += all;
-                bmv = lane < 2 * kJoinSpan && j0 + lane < sg.bm_words ? __ldg(body + sg.bm + (j0 + lane) * 32 + r) : 0u;
-            }
-            if (lane == r) col = last ? c_row : stop;
-        }
-        __syncthreads();
-    }
-}
-
 }  // namespace cass
 
 using namespace cass;
@@ -624,12 +483,10 @@ extern "C" int cass_decode_full(const void* blob, const cass_blob_info* bi, cons
     const JoinGeom jg{bi->rows, bi->cols, ceil_div(bi->cols, 32) * 32, bi->seg_cols, bi->n_seg, n_ch,
                       bi->n_rowblocks * bi->n_seg * n_ch, vdata_lo_words(bi->kept_per_row, bi->trunc_bits),
                       vdata_row_words(bi->cols, bi->kept_per_row, bi->trunc_bits), bi->cols - bi->kept_per_row};
-    const bool team = jg.n_tasks < kJoinTeamMax;
-    const bool by_rows = jg.n_tasks <= kJoinRowsMax || (jg.k % 2 && !team && jg.n_tasks <= 2 * kJoinRowsMax);
+    const bool team = jg.n_tasks <= kJoinTeamMax;
 #define CASS_JOIN(T_)                                                                                                               \
     do {                                                                                                                            \
-        if (by_rows) CASS_PDL_LAUNCH(k_join_rows<T_>, dim3(jg.n_tasks), dim3(32 * kJoinWarps), 0, stream, b32, v32, o16, jg);       \
-        else if (team) CASS_PDL_LAUNCH((k_join<T_, true>), dim3(jg.n_tasks), dim3(32 * kJoinWarps), 0, stream, b32, v32, o16, jg);        \
+        if (team) CASS_PDL_LAUNCH((k_join<T_, true>), dim3(jg.n_tasks), dim3(32 * kJoinWarps), 0, stream, b32, v32, o16, jg);        \
         else CASS_PDL_LAUNCH((k_join<T_, false>), dim3(ceil_div(jg.n_tasks, kJoinWarps)), dim3(32 * kJoinWarps), 0, stream, b32, v32, o16, jg); \
     } while (0)
     switch (bi->trunc_bits) {
