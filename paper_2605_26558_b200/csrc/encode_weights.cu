@@ -1079,10 +1079,12 @@ extern "C" int cass_encode_weights(const cass_format* fmt, const void* W_bf16, c
         };
         return ends % 16 == 0 ? pack(uint4{}) : ends % 4 == 0 ? pack(uint32_t{}) : pack(uint16_t{});
     }
+    // (t = 4 without lanes: few columns, or rows off 16-byte boundaries with a place for every superblock; with field places computed at run
+    // time 5000 x 512 took 44 us instead of 40, 20000 x 501 107 instead of 98, 9000 x 641 69 instead of 65)
     if (n_sb <= kSms) rc = g.mx ? (g.t == 4 ? launch_pack(k_pack<true, 4, 1024>, 1024) : launch_pack(k_pack<true, -1, 1024>, 1024))
                                : (g.t == 4 ? launch_pack(k_pack<false, 4, 1024>, 1024) : launch_pack(k_pack<false, -1, 1024>, 1024));
     else rc = g.mx ? (g.t == 4 ? launch_pack(k_pack<true, 4, 512>, 512) : launch_pack(k_pack<true, -1, 512>, 512))
-                   : launch_pack(k_pack<false, -1, 512>, 512);      // t = 4: by lanes
+                   : (g.t == 4 ? launch_pack(k_pack<false, 4, 512>, 512) : launch_pack(k_pack<false, -1, 512>, 512));
     if (rc) return rc;
     return CASS_OK;
 }
