@@ -77,7 +77,7 @@ def test_rows_in_turn(cass, rows, cols):
 
 @pytest.mark.parametrize("rows,cols,p,seg,chunk", [(9000, 520, 400, 0, 0), (41601, 200, 400, 0, 0), (21000, 470, 300, 0, 0), (2410, 2569, 400, 0, 0),
                                                     (2410, 2570, 600, 0, 0), (1600, 5300, 0, 0, 0), (3000, 2056, 400, 1024, 32), (1600, 4100, 990, 0, 0),
-                                                    (4801, 512, 400, 0, 0), (4737, 641, 600, 0, 0)])
+                                                    (4801, 512, 400, 0, 0), (4737, 641, 600, 0, 0), (4801, 1300, 400, 0, 0)])
 def test_blobs_by_lanes(cass, rows, cols, p, seg, chunk):
     """Matrices of so many blocks that sizes and packing go by lanes: 2 to 16 warps a superblock, rows on 16-, 4- and 2-byte
     boundaries, chunks of few values, a last row block that is not full; rows of one value, of none, and with codes longer than a word.
