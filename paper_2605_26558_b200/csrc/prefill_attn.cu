@@ -204,14 +204,14 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_prefill_attn(const __grid_con
             __syncwarp();
             if (lane == 0) pa_arrive(bar);
         };
-        // 32 scores from token t of chunk c on; those beyond the pair's position -inf (none in a chunk that the first row sees whole)
-        auto load = [&](int u, int c, int t, float (&a)[32]) {
+        // 32 scores from token t of chunk c on; those beyond the position `to` -inf, where some lane's chunk is cut
+        auto load = [&](int u, int c, int t, int to, bool cut, float (&a)[32]) {
             uint32_t v[32];
             tmem_ld32(lanes + kPaS + (u & 1) * 128 + t, v);
 #pragma unroll
             for (int i = 0; i < 32; ++i) a[i] = __uint_as_float(v[i]);
-            if (c * kPaTok + kPaTok - 1 > len) {
-                const int left = lim - (c * kPaTok + t);                     // tokens 0 .. left are seen
+            if (cut) {
+                const int left = to - (c * kPaTok + t);                      // tokens 0 .. left are seen
 #pragma unroll
                 for (int i = 0; i < 32; ++i) a[i] = i <= left ? a[i] : -INFINITY;
             }
@@ -220,11 +220,11 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_prefill_attn(const __grid_con
         for (int u = wg; u < n && ok; u += 2) {
             wait(&s_full[u & 1], u >> 1);
             if (!ok) break;
-            float m = -INFINITY;
+            float m = __int_as_float(0x7FFFFFFF);                            // NaN: left only where all 128 are
 #pragma unroll 1
             for (int t = 0; t < kPaTok; t += 32) {
                 float a[32];
-                load(u, u, t, a);
+                load(u, u, t, lim, u * kPaTok + kPaTok - 1 > len, a);            // cut: the first row does not see the whole chunk
 #pragma unroll
                 for (int i = 0; i < 32; ++i) m = fmaxf(m, a[i]);
             }
@@ -281,7 +281,10 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_prefill_attn(const __grid_con
             const int u = n + i;
             if (i > 0) c = next_chunk(c_prev);
             if ((u & 1) == wg) {
-                const float mc = __ldcg(sm + (size_t)c * kPaPairs), m = mc == -INFINITY ? 0.f : mc;      // nothing seen: exp(-inf) = 0
+                // no maximum (nothing seen, or beside what is not seen NaN alone): numerators 0, as in the verification kernel
+                const float mc = __ldcg(sm + (size_t)c * kPaPairs), m = mc == -INFINITY ? 0.f : mc;
+                const int to = mc == -INFINITY ? -1 : lim;
+                const bool cut = __any_sync(0xffffffffu, mc == -INFINITY) || c * kPaTok + kPaTok - 1 > len;
                 wait(&s_full[u & 1], u >> 1);
                 if (!ok) break;
                 float l[32];
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) k_prefill_attn(const __grid_con
                 for (int t = 0; t < kPaTok; t += 32) {
                     float a[32];
                     uint32_t hi[16], lo[16];
-                    load(u, c, t, a);
+                    load(u, c, t, to, cut, a);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) {
                         float e[2], h[2];

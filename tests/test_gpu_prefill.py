@@ -151,6 +151,39 @@ def test_prefill_attention_of_every_group(cass, heads, kv, batch, n):
     b.close()
 
 
+@pytest.mark.parametrize("heads,kv", [(8, 2), (2, 2)])
+@pytest.mark.parametrize("first,last", [(256, 300), (0, 128), (290, 300)])
+def test_scores_that_are_no_numbers(cass, heads, kv, first, last):
+    """K of some tokens overflows to infinities of both signs, and all scores there are NaN.  Both paths pass over a chunk that such
+    tokens begin and the causal limit ends, and lose a row to one that they fill."""
+    n, d, hidden = 300, 128, 256
+    shape = synth.ModelShape(n_layers=1, hidden=hidden, n_q_heads=heads, n_kv_heads=kv, head_dim=d, ffn=256, vocab=512)
+    wt = synth.model_weights(shape, 6, device="cuda")
+    gw = {"layers": [cass.engine.fuse_layer_weights(lw) for lw in wt["layers"]], "embed": wt["embed"].clone(), "lm_head": wt["lm_head"],
+          "norm_final": wt["norm_final"]}
+    layer, wide = gw["layers"][0], 7                                       # input channel `wide`: 1e36 of it, for K alone
+    gw["embed"][:, wide] = 0.0
+    gw["embed"][0, wide] = gw["embed"][0].abs().max()
+    layer["norm_attn"] = layer["norm_attn"].clone()
+    layer["norm_attn"][wide] = 1e36
+    layer["wqkv"] = layer["wqkv"].clone()
+    layer["wqkv"][:, wide] = 0.0
+    layer["wqkv"][heads * d: (heads + kv) * d, wide] = 1e4 * (1 - 2 * (torch.arange(kv * d, device="cuda") % 2)).to(torch.bfloat16)
+    prompt = synth.random_prompt(n, shape.vocab - 1, 70) + 1
+    prompt[first: last] = 0
+    a, b = (cass.engine.Engine(shape, gw, max_seq=384, gamma_max=4) for _ in range(2))
+    a.prefill(prompt)
+    _, rows = _chunked(cass, b, prompt)
+    assert a.status()[0] == b.status()[0] == 0
+    k, v = _cache(cass, a, n)
+    k = k.view(n, -1)
+    assert not torch.isfinite(k[first: last]).any() and torch.isfinite(k[:first]).all() and torch.isfinite(k[last:]).all() and torch.isfinite(v).all()
+    x, y = (_activation(cass, e, 1, rows) for e in (a, b))
+    assert torch.isfinite(y).all() == (first == 256) and torch.equal(x.view(torch.int16), y.view(torch.int16))
+    a.close()
+    b.close()
+
+
 def test_two_bf16_terms_are_as_accurate_as_the_fp32_pipes(cass):
     """Five query heads a KV head at head size 128: verification takes 16 rows to the fp32 pipes, the wide pass to the tensor
     cores with P in two bf16 terms.  On the same queries and caches both differ from 64 bits by the rounding of the output alone
