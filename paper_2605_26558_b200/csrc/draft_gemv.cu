@@ -671,9 +671,11 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
     if (out != 2) return;
     cg::cluster_group cluster = cg::this_cluster();
     cluster.sync();                                     // every CTA comes here, also one that gave up
-    if (done && cluster.block_rank() == 0) {
+    // One vector: by the first warp, without a loop.  (As a loop over warps it cost the instantiations for t = 0 and 4 above 52 % pruning, whose
+    // windows' code the compiler then lays out otherwise: 512 x 512 at 53 % 4.4 -> 6.1 us, 4096 x 2048 6.6 -> 8.1, 28672 x 4096 at 60 % 39.3 -> 40.9.)
+    if (done && cluster.block_rank() == 0 && (NB > 1 || threadIdx.x < 32)) {
         const int row = (int)blockIdx.y * kRowsPerBlock + lane;
-        for (int b = threadIdx.x >> 5; b < NB; b += (int)blockDim.x >> 5) {
+        for (int b = NB > 1 ? (int)threadIdx.x >> 5 : 0; b < NB; b += NB > 1 ? (int)blockDim.x >> 5 : 1) {
             float part[8];
 #pragma unroll
             for (int s = 0; s < 8; ++s) part[s] = *cluster.map_shared_rank(&s_sum[b][lane], min(s, n_seg - 1));
