@@ -241,36 +241,42 @@ static int launch_wide(const CUtensorMap& mw, const CUtensorMap& mx, uint16_t* o
 
 // Rows of a tile: the one whose rounds of all pairs take least, a K block of a round being 0.22, 0.27 and 0.37 us at 128, 192 and 256
 // rows (4096 x 14336, 1000 rows).  1000 rows: 28672 x 4096 186, 178 and 168 us, 6144 x 4096 49, 43 and 56.
-static int wide_gemm_plan(int rows, int n, int* rounds_us100) {
+struct WidePlan { int bn, rounds, block_us100; };
+static WidePlan wide_gemm_plan(int rows, int n) {
     const int us100[3] = {37, 27, 22};
-    int best = 256;
+    WidePlan best{0, 0, 0};
     for (int i = 0; i < 3; ++i) {
-        const int bn = 256 - 64 * i, c = ceil_div(ceil_div(n, 2 * kWgBM) * ceil_div(rows, bn), kPairs) * us100[i];
-        if (i == 0 || c < *rounds_us100) { *rounds_us100 = c; best = bn; }
+        const int bn = 256 - 64 * i, rounds = ceil_div(ceil_div(n, 2 * kWgBM) * ceil_div(rows, bn), kPairs);
+        if (i == 0 || rounds * us100[i] < best.rounds * best.block_us100) best = WidePlan{bn, rounds, us100[i]};
     }
     return best;
 }
 
-// Where the split-K kernel takes the rows too (up to kSplitRows): it spreads the K ranges over the chip but writes each one's sums,
-// which take longer the more rows there are.  us = rounds x (K blocks of a range x x + e) against 2 + K blocks x the above; measured, split-K
-// with its addition / this one: 6144 x 4096 16 / 21 us for 64 rows, 21 / 21 for 128, 33 / 21 for 256; 4096 x 14336 49 / 51 for 256;
-// 28672 x 4096 55 / 46 for 40; 256 x 688 13 / 9 for 256.
+// Where the split-K kernel takes the rows too (up to kSplitRows): it spreads the K ranges over the chip but writes each one's sums, which
+// the next kernel reads; here they follow one another, each at least as long as its sums' addition to the registers (1.2 us for 128 rows).
+// Both sides in hundredths of a us, fitted to kernel times (split-K with what its parts cost the next kernel) of six models' projections, 256 to
+// 5120 wide, at 33 to 256 rows: the faster one is chosen but for 10 of 216, by 0.2 % of the time over all.  Split-K / this one: 256 x 688
+// 5 / 9 us for 64 rows, 11 / 10 for 160; 2048 x 2048 6 / 17 for 64, 12 / 17 for 256; 6144 x 4096 17 / 22 for 128, 26 / 22 for 256; 28672 x
+// 4096 52 / 48 for 64, 92 / 62 for 256; 4096 x 14336 36 / 53 for 256.
 bool wide_gemm_pays(int rows, int n, int k) {
     if (rows > kSplitRows) return true;
     if (rows <= 32) return false;
-    int kbt, kbs, ns, wide;
+    int kbt, kbs, ns;
     verify_gemm_split(n, k, &kbt, &kbs, &ns);
-    wide_gemm_plan(rows, n, &wide);
-    const int x = rows <= 64 ? 86 : rows <= 128 ? 91 : 111, e = rows <= 64 ? 280 : rows <= 128 ? 690 : 1680;      // hundredths of a us
-    return 200 + wide * kbt < ceil_div(ceil_div(n, kWgBM) * ns, 2 * kSms) * (kbs * x + e);
+    const WidePlan plan = wide_gemm_plan(rows, n);
+    const int range = kbs * plan.block_us100, add = 120 * plan.bn / 128;
+    const int c = rows <= 64 ? 0 : rows <= 128 ? 1 : 2;                      // columns of the split-K kernel's tile: 64, 128, 256
+    constexpr int kCall[3] = {200, 350, 500}, kBlock[3] = {74, 74, 98}, kRound[3] = {0, 0, 400}, kParts[3] = {16, 12, 8};
+    const int rounds = ceil_div(ceil_div(n, kWgBM) * ns, 2 * kSms);
+    return 700 + plan.rounds * ns * (range > add ? range : add) <
+           kCall[c] + rounds * (kbs * kBlock[c] + kRound[c]) + (long long)ns * rows * n * kParts[c] / 100000;
 }
 
 int launch_wide_gemm(const uint16_t* W, const uint16_t* X, int x_rows, int rows, int n, int k, uint16_t* out, int32_t* d_status, cudaStream_t s,
                      int w_static) {
     if (rows < 1 || rows > x_rows || (k % 8) || n < 1 || !out || !d_status) return CASS_ERR_INVALID_ARG;
     if (((uintptr_t)W & 15) || ((uintptr_t)X & 15)) return CASS_ERR_INVALID_ARG;
-    int us;
-    const int bn = wide_gemm_plan(rows, n, &us);
+    const int bn = wide_gemm_plan(rows, n).bn;
     CUtensorMap mw, mx;
     int rc = tc_matrix_map(&mw, W, n, k, kWgBM);
     if (rc) return rc;

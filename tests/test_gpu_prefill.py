@@ -128,6 +128,26 @@ def test_wide_projections_equal_verification_calls(cass, batch, n):
     b.close()
 
 
+@pytest.mark.parametrize("n", [33, 64, 65, 128, 129, 192, 193, 256])
+def test_wide_projection_of_few_rows_between_split_ones(cass, n):
+    """A projection of so many features that few rows pay in the wide form (tiles of 128 and 192 rows, K and features off the tiles'
+    multiples) among others that are split: bf16 results and parts in one layer."""
+    shape = synth.ModelShape(n_layers=1, hidden=1288, n_q_heads=4, n_kv_heads=2, head_dim=64, ffn=10328, vocab=512)
+    wt = synth.model_weights(shape, 8, device="cuda")
+    gw = {"layers": [cass.engine.fuse_layer_weights(lw) for lw in wt["layers"]], "embed": wt["embed"], "lm_head": wt["lm_head"],
+          "norm_final": wt["norm_final"]}
+    prompt = synth.random_prompt(n, shape.vocab, 80)
+    a, b = (cass.engine.Engine(shape, gw, max_seq=288, gamma_max=4) for _ in range(2))
+    first = a.prefill(prompt)
+    want, rows = _chunked(cass, b, prompt)
+    assert [first] == want and a.status()[0] == b.status()[0] == 0
+    assert all(torch.equal(x, y) for x, y in zip(_cache(cass, a, n), _cache(cass, b, n)))
+    for w in (0, 1, 2):
+        assert torch.equal(_activation(cass, a, w, rows), _activation(cass, b, w, rows)), w
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("heads,kv,batch,n", [(2, 2, 1, 127), (2, 2, 1, 257), (2, 1, 1, 1025), (3, 1, 2, 129), (3, 1, 1, 1190), (4, 1, 4, 300), (8, 1, 1, 300), (7, 1, 1, 1100)])
 def test_prefill_attention_of_every_group(cass, heads, kv, batch, n):
     """Head size 128: groups that leave lanes of a CTA without a pair, ends of chunks and of CTAs, more than eight chunks (chains of
