@@ -117,7 +117,8 @@ __device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t v) {
 }
 
 // LANES: the bitmap goes to 32 rows' words side by side (decided at run time it took a value's address two multiplications: 15000 x 512 72.7
-// us instead of 70.7, 9000 x 641 at 60 % 64.5 instead of 62.5, 12000 x 513 by lanes 78.8 instead of 76.9).
+// us instead of 70.7, 9000 x 641 at 60 % 64.5 instead of 62.5, 12000 x 513 by lanes 78.8 instead of 76.9).  Rows of several warps wait for one
+// another instead, and are faster so (4096 x 14336 140.8 us, as a constant 142.9): WIDE asks the geometry.
 template <int NV, bool WIDE, bool LANES>
 __global__ void __launch_bounds__(!WIDE ? 128 : NV == 128 ? 32 * kSelWarps : 32 * kSelWarps64, !WIDE ? 6 : NV == 128 ? 1 : 2)
     k_select(const uint16_t* __restrict__ W, const float* __restrict__ act, EncGeom g, uint32_t* __restrict__ keepbm,
@@ -280,8 +281,10 @@ __global__ void __launch_bounds__(!WIDE ? 128 : NV == 128 ? 32 * kSelWarps : 32 
         }
         // kept: the values above the shared upper half, and those of the list from the threshold on
         const __nv_bfloat162 t2 = as_bf162(top ? top | (top << 16) : 0x007F007Fu);
-        const size_t row_at = LANES ? (size_t)(row / kRowsPerBlock) * kRowsPerBlock * row_bytes + (size_t)(row % kRowsPerBlock) * 4 : (size_t)row * row_bytes;
+        const bool lanes = WIDE ? g.lanes != 0 : LANES;
+        const size_t row_at = lanes ? (size_t)(row / kRowsPerBlock) * kRowsPerBlock * row_bytes + (size_t)(row % kRowsPerBlock) * 4 : (size_t)row * row_bytes;
         uint8_t* keep_row = reinterpret_cast<uint8_t*>(keepbm) + row_at;
+        const int word_at = lanes ? 4 * kRowsPerBlock : 4;               // bytes between a row's words
 #pragma unroll
         for (int q = 0; q < NG; ++q) {
             const int c = col_of(q * 8);
@@ -298,7 +301,7 @@ __global__ void __launch_bounds__(!WIDE ? 128 : NV == 128 ? 32 * kSelWarps : 32 
                 kb = c + 8 <= g.k ? 0xFFu : c < g.k ? (0xFF00u >> (g.k - c)) & 0xFFu : 0u;
             }
             // byte of column c in its word: the first column at the most significant end
-            if (c / 8 < row_bytes) keep_row[LANES ? c / 32 * (4 * kRowsPerBlock) + ((c / 8 & 3) ^ 3) : (c / 8) ^ 3] = (uint8_t)kb;
+            if (c / 8 < row_bytes) keep_row[(size_t)(c / 32) * word_at + ((c / 8 & 3) ^ 3)] = (uint8_t)kb;
             if (!g.mx) {
                 uint32_t v[4];
                 row_load8(wr + c, kb, vec, v);
@@ -933,8 +936,8 @@ static int launch_select(const uint16_t* W, const float* act, const EncGeom& g, 
     if (k <= 512) return launch_select_as<16, false, LANES>(W, act, g, ws, stream);
     if (k <= 1024) return launch_select_as<32, false, LANES>(W, act, g, ws, stream);
     if (k <= 2048) return launch_select_as<64, false, LANES>(W, act, g, ws, stream);
-    if (k <= 2048 * kSelWarps64) return launch_select_as<64, true, LANES>(W, act, g, ws, stream);
-    return launch_select_as<128, true, LANES>(W, act, g, ws, stream);
+    if (k <= 2048 * kSelWarps64) return launch_select_as<64, true, false>(W, act, g, ws, stream);
+    return launch_select_as<128, true, false>(W, act, g, ws, stream);
 }
 
 // ---- test hook: zero-padded reconstruction of the whole blob ---------------------------------------------
