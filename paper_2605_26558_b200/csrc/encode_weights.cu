@@ -380,6 +380,8 @@ __global__ void __launch_bounds__(1024) k_sizes(const uint16_t* __restrict__ W, 
 // the whole encoder 332 -> 258.  Bitmaps in rows (each lane's word in a line of its own): packing 125, sizes 52; tiles of 128 columns, three
 // CTAs an SM for two and a bit rounds: 97 and 43; sizes without the next tile's loads under way 43.
 constexpr int kBlkCols = 128, kSegBlks = 2048 / kBlkCols;
+template <int N>
+using Int = std::integral_constant<int, N>;
 constexpr int kTileCols = 64, kTileWords = kTileCols / 32, kBlkTiles = kBlkCols / kTileCols;
 constexpr int kLaneRow = 16 + 2 * kTileCols;             // bytes of a row: up to 7 values left of the tile before, and the tile's
 constexpr int kLaneTile = 32 * kLaneRow;
@@ -512,10 +514,10 @@ __global__ void __launch_bounds__(32 * kSizeWarps) k_sizes_lanes(const uint16_t*
     }
 }
 
-// One CTA a superblock of t = 4, NW warps of kSegBlks / NW blocks each.  A block's kept values move to the front of the row, behind those
+// One CTA a superblock of t = 4, NW warps of PER blocks each.  A block's kept values move to the front of the row, behind those
 // that were left over (no branches: every value is stored, the next one takes its place if it is pruned), and leave as groups of 8: a field word,
 // and code bits in one word that goes to the row's code stream.  A word that two warps fill is zero before either adds to it.
-template <int NW, class V>
+template <int NW, int PER, class V>
 __global__ void __launch_bounds__(32 * NW) k_pack_lanes(const uint16_t* __restrict__ W, EncGeom g, const uint32_t* __restrict__ keepbm,
                                                         const uint8_t* __restrict__ exp_to_rank, const uint32_t* __restrict__ blk_size,
                                                         uint32_t* __restrict__ blob, const uint32_t* __restrict__ abort_flag) {
@@ -536,10 +538,10 @@ __global__ void __launch_bounds__(32 * NW) k_pack_lanes(const uint16_t* __restri
     const uint32_t* bmr = keepbm + ((size_t)rb * (g.k_pad / 32) + w0) * 32 + lane;
     auto bm_word = [&](int j) { return row < g.n && j < nw ? __ldg(bmr + j * 32) : 0u; };
     // where the warp's blocks begin: kept values and code bits of the row before them
-    const int b0 = warp * (kSegBlks / NW), b1 = b0 + kSegBlks / NW;
+    const int b0 = warp * PER, b1 = b0 + PER;
     uint32_t k = 0, pos = 0, all_k = 0, all_bits = 0;
 #pragma unroll
-    for (int b = 0; b < kSegBlks; ++b) {
+    for (int b = 0; b < NW * PER; ++b) {
         const uint32_t v = b * (kBlkCols / 32) < nw ? __ldg(blk_size + ((size_t)sb * kSegBlks + b) * 32 + lane) : 0u;
         all_k += v >> 16;
         all_bits += v & 0xFFFFu;
@@ -1068,19 +1070,24 @@ extern "C" int cass_encode_weights(const cass_format* fmt, const void* W_bf16, c
         return CASS_OK;
     };
     if (g.lanes) {
-        // warps a superblock: some 3000 of them in all, no more than it has blocks
-        const int blks = ceil_div(g.seg_cols, kBlkCols), nw = blks <= 2 ? 2 : blks <= 4 || n_sb >= 750 ? 4 : blks <= 8 || n_sb >= 375 ? 8 : 16;
-        auto pack_as = [&](auto warps, auto piece) -> int {
-            constexpr int NW = decltype(warps)::value;
+        // warps a superblock: some 3000 of them in all, no more than it has blocks.  The blocks that it has are what they share: of the 16 of
+        // 2048 columns each, half or more of the warps of a shorter segment had none (45000 x 256 112.6 -> 104.4 us, 30000 x 301 110.6 -> 99.0,
+        // 32000 x 512 108.6 -> 96.3, 20000 x 640 106.5 -> 92.1, 12000 x 520 65.6 -> 61.2)
+        const int blks = ceil_div(g.seg_cols, kBlkCols);
+        auto pack_as = [&](auto warps, auto blocks, auto piece) -> int {
+            constexpr int NW = decltype(warps)::value, PER = decltype(blocks)::value;
             using V = decltype(piece);
-            CASS_ALLOW_SMEM(k_pack_lanes<NW, V>);
-            CASS_PDL_LAUNCH((k_pack_lanes<NW, V>), dim3((unsigned)n_sb), dim3(32 * NW), (size_t)(NW * kLaneTile), stream, W, g, (const uint32_t*)ws.keepbm,
+            CASS_ALLOW_SMEM(k_pack_lanes<NW, PER, V>);
+            CASS_PDL_LAUNCH((k_pack_lanes<NW, PER, V>), dim3((unsigned)n_sb), dim3(32 * NW), (size_t)(NW * kLaneTile), stream, W, g, (const uint32_t*)ws.keepbm,
                             (const uint8_t*)ws.exp_to_rank, (const uint32_t*)ws.blk_size, b32, (const uint32_t*)ws.abort_flag);
             return CASS_OK;
         };
         auto pack = [&](auto piece) {
-            return nw == 2 ? pack_as(std::integral_constant<int, 2>{}, piece) : nw == 4 ? pack_as(std::integral_constant<int, 4>{}, piece)
-                   : nw == 8 ? pack_as(std::integral_constant<int, 8>{}, piece) : pack_as(std::integral_constant<int, 16>{}, piece);
+            if (blks <= 2) return pack_as(Int<2>{}, Int<1>{}, piece);
+            if (blks <= 4) return pack_as(Int<4>{}, Int<1>{}, piece);
+            if (n_sb >= 750) return blks <= 8 ? pack_as(Int<4>{}, Int<2>{}, piece) : blks <= 12 ? pack_as(Int<4>{}, Int<3>{}, piece) : pack_as(Int<4>{}, Int<4>{}, piece);
+            if (blks <= 8) return pack_as(Int<8>{}, Int<1>{}, piece);
+            return n_sb >= 375 ? pack_as(Int<8>{}, Int<2>{}, piece) : pack_as(Int<16>{}, Int<1>{}, piece);
         };
         return ends % 16 == 0 ? pack(uint4{}) : ends % 4 == 0 ? pack(uint32_t{}) : pack(uint16_t{});
     }

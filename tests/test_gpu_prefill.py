@@ -171,6 +171,44 @@ def test_prefill_attention_of_every_group(cass, heads, kv, batch, n):
     b.close()
 
 
+@pytest.mark.parametrize("n,max_seq", [(4097, 4224), (4240, 8448), (8300, 8448), (300, 32896)])
+def test_prefill_attention_of_many_chunks(cass, n, max_seq):
+    """Head size 128: more than 32 and 64 chunks of 128 positions, whose sums are added 32 at a time, and a cache of 257, which the
+    one-CTA attention does not take."""
+    shape = synth.ModelShape(n_layers=1, hidden=256, n_q_heads=2, n_kv_heads=1, head_dim=128, ffn=256, vocab=512)
+    wt = synth.model_weights(shape, 9, device="cuda")
+    gw = {"layers": [cass.engine.fuse_layer_weights(lw) for lw in wt["layers"]], "embed": wt["embed"], "lm_head": wt["lm_head"],
+          "norm_final": wt["norm_final"]}
+    prompt = synth.random_prompt(n, shape.vocab, 90)
+    a, b = (cass.engine.Engine(shape, gw, max_seq=max_seq, gamma_max=4) for _ in range(2))
+    first = a.prefill(prompt)
+    want, rows = _chunked(cass, b, prompt)
+    assert [first] == want and a.status()[0] == b.status()[0] == 0
+    for w in (0, 1, 2):
+        assert torch.equal(_activation(cass, a, w, rows), _activation(cass, b, w, rows)), w
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("hidden", [4232, 5120, 8192])
+@pytest.mark.parametrize("n", [296, 300])
+def test_norms_of_wide_rows(cass, hidden, n):
+    """Rows of more than 4096 values take two turns of the norm's threads; from 297 rows on a quarter as many."""
+    shape = synth.ModelShape(n_layers=1, hidden=hidden, n_q_heads=4, n_kv_heads=2, head_dim=64, ffn=264, vocab=512)
+    wt = synth.model_weights(shape, 10, device="cuda")
+    gw = {"layers": [cass.engine.fuse_layer_weights(lw) for lw in wt["layers"]], "embed": wt["embed"], "lm_head": wt["lm_head"],
+          "norm_final": wt["norm_final"]}
+    prompt = synth.random_prompt(n, shape.vocab, 91)
+    a, b = (cass.engine.Engine(shape, gw, max_seq=384, gamma_max=4) for _ in range(2))
+    first = a.prefill(prompt)
+    want, rows = _chunked(cass, b, prompt)
+    assert [first] == want and a.status()[0] == b.status()[0] == 0
+    for w in (0, 1, 2):
+        assert torch.equal(_activation(cass, a, w, rows), _activation(cass, b, w, rows)), w
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("heads,kv", [(8, 2), (2, 2)])
 @pytest.mark.parametrize("first,last", [(256, 300), (0, 128), (290, 300)])
 def test_scores_that_are_no_numbers(cass, heads, kv, first, last):
