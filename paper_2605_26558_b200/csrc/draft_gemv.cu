@@ -671,11 +671,14 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
     if (out != 2) return;
     cg::cluster_group cluster = cg::this_cluster();
     cluster.sync();                                     // every CTA comes here, also one that gave up
-    // One vector: by the first warp, without a loop.  (As a loop over warps it cost the instantiations for t = 0 and 4 above 52 % pruning, whose
-    // windows' code the compiler then lays out otherwise: 512 x 512 at 53 % 4.4 -> 6.1 us, 4096 x 2048 6.6 -> 8.1, 28672 x 4096 at 60 % 39.3 -> 40.9.)
-    if (done && cluster.block_rank() == 0 && (NB > 1 || threadIdx.x < 32)) {
+    // Vector b by warp b, or by the first without a loop: the same additions, but the compiler lays the walk out otherwise for either, and one
+    // vector takes the one with which its walk is faster, loop / first warp.  More than 52 % pruned: 512 x 512 at 53 % 6.2 / 4.6 us, 28672 x 4096 at
+    // 60 % 41.0 / 39.2.  Else 28672 x 4096 at t = 4 47.8 / 48.1, t = 0 49.8 / 50.3, t = 6 397 / 420, Cassandra-2 39.15 / 39.46, but t = 1 73.7 / 69.3,
+    // t = 2 93.4 / 91.3, t = 5 (30 %) 101.8 / 100.1, and 4096 x 4096 at t = 3 24.8 / 24.5.
+    constexpr bool kByWarps = NB > 1 || (!WIDE && T != 1 && T != 2 && T != 3 && T != 5);
+    if (done && cluster.block_rank() == 0 && (kByWarps || threadIdx.x < 32)) {
         const int row = (int)blockIdx.y * kRowsPerBlock + lane;
-        for (int b = NB > 1 ? (int)threadIdx.x >> 5 : 0; b < NB; b += NB > 1 ? (int)blockDim.x >> 5 : 1) {
+        for (int b = kByWarps ? (int)threadIdx.x >> 5 : 0; b < NB; b += kByWarps ? (int)blockDim.x >> 5 : 1) {
             float part[8];
 #pragma unroll
             for (int s = 0; s < 8; ++s) part[s] = *cluster.map_shared_rank(&s_sum[b][lane], min(s, n_seg - 1));
