@@ -58,14 +58,18 @@ static int make_geom(const cass_format* fmt, int rows, int cols, EncGeom* g) {
     g->n_rb = ceil_div(rows, kRowsPerBlock);
     g->n_pad = g->n_rb * kRowsPerBlock;
     g->n_prune = (int)(((long long)cols * p) / 1000);
-    // Sizes and packing by lanes (a warp's chain is long) or by warps, by the blocks of 128 columns of 32 rows there are: 104 -> 76 us by
-    // lanes for 2400 x 3000 (1800 blocks), 61 -> 56 for 900 x 8192 (1856), 79 -> 60 for 12000 x 520 (1875), but 34 and 34 for 1000 x 1000
-    // (256).  Rows of few columns take a warp little: 40 -> 52 for 5000 x 512 (628), 42 -> 54 for 9000 x 400 (1124), 88 -> 93 for
-    // 20000 x 501 (2500), 120 -> 103 for 30000 x 301 (2814).  Rows off 16-byte boundaries take lanes longer (4692 x 1184: 52, x 1185: 70), and
-    // they then lose to warps where those have a place on the chip for every superblock at once: 63 -> 70 for 4692 x 1185 (147
-    // superblocks), 75 -> 78 for 900 x 8191 (116), 65 -> 72 for 9000 x 641 (282), but 88 -> 79 for 4800 x 1185 (150), 89 -> 79 for 12000 x 513 (375).
-    const long long blocks = (long long)g->n_rb * ceil_div(g->k_pad, 128), places = kSms * (g->seg_cols > 768 ? 1 : 2);
-    g->lanes = !g->mx && t == 4 && blocks >= (g->seg_cols > 512 ? 1400 : 2600) && (cols % 8 == 0 || (long long)g->n_rb * g->n_seg > places);
+    // Sizes and packing by lanes or by warps, measured both ways (us by warps / by lanes).  By warps a superblock is a CTA's, up to one an SM with
+    // 1024 threads, then two with 512; by lanes a CTA has 2 to 16 warps, a warp's chain is long and longer for rows off 16- and 4-byte boundaries.
+    //   up to one superblock an SM: 256 x 2048 55.3 / 48.8, 1000 x 1000 38.9 / 38.9, 900 x 8190 79.8 / 73.8, but with odd columns 4700 x 1001 53.2 /
+    //     57.4, 900 x 8191 79.8 / 86.0, and in short segments 3000 x 768 38.5 / 38.9, 3000 x 512 32.8 / 34.8, 1376 x 256 26.6 / 30.7
+    //   up to two: 5000 x 512 45.0 / 38.9, 5000 x 515 55.3 / 53.2, 5200 x 641 59.4 / 57.3, 4800 x 1185 86 / 84, but 6000 x 128 36.9 / 38.9, 9000 x 257 49.2 / 53.2
+    //   more: 9600 x 64 47.1 / 40.7, 9500 x 501 65.5 / 57.3, 20000 x 512 92.2 / 69.7, 12000 x 513 88.1 / 73.7, 32000 x 512 125 / 96
+    // Rows that keep more have longer chains still: unpruned 1000 x 1024 38.9 / 49.2, 5000 x 512 43.0 / 49.2, 4096 x 4096 114.7 / 104.4, at 30 % 38.9 / 38.9,
+    // 46 / 40 and 120.6 / 100.3.  There it takes as many blocks of 128 columns as it did when lanes shared them out worse.
+    const long long n_sb = (long long)g->n_rb * g->n_seg, blocks = (long long)g->n_rb * ceil_div(g->k_pad, 128);
+    const bool many = n_sb > 2 * kSms || (n_sb > kSms ? g->seg_cols > 512 || (g->seg_cols > 256 && cols % 8 == 0) : g->seg_cols > 768 && cols % 2 == 0);
+    const bool chains = p >= 300 || (blocks >= (g->seg_cols > 512 ? 1400 : 2600) && (cols % 8 == 0 || n_sb > kSms * (g->seg_cols > 768 ? 1 : 2)));
+    g->lanes = !g->mx && t == 4 && many && chains;
     return CASS_OK;
 }
 
@@ -1091,8 +1095,8 @@ extern "C" int cass_encode_weights(const cass_format* fmt, const void* W_bf16, c
         };
         return ends % 16 == 0 ? pack(uint4{}) : ends % 4 == 0 ? pack(uint32_t{}) : pack(uint16_t{});
     }
-    // (t = 4 without lanes: few columns, or rows off 16-byte boundaries with a place for every superblock; with field places computed at run
-    // time 5000 x 512 took 44 us instead of 40, 20000 x 501 107 instead of 98, 9000 x 641 69 instead of 65)
+    // (t = 4 without lanes: see make_geom; with field places computed at run time 5000 x 512 took 44 us by warps instead of 40, 20000 x 501 107
+    // instead of 98, 9000 x 641 69 instead of 65)
     if (n_sb <= kSms) rc = g.mx ? (g.t == 4 ? launch_pack(k_pack<true, 4, 1024>, 1024) : launch_pack(k_pack<true, -1, 1024>, 1024))
                                : (g.t == 4 ? launch_pack(k_pack<false, 4, 1024>, 1024) : launch_pack(k_pack<false, -1, 1024>, 1024));
     else rc = g.mx ? (g.t == 4 ? launch_pack(k_pack<true, 4, 512>, 512) : launch_pack(k_pack<true, -1, 512>, 512))

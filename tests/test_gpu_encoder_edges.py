@@ -78,12 +78,14 @@ def test_rows_in_turn(cass, rows, cols):
 @pytest.mark.parametrize("rows,cols,p,seg,chunk", [(9000, 520, 400, 0, 0), (41601, 200, 400, 0, 0), (21000, 470, 300, 0, 0), (2410, 2569, 400, 0, 0),
                                                     (2410, 2570, 600, 0, 0), (1600, 5300, 0, 0, 0), (3000, 2056, 400, 1024, 32), (1600, 4100, 990, 0, 0),
                                                     (4801, 512, 400, 0, 0), (4737, 641, 600, 0, 0), (4801, 1300, 400, 0, 0),
-                                                    (83201, 64, 400, 0, 0), (30000, 301, 999, 0, 0), (12000, 513, 400, 0, 0), (16640, 632, 400, 256, 256)])
+                                                    (83201, 64, 400, 0, 0), (30000, 301, 999, 0, 0), (12000, 513, 400, 0, 0), (16640, 632, 400, 256, 256),
+                                                    (4737, 256, 400, 0, 0), (4737, 501, 400, 0, 0), (4736, 1025, 300, 0, 0), (4737, 1025, 300, 0, 0), (4736, 1026, 300, 0, 0),
+                                                    (6000, 512, 299, 0, 0), (9473, 65, 300, 0, 0), (40, 3000, 300, 0, 0), (9, 1032, 400, 1024, 1024)])
 def test_blobs_by_lanes(cass, rows, cols, p, seg, chunk):
-    """Matrices of so many blocks that sizes and packing go by lanes: 2 to 16 warps a superblock, rows on 16-, 4- and 2-byte
-    boundaries, chunks of few values, a last row block that is not full; rows of one value, of none, and with codes longer than a word.
-    The ninth and tenth by warps: of few columns a row, and off 16-byte boundaries.  The last four: fewer blocks of 128 columns than
-    warps, blocks that do not share out evenly, and a last segment of one."""
+    """Sizes and packing by lanes: 2 to 16 warps a superblock, rows on 16-, 4- and 2-byte boundaries, chunks of few values, a last row
+    block that is not full; rows of one value, of none, and with codes longer than a word; fewer blocks of 128 columns than warps,
+    blocks that do not share out evenly, a last segment of one.  By warps: of one and two superblocks an SM (4736 rows and more), short
+    segments, odd columns and rows that keep more than 70 %."""
     w = synth.student_t_weight(rows, cols, 2, f"lanes/{rows}x{cols}").float()
     w[1] = 0.25
     w[2] = 0.0
