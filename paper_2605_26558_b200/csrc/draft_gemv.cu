@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
         float* xs = reinterpret_cast<float*>(kCompact ? smem_raw : smem_raw + (size_t)kGemvStages * stage_bytes);
         uint32_t* lut = reinterpret_cast<uint32_t*>(kCompact ? stage0 + (size_t)kGemvStages * stage_bytes
                                                              : reinterpret_cast<uint8_t*>(xs) + (size_t)(seg_cols + kXSlack) * x_col_bytes(NB));
-        float* red = kCompact ? reinterpret_cast<float*>(stage0) : reinterpret_cast<float*>(lut + 256);      // NB = 1: [2][n_warps][32], else [NB][n_warps][32]
+        float* red = kCompact ? reinterpret_cast<float*>(stage0) : reinterpret_cast<float*>(lut + 256);      // NB = 1: [turn][n_warps][32], else [NB][n_warps][32]
         uint64_t* bar = reinterpret_cast<uint64_t*>(lut + 256 + (kCompact ? 0 : 2 * n_warps * 32));    // [kGemvStages]
         const int x_cols = kCompact ? seg_cols : seg_cols + kXSlack;
         __shared__ int s_skip[kGemvStages], s_bad;
@@ -671,10 +671,10 @@ __global__ void __launch_bounds__(1024, T == 104 && NB == 2 ? 1 : 0) k_draft_gem
     if (out != 2) return;
     cg::cluster_group cluster = cg::this_cluster();
     cluster.sync();                                     // every CTA comes here, also one that gave up
-    // Vector b by warp b, or by the first without a loop: the same additions, but the compiler lays the walk out otherwise for either, and one
-    // vector takes the one with which its walk is faster, loop / first warp.  More than 52 % pruned: 512 x 512 at 53 % 6.2 / 4.6 us, 28672 x 4096 at
-    // 60 % 41.0 / 39.2.  Else 28672 x 4096 at t = 4 47.8 / 48.1, t = 0 49.8 / 50.3, t = 6 397 / 420, Cassandra-2 39.15 / 39.46, but t = 1 73.7 / 69.3,
-    // t = 2 93.4 / 91.3, t = 5 (30 %) 101.8 / 100.1, and 4096 x 4096 at t = 3 24.8 / 24.5.
+    // Vector b by warp b, or the one vector by the first warp without a loop: the same additions, but the time of the whole kernel differs by more
+    // than they take, and each instantiation has the faster one.  Loop / first warp, more than 52 % pruned: 512 x 512 at 53 % 6.2 / 4.6 us, 28672
+    // x 4096 at 60 % 41.0 / 39.2; else 28672 x 4096 at t = 4 47.8 / 48.1, t = 0 49.8 / 50.3, t = 6 397 / 420, Cassandra-2 39.15 / 39.46, but
+    // t = 1 73.7 / 69.3, t = 2 93.4 / 91.3, t = 5 (30 %) 101.8 / 100.1, and 4096 x 4096 at t = 3 24.8 / 24.5.
     constexpr bool kByWarps = NB > 1 || (!WIDE && T != 1 && T != 2 && T != 3 && T != 5);
     if (done && cluster.block_rank() == 0 && (kByWarps || threadIdx.x < 32)) {
         const int row = (int)blockIdx.y * kRowsPerBlock + lane;

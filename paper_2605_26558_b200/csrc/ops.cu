@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(128) k_swiglu(Partials pp, uint16_t* __restric
     }
 }
 
-// The same of bf16 projections (a prefill pass), eight features a thread: two 16-byte loads under way and one store; rows of the grid are
-// taken in turn.  Four features a thread: 32 us for 1000 rows of 14336, 86 MB, 21 so.
+// The same of bf16 projections (a prefill pass), eight features of one row a thread: two 16-byte loads under way and one store.  Four
+// features a thread: 32 us for 1000 rows of 14336, 86 MB, 21 so.
 __global__ void __launch_bounds__(256) k_swiglu_rows(const uint16_t* __restrict__ gu, uint16_t* __restrict__ act, int ffn, int n_items) {
     pdl_wait();
     pdl_early<0>();

@@ -11,6 +11,7 @@
 // Bound: latency and issue (33 % of the slots with 8 warps at work): 1000 rows of 32 heads are 16 M exponentials, 28 instructions a score.
 // 1000 rows of an 8B-shaped layer, cold: 62 us; the verification kernel and its merge took 210 (two launches of the scratch's
 // room, 74 MB of partial outputs).  The heaviest CTAs first in the grid: 77 -> 62.
+// 168 registers, what ten warps leave a thread; P in two terms spills 11 words.
 #include "tc.cuh"
 #include "kernels.cuh"
 

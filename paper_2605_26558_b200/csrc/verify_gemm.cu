@@ -7,8 +7,8 @@
 // BNx64 activation tile through a ring of TMA loads (128-byte swizzle), warp 1 issues the MMAs, warps 2-5 read the
 // accumulator back and store fp32 partial sums; a second kernel adds the K ranges in fixed order.
 //
-// The issuing threads are found by elect.sync: of a thread found by its lane the compiler does not know that it is alone, and wraps
-// every issue in a loop (20 rows of two Qwen-shaped layers 558 -> 549 us).
+// The issuing threads are found by elect.sync instead of their lane's number: 20 rows of two Qwen-shaped layers 558 -> 549 us; a single
+// product of few rows is as fast either way (5 rows of 6144 x 4096 10.6 us a call).
 //
 // Row-count invariance: an accumulator column belongs to one token row, the tile shape, the K ranges and the order
 // of the MMAs depend on (n, k) only, so a row gives the same bits whether it is verified alone or with others.

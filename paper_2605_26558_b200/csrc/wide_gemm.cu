@@ -14,8 +14,9 @@
 // Bound: the tensor pipe and the steps around it.  28672 x 4096 with 1000 rows 168 us (1.40 PFLOP/s, 85 % of measured with 6.05 rounds
 // of the pairs taken as 7), four calls of the split-K kernel with their additions 501; four layers' prompt of 1000 tokens 4.28 -> 2.69 ms.
 // A stage's barriers and commit cost some 0.2 us, hence two K blocks a stage where those are small (128 rows: 4096 x 14336 140 -> 99 us;
-// at 256 rows six stages of one block are as fast), and one thread found by elect.sync issues, for which the compiler needs no loop over
-// lanes (140 -> 116 us of that).
+// at 256 rows six stages of one block are as fast), and the issuing thread is found by elect.sync instead of its lane's
+// number (140 -> 116 us of that).  Ten warps are three on one quarter of the SM, which leaves a thread 168 registers; at 256 rows the 128 sums do
+// not quite fit beside the rest (11 words spilled).
 #include "tc.cuh"
 #include "kernels.cuh"
 
