@@ -128,12 +128,12 @@ __global__ void __launch_bounds__(32 * kSplitWarps) k_split(const uint32_t* __re
 //     columns begin; each then takes the next of either, and the eight leave in one store, but for a chunk's first and last columns.
 // Kept and pruned values of a window are 64 together, so the buffer is 82 halfwords a row, whatever the matrix looks like, and 28 warps
 // fit an SM (72 registers; with 80 and 24 warps 20000 x 1528 takes 71 us instead of 64, with 64 and 32 28672 x 4096 258 instead of 217).
-// Bound: instruction issue (62 %) and the latency of a window's steps: 33 M warp instructions for 6144 x 4096 (49 M with a list of a
+// Bound: instruction issue (62 %) and the latency of a window's steps: 31 M warp instructions for 6144 x 4096 (49 M with a list of a
 // whole chunk's values, which 20 warps an SM had room for, and one row after the other with its loads).  6144 x 4096 at 40 %
-// pruning 109 -> 58 us, at 30 % 217 -> 61 (a chunk took a second turn), at 60 % 109 -> 54; 28672 x 4096 374 -> 209.
+// pruning 130 -> 56 us, at 30 % 243 -> 60 (a chunk took a second turn), at 60 % 129 -> 57; 28672 x 4096 374 -> 199.
 constexpr int kJoinWarps = 4;
-// Chunks up to which teams: as long as all have a place at once, seven CTAs an SM.  23 and 32 us with and without for 3908 x 1528 (738 chunks), 20 and 27
-// for 9000 x 600 (846), but 43 and 41 for 640 x 14336 (1120), 40 and 37 for 2171 x 4088 (1088), 76 and 61 for 5979 x 4088 (2976).
+// Chunks up to which teams: as long as all have a place at once, seven CTAs an SM.  26 and 35 us with and without for 3908 x 1528 (738 chunks), 22 and 28
+// for 9000 x 600 (846), 26 and 32 for 33000 x 256 (1032), but 45 and 40 for 640 x 14336 (1120), 43 and 36 for 2171 x 4088 (1088), 74 and 55 for 5979 x 4088 (2976).
 constexpr int kJoinTeamMax = 7 * kSms;
 // Halfwords: a row's windows begin where its output is on a 16-byte boundary, so that whatever the width eight columns leave in one store.
 // With windows from bitmap words on and one store width for the whole matrix 8987 x 4089 took 139 us instead of 86, 19995 x 4090 171 instead of 160, and
@@ -240,17 +240,22 @@ struct JoinGroups {
             used -= q;
             uv = __funnelshift_r(0u, uv, q);
         }
-        if ((int32_t)q < 0) {                                           // the codes did not fit the window: one by one
-            uint32_t ub = upos;
-            const int cnt = (int)(__ldg(rows + (bm - 32)) >> 20) - k_first;     // kept values of the segment from the chunk's first on
+        if ((int32_t)q < 0) {                                           // eight codes did not fit the window
+            // Kept values of the segment from this group on.  The last group's may be fewer than eight, and their codes there: one by one all the
+            // same, the last group of every row and segment took 4 us of a small matrix (512 x 512 19.1 -> 15.7, 256 x 4096 22.9 -> 16.8), and
+            // 6144 x 4096 62 instead of 56
+            const int cnt = (int)(__ldg(rows + (bm - 32)) >> 20) - k_first - g;
+            if (__popc(__funnelshift_l(u1, u0, upos)) < min(cnt, 8)) {  // one by one
+                uint32_t ub = upos;
 #pragma unroll 1
-            for (int i = 0; i < 8; ++i) {
-                uint32_t x = 0;
-                if (g + i < cnt) x = lut[read_unary(rows + un, ub, (uint32_t)(last + 32 - un)) & 255];
+                for (int i = 0; i < 8; ++i) {
+                    uint32_t x = 0;
+                    if (i < cnt) x = lut[read_unary(rows + un, ub, (uint32_t)(last + 32 - un)) & 255];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = i == j ? x : v[j];
+                    for (int j = 0; j < 8; ++j) v[j] = i == j ? x : v[j];
+                }
+                used = ub - upos;
             }
-            used = ub - upos;
         }
         const int was = (int)(upos >> 5);
         upos += used;
