@@ -98,6 +98,25 @@ def test_blobs_by_lanes(cass, rows, cols, p, seg, chunk):
     assert np.array_equal(got, layout.encode_weight_blob(_bits(w), act, p, 4, *((seg, chunk) if seg else ()))[0])
 
 
+@pytest.mark.parametrize("rows,cols", [(9473, 1), (9473, 2), (9473, 8), (9473, 33)])
+def test_blobs_of_next_to_no_columns_by_lanes(cass, rows, cols):
+    w = synth.student_t_weight(rows, cols, 4, f"narrow/{cols}")
+    w[1] = 0.0
+    act = (np.abs(np.random.default_rng(cols).standard_normal(cols)) + 0.05).astype(np.float32)
+    assert np.array_equal(_blob(cass, w, act, cass.default_format()), layout.encode_weight_blob(_bits(w), act, 400, 4)[0])
+
+
+@pytest.mark.parametrize("rows,cols", [(70, 2056), (4801, 512)])
+@pytest.mark.parametrize("shift", [1, 2, 4])
+def test_matrix_off_16_byte_boundaries_by_lanes(cass, rows, cols, shift):
+    w = synth.student_t_weight(rows, cols, 5, f"shift/{cols}").cuda()
+    act = (np.abs(np.random.default_rng(shift).standard_normal(cols)) + 0.05).astype(np.float32)
+    off = torch.empty(rows * cols + 8, dtype=torch.bfloat16, device="cuda")[shift: shift + rows * cols].view(rows, cols)
+    off.copy_(w)
+    fmt = cass.default_format()
+    assert np.array_equal(_blob(cass, off, act, fmt), _blob(cass, w, act, fmt))
+
+
 def test_constant_rows_and_no_pruning(cass):
     w = torch.full((40, 3000), 0.5, dtype=torch.bfloat16)
     w[7] = 0.0

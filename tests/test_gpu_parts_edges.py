@@ -79,6 +79,7 @@ def test_join_of_every_truncation(cass, rows, cols, t):
     cass.cass_encode_weights(fmt, wd, None, blob, torch.zeros(ws_bytes, dtype=torch.uint8, device="cuda"), status)
     info = cass.cass_weight_blob_info(blob)
     assert int(status.item()) == 0
+    assert info.n_rowblocks * info.n_seg * (info.seg_cols // info.chunk_cols) == (992 if rows == 992 else 1216)      # teams up to 1036
     vdata = torch.zeros(cass.cass_verification_data_bytes(info) // 4, dtype=torch.int32, device="cuda")
     cass.cass_encode_verification_data(blob, info, wd, vdata)
     _join_at_every_phase(cass, blob, info, vdata, _bits(w))
